@@ -167,6 +167,8 @@ struct fe_mesh_s {
   double* relp = nullptr;    // [ne][4]
   double* red = nullptr;     // reduction partials [RED_SLOTS]
   unsigned* red_ticket = nullptr;
+  void* xch = nullptr;       // grid exchange words of the register-resident Arnoldi steps [2][XCH_BLOCKS][BMGS_P] x 16 bytes
+  uint32_t xch_used = 0;     // grid sums issued since the exchange state was last reset
   double* scal = nullptr;    // device scalars [64]
   int* err = nullptr;        // device error word
   unsigned* bar = nullptr;   // grid reduction state [BAR_WORDS]: count, seq, slot[2] (u64); blocked-MGS seq, pub[2][8] (u64)
@@ -226,6 +228,8 @@ constexpr int SCAL_N = 64;
 constexpr int LBFGS_MAX = 1000;  // largest number of stored secant pairs
 constexpr int BMGS_P = 8;        // basis vectors per block of the blocked MGS step
 constexpr int BAR_WORDS = 64;    // u32 words of the grid reduction state
+constexpr int XCH_BLOCKS = 256;  // largest grid of the grid exchange
+constexpr int XCH_SEQ_WORD = 48; // its sequence number in the grid reduction state
 
 // Tangent values: tiles of 32 consecutive blocks, component-major inside a
 // tile.  Entry c = 3i + k of block p lives at (p / 32) 288 + 32 c + p % 32,

@@ -161,17 +161,6 @@ __device__ __forceinline__ double block_sum0(double v, double* sh) {
   return t;
 }
 
-// ---------------------------------------------------------------- persistent Arnoldi (MGS)
-// Step j.  Block b owns the contiguous slice [b*S, min((b+1)*S, n)) of every
-// vector (S = NPT*blockDim values, NPT a multiple of 3, so slices hold whole
-// nodes); w's slice lives in shared memory for the whole sweep.  For
-// i = 0..j: h_ij = <w, V_i> (warp sums -> one block barrier -> warp 0 adds the
-// warp sums and runs the grid reduction -> one block barrier), w -= h_ij V_i;
-// V_{i+1}'s slice is loaded into registers before the reduction.  Then
-// h_{j+1,j} = ||w||, V_{j+1} = w / h_{j+1,j}, optionally z = D^{-1} V_{j+1}
-// (nodal block-Jacobi, the input of the next SpMV), and block 0 applies the
-// previous Givens rotations to column j, forms the new one and updates g.
-// Rows of V have a leading dimension rounded up to 32 values (256 bytes).
 // warp 0 only: grid reduction of the block total `b` (valid in every lane);
 // publishes or waits; lane 0 leaves the total in *s_val
 __device__ __forceinline__ void grid_reduce_w0(const GridSync& gs, double* part, unsigned seq, double b, double* s_val,
@@ -209,8 +198,649 @@ __device__ __forceinline__ void grid_reduce_w0(const GridSync& gs, double* part,
   }
 }
 
+// ---------------------------------------------------------------- grid exchange
+// Grid-wide sums of the register-resident Arnoldi steps.  Every block posts
+// its P partial sums as 16-byte words {lo, tag, hi, tag} (the two halves of
+// the FP64 value, each beside the step's sequence number, so each 8-byte
+// half carries its own validity and no fence or counter is needed), and
+// every block polls the words of all blocks and adds them in block order:
+// one L2 round trip instead of the three of an arrival counter, a last
+// block's sum and a published total.  Two sets alternate by the parity of
+// the sequence number: a block posts step s + 2 only after it has read all
+// of step s + 1, which every block posts after it has read all of step s.
+// The sequence number lives in device memory across launches and grows with
+// every sum; the host resets it long before it wraps (xch_reserve).  Waits
+// are bounded as in grid_arrive's scheme (fe_set_wait_limit).
+// Measured alone (a loop of sums): 1.3 us on 16 blocks, 1.5 us on 76, 2.0 us
+// on 152 for 1 or 8 values; two levels of blocks 3.4-4.4 us, clusters with
+// distributed shared memory below the exchange 3.0-5.8 us, 4 to 16 copies of
+// the words against polling contention 2.1-2.4 us.
+struct XchSync {
+  uint4* slots;    // [2][XCH_BLOCKS][BMGS_P]
+  unsigned* seq;   // sequence number of the next sum
+  int* err;
+  unsigned limit;  // polls before a wait gives up (fe_set_wait_limit)
+};
+
+__device__ __forceinline__ uint4 ld_relaxed_v4(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed_v4(uint4* p, uint4 v) {
+  asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+               : "memory");
+}
+__device__ __forceinline__ void xch_post(uint4* p, double v, unsigned tag) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+  st_relaxed_v4(p, make_uint4((unsigned)u, tag, (unsigned)(u >> 32), tag));
+}
+// Sum of the words idx, idx + step, ... (< cnt) of a set, in that order, once
+// each carries `tag`; up to FL polls in flight.  false: a wait ran out.
+template <int FL>
+__device__ __forceinline__ bool xch_gather(const XchSync& xs, const uint4* set, int idx, int step, int cnt,
+                                           unsigned tag, double& sum) {
+  sum = 0.0;
+  for (; idx < cnt; idx += FL * step) {
+    uint4 v[FL];
+    unsigned spins = 0;
+    for (;;) {
+      bool all = true;
+#pragma unroll
+      for (int q = 0; q < FL; q++)
+        if (idx + q * step < cnt) v[q] = ld_relaxed_v4(set + idx + q * step);
+#pragma unroll
+      for (int q = 0; q < FL; q++)
+        if (idx + q * step < cnt) all = all && v[q].y == tag && v[q].w == tag;
+      if (all) break;
+      if (++spins > xs.limit || *(volatile int*)xs.err != DEV_OK) {
+        atomicCAS(xs.err, DEV_OK, DEV_ERR_TIMEOUT);
+        return false;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < FL; q++)
+      if (idx + q * step < cnt)
+        sum += __longlong_as_double((long long)(((unsigned long long)v[q].z << 32) | v[q].x));
+  }
+  return true;
+}
+
+// Warp reduce-scatter of P values per lane: returns, in every lane, the warp
+// total of value index lane / (32 / P).  Each of the first log2(P) exchange
+// steps halves the values a lane carries (it keeps the half selected by its
+// lane bit and adds the partner's copy of that half), then plain xor steps
+// finish the sum: P - 1 + 5 - log2(P) shuffles instead of 5 P.
+template <int P>
+__device__ __forceinline__ double warp_reduce_scatter(double (&v)[P], int lane) {
+#pragma unroll
+  for (int cnt = P, o = 16; cnt > 1; cnt >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < cnt / 2; k++) {
+      const double send = up ? v[k] : v[k + cnt / 2];
+      const double keep = up ? v[k + cnt / 2] : v[k];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  double t = v[0];
+#pragma unroll
+  for (int o = 16 / P; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
+}
+
+// shared memory of one Arnoldi step
+struct ArnShared {
+  double wpart[BMGS_P][16];  // block partials by warp (at most 16 warps)
+  double wsum[16][BMGS_P];   // gathered partials by warp
+  double part[512];          // one value per thread (sums of one value)
+  double h[BMGS_P];          // the last sum's results
+  double inv;                // 1 / |w|
+  double gj;                 // block 0: g_j
+  double carry;              // block 0: column j's entry above the new one after the earlier rotations
+  double trow[BMGS_P][BMGS_P];
+  double col[1024], cs[1024], sn[1024];  // block 0: column j of H and the earlier rotations
+  int fail;
+};
+
+// Grid sums of the P values in loc (every thread of the block calls it);
+// results in sh.h[0..P).  With `solve` the results are h = T_B s, the block's
+// MGS coefficients from its inner products s (sh.trow[m][l], l < m < nc: the
+// block's rows of T_B).  `last`: the step's final sum, sh.h[0] = |w| (its
+// square arrives) and sh.inv = 1 / |w|, formed by one warp (a square root and
+// a division in every warp are 25 FP64 instructions each, 1-3 us).  FL: polls
+// in flight per thread.  idle() runs in the block's last warp between the
+// post and its gather, for work that hides behind the exchange.  false: a
+// wait ran out.
+template <int P, int FL, class Idle>
+__device__ __forceinline__ bool xch_reduce(const XchSync& xs, unsigned& seq, double (&loc)[P], ArnShared& sh,
+                                           bool solve, int nc, bool last, Idle idle) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int G = gridDim.x;
+  uint4* set = xs.slots + (size_t)(seq & 1u) * XCH_BLOCKS * BMGS_P;
+  double t = 0.0;
+  if (P == 1) {
+    // one value: through shared memory, then one warp (a warp sum in every
+    // warp first would cost five more dependent FP64 steps)
+    sh.part[threadIdx.x] = loc[0];
+    __syncthreads();
+    if (wid == 0) {
+      for (int q = 0; q < nw; q++) t += sh.part[32 * q + lane];
+      t = warp_sum(t);
+      if (G > 1 && lane == 0) xch_post(set + blockIdx.x, t, seq);
+    }
+  } else {
+    const double r = warp_reduce_scatter<P>(loc, lane);
+    if ((lane & (32 / P - 1)) == 0) sh.wpart[lane / (32 / P)][wid] = r;
+    __syncthreads();
+    if (wid == 0) {
+      for (int q = lane / P; q < nw; q += 32 / P) t += sh.wpart[lane % P][q];
+#pragma unroll
+      for (int o = P; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (G > 1 && lane < P) xch_post(set + blockIdx.x * P + lane, t, seq);
+    }
+  }
+  if (wid == nw - 1) idle();
+  if (G > 1) {
+    if (P == 1) {  // few words: one warp gathers them
+      if (wid == 0) {
+        if (!xch_gather<FL>(xs, set, lane, 32, G, seq, t)) sh.fail = 1;
+        t = warp_sum(t);
+      }
+    } else {
+      double a;
+      if (!xch_gather<FL>(xs, set, threadIdx.x, blockDim.x, G * P, seq, a)) sh.fail = 1;
+#pragma unroll
+      for (int o = P; o < 32; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      if (lane < P) sh.wsum[wid][lane] = a;
+      __syncthreads();
+      if (wid == 0) {
+        t = 0.0;
+        for (int q = lane / P; q < nw; q += 32 / P) t += sh.wsum[q][lane % P];
+#pragma unroll
+        for (int o = P; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      }
+    }
+    seq++;
+  }
+  if (wid == 0) {
+    if (solve) {  // h_m = s_m + sum_{l<m} T[m][l] s_l
+      double hm = t;
+#pragma unroll
+      for (int l = 0; l < P - 1; l++) {
+        const double sl = __shfl_sync(0xffffffffu, t, l);
+        if (lane > l && lane < nc) hm += sh.trow[lane][l] * sl;
+      }
+      t = hm;
+    }
+    if (last && lane == 0) {
+      const double inv = t > 0.0 ? rsqrt(t) : 0.0;
+      if (t > 0.0) t *= inv;  // (a NaN stays a NaN)
+      sh.inv = inv;
+    }
+    if (lane < P) sh.h[lane] = t;
+  }
+  __syncthreads();
+  return sh.fail == 0;
+}
+
+// One warp of block 0: the inner products sh.col[0..j] of column j of H
+// through the j earlier rotations; leaves the last entry in sh.carry.  The
+// rotations act on the column as the recurrence c_{i+1} = -sn_i c_i + cs_i
+// h_{i+1} with R_i = cs_i c_i + sn_i h_{i+1}: a scan over affine maps, 32
+// rotations per pass, instead of one thread's chain of j dependent FP64
+// steps and loads.  It needs nothing of the step's final sum and runs while
+// that one is exchanged.
+__device__ __forceinline__ void arnoldi_rotate(ArnShared& sh, int j, double* __restrict__ Hcol) {
+  const int lane = threadIdx.x & 31;
+  double carry = sh.col[0];
+  for (int b = 0; b < j; b += 32) {
+    const int i = b + lane;
+    const bool in = i < j;
+    const double c = in ? sh.cs[i] : 0.0, s = in ? sh.sn[i] : 0.0, h1 = in ? sh.col[i + 1] : 0.0;
+    double A = -s, B = c * h1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double Ap = __shfl_up_sync(0xffffffffu, A, o), Bp = __shfl_up_sync(0xffffffffu, B, o);
+      if (lane >= o) {
+        B += A * Bp;
+        A *= Ap;
+      }
+    }
+    const double next = A * carry + B;  // c_{i+1}
+    double ci = __shfl_up_sync(0xffffffffu, next, 1);
+    if (lane == 0) ci = carry;
+    if (in) Hcol[i] = c * ci + s * h1;
+    carry = __shfl_sync(0xffffffffu, next, min(31, j - 1 - b));
+  }
+  if (lane == 0) sh.carry = carry;
+}
+
+// Block 0, warp 0: the new rotation, the rotated right-hand side and the
+// stopping test.
+__device__ __forceinline__ void arnoldi_givens(const ArnShared& sh, int j, double hn,
+                                               double* __restrict__ Hcol, double* __restrict__ cs,
+                                               double* __restrict__ sn, double* __restrict__ g,
+                                               double* __restrict__ out, double target, int kmax, int it0, int max_it) {
+  const int lane = threadIdx.x & 31;
+  const double a = sh.carry, c = hn, gj = sh.gj;
+  const double r = hypot(a, c);
+  const double q = (lane == 0 ? a : c) / r;  // lane 0: the cosine, lane 1: the sine
+  const double sj = __shfl_sync(0xffffffffu, q, 1);
+  if (lane == 0) {
+    cs[j] = q;
+    sn[j] = sj;
+    Hcol[j] = r;
+    Hcol[j + 1] = 0.0;
+    g[j + 1] = -sj * gj;
+    g[j] = q * gj;
+    const double res = fabs(sj * gj);
+    out[0] = res;
+    out[1] = hn;
+    out[8] = (double)(j + 1);  // steps completed in this cycle
+    if (!(res > target) || hn == 0.0 || j + 1 >= kmax || it0 + j + 1 >= max_it) out[7] = 1.0;
+  }
+}
+
+__device__ __forceinline__ void prefetch_l2(const double* p, int64_t count) {
+  // bulk L2 prefetch of a 16-byte aligned run (rows of V are 256-byte aligned
+  // and zero-padded, so rounding the size up stays inside the row)
+  const uint32_t bytes = (uint32_t)(((count * 8) + 15) & ~(int64_t)15);
+  if (bytes) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
+// A thread owns NPT / 2 pairs of consecutive values of its block's slice:
+// values s = 2q, 2q + 1 sit at slice offset bm_off(q) and bm_off(q) + 1, so
+// each pair is one 16-byte load (slices start at even offsets of 256-byte
+// aligned rows).
+__device__ __forceinline__ int64_t bm_off(int q) { return 2 * (threadIdx.x + (int64_t)q * blockDim.x); }
+
+// this thread's NPT values of a vector slice (0 past its end)
+template <int NPT>
+__device__ __forceinline__ void load_slice(double (&r)[NPT], const double* __restrict__ v, int64_t len) {
+#pragma unroll
+  for (int q = 0; q < NPT / 2; q++) {
+    const int64_t k = bm_off(q);
+    if (k + 1 < len) {
+      const double2 p = __ldcg(reinterpret_cast<const double2*>(v + k));
+      r[2 * q] = p.x;
+      r[2 * q + 1] = p.y;
+    } else {
+      r[2 * q] = k < len ? __ldcg(v + k) : 0.0;
+      r[2 * q + 1] = 0.0;
+    }
+  }
+}
+
+// The tail of a step: V_{j+1} = w / |w|, optionally z = D^{-1} V_{j+1} (nodal
+// block-Jacobi, the input of the next SpMV; through the slice's copy in
+// shared memory, slices hold whole nodes).
 template <int NPT, class DT, class ZT>
-__global__ void __launch_bounds__(NPT <= 6 ? 1024 : (NPT <= 12 ? 512 : 256))
+__device__ __forceinline__ void arnoldi_tail(const double (&wr)[NPT], double inv, double* ws, double* vnx, int64_t base,
+                                             int64_t len, const DT* __restrict__ Dinv, ZT* __restrict__ z) {
+#pragma unroll
+  for (int q = 0; q < NPT / 2; q++) {
+    const int64_t k = bm_off(q);
+    const double v0 = wr[2 * q] * inv, v1 = wr[2 * q + 1] * inv;
+    if (z) {
+      ws[k] = v0;
+      ws[k + 1] = v1;
+    }
+    if (k + 1 < len) *reinterpret_cast<double2*>(vnx + k) = make_double2(v0, v1);
+    else if (k < len) vnx[k] = v0;
+  }
+  if (!z) return;
+  __syncthreads();
+  for (int64_t a = threadIdx.x; a < len / 3; a += blockDim.x) {
+    const DT* D = Dinv + ((base / 3) + a) * 9;
+    const double x0 = ws[3 * a], x1 = ws[3 * a + 1], x2 = ws[3 * a + 2];
+    ZT* zo = z + base + 3 * a;
+    if constexpr (sizeof(DT) == 8) {
+      zo[0] = (ZT)(D[0] * x0 + D[1] * x1 + D[2] * x2);
+      zo[1] = (ZT)(D[3] * x0 + D[4] * x1 + D[5] * x2);
+      zo[2] = (ZT)(D[6] * x0 + D[7] * x1 + D[8] * x2);
+    } else {
+      const float f0 = (float)x0, f1 = (float)x1, f2 = (float)x2;
+      zo[0] = (ZT)(D[0] * f0 + D[1] * f1 + D[2] * f2);
+      zo[1] = (ZT)(D[3] * f0 + D[4] * f1 + D[5] * f2);
+      zo[2] = (ZT)(D[6] * f0 + D[7] * f1 + D[8] * f2);
+    }
+  }
+}
+
+// block 0 at the end of a step: the new rotation and, in the last warp, the
+// new row of T_B (blocked form, ng > 0)
+//   T[j+1][c] = -(g_c + sum_{c<l<ng} g_l T[b0+l][c]), g_l = <v_{j+1}, v_{b0+l}>
+__device__ __forceinline__ void arnoldi_finish(ArnShared& sh, int j, int ng, double hn,
+                                               double* __restrict__ T, double* __restrict__ Hcol,
+                                               double* __restrict__ cs, double* __restrict__ sn,
+                                               double* __restrict__ g, double* __restrict__ out, double target,
+                                               int kmax, int it0, int max_it) {
+  if (blockIdx.x != 0) return;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (wid == (int)(blockDim.x >> 5) - 1 && hn > 0.0 && lane < ng) {
+    const int c = lane, b0 = j / BMGS_P * BMGS_P;
+    double acc = sh.h[1 + c] * sh.inv;
+    for (int l = c + 1; l < ng; l++) acc += sh.h[1 + l] * sh.inv * T[(int64_t)(b0 + l) * BMGS_P + c];
+    T[(int64_t)(j + 1) * BMGS_P + c] = -acc;
+  }
+  if (wid == 0) arnoldi_givens(sh, j, hn, Hcol, cs, sn, g, out, target, kmax, it0, max_it);
+}
+
+// ---------------------------------------------------------------- persistent Arnoldi step, block in registers
+// Step j for vectors whose slices are short (at most 6 values per thread of
+// 256): block b of the grid owns the slice [b S, min((b+1) S, n)) of every
+// vector, S a multiple of 6 (whole nodes, 16-byte pairs).  The basis is taken
+// in blocks of 8 vectors whose slices sit in registers, so each basis value
+// is loaded once per step and the next block's loads are in flight during
+// the current block's grid sum.
+//
+// Blocked form (SEQ false): modified Gram-Schmidt over the basis in blocks of
+// P vectors.  Inside a block the sequential MGS coefficients follow from the
+// block's inner products with the current w and from its own Gram entries:
+//   <w - sum_{l<m} h_l v_l, v_m> = <w, v_m> - sum_{l<m} h_l <v_l, v_m>,
+// i.e. h_B = (I + L_B)^{-1} V_B^T w with L_B the strictly lower triangle of
+// V_B^T V_B (the compact-WY identity of the low-synchronisation step, applied
+// per block; equal to the MGS coefficients in exact arithmetic).  Between
+// blocks w is updated before the next block's inner products, as in MGS.  The
+// entries <v_{j+1}, v_l>, v_l in the block of v_{j+1}, are summed together
+// with ||w||^2 at the end of step j, and the new row of T_B = (I + L_B)^{-1}
+// is stored, so step j takes ceil((j+1)/P) + 1 grid sums instead of j + 2.
+//
+// Sequential form (SEQ): for i = 0..j: h_ij = <w, V_i>, w -= h_ij V_i, one
+// grid sum each.
+//
+// Then h_{j+1,j} = ||w||, V_{j+1} = w / h_{j+1,j}, z, and block 0 applies the
+// rotations.
+//
+// GB300 issues about two FP64 lane-operations per clock per SM, so a step
+// costs 2 (j+1) n / grid FP64 cycles plus its grid sums: the slice is spread
+// over every SM as soon as the vector is longer than a few hundred values
+// (launch_arnoldi_new), with only as many threads as the slice has values
+// for (idle lanes of a warp cost FP64 issue like busy ones, and so does every
+// step of a warp sum: one FP64 warp instruction holds its SM quarter 64
+// cycles, dependent or not).
+//
+// Measured per launch (before: slices of 6,144 values in shared memory or
+// registers on as few blocks as hold the vector): blocked, 94,800 unknowns,
+// j < 16: 88 -> 28 us; sequential, 178,689 unknowns, j = 24: 173 -> 101 us;
+// sequential, 729 unknowns, j = 95: 402 -> 125 us.
+template <int NPT, bool SEQ, class DT, class ZT>
+__global__ void __launch_bounds__(256)
+    k_arnoldi_reg(int64_t n, int64_t S, int j, double* __restrict__ V, int64_t ldv, const double* __restrict__ w,
+                  double* __restrict__ Hcol, XchSync xs, double* __restrict__ T, double* __restrict__ cs,
+                  double* __restrict__ sn, double* __restrict__ g, double* __restrict__ out,
+                  const DT* __restrict__ Dinv, ZT* __restrict__ z, double target, int kmax, int it0, int max_it) {
+  constexpr int P = BMGS_P;
+  extern __shared__ __align__(16) double ws[];
+  __shared__ ArnShared sh;
+  // speculative batches: a step queued after the cycle ended does nothing
+  // (checked once the first loads are in flight)
+  const double stop = *(volatile double*)(out + 7);
+  unsigned seq = *(volatile unsigned*)xs.seq;  // no sum completes before every block has read it
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t base = (int64_t)blockIdx.x * S;
+  const int64_t len = n - base < S ? n - base : S;
+  const int nb = j / P + 1;                     // blocks of the basis v_0..v_j
+  const int nlast = j + 1 - (nb - 1) * P;       // vectors in the last block
+  const int ng = SEQ || (j + 1) % P == 0 ? 0 : nlast;  // Gram entries of v_{j+1} (its block is the last one)
+  if (threadIdx.x == 0) sh.fail = 0;
+  if (blockIdx.x == 0) {
+    if (threadIdx.x == 0) sh.gj = g[j];
+    for (int i = threadIdx.x; i < j; i += blockDim.x) {
+      sh.cs[i] = cs[i];
+      sh.sn[i] = sn[i];
+    }
+  }
+  double wr[NPT], cur[P][NPT], nxt[P][NPT];
+  load_slice<NPT>(wr, w + base, len);
+#pragma unroll
+  for (int m = 0; m < P; m++) load_slice<NPT>(cur[m], V + (int64_t)m * ldv + base, m <= j ? len : 0);
+#pragma unroll
+  for (int m = 0; m < P; m++)
+#pragma unroll
+    for (int s = 0; s < NPT; s++) nxt[m][s] = 0.0;
+  if (stop != 0.0) return;
+  __syncthreads();
+  auto none = [] {};
+  auto rotate = [&] {
+    if (blockIdx.x == 0) arnoldi_rotate(sh, j, Hcol);
+  };
+  for (int kb = 0; kb < nb; kb++) {
+    const int nc = kb == nb - 1 ? nlast : P;
+    if (SEQ) {
+      if (kb + 1 < nb)
+#pragma unroll
+        for (int m = 0; m < P; m++)
+          load_slice<NPT>(nxt[m], V + (int64_t)((kb + 1) * P + m) * ldv + base, (kb + 1) * P + m <= j ? len : 0);
+#pragma unroll
+      for (int m = 0; m < P; m++)
+        if (m < nc) {
+          double a[1] = {0.0};
+#pragma unroll
+          for (int s = 0; s < NPT; s++) a[0] += wr[s] * cur[m][s];
+          if (!xch_reduce<1, 5>(xs, seq, a, sh, false, 0, false, none)) return;
+          const double h = sh.h[0];
+          if (blockIdx.x == 0 && threadIdx.x == 0) sh.col[kb * P + m] = h;
+#pragma unroll
+          for (int s = 0; s < NPT; s++) wr[s] -= h * cur[m][s];
+        }
+    } else {
+      double loc[P];
+#pragma unroll
+      for (int m = 0; m < P; m++) {
+        loc[m] = 0.0;
+#pragma unroll
+        for (int s = 0; s < NPT; s++) loc[m] += wr[s] * cur[m][s];
+      }
+      if (kb + 1 < nb)
+#pragma unroll
+        for (int m = 0; m < P; m++)
+          load_slice<NPT>(nxt[m], V + (int64_t)((kb + 1) * P + m) * ldv + base, (kb + 1) * P + m <= j ? len : 0);
+      if (wid == 0 && lane < nc) {  // T rows of the block (lane m: row kb P + m, entries l < m)
+        const double* tr = T + (int64_t)(kb * P + lane) * P;
+#pragma unroll
+        for (int l = 0; l < P - 1; l++)
+          if (l < lane) sh.trow[lane][l] = tr[l];
+      }
+      if (!xch_reduce<P, 5>(xs, seq, loc, sh, true, nc, false, none)) return;
+      if (blockIdx.x == 0 && (int)threadIdx.x < nc) sh.col[kb * P + threadIdx.x] = sh.h[threadIdx.x];
+#pragma unroll
+      for (int m = 0; m < P; m++) {
+        const double h = m < nc ? sh.h[m] : 0.0;
+#pragma unroll
+        for (int s = 0; s < NPT; s++) wr[s] -= h * cur[m][s];
+      }
+    }
+    if (kb + 1 < nb)
+#pragma unroll
+      for (int m = 0; m < P; m++)
+#pragma unroll
+        for (int s = 0; s < NPT; s++) cur[m][s] = nxt[m][s];
+  }
+  // final sum: ||w||^2 and, in the blocked form, the Gram row against the last block
+  if (SEQ) {
+    double a[1] = {0.0};
+#pragma unroll
+    for (int s = 0; s < NPT; s++) a[0] += wr[s] * wr[s];
+    if (!xch_reduce<1, 5>(xs, seq, a, sh, false, 0, true, rotate)) return;
+  } else {
+    double loc[P];
+#pragma unroll
+    for (int m = 0; m < P; m++) {
+      loc[m] = 0.0;
+      if (m == 0 || m - 1 < ng)
+#pragma unroll
+        for (int s = 0; s < NPT; s++) loc[m] += wr[s] * (m == 0 ? wr[s] : cur[m > 0 ? m - 1 : 0][s]);
+    }
+    if (!xch_reduce<P, 5>(xs, seq, loc, sh, false, 0, true, rotate)) return;
+  }
+  const double hn = sh.h[0];
+  if (blockIdx.x == 0 && threadIdx.x == 0) *(volatile unsigned*)xs.seq = seq;
+  if (hn > 0.0) arnoldi_tail<NPT, DT, ZT>(wr, sh.inv, ws, V + (int64_t)(j + 1) * ldv + base, base, len, Dinv, z);
+  arnoldi_finish(sh, j, ng, hn, T, Hcol, cs, sn, g, out, target, kmax, it0, max_it);
+}
+
+// ---------------------------------------------------------------- persistent Arnoldi step, long slices
+// The same step for slices of up to 12 values per thread of 512 (6,144 per
+// block, 152 x 6,144 = 933,888 unknowns with one block per SM): w stays in
+// registers; each sweep applies the previous block's update and accumulates
+// the current block's inner products, one vector per pass, with the next
+// pass's vector loaded while the current one is used (a block's second pass
+// over its vectors reads L2).  SEQ: one vector per pass, inner product, grid
+// sum, update.
+template <int NPT, bool SEQ, class DT, class ZT>
+__global__ void __launch_bounds__(512)
+    k_arnoldi_bm(int64_t n, int64_t S, int j, double* __restrict__ V, int64_t ldv, const double* __restrict__ w,
+                 double* __restrict__ Hcol, XchSync xs, double* __restrict__ T, double* __restrict__ cs,
+                 double* __restrict__ sn, double* __restrict__ g, double* __restrict__ out,
+                 const DT* __restrict__ Dinv, ZT* __restrict__ z, double target, int kmax, int it0, int max_it) {
+  constexpr int P = BMGS_P;
+  extern __shared__ __align__(16) double ws[];
+  __shared__ ArnShared sh;
+  const double stop = *(volatile double*)(out + 7);  // a step queued after the cycle ended does nothing
+  unsigned seq = *(volatile unsigned*)xs.seq;  // no sum completes before every block has read it
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t base = (int64_t)blockIdx.x * S;
+  const int64_t len = n - base < S ? n - base : S;
+  const int nb = j / P + 1;                // blocks of the basis v_0..v_j
+  const int nlast = j + 1 - (nb - 1) * P;  // vectors in the last block
+  const int ng = SEQ || (j + 1) % P == 0 ? 0 : nlast;  // Gram entries of v_{j+1} (its block is the last one)
+  if (threadIdx.x == 0) sh.fail = 0;
+  if (threadIdx.x < P) sh.h[threadIdx.x] = 0.0;
+  if (threadIdx.x < P && (int)threadIdx.x <= j) prefetch_l2(V + (int64_t)threadIdx.x * ldv + base, len);
+  if (blockIdx.x == 0) {
+    if (threadIdx.x == 0) sh.gj = g[j];
+    for (int i = threadIdx.x; i < j; i += blockDim.x) {
+      sh.cs[i] = cs[i];
+      sh.sn[i] = sn[i];
+    }
+  }
+  double wr[NPT];
+  load_slice<NPT>(wr, w + base, len);
+  double cur[NPT], nxt[NPT];
+#pragma unroll
+  for (int s = 0; s < NPT; s++) nxt[s] = 0.0;
+  load_slice<NPT>(cur, V + base, len);  // first pass: the inner product with v_0
+  if (stop != 0.0) return;
+  __syncthreads();
+  auto none = [] {};
+  auto rotate = [&] {
+    if (blockIdx.x == 0) arnoldi_rotate(sh, j, Hcol);
+  };
+  if (SEQ) {
+    for (int i = 0; i <= j; i++) {
+      double a[1] = {0.0};
+      double b = 0.0;
+#pragma unroll
+      for (int s = 0; s < NPT; s += 2) {
+        a[0] += wr[s] * cur[s];
+        b += wr[s + 1] * cur[s + 1];
+      }
+      a[0] += b;
+      if (i < j) load_slice<NPT>(nxt, V + (int64_t)(i + 1) * ldv + base, len);
+      if (i + P <= j && threadIdx.x == 0) prefetch_l2(V + (int64_t)(i + P) * ldv + base, len);
+      if (!xch_reduce<1, 3>(xs, seq, a, sh, false, 0, false, none)) return;
+      const double h = sh.h[0];
+      if (blockIdx.x == 0 && threadIdx.x == 0) sh.col[i] = h;
+#pragma unroll
+      for (int s = 0; s < NPT; s++) {
+        wr[s] -= h * cur[s];
+        cur[s] = nxt[s];
+      }
+    }
+    double a[1] = {0.0};
+#pragma unroll
+    for (int s = 0; s < NPT; s++) a[0] += wr[s] * wr[s];
+    if (!xch_reduce<1, 3>(xs, seq, a, sh, false, 0, true, rotate)) return;
+  } else {
+    for (int kb = 0; kb <= nb; kb++) {
+      const int np = kb == 0 ? 0 : (kb == nb ? nlast : P);        // previous block: update
+      const int nc = kb == nb ? ng : (kb == nb - 1 ? nlast : P);  // current block (final sweep: Gram row)
+      const double* Vp = V + (int64_t)(kb > 0 ? kb - 1 : 0) * P * ldv + base;
+      const double* Vc = kb < nb ? V + (int64_t)kb * P * ldv + base : Vp;
+      // Passes over one vector each: np update passes (w -= h_m v_m, block B-1),
+      // then nc inner-product passes (block B; final sweep: the Gram row against
+      // block B-1).  The slice of the next pass's vector is loaded into registers
+      // while the current one is used.
+      const int nq = np + nc;
+#pragma unroll
+      for (int m = 0; m < P; m++) {
+        if (m < np) {
+          if (m + 1 < nq) load_slice<NPT>(nxt, m + 1 < np ? Vp + (int64_t)(m + 1) * ldv : Vc, len);
+          const double h = sh.h[m];
+#pragma unroll
+          for (int s = 0; s < NPT; s++) wr[s] -= h * cur[s];
+#pragma unroll
+          for (int s = 0; s < NPT; s++) cur[s] = nxt[s];
+        }
+      }
+      double loc[P];
+#pragma unroll
+      for (int m = 0; m < P; m++) loc[m] = 0.0;
+#pragma unroll
+      for (int m = 0; m < P; m++) {
+        if (m < nc) {
+          if (m + 1 < nc) load_slice<NPT>(nxt, Vc + (int64_t)(m + 1) * ldv, len);
+          double a[2] = {0.0, 0.0};  // two chains: each extra one costs an FP64 add per vector
+#pragma unroll
+          for (int s = 0; s < NPT; s++) a[s & 1] += wr[s] * cur[s];
+          loc[m] = a[0] + a[1];
+#pragma unroll
+          for (int s = 0; s < NPT; s++) cur[s] = nxt[s];
+        }
+      }
+      if (kb == nb) {  // final sweep: [||w||^2, Gram row]
+        double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+        for (int s = 0; s < NPT; s++) a[s & 3] += wr[s] * wr[s];
+#pragma unroll
+        for (int m = P - 1; m > 0; m--) loc[m] = loc[m - 1];
+        loc[0] = (a[0] + a[1]) + (a[2] + a[3]);
+      } else {
+        // first pass of the next sweep: the update with this block's v_{kb P}
+        load_slice<NPT>(cur, V + (int64_t)kb * P * ldv + base, len);
+      }
+      // the next block's vectors are read from HBM by the next sweep: start them now
+      if (kb + 1 < nb && threadIdx.x < P && (kb + 1) * P + (int)threadIdx.x <= j)
+        prefetch_l2(V + (int64_t)((kb + 1) * P + threadIdx.x) * ldv + base, len);
+      // T rows of the current block (lane m: row kb P + m, entries l < m)
+      const bool solve = kb < nb;
+      if (wid == 0 && solve && lane < nc) {
+        const double* tr = T + (int64_t)(kb * P + lane) * P;
+#pragma unroll
+        for (int l = 0; l < P - 1; l++)
+          if (l < lane) sh.trow[lane][l] = tr[l];
+      }
+      auto rotate_last = [&] {
+        if (kb == nb) rotate();
+      };
+      if (!xch_reduce<P, 3>(xs, seq, loc, sh, solve, nc, !solve, rotate_last)) return;
+      if (solve && blockIdx.x == 0 && (int)threadIdx.x < nc) sh.col[kb * P + threadIdx.x] = sh.h[threadIdx.x];
+    }
+  }
+  // sh.h[0] = ||w||, sh.h[1..ng] = <w, v_l> for the last block's vectors
+  const double hn = sh.h[0];
+  if (blockIdx.x == 0 && threadIdx.x == 0) *(volatile unsigned*)xs.seq = seq;
+  if (hn > 0.0) arnoldi_tail<NPT, DT, ZT>(wr, sh.inv, ws, V + (int64_t)(j + 1) * ldv + base, base, len, Dinv, z);
+  arnoldi_finish(sh, j, ng, hn, T, Hcol, cs, sn, g, out, target, kmax, it0, max_it);
+}
+
+// ---------------------------------------------------------------- persistent Arnoldi (MGS), longest vectors
+// Sequential sweep for vectors beyond one register-resident block per SM.
+// Step j.  Block b owns the contiguous slice [b*S, min((b+1)*S, n)) of every
+// vector (S = NPT*blockDim values, NPT a multiple of 3, so slices hold whole
+// nodes), several blocks per SM; w's slice lives in shared memory for the
+// whole sweep.  For i = 0..j: h_ij = <w, V_i> (warp sums -> one block barrier
+// -> warp 0 adds the warp sums and runs the grid reduction -> one block
+// barrier), w -= h_ij V_i; V_{i+1}'s slice is loaded into registers before
+// the reduction.  The rest of the step as in k_arnoldi_reg, the rotations by
+// one thread.
+template <int NPT, class DT, class ZT>
+__global__ void __launch_bounds__(256)
     k_arnoldi(int64_t n, int j, double* __restrict__ V, int64_t ldv, const double* __restrict__ w,
               double* __restrict__ Hcol, double* part, GridSync gs,
               double* __restrict__ cs, double* __restrict__ sn, double* __restrict__ g, double* __restrict__ out,
@@ -527,27 +1157,12 @@ __global__ void __launch_bounds__(NPT <= 6 ? 1024 : (NPT <= 12 ? 512 : 256))
   }
 }
 
-// ---------------------------------------------------------------- blocked MGS step
-// Modified Gram-Schmidt over the basis in blocks of P vectors.  Inside a
-// block the sequential MGS coefficients follow from the block's inner
-// products with the current w and from the block's own Gram entries:
-//   <w - sum_{l<m} h_l v_l, v_m> = <w, v_m> - sum_{l<m} h_l <v_l, v_m>,
-// i.e. h_B = (I + L_B)^{-1} V_B^T w with L_B the strictly lower triangle of
-// V_B^T V_B (the compact-WY identity of the low-synchronisation step,
-// applied per block; equal to the MGS coefficients in exact arithmetic, the
-// sequential MGS sweep for P = 1).  Between blocks w is updated before the
-// next block's inner products, as in MGS.  The entries <v_{j+1}, v_l>, v_l in
-// the block of v_{j+1}, are reduced together with ||w||^2 at the end of step
-// j, and the new row of T_B = (I + L_B)^{-1} is stored, so step j takes
-// ceil((j+1)/P) + 1 grid reductions instead of j + 2, at the same 2 FMAs per
-// entry and basis vector (plus at most P - 1 inner products for the Gram
-// row).  w stays in registers; each sweep applies the previous block's
-// update and accumulates the current block's inner products, one vector per
-// pass, with the next pass's vector loaded while the current one is used.
-//
-// The reductions have their own step sequence and two sets of P published
-// slots (bar[6], bar[8..]) so that other persistent kernels' use of the
-// shared slots cannot leave a stale value in a slot this kernel polls.
+// ---------------------------------------------------------------- blocked MGS step, longest vectors
+// The blocked form for vectors too long for one register-resident block per
+// SM.  Its reductions (the arrival counter and published totals described
+// above) have their own step sequence and two sets of P published slots
+// (bar[6], bar[8..]) so that other persistent kernels' use of the shared
+// slots cannot leave a stale value in a slot this kernel polls.
 struct BlockSync {
   unsigned* count;           // arrival counter (shared with GridSync)
   unsigned* seq;             // this kernel's step sequence
@@ -555,29 +1170,6 @@ struct BlockSync {
   int* err;
   unsigned limit;            // polls before a wait gives up (fe_set_wait_limit)
 };
-
-// Warp reduce-scatter of P values per lane: returns, in every lane, the warp
-// total of value index lane / (32 / P).  Each of the first log2(P) exchange
-// steps halves the values a lane carries (it keeps the half selected by its
-// lane bit and adds the partner's copy of that half), then plain xor steps
-// finish the sum: P - 1 + 5 - log2(P) shuffles instead of 5 P.
-template <int P>
-__device__ __forceinline__ double warp_reduce_scatter(double (&v)[P], int lane) {
-#pragma unroll
-  for (int cnt = P, o = 16; cnt > 1; cnt >>= 1, o >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int k = 0; k < cnt / 2; k++) {
-      const double send = up ? v[k] : v[k + cnt / 2];
-      const double keep = up ? v[k + cnt / 2] : v[k];
-      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-  double t = v[0];
-#pragma unroll
-  for (int o = 16 / P; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  return t;
-}
 
 // warp 0 of every block.  Lane l holds the block total of value l % P.  The
 // last block to arrive adds the partials of all blocks in block order, and
@@ -638,205 +1230,8 @@ __device__ __forceinline__ bool bm_reduce_w0(const BlockSync& bs, double* part, 
   return true;
 }
 
-__device__ __forceinline__ void prefetch_l2(const double* p, int64_t count) {
-  // bulk L2 prefetch of a 16-byte aligned run (rows of V are 256-byte aligned
-  // and zero-padded, so rounding the size up stays inside the row)
-  const uint32_t bytes = (uint32_t)(((count * 8) + 15) & ~(int64_t)15);
-  if (bytes) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
-// A thread owns NPT / 2 pairs of consecutive values of its block's slice:
-// values s = 2q, 2q + 1 sit at slice offset bm_off(q) and bm_off(q) + 1, so
-// each pair is one 16-byte load (slices start at even offsets of 256-byte
-// aligned rows).
-__device__ __forceinline__ int64_t bm_off(int q) { return 2 * (threadIdx.x + (int64_t)q * blockDim.x); }
-
-// this thread's NPT values of a vector slice (0 past its end)
-template <int NPT>
-__device__ __forceinline__ void load_slice(double (&r)[NPT], const double* __restrict__ v, int64_t len) {
-#pragma unroll
-  for (int q = 0; q < NPT / 2; q++) {
-    const int64_t k = bm_off(q);
-    if (k + 1 < len) {
-      const double2 p = __ldcg(reinterpret_cast<const double2*>(v + k));
-      r[2 * q] = p.x;
-      r[2 * q + 1] = p.y;
-    } else {
-      r[2 * q] = k < len ? __ldcg(v + k) : 0.0;
-      r[2 * q + 1] = 0.0;
-    }
-  }
-}
-
-template <int NPT, int P, class DT, class ZT>
-__global__ void __launch_bounds__(NPT <= 12 ? 512 : 256)
-    k_arnoldi_bm(int64_t n, int j, double* __restrict__ V, int64_t ldv, const double* __restrict__ w,
-                 double* __restrict__ Hcol, double* part, BlockSync bs, double* __restrict__ T,
-                 double* __restrict__ cs, double* __restrict__ sn, double* __restrict__ g, double* __restrict__ out,
-                 const DT* __restrict__ Dinv, ZT* __restrict__ z, double target, int kmax, int it0, int max_it) {
-  static_assert(P == 2 || P == 4 || P == 8, "block of 2, 4 or 8 basis vectors");
-  extern __shared__ __align__(16) double ws[];
-  __shared__ double wpart[P][32];
-  __shared__ double s_h[P];       // the last reduction's results (h of the block, or the final norm/Gram row)
-  __shared__ double s_trow[P][P];
-  __shared__ int s_fail;
-  if (*(volatile double*)(out + 7) != 0.0) return;
-  unsigned seq = *(volatile unsigned*)bs.seq;  // no reduction completes before every block has read it
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int64_t S = (int64_t)NPT * blockDim.x;
-  const int64_t base = (int64_t)blockIdx.x * S;
-  const int64_t len = n - base < S ? n - base : S;
-  const int nb = j / P + 1;                // blocks of the basis v_0..v_j
-  const int nlast = j + 1 - (nb - 1) * P;  // vectors in the last block
-  const int ng = (j + 1) % P ? nlast : 0;  // Gram entries of v_{j+1} (its block is the last one)
-  if (threadIdx.x == 0) s_fail = 0;
-  if (threadIdx.x < P) s_h[threadIdx.x] = 0.0;
-  if (threadIdx.x < P && (int)threadIdx.x <= j) prefetch_l2(V + (int64_t)threadIdx.x * ldv + base, len);
-  double wr[NPT];
-  load_slice<NPT>(wr, w + base, len);
-  double cur[NPT], nxt[NPT];
-#pragma unroll
-  for (int s = 0; s < NPT; s++) nxt[s] = 0.0;
-  load_slice<NPT>(cur, V + base, len);  // first pass: the inner product with v_0
-  for (int kb = 0; kb <= nb; kb++) {
-    const int np = kb == 0 ? 0 : (kb == nb ? nlast : P);        // previous block: update
-    const int nc = kb == nb ? ng : (kb == nb - 1 ? nlast : P);  // current block (final sweep: Gram row)
-    const double* Vp = V + (int64_t)(kb > 0 ? kb - 1 : 0) * P * ldv + base;
-    const double* Vc = kb < nb ? V + (int64_t)kb * P * ldv + base : Vp;
-    // Passes over one vector each: np update passes (w -= h_m v_m, block B-1),
-    // then nc inner-product passes (block B; final sweep: the Gram row against
-    // block B-1).  The slice of the next pass's vector is loaded into registers
-    // while the current one is used.
-    const int nq = np + nc;
-#pragma unroll
-    for (int m = 0; m < P; m++) {
-      if (m < np) {
-        if (m + 1 < nq) load_slice<NPT>(nxt, m + 1 < np ? Vp + (int64_t)(m + 1) * ldv : Vc, len);
-        const double h = s_h[m];
-#pragma unroll
-        for (int s = 0; s < NPT; s++) wr[s] -= h * cur[s];
-#pragma unroll
-        for (int s = 0; s < NPT; s++) cur[s] = nxt[s];
-      }
-    }
-    double loc[P];
-#pragma unroll
-    for (int m = 0; m < P; m++) loc[m] = 0.0;
-#pragma unroll
-    for (int m = 0; m < P; m++) {
-      if (m < nc) {
-        if (m + 1 < nc) load_slice<NPT>(nxt, Vc + (int64_t)(m + 1) * ldv, len);
-        double a[2] = {0.0, 0.0};  // two chains: each extra one costs an FP64 add per vector
-#pragma unroll
-        for (int s = 0; s < NPT; s++) a[s & 1] += wr[s] * cur[s];
-        loc[m] = a[0] + a[1];
-#pragma unroll
-        for (int s = 0; s < NPT; s++) cur[s] = nxt[s];
-      }
-    }
-    if (kb == nb) {  // final sweep: [||w||^2, Gram row]
-      double a[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-      for (int s = 0; s < NPT; s++) a[s & 3] += wr[s] * wr[s];
-#pragma unroll
-      for (int m = P - 1; m > 0; m--) loc[m] = loc[m - 1];
-      loc[0] = (a[0] + a[1]) + (a[2] + a[3]);
-    } else {
-      // first pass of the next sweep: the update with this block's v_{kb P}
-      load_slice<NPT>(cur, V + (int64_t)kb * P * ldv + base, len);
-    }
-    // the next block's vectors are read from HBM by the next sweep: start them now
-    if (kb + 1 < nb && threadIdx.x < P && (kb + 1) * P + (int)threadIdx.x <= j)
-      prefetch_l2(V + (int64_t)((kb + 1) * P + threadIdx.x) * ldv + base, len);
-    // T rows of the current block (lane m: row kb P + m, entries l < m)
-    const bool solve = kb < nb;
-    if (wid == 0 && solve && lane < nc) {
-      const double* tr = T + (int64_t)(kb * P + lane) * P;
-#pragma unroll
-      for (int l = 0; l < P - 1; l++)
-        if (l < lane) s_trow[lane][l] = tr[l];
-    }
-    const double r = warp_reduce_scatter<P>(loc, lane);
-    if ((lane & (32 / P - 1)) == 0) wpart[lane / (32 / P)][wid] = r;
-    __syncthreads();
-    if (wid == 0) {
-      double t = 0.0;
-      for (int q = lane / P; q < nw; q += 32 / P) t += wpart[lane % P][q];
-#pragma unroll
-      for (int x = P; x < 32; x <<= 1) t += __shfl_xor_sync(0xffffffffu, t, x);
-      __syncwarp();
-      if (!bm_reduce_w0<P>(bs, part, seq, t, s_trow, solve, nc, s_h) && lane == 0) s_fail = 1;
-    }
-    if (gridDim.x > 1) seq++;
-    __syncthreads();
-    if (s_fail) return;
-    if (solve && blockIdx.x == 0 && threadIdx.x < nc) Hcol[kb * P + threadIdx.x] = s_h[threadIdx.x];
-  }
-  // s_h[0] = ||w||^2, s_h[1..ng] = <w, v_l> for the last block's vectors
-  const double hn = sqrt(s_h[0]);
-  if (hn > 0.0) {
-    const double inv = 1.0 / hn;
-    double* vnx = V + (int64_t)(j + 1) * ldv + base;
-#pragma unroll
-    for (int q = 0; q < NPT / 2; q++) {
-      const int64_t k = bm_off(q);
-      const double v0 = wr[2 * q] * inv, v1 = wr[2 * q + 1] * inv;
-      ws[k] = v0;
-      ws[k + 1] = v1;
-      if (k + 1 < len) *reinterpret_cast<double2*>(vnx + k) = make_double2(v0, v1);
-      else if (k < len) vnx[k] = v0;
-    }
-    if (z) {
-      __syncthreads();
-      for (int64_t a = threadIdx.x; a < len / 3; a += blockDim.x) {
-        const DT* D = Dinv + ((base / 3) + a) * 9;
-        double x0 = ws[3 * a], x1 = ws[3 * a + 1], x2 = ws[3 * a + 2];
-        ZT* zo = z + base + 3 * a;
-        if constexpr (sizeof(DT) == 8) {
-          zo[0] = (ZT)(D[0] * x0 + D[1] * x1 + D[2] * x2);
-          zo[1] = (ZT)(D[3] * x0 + D[4] * x1 + D[5] * x2);
-          zo[2] = (ZT)(D[6] * x0 + D[7] * x1 + D[8] * x2);
-        } else {
-          float f0 = (float)x0, f1 = (float)x1, f2 = (float)x2;
-          zo[0] = (ZT)(D[0] * f0 + D[1] * f1 + D[2] * f2);
-          zo[1] = (ZT)(D[3] * f0 + D[4] * f1 + D[5] * f2);
-          zo[2] = (ZT)(D[6] * f0 + D[7] * f1 + D[8] * f2);
-        }
-      }
-    }
-    // new row of T_B: T[j+1][c] = -(g_c + sum_{c<l<ng} g_l T[b0+l][c]), g_l = <v_{j+1}, v_{b0+l}>
-    if (blockIdx.x == 0 && threadIdx.x < ng) {
-      const int c = threadIdx.x, b0 = (nb - 1) * P;
-      double acc = s_h[1 + c] * inv;
-      for (int l = c + 1; l < ng; l++) acc += s_h[1 + l] * inv * T[(int64_t)(b0 + l) * P + c];
-      T[(int64_t)(j + 1) * P + c] = -acc;
-    }
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    Hcol[j + 1] = hn;
-    for (int i = 0; i < j; i++) {
-      double a = Hcol[i], c = Hcol[i + 1];
-      Hcol[i] = cs[i] * a + sn[i] * c;
-      Hcol[i + 1] = -sn[i] * a + cs[i] * c;
-    }
-    double a = Hcol[j], c = Hcol[j + 1];
-    double r = hypot(a, c);
-    cs[j] = a / r;
-    sn[j] = c / r;
-    Hcol[j] = r;
-    Hcol[j + 1] = 0.0;
-    g[j + 1] = -sn[j] * g[j];
-    g[j] = cs[j] * g[j];
-    double res = fabs(g[j + 1]);
-    out[0] = res;
-    out[1] = hn;
-    out[8] = (double)(j + 1);
-    if (!(res > target) || hn == 0.0 || j + 1 >= kmax || it0 + j + 1 >= max_it) out[7] = 1.0;
-  }
-}
-
 // The blocked MGS step for vectors too long for a register-resident grid:
-// the same passes, reductions and tail as k_arnoldi_bm, with the block's
+// the same passes and tail as k_arnoldi_bm, with the block's
 // slice of w in shared memory (NPT values per thread, up to 18,432 per
 // block) and each basis slice read straight from L2/HBM in 16-byte pairs
 // (the next block of basis vectors is prefetched into L2 as before).  One
@@ -1575,30 +1970,30 @@ __global__ void k_scale(int64_t n, const double* __restrict__ s, double* __restr
   if (i < glen) g[i] = (i == 0) ? beta : 0.0;
 }
 
-// back substitution y = H^{-1} g on the k x k upper triangle (one block)
 // back substitution R y = g (R upper triangular, column j at H + j ldh), one
-// block of 1024 threads, thread r owns row r (k <= 1000): g and the diagonal
-// sit in shared memory and each thread loads its entry of the next column
-// while the current one is applied, so a column costs one block barrier
-// instead of a global-memory round trip
+// block, thread r owns row r (k <= 1000): g sits in shared memory, each
+// thread loads its entry of the next column while the current one is applied,
+// so a column costs one block barrier and one FP64 product per row.  The
+// divisions by the diagonal become products with its reciprocals, formed
+// once in parallel: a division per column in every thread kept the FP64 pipe
+// busy for 2 us per column (k = 60: 133 us; Cook P2 40x33x5).
 __global__ void __launch_bounds__(1024) k_trisolve(int k, int ldh, const double* __restrict__ H,
                                                    const double* __restrict__ g, double* __restrict__ y) {
   __shared__ double gs[1024], dg[1024];
   const int r = threadIdx.x;
   if (r < k) {
     gs[r] = g[r];
-    dg[r] = H[(int64_t)r * ldh + r];
+    dg[r] = 1.0 / H[(int64_t)r * ldh + r];
   }
   double h = (r < k - 1) ? H[(int64_t)(k - 1) * ldh + r] : 0.0;
   __syncthreads();
   for (int i = k - 1; i >= 0; i--) {
-    const double yi = gs[i] / dg[i];
     const double hn = (i >= 1 && r < i - 1) ? H[(int64_t)(i - 1) * ldh + r] : 0.0;
-    if (r < i) gs[r] -= h * yi;
-    if (r == 0) y[i] = yi;
+    if (r < i) gs[r] -= h * (gs[i] * dg[i]);
     h = hn;
     __syncthreads();
   }
+  if (r < k) y[r] = gs[r] * dg[r];
 }
 
 // u = sum_i y_i V_i
@@ -1674,21 +2069,106 @@ static GridSync grid_sync(fe_mesh m) {
   return gs;
 }
 
-template <int NPT, class DT, class ZT>
-static const void* arnoldi_fn() { return (const void*)k_arnoldi<NPT, DT, ZT>; }
+static XchSync xch_sync(fe_mesh m) {
+  XchSync xs;
+  xs.slots = (uint4*)m->xch;
+  xs.seq = m->bar + XCH_SEQ_WORD;
+  xs.err = m->err;
+  xs.limit = m->wait_limit;
+  return xs;
+}
 
-// Picks the smallest slice width (NPT values per thread, a multiple of 3)
-// whose grid of ceil(n / S) blocks can be co-resident, then launches the
-// step cooperatively.  fuse_pc: also write z = D^{-1} V_{j+1} into zx.
+// The sequence numbers of the grid exchange are 32 bits: before they can
+// wrap (2^31 sums), the exchange state starts anew.
+static int xch_reserve(fe_mesh m, int sums) {
+  if (m->xch_used + (uint32_t)sums >= (1u << 31)) FE_TRY(fe_reset_grid_sync(m));
+  m->xch_used += (uint32_t)sums;
+  return FE_OK;
+}
+
+// Register-resident Arnoldi step (k_arnoldi_reg, k_arnoldi_bm) for vectors of
+// up to 6,144 values per SM; returns 1 without launching for longer ones.
+// fuse_pc: also write z = D^{-1} V_{j+1} into zx.
+//
+// Grid.  A step costs about 16 (blocked: 8 vectors' products and updates) or
+// 2 (sequential) FP64 passes of S / 2 cycles over a block's slice of S values
+// per grid sum, and a grid sum about 3,000 cycles more on several blocks than
+// on one: one block up to 384 (blocked) or 1,536 (sequential) values, above
+// that slices of at least 256 or 512 values on as many SMs as there are.
+// Threads: of the (threads, values per thread) pairs that hold the slice, the
+// one with the least FP64 issue per SM quarter (the passes, and 9 or 6 steps
+// per warp for the sums).
+template <bool SEQ, class DT, class ZT>
+static int launch_arnoldi_new(fe_mesh m, int j, int kmax, bool fuse_pc, const DT* Dinv, double target, int it0,
+                              int max_it) {
+  const int64_t n = m->ndof;
+  const int sms = std::min(m->sm_count, XCH_BLOCKS);
+  int64_t G = 1;
+  if (n > (SEQ ? 1536 : 384)) G = std::min<int64_t>(sms, (n + (SEQ ? 511 : 255)) / (SEQ ? 512 : 256));
+  const int64_t S = ((n + G - 1) / G + 5) / 6 * 6;
+  if (S > 6144) return 1;
+  const int grid = (int)((n + S - 1) / S);
+  const void* fn = nullptr;
+  int nt = 0, npt = 0;
+  if (S <= 1536) {
+    const void* fns[3] = {(const void*)k_arnoldi_reg<2, SEQ, DT, ZT>, (const void*)k_arnoldi_reg<4, SEQ, DT, ZT>,
+                          (const void*)k_arnoldi_reg<6, SEQ, DT, ZT>};
+    int best = INT_MAX;
+    for (int t = 128; t <= 256; t += 128)
+      for (int q = 0; q < 3; q++) {
+        const int v = 2 * (q + 1), cost = t / 128 * (16 * v + (SEQ ? 48 : 9));
+        if ((int64_t)t * v >= S && cost < best) {
+          best = cost;
+          fn = fns[q];
+          nt = t;
+          npt = v;
+        }
+      }
+  } else {
+    fn = (const void*)k_arnoldi_bm<12, SEQ, DT, ZT>;
+    npt = 12;
+    nt = (int)((S + 12 * 128 - 1) / (12 * 128) * 128);
+  }
+  const size_t smem = (size_t)npt * nt * sizeof(double);
+  FE_TRY(fe_kernel_smem(fn, (int)smem));
+  int per_sm = 0;
+  FE_TRY(fe_kernel_occupancy(fn, nt, smem, &per_sm));
+  if ((int64_t)per_sm * m->sm_count < grid) return 1;
+  FE_TRY(xch_reserve(m, j + 2));
+  double* V = m->V;
+  int64_t ldv = m->ldv;
+  double* Hcol = m->H + (int64_t)j * (kmax + 1);
+  double* cs = m->gv;
+  double* sn = m->gv + (kmax + 2);
+  double* g = m->gv + 2 * (kmax + 2);
+  double* out = m->scal + 3;
+  double* T = m->Tbm;
+  const DT* D = fuse_pc ? Dinv : nullptr;
+  ZT* z = fuse_pc ? (ZT*)m->zx : nullptr;
+  XchSync xs = xch_sync(m);
+  void* args[] = {(void*)&n, (void*)&S, (void*)&j, (void*)&V, (void*)&ldv, (void*)&m->w64, (void*)&Hcol,
+                  (void*)&xs, (void*)&T, (void*)&cs, (void*)&sn, (void*)&g, (void*)&out,
+                  (void*)&D, (void*)&z, (void*)&target, (void*)&kmax, (void*)&it0, (void*)&max_it};
+  // flops: (j+1) inner products and axpys (4 per entry), the norm (2) and the scaling (1) per
+  // entry, the blocked form's Gram row, plus 18 per node for the fused block-Jacobi product
+  const int ng = SEQ ? 0 : (j + 1) % BMGS_P;
+  FE_SCOPE_F(m, FE_PROF_ARNOLDI, 8.0 * (double)n * (j + 3) + (fuse_pc ? (double)n * (3.0 * sizeof(DT) + sizeof(ZT)) : 0.0),
+             (double)n * (4.0 * (j + 1) + 3.0 + 2.0 * ng) + (fuse_pc ? 6.0 * n : 0.0));
+  FE_CUDA(cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(nt), args, smem, m->stream));
+  return FE_OK;
+}
+
+// Sequential sweep for longer vectors: several blocks of 256 threads per SM.
 template <class DT, class ZT>
 static int launch_arnoldi_t(fe_mesh m, int j, int kmax, bool fuse_pc, const DT* Dinv, double target, int it0,
                             int max_it) {
   const int64_t n = m->ndof;
-  const void* fns[3] = {arnoldi_fn<24, DT, ZT>(), arnoldi_fn<12, DT, ZT>(), arnoldi_fn<6, DT, ZT>()};
-  const int npts[3] = {24, 12, 6};
-  const int bds[3] = {256, 512, 1024};
+  const void* fns[1] = {(const void*)k_arnoldi<24, DT, ZT>};
+  const int npts[1] = {24};
+  const int bds[1] = {256};
   int which = -1, grid = 0;
-  for (int q = 0; q < 3; q++) {
+  {
+    const int q = 0;
     size_t smem = (size_t)npts[q] * bds[q] * sizeof(double);
     FE_TRY(fe_kernel_smem(fns[q], (int)smem));
     int per_sm = 0;
@@ -1697,7 +2177,6 @@ static int launch_arnoldi_t(fe_mesh m, int j, int kmax, bool fuse_pc, const DT* 
     if (per_sm >= 1 && need <= (int64_t)per_sm * m->sm_count && need <= RED_SLOTS) {
       which = q;
       grid = (int)need;
-      break;
     }
   }
   if (which < 0) return fe_set_error("vector too long for the persistent Arnoldi kernel (n = %lld)", (long long)n), FE_ERR_ARG;
@@ -1779,8 +2258,6 @@ static int launch_arnoldi_ls_t(fe_mesh m, int j, int kmax, bool fuse_pc, const D
 }
 
 template <int NPT, class DT, class ZT>
-static const void* arnoldi_bm_fn() { return (const void*)k_arnoldi_bm<NPT, BMGS_P, DT, ZT>; }
-template <int NPT, class DT, class ZT>
 static const void* arnoldi_bm_ws_fn() { return (const void*)k_arnoldi_bm_ws<NPT, BMGS_P, DT, ZT>; }
 
 static BlockSync block_sync(fe_mesh m) {
@@ -1793,23 +2270,19 @@ static BlockSync block_sync(fe_mesh m) {
   return bs;
 }
 
-// Slice selection as in launch_arnoldi_t: first the register-resident
-// kernels (w, the current and the next basis slice in registers), then, for
-// longer vectors, the shared-memory slices of k_arnoldi_bm_ws (48 or 72
-// values per thread); returns 1 without launching when no co-resident grid
-// exists, and the caller takes the sequential sweep.
+// The shared-memory slices of k_arnoldi_bm_ws (48 or 72 values per thread)
+// for vectors beyond the register-resident kernels; returns 1 without
+// launching when no co-resident grid exists, and the caller takes the
+// sequential sweep.
 template <class DT, class ZT>
 static int launch_arnoldi_bm_t(fe_mesh m, int j, int kmax, bool fuse_pc, const DT* Dinv, double target, int it0,
                                int max_it) {
   const int64_t n = m->ndof;
-  // 512 threads of 12 values first: four warps per SM sub-partition keep
-  // the FP64 pipe busier than two
-  const void* fns[4] = {arnoldi_bm_fn<12, DT, ZT>(), arnoldi_bm_fn<24, DT, ZT>(), arnoldi_bm_ws_fn<48, DT, ZT>(),
-                        arnoldi_bm_ws_fn<72, DT, ZT>()};
-  const int npts[4] = {12, 24, 48, 72};
-  const int bds[4] = {512, 256, 256, 256};
+  const void* fns[2] = {arnoldi_bm_ws_fn<48, DT, ZT>(), arnoldi_bm_ws_fn<72, DT, ZT>()};
+  const int npts[2] = {48, 72};
+  const int bds[2] = {256, 256};
   int which = -1, grid = 0;
-  for (int q = 0; q < 4; q++) {
+  for (int q = 0; q < 2; q++) {
     size_t smem = (size_t)npts[q] * bds[q] * sizeof(double);
     FE_TRY(fe_kernel_smem(fns[q], (int)smem));
     int per_sm = 0;
@@ -1847,6 +2320,18 @@ static int launch_arnoldi_bm_t(fe_mesh m, int j, int kmax, bool fuse_pc, const D
 }
 
 static int launch_arnoldi(fe_mesh m, int j, int kmax, bool fuse_pc, double target, int it0, int max_it) {
+  if (m->orthog != 1) {
+    int r;
+    if (m->orthog == 2)
+      r = m->prec == FE_PREC_FP64
+              ? launch_arnoldi_new<false, double, double>(m, j, kmax, fuse_pc, m->Dinv64, target, it0, max_it)
+              : launch_arnoldi_new<false, float, float>(m, j, kmax, fuse_pc, m->Dinv32, target, it0, max_it);
+    else
+      r = m->prec == FE_PREC_FP64
+              ? launch_arnoldi_new<true, double, double>(m, j, kmax, fuse_pc, m->Dinv64, target, it0, max_it)
+              : launch_arnoldi_new<true, float, float>(m, j, kmax, fuse_pc, m->Dinv32, target, it0, max_it);
+    if (r <= 0) return r;
+  }
   if (m->orthog == 2) {
     int r = m->prec == FE_PREC_FP64
                 ? launch_arnoldi_bm_t<double, double>(m, j, kmax, fuse_pc, m->Dinv64, target, it0, max_it)
@@ -1979,7 +2464,7 @@ int fe_gmres_dev(fe_mesh m, const double* b, double* x, double rtol, double atol
     done = it >= max_it || m->h_scal[4] == 0.0 || !std::isfinite(resid) || (resid <= target && !refine);
     {
       FE_SCOPE(m, FE_PROF_VECTOR, 8.0 * j * (j + 1));
-      k_trisolve<<<1, 1024, 0, m->stream>>>(j, kmax + 1, m->H, g, y);
+      k_trisolve<<<1, (j + 31) / 32 * 32, 0, m->stream>>>(j, kmax + 1, m->H, g, y);
     }
     {
       FE_SCOPE(m, FE_PROF_VECTOR, 8.0 * n * (j + 1));

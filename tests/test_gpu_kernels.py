@@ -1,0 +1,47 @@
+"""Launch rules of the kernels at the sizes where they change: edges of
+tiles, remainders and the smallest and largest sizes of each branch, against
+the CPU oracle or against the general path."""
+import numpy as np
+import pytest
+
+import oracle as O
+import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fe():
+    import __graft_entry__ as g
+    g.build()
+    import paper_2203_05610_gb300 as fe
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    return fe
+
+
+# unknowns 150 (one block in both forms), 729 and 1,500 (several blocks only
+# in the blocked form), 1,800 (several in both), 39,375 (a slice of 264 per
+# SM), 151,290 (996 values: 256 threads x 4), 249,696 (1,644: the long-slice
+# kernel)
+@pytest.mark.parametrize("orthog", [0, 2])
+@pytest.mark.parametrize("size", [(4, 4, 1), (8, 8, 2), (9, 9, 4), (9, 9, 5), (24, 24, 20), (40, 40, 29),
+                                  (50, 50, 31)])
+def test_arnoldi_launch_shapes(fe, size, orthog):
+    # both sides run exactly 24 iterations in cycles of 13 (a full block of
+    # eight basis vectors and a part of one); the projections are the same, so
+    # the iterates differ by rounding (FP64 sums of n terms in another order:
+    # below 1e-9 relative, the bound of the longer multi-block test)
+    w = W.cook(*size, order=1, nu=0.3)
+    m, om = fe.Mesh(w), O.Mesh(w)
+    d = 0.02 * np.random.default_rng(3).standard_normal(om.ndof)
+    om.apply_dirichlet(d)
+    dg = torch.from_numpy(d).cuda()
+    om.tangent(d)
+    m.tangent(dg)
+    b = np.random.default_rng(4).standard_normal(om.ndof)
+    x, it, res = om.gmres(b, rtol=1e-14, atol=0.0, restart=13, max_it=24)
+    xg, itg, resg = m.gmres(torch.from_numpy(b).cuda(), rtol=1e-14, atol=0.0, restart=13, max_it=24, orthog=orthog)
+    assert it == itg == 24
+    assert abs(resg - res) <= 1e-8 * res, (resg, res)
+    assert np.linalg.norm(xg.cpu().numpy() - x) <= 1e-9 * np.linalg.norm(x)
