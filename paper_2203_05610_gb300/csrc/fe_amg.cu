@@ -53,6 +53,7 @@
 #include <vector>
 
 #include "fe_internal.h"
+#include "fe_stream.cuh"
 
 namespace {
 
@@ -107,7 +108,8 @@ struct AmgLevel {
   float* pt32 = nullptr;
   double* coef64 = nullptr;  // Chebyshev coefficients {1/theta, c1, c2} in device memory, so
   float* coef32 = nullptr;   // a captured V-cycle stays valid when a new tangent changes them
-  // V-cycle vectors [n*b] in the V-cycle precision
+  // V-cycle vectors [n*b] in the V-cycle precision (level 0: x is the mesh's
+  // SpMV input zx)
   void *x = nullptr, *r = nullptr, *d0 = nullptr, *d1 = nullptr, *e = nullptr;
 };
 
@@ -121,13 +123,19 @@ struct AmgHier {
   std::vector<void*> allocs; // device buffers owned by the hierarchy
   int64_t bytes = 0;         // their size (counted in the mesh's device bytes)
   bool ready = false;        // numbers formed for the current tangent
-  // the V-cycle captured as a CUDA graph: input vin (FP64), output lev[0].x
-  double* vin = nullptr;
+  // the V-cycle captured as a CUDA graph, output lev[0].x; its first kernel
+  // reads the caller's vector (argument `root_arg` of node `root`, set before
+  // each launch)
+  cudaGraph_t graph = nullptr;
+  cudaGraphNode_t root = nullptr;
+  int root_arg = 0;
+  StreamShape shape0{};             // the streamed level-0 step's launch and row ranges
+  int* part0 = nullptr;             // [shape0.ranges + 1]
+  int part0_len = 0;
   cudaStream_t cap = nullptr;       // capture stream (the mesh's may be the legacy stream)
   cudaGraphExec_t exec = nullptr;
   int exec_prec = -1;               // tangent precision the graph was captured for
   double vc_bytes = 0, vc_flops = 0; // algorithmic bytes and flops of one V-cycle
-  unsigned grid0 = 0;               // one wave of the streamed level-0 kernel
 };
 
 namespace {
@@ -673,51 +681,125 @@ __global__ void k_amg_tile(int64_t nblocks, const T* __restrict__ src, T* __rest
 enum { VC_SETX = 1, VC_FINAL = 2, VC_KEEPX = 4, VC_START = 8 };
 
 
-// Chebyshev epilogue of block row `row` with row sum s = (A g)_row
-template <class T, int B>
-__device__ __forceinline__ void cheb_rows(int64_t row, const T (&s)[B], const T* __restrict__ dinv,
-                                          const T* __restrict__ g, T* __restrict__ x, T* __restrict__ r,
-                                          T* __restrict__ dout, T cx, const T* __restrict__ coef, int flags) {
-  const int64_t o = (int64_t)B * row;
-  T rn[B], gi[B], xi[B];
-#pragma unroll
-  for (int q = 0; q < B; q++) {
-    gi[q] = g[o + q];
-    rn[q] = r[o + q] - s[q];
-    r[o + q] = rn[q];
-  }
-  const bool wx = !(flags & VC_KEEPX);
-#pragma unroll
-  for (int q = 0; q < B; q++) xi[q] = ((flags & VC_SETX) ? T(0) : (wx ? x[o + q] : T(0))) + cx * gi[q];
-  if (dout) {
-    const T c1 = (flags & VC_START) ? T(0) : coef[1];
-    const T c2 = (flags & VC_START) ? coef[0] : coef[2];
-#pragma unroll
-    for (int q = 0; q < B; q++) {
-      T t = T(0);
-#pragma unroll
-      for (int j = 0; j < B; j++) t += dinv[row * B * B + B * q + j] * rn[j];
-      const T dn = c1 * gi[q] + c2 * t;
-      dout[o + q] = dn;
-      if (flags & VC_FINAL) xi[q] += dn;
+// Level-0 Chebyshev step: the streamed product of fe_stream.cuh with the row
+// updates as its epilogue; a window's g, r, x and block-Jacobi inverses are
+// copied to shared memory while its tiles are multiplied.  Every row of A
+// holds its diagonal block, so no row is empty.  Five blocks per SM (96
+// registers) in FP32: with six the operands spill (48x48x8: 312 against 278 us
+// per V-cycle).
+template <class T>
+__host__ __device__ constexpr int cheb0_blocks_per_sm() { return sizeof(T) == 8 ? 3 : 5; }
+
+template <class T>
+struct ChebStage {  // operands of up to 16 rows of a window
+  T g[48], r[48], x[48], d[144];
+};
+
+template <class T>
+struct EpiCheb {
+  const T* dinv;
+  const T* g;
+  T* x;
+  T* r;
+  T* dout;
+  T cx, k1, k2;
+  int flags;
+  ChebStage<T>* st;
+  T gi[3], ri[3], xo[3], di[9];
+  // copies a window's rows into the stage while its tiles are multiplied
+  __device__ __forceinline__ void prefetch(int r0, int rb, int lane) {
+    const int m = min(16, rb - r0);
+    const int64_t o = 3 * (int64_t)r0;
+    for (int i = lane; i < 3 * m; i += 32) {
+      cp_async(st->g + i, g + o + i);
+      cp_async(st->r + i, r + o + i);
+      if (!(flags & (VC_KEEPX | VC_SETX))) cp_async(st->x + i, x + o + i);
     }
+    if (dout)
+      for (int i = lane; i < 9 * m; i += 32) cp_async(st->d + i, dinv + 3 * o + i);
   }
-  if (wx)
+  __device__ __forceinline__ void load(int r0, int i0, int nd, int lane) {
+    cp_async_wait();
+    __syncwarp();  // (a lane reads what other lanes copied)
+    if (lane >= nd) return;
+    const bool in = i0 + lane < 16;
+    const int64_t o = 3 * (int64_t)(r0 + lane);
+    const int i = i0 + lane;
 #pragma unroll
-    for (int q = 0; q < B; q++) x[o + q] = xi[q];
+    for (int q = 0; q < 3; q++) {
+      gi[q] = in ? st->g[3 * i + q] : g[o + q];
+      ri[q] = in ? st->r[3 * i + q] : r[o + q];
+      xo[q] = (flags & (VC_KEEPX | VC_SETX)) ? T(0) : (in ? st->x[3 * i + q] : x[o + q]);
+    }
+    if (dout)
+#pragma unroll
+      for (int q = 0; q < 9; q++) di[q] = in ? st->d[9 * i + q] : dinv[3 * o + q];
+  }
+  __device__ __forceinline__ void finish(int row, const T (&s)[3]) {
+    const int64_t o = 3 * (int64_t)row;
+    T rn[3], xi[3];
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      rn[q] = ri[q] - s[q];
+      r[o + q] = rn[q];
+      xi[q] = xo[q] + cx * gi[q];
+    }
+    if (dout) {
+#pragma unroll
+      for (int q = 0; q < 3; q++) {
+        T t = T(0);
+#pragma unroll
+        for (int j = 0; j < 3; j++) t += di[3 * q + j] * rn[j];
+        const T dn = k1 * gi[q] + k2 * t;
+        if (flags & VC_FINAL) xi[q] += dn;  // (the final direction is in x already)
+        else dout[o + q] = dn;
+      }
+    }
+    if (!(flags & VC_KEEPX))
+#pragma unroll
+      for (int q = 0; q < 3; q++) x[o + q] = xi[q];
+  }
+};
+
+template <class V, class T>
+__global__ void __launch_bounds__(STREAM_THREADS, cheb0_blocks_per_sm<T>())
+    k_vc_cheb0(int n, int warps, int ranges, const int* __restrict__ part, const int* __restrict__ row_ptr,
+               const int* __restrict__ col, const V* __restrict__ val, const T* __restrict__ dinv,
+               const T* __restrict__ g, T* __restrict__ x, T* __restrict__ r, T* __restrict__ dout, T cx,
+               const T* __restrict__ coef, int flags) {
+  __shared__ StreamShared<T> sh;
+  __shared__ __align__(16) ChebStage<T> stage[STREAM_WARPS];
+  const int warp = (int)blockIdx.x * STREAM_WARPS + (threadIdx.x >> 5);
+  if (warp >= warps) return;
+  EpiCheb<T> epi;
+  epi.st = &stage[threadIdx.x >> 5];
+  epi.dinv = dinv;
+  epi.g = g;
+  epi.x = x;
+  epi.r = r;
+  epi.dout = dout;
+  epi.cx = cx;
+  epi.k1 = (flags & VC_START) ? T(0) : coef[1];
+  epi.k2 = (flags & VC_START) ? coef[0] : coef[2];
+  epi.flags = flags;
+  stream_rows<V, T, T>(n, warp, warps, ranges, part, row_ptr, col, val, g, sh.prod[threadIdx.x >> 5], epi);
 }
 
-// Level-0 Chebyshev step, streamed like the SpMV: a warp takes groups of 16
+// The same step for the largest FP32 levels: a warp takes groups of 16
 // consecutive block rows and walks their (contiguous) blocks in chunks of 32,
 // one block per lane, forming the row sums by a segmented scan across the
 // lanes and carrying a row's partial sum into the next chunk; values, column
-// indices and the gather of g run two chunks ahead.  A row's sum goes to
-// shared memory when its last block is reached; the group's 16 Chebyshev
-// row updates (cheb_rows' arithmetic) run together after its last chunk,
-// lane i on row i, with the rows' g, r, x and block-Jacobi inverse loaded
-// when the group starts: one memory latency per group for the updates
-// instead of one per chunk that ends a row.  Every row of A holds its
-// diagonal block, so no row is empty.
+// indices and the gather of g run ahead.  A row's sum goes to shared memory
+// when its last block is reached; the group's 16 Chebyshev row updates run
+// together after its last chunk, lane i on row i, with the rows' g, r, x and
+// block-Jacobi inverse loaded when the group starts.
+//
+// The loads of a group never wait for a phase of row sums, which is worth 7%
+// of the V-cycle where HBM bounds it, but groups of 16 rows must fill the
+// wave several times: per V-cycle, scan against window form, FP32: Cook P2
+// 64x64x8 (4.8 groups per warp) 417 and 446 us, 48x48x8 (2.7) 288 and 278,
+// 30x26x6 (one) 113 and 87, cardiac shell 72 and 71; FP64: 2,420 and 1,688,
+// 1,518 and 995, 609 and 332, 363 and 316 us (the scan's adds, 15 per block).
 constexpr int VC_RPW = 16;
 
 template <class V, class T>
@@ -742,7 +824,7 @@ __device__ __forceinline__ void vc_load_g(const T* __restrict__ g, int c, T (&x)
 }
 
 template <class V, class T>
-__global__ void __launch_bounds__(256) k_vc_cheb0(int n, const int* __restrict__ row_ptr, const int* __restrict__ col,
+__global__ void __launch_bounds__(256) k_vc_cheb0_scan(int n, const int* __restrict__ row_ptr, const int* __restrict__ col,
                                                   const V* __restrict__ val, const T* __restrict__ dinv,
                                                   const T* __restrict__ g, T* __restrict__ x, T* __restrict__ r,
                                                   T* __restrict__ dout, T cx, const T* __restrict__ coef,
@@ -975,15 +1057,16 @@ __global__ void k_vc_init0(int n, const T* __restrict__ dinv, const double* __re
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const T inv_theta = coef[0];
-  T bi[3];
-  for (int q = 0; q < 3; q++) {
-    bi[q] = (T)b[3 * (int64_t)i + q];
-    r[3 * (int64_t)i + q] = bi[q];
-  }
+  T bi[3], di[3];
+  for (int q = 0; q < 3; q++) bi[q] = (T)b[3 * (int64_t)i + q];
   for (int q = 0; q < 3; q++) {
     T t = T(0);
     for (int j = 0; j < 3; j++) t += dinv[(int64_t)i * 9 + 3 * q + j] * bi[j];
-    d[3 * (int64_t)i + q] = t * inv_theta;
+    di[q] = t * inv_theta;
+  }
+  for (int q = 0; q < 3; q++) {
+    r[3 * (int64_t)i + q] = bi[q];
+    d[3 * (int64_t)i + q] = di[q];
   }
 }
 
@@ -1208,7 +1291,6 @@ __global__ void k_vc_convert(int64_t n, const A* __restrict__ a, B* __restrict__
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) b[i] = (B)a[i];
 }
-
 // ---------------------------------------------------------------- host drivers
 template <class X>
 int dev_alloc(fe_mesh m, X** p, size_t count) {
@@ -1485,8 +1567,10 @@ int ensure_vectors(fe_mesh m, int elem) {
   for (int q = 0; q < h->nlev; q++) {
     AmgLevel& L = h->lev[q];
     const size_t bytes = (size_t)L.n * L.b * elem;
-    void** vs[5] = {&L.x, &L.r, &L.d0, &L.d1, &L.e};
+    if (q == 0) L.x = m->zx;  // allocated before any preconditioner application
+    void** vs[5] = {&L.r, &L.d0, &L.d1, &L.e, &L.x};
     for (void** v : vs) {
+      if (q == 0 && v == &L.x) continue;
       char* p = nullptr;
       FE_TRY(dev_alloc(m, &p, bytes));
       *v = p;
@@ -1530,8 +1614,9 @@ int store_coeffs(fe_mesh m) {
 }
 
 // The kernels of one V-cycle in precision T, level-0 values of type V
-// (tiled), on stream st: input b (FP64 [3 nn]), result in lev[0].x.  Adds
-// the algorithmic bytes and flops of its kernels to *bytes, *flops.
+// (tiled), on stream st: input b (FP64 [3 nn], read by the first kernel
+// alone), result in lev[0].x.  Adds the algorithmic bytes and flops of its
+// kernels to *bytes, *flops.
 template <class T, class V>
 int vcycle_launches(fe_mesh m, cudaStream_t st, const V* K0, const double* b, double* bytes, double* flops) {
   AmgHier* h = m->amg;
@@ -1545,15 +1630,26 @@ int vcycle_launches(fe_mesh m, cudaStream_t st, const V* K0, const double* b, do
   auto coef = [&](int q) -> const T* { return D ? (const T*)h->lev[q].coef64 : (const T*)h->lev[q].coef32; };
   auto X = [&](int q) { return (T*)h->lev[q].x; };
   const double sv = sizeof(T), s0 = sizeof(V);
+  // level 0: the scan form where its 16-row groups fill the wave four times
+  // (FP32 and BF16 values; see k_vc_cheb0_scan)
+  int per_sm = 0;
+  FE_TRY(fe_kernel_occupancy((const void*)k_vc_cheb0_scan<V, T>, 256, 0, &per_sm));
+  const int64_t groups = ((int64_t)m->nn + VC_RPW - 1) / VC_RPW, wave = (int64_t)std::max(per_sm, 1) * m->sm_count;
+  const bool scan = !D && groups >= 4 * 8 * wave;
+  const unsigned grid_scan = (unsigned)wave;
   // Chebyshev step on level q (fused SpMV)
   auto step = [&](int q, const T* g, T* dout, double cx, int flags) -> int {
     AmgLevel& Lq = h->lev[q];
     const int B = Lq.b;
     *bytes += (double)Lq.nnz * (B * B * (q == 0 ? s0 : sv) + 4) + 4.0 * (Lq.n + 1) + (double)Lq.n * B * (sv * 5 + B * sv);
     *flops += 2.0 * Lq.nnz * B * B;
-    if (q == 0)
-      k_vc_cheb0<V, T><<<h->grid0, 256, 0, st>>>(Lq.n, Lq.ptr, Lq.col, K0, dinv(0), g, X(0), (T*)Lq.r, dout, (T)cx,
-                                                 coef(0), flags);
+    if (q == 0 && scan)
+      k_vc_cheb0_scan<V, T><<<grid_scan, 256, 0, st>>>(Lq.n, Lq.ptr, Lq.col, K0, dinv(0), g, X(0), (T*)Lq.r, dout,
+                                                       (T)cx, coef(0), flags);
+    else if (q == 0)
+      k_vc_cheb0<V, T><<<stream_grid(h->shape0.warps), STREAM_THREADS, 0, st>>>(
+          Lq.n, h->shape0.warps, h->shape0.ranges, h->part0, Lq.ptr, Lq.col, K0, dinv(0), g, X(0), (T*)Lq.r, dout,
+          (T)cx, coef(0), flags);
     else
       k_vc_cheb<T, AMG_NS><<<blocks_for((int64_t)Lq.n * 32, 256), 256, 0, st>>>(
           Lq.n, Lq.ptr, Lq.col, vals(q), dinv(q), g, X(q), (T*)Lq.r, dout, (T)cx, coef(q), flags);
@@ -1670,27 +1766,54 @@ int vcycle_launches(fe_mesh m, cudaStream_t st, const V* K0, const double* b, do
   return FE_OK;
 }
 
+void drop_graph(AmgHier* h) {
+  if (h->exec) cudaGraphExecDestroy(h->exec);
+  if (h->graph) cudaGraphDestroy(h->graph);
+  h->exec = nullptr;
+  h->graph = nullptr;
+  h->root = nullptr;
+}
+
+// The captured graph's first kernel (k_vc_init0 or, with one level,
+// k_vc_convert) and the place of the input vector among its arguments.
+int find_root(AmgHier* h) {
+  size_t n = 1;
+  if (cudaGraphGetRootNodes(h->graph, &h->root, &n) != cudaSuccess || n != 1)
+    return fe_set_error("the V-cycle graph has no single first kernel"), FE_ERR_CUDA;
+  h->root_arg = h->nlev == 1 ? 1 : 2;
+  return FE_OK;
+}
+
+// lets the graph's next launches read b
+int set_input(AmgHier* h, const double* b) {
+  cudaKernelNodeParams p{};
+  FE_CUDA(cudaGraphKernelNodeGetParams(h->root, &p));
+  void* args[8];
+  for (int i = 0; i < (h->nlev == 1 ? 3 : 6); i++) args[i] = p.kernelParams[i];
+  args[h->root_arg] = (void*)&b;
+  p.kernelParams = args;
+  FE_CUDA(cudaGraphExecKernelNodeSetParams(h->exec, h->root, &p));
+  return FE_OK;
+}
+
 // capture the V-cycle of the current precision into a CUDA graph
 template <class T, class V>
-int capture(fe_mesh m, const V* K0) {
+int capture(fe_mesh m, const V* K0, const double* b) {
   AmgHier* h = m->amg;
-  if (h->exec) {
-    cudaGraphExecDestroy(h->exec);
-    h->exec = nullptr;
-  }
+  drop_graph(h);
   if (!h->cap) FE_CUDA(cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking));
   FE_CUDA(cudaStreamSynchronize(m->stream));
-  {  // one wave of resident blocks, no more warps than 16-row groups
-    int per_sm = 0;
-    FE_TRY(fe_kernel_occupancy((const void*)k_vc_cheb0<V, T>, 256, 0, &per_sm));
-    const int64_t groups = ((int64_t)m->nn + VC_RPW - 1) / VC_RPW;
-    h->grid0 = (unsigned)std::max<int64_t>(1, std::min<int64_t>((groups + 7) / 8, (int64_t)std::max(per_sm, 1) * m->sm_count));
+  h->shape0 = stream_shape(cheb0_blocks_per_sm<T>(), m->sm_count, m->nnzb);
+  if (h->part0_len < h->shape0.ranges + 1) {
+    FE_TRY(dev_alloc(m, &h->part0, (size_t)h->shape0.ranges + 1));
+    h->part0_len = h->shape0.ranges + 1;
   }
+  FE_TRY(fe_stream_partition(m, h->shape0.ranges, h->part0));
   double bytes = 0.0, flops = 0.0;
   m->prof_suspend++;
   cudaGraph_t g = nullptr;
   cudaError_t e0 = cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal);
-  int rc = e0 == cudaSuccess ? vcycle_launches<T, V>(m, h->cap, K0, h->vin, &bytes, &flops) : FE_ERR_CUDA;
+  int rc = e0 == cudaSuccess ? vcycle_launches<T, V>(m, h->cap, K0, b, &bytes, &flops) : FE_ERR_CUDA;
   cudaError_t e1 = e0 == cudaSuccess ? cudaStreamEndCapture(h->cap, &g) : e0;
   m->prof_suspend--;
   if (rc != FE_OK) {
@@ -1699,9 +1822,14 @@ int capture(fe_mesh m, const V* K0) {
   }
   if (e1 != cudaSuccess)
     return fe_set_error("capturing the V-cycle failed: %s", cudaGetErrorString(e1)), FE_ERR_CUDA;
+  h->graph = g;
   cudaError_t e2 = cudaGraphInstantiate(&h->exec, g, 0);
-  cudaGraphDestroy(g);
-  if (e2 != cudaSuccess) return fe_set_error("instantiating the V-cycle graph failed: %s", cudaGetErrorString(e2)), FE_ERR_CUDA;
+  if (e2 != cudaSuccess) {
+    h->exec = nullptr;
+    drop_graph(h);
+    return fe_set_error("instantiating the V-cycle graph failed: %s", cudaGetErrorString(e2)), FE_ERR_CUDA;
+  }
+  FE_TRY(find_root(h));
   h->exec_prec = m->prec;
   h->vc_bytes = bytes;
   h->vc_flops = flops;
@@ -1727,44 +1855,39 @@ int fe_amg_setup(fe_mesh m) {
   return FE_OK;
 }
 
-int fe_amg_apply(fe_mesh m, const double* x, void* z, bool z_double) {
+int fe_amg_apply(fe_mesh m, const double* x, double* z) {
   if (!m->amg || !m->amg->ready) return fe_set_error("AMG hierarchy not set up"), FE_ERR_STATE;
   AmgHier* h = m->amg;
-  const int64_t N = (int64_t)m->nn * 3;
   const bool d64 = m->prec == FE_PREC_FP64;
   FE_TRY(ensure_vectors(m, d64 ? 8 : 4));
-  if (!h->vin) FE_TRY(dev_alloc(m, &h->vin, (size_t)N));
   // pc_type 2 with the FP32 tangent: the smoother reads a BF16 copy of the
   // fine level (half the bytes of the V-cycle's dominant passes); coarse
   // levels, transfers and vectors stay FP32
   const bool bf_smooth = m->pc_type == 2 && m->prec == FE_PREC_MIXED_FP32;
   const int variant = bf_smooth ? 16 : m->prec;
   if (!h->exec || h->exec_prec != variant) {
-    if (d64) FE_TRY((capture<double, double>(m, m->K64)));
-    else if (m->prec == FE_PREC_MIXED_BF16 || bf_smooth) FE_TRY((capture<float, __nv_bfloat16>(m, m->K16)));
-    else FE_TRY((capture<float, float>(m, m->K32)));
+    if (d64) FE_TRY((capture<double, double>(m, m->K64, x)));
+    else if (m->prec == FE_PREC_MIXED_BF16 || bf_smooth) FE_TRY((capture<float, __nv_bfloat16>(m, m->K16, x)));
+    else FE_TRY((capture<float, float>(m, m->K32, x)));
     h->exec_prec = variant;
   }
-  FE_CUDA(cudaMemcpyAsync(h->vin, x, N * sizeof(double), cudaMemcpyDeviceToDevice, m->stream));
+  FE_TRY(set_input(h, x));
   {
     FE_SCOPE_F(m, FE_PROF_PC, h->vc_bytes, h->vc_flops);
     FE_CUDA(cudaGraphLaunch(h->exec, m->stream));
   }
-  const unsigned g = blocks_for(N, 256);
-  if (d64) {
-    if (z_double) FE_CUDA(cudaMemcpyAsync(z, h->lev[0].x, N * sizeof(double), cudaMemcpyDeviceToDevice, m->stream));
-    else k_vc_convert<double, float><<<g, 256, 0, m->stream>>>(N, (const double*)h->lev[0].x, (float*)z);
-  } else {
-    if (z_double) k_vc_convert<float, double><<<g, 256, 0, m->stream>>>(N, (const float*)h->lev[0].x, (double*)z);
-    else FE_CUDA(cudaMemcpyAsync(z, h->lev[0].x, N * sizeof(float), cudaMemcpyDeviceToDevice, m->stream));
+  if (z) {
+    const int64_t N = (int64_t)m->nn * 3;
+    if (d64) FE_CUDA(cudaMemcpyAsync(z, m->zx, N * sizeof(double), cudaMemcpyDeviceToDevice, m->stream));
+    else k_vc_convert<float, double><<<blocks_for(N, 256), 256, 0, m->stream>>>(N, (const float*)m->zx, z);
+    FE_CUDA(cudaGetLastError());
   }
-  FE_CUDA(cudaGetLastError());
   return FE_OK;
 }
 
 void fe_amg_free(fe_mesh m) {
   if (!m->amg) return;
-  if (m->amg->exec) cudaGraphExecDestroy(m->amg->exec);
+  drop_graph(m->amg);
   if (m->amg->cap) cudaStreamDestroy(m->amg->cap);
   for (void* p : m->amg->allocs) cudaFreeAsync(p, m->stream);
   m->device_bytes -= m->amg->bytes;

@@ -104,6 +104,9 @@ struct fe_mesh_s {
   int* col = nullptr;      // [nnzb]
   int* diag_pos = nullptr; // [nn]
   int* emap = nullptr;     // [ne][nen*nen]
+  int* part32 = nullptr;   // [ranges+1] row ranges of the streamed products (fe_stream.cuh) by accumulation type
+  int* part64 = nullptr;
+  int warps32 = 0, warps64 = 0, ranges32 = 0, ranges64 = 0;
   // u-p coupling pattern (u rows, vertex columns) and its transpose
   int64_t nnz_up = 0;
   int* up_ptr = nullptr;   // [nn+1]
@@ -189,7 +192,7 @@ struct fe_mesh_s {
   double* w64 = nullptr;     // [ndof]
   double* t64 = nullptr;     // [ndof]
   double* u64 = nullptr;     // [ndof]
-  void* zx = nullptr;        // [ndof] SpMV input (FP32 or FP64)
+  void* zx = nullptr;        // [ndof] SpMV input (FP32 or FP64); also the V-cycle's level-0 iterate
   int lb_m = 0;
   double* S = nullptr;       // [m][ndof]
   double* Yv = nullptr;      // [m][ndof]
@@ -318,10 +321,11 @@ int fe_spmv_preload(fe_mesh m);  // loads every SpMV kernel and caches its launc
 // fe_amg.cu: smoothed-aggregation AMG.  fe_amg_setup builds the hierarchy
 // for the tangent just assembled (its structure once per mesh, on the host;
 // its numbers every time, on the device); fe_amg_apply runs one V-cycle on
-// the displacement part of x (FP64) into z (FP64 or FP32, z_double says
-// which); fe_amg_free releases everything.
+// the displacement part of x (FP64) into m->zx (the SpMV input, in the
+// tangent's precision) and, when z is given, into z (FP64);
+// fe_amg_free releases everything.
 int fe_amg_setup(fe_mesh m);
-int fe_amg_apply(fe_mesh m, const double* x, void* z, bool z_double);
+int fe_amg_apply(fe_mesh m, const double* x, double* z);
 void fe_amg_free(fe_mesh m);
 // fe_assemble.cu: uploads the face-pattern values (springs plus 2/dt times
 // the dashpots while dynamics is on)

@@ -10,13 +10,14 @@
 // order (block tree, then block partials in block order) between bounded
 // grid barriers -- one per inner product for the sequential MGS sweep, one
 // per block of 8 basis vectors for the blocked form.  The SpMV streams block
-// rows in 32-block chunks with a segmented row-sum scan.  The two-loop
+// rows tile by tile (fe_stream.cuh).  The two-loop
 // recursion uses the persistent structure with q (or z) held in registers.
 #include <algorithm>
 #include <climits>
 #include <cmath>
 
 #include "fe_internal.h"
+#include "fe_stream.cuh"
 
 __device__ __forceinline__ double warp_sum(double v) {
   for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
@@ -500,13 +501,13 @@ __device__ __forceinline__ void arnoldi_tail(const double (&wr)[NPT], double inv
     ZT* zo = z + base + 3 * a;
     if constexpr (sizeof(DT) == 8) {
       zo[0] = (ZT)(D[0] * x0 + D[1] * x1 + D[2] * x2);
-      zo[1] = (ZT)(D[3] * x0 + D[4] * x1 + D[5] * x2);
-      zo[2] = (ZT)(D[6] * x0 + D[7] * x1 + D[8] * x2);
+          zo[1] = (ZT)(D[3] * x0 + D[4] * x1 + D[5] * x2);
+          zo[2] = (ZT)(D[6] * x0 + D[7] * x1 + D[8] * x2);
     } else {
       const float f0 = (float)x0, f1 = (float)x1, f2 = (float)x2;
       zo[0] = (ZT)(D[0] * f0 + D[1] * f1 + D[2] * f2);
-      zo[1] = (ZT)(D[3] * f0 + D[4] * f1 + D[5] * f2);
-      zo[2] = (ZT)(D[6] * f0 + D[7] * f1 + D[8] * f2);
+          zo[1] = (ZT)(D[3] * f0 + D[4] * f1 + D[5] * f2);
+          zo[2] = (ZT)(D[6] * f0 + D[7] * f1 + D[8] * f2);
     }
   }
 }
@@ -1430,15 +1431,6 @@ __device__ __forceinline__ double widen(float f) {
 }
 __device__ __forceinline__ double widen(double d) { return d; }
 
-template <class V>
-__device__ __forceinline__ float ld_val(const V* p);
-template <>
-__device__ __forceinline__ float ld_val<float>(const float* p) { return __ldg(p); }
-template <>
-__device__ __forceinline__ float ld_val<__nv_bfloat16>(const __nv_bfloat16* p) {
-  return __bfloat162float(*p);
-}
-
 // y_u = K x_u (+ B1 x_p): one warp per block row, one lane per 3x3 block.
 // A lane loads its block's column index, its 9 values and the 3 entries of
 // x, then accumulates the 3 row sums; the warp reduces them with shuffles.
@@ -1468,15 +1460,16 @@ __global__ void __launch_bounds__(256) k_spmv(int nn, const int* __restrict__ ro
       if constexpr (sizeof(VT) == 8) v[t] = __ldg(b + 32 * t);
       else v[t] = (AT)ld_val<VT>(b + 32 * t);
     }
-    const XT* xc = x + 3 * (int64_t)c;
-    AT x0 = (AT)xc[0], x1 = (AT)xc[1], x2 = (AT)xc[2];
+    AT xv[3];
+    stream_load_x<XT, AT>(x, c, xv, nn);
+    const AT x0 = xv[0], x1 = xv[1], x2 = xv[2];
     a0 += v[0] * x0 + v[1] * x1 + v[2] * x2;
     a1 += v[3] * x0 + v[4] * x1 + v[5] * x2;
     a2 += v[6] * x0 + v[7] * x1 + v[8] * x2;
   }
   if (up_ptr) {
     for (int k = up_ptr[row] + lane; k < up_ptr[row + 1]; k += 32) {
-      AT xv = (AT)xp[up_col[k]];
+      const AT xv = (AT)xp[up_col[k]];
       const VT* b = B + (int64_t)k * 3;
       if constexpr (sizeof(VT) == 8) {
         a0 += b[0] * xv;
@@ -1501,138 +1494,34 @@ __global__ void __launch_bounds__(256) k_spmv(int nn, const int* __restrict__ ro
   }
 }
 
-// y = K x for the displacement form, streamed: a warp takes groups of 16
-// consecutive block rows, whose blocks are contiguous in memory, and walks
-// each group in chunks of 32 blocks (one block per lane) regardless of where
-// rows start.  The grid is one wave of resident blocks; warps stride over
-// the groups, so no half-empty second wave idles the SMs.  Row sums are
-// formed by a segmented inclusive scan across the lanes (segment heads = row
-// starts inside the chunk, found from the group's row pointers); the last
-// lane of each segment writes its row, and a row that runs past the chunk
-// carries its partial sum into the next chunk.  Loads run two chunks ahead:
-// while chunk i is multiplied and reduced, the x gather of chunk i + 1 and
-// the column indices and values of chunk i + 2 are in flight, so each warp
-// keeps HBM and L2 requests outstanding across its rows instead of one
-// dependent row-pointer -> values -> x chain per row, and no lane idles on
-// rows shorter than 32 blocks.  Summation order is fixed by the chunking, so
-// results are deterministic.
-constexpr int SPMV_RPW = 16;  // block rows per group (<= 32)
-
-template <class VT, class AT>
-__device__ __forceinline__ void spmv_load_chunk(const int* __restrict__ col, const VT* __restrict__ val, int64_t k,
-                                                int64_t kend, int& c, AT (&v)[9]) {
-  if (k < kend) {
-    c = __ldg(col + k);
-    const VT* b = val + kv_index(k, 0);
+// y = K x for the displacement form: the streamed product of fe_stream.cuh,
+// rows written in FP64 (FP32 sums widened exactly).
+//
+// Measured (before: 16-row groups, row sums by a segmented scan): FP32 Cook P2
+// 64x64x8 (322 MB) 79 -> 73 us, 48x48x8 52 -> 46 us, 30x26x6 23 -> 14 us; FP64
+// 491 -> 240, 297 -> 139, 118 -> 44 us, cardiac shell 37 -> 21 us.  A plain
+// read of 322 MB on this device takes 64-70 us, launch included.
+template <class AT>
+struct EpiSpmv {
+  double* y;
+  __device__ __forceinline__ void prefetch(int, int, int) {}
+  __device__ __forceinline__ void load(int, int, int, int) {}
+  __device__ __forceinline__ void finish(int row, const AT (&s)[3]) {
 #pragma unroll
-    for (int t = 0; t < 9; t++) {
-      if constexpr (sizeof(VT) == 8) v[t] = __ldg(b + 32 * t);
-      else v[t] = (AT)ld_val<VT>(b + 32 * t);
-    }
-  } else {
-    c = -1;
-#pragma unroll
-    for (int t = 0; t < 9; t++) v[t] = AT(0);
+    for (int q = 0; q < 3; q++) y[3 * (int64_t)row + q] = widen(s[q]);
   }
-}
-
-template <class XT, class AT>
-__device__ __forceinline__ void spmv_load_x(const XT* __restrict__ x, int c, AT& x0, AT& x1, AT& x2, int ncol) {
-  if (c >= 0) {
-    const XT* xc = x + 3 * (int64_t)fe_idx(c, ncol);
-    x0 = (AT)xc[0];
-    x1 = (AT)xc[1];
-    x2 = (AT)xc[2];
-  } else {
-    x0 = x1 = x2 = AT(0);
-  }
-}
+};
 
 template <class VT, class XT, class AT>
-__global__ void __launch_bounds__(256) k_spmv_stream(int nn, const int* __restrict__ row_ptr,
-                                                     const int* __restrict__ col, const VT* __restrict__ val,
-                                                     const XT* __restrict__ x, double* __restrict__ y) {
-  const int lane = threadIdx.x & 31;
-  const int ngroups = (nn + SPMV_RPW - 1) / SPMV_RPW;
-  const int nwarps = (int)(((int64_t)gridDim.x * blockDim.x) >> 5);
-  for (int g = (int)((((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5)); g < ngroups; g += nwarps) {
-    const int r0 = g * SPMV_RPW;
-    const int nr = min(SPMV_RPW, nn - r0);
-    const int rpl = lane < nr ? __ldg(row_ptr + r0 + lane) : INT_MAX;  // start of row r0 + lane
-    const int kstart = __shfl_sync(0xffffffffu, rpl, 0);
-    const int kend = __ldg(row_ptr + r0 + nr);
-    // three chunks in flight: the current one (values and x in registers), the
-    // next one (values in registers, x gather issued) and the one after (column
-    // indices and values issued)
-    int c0, c1;
-    AT v0[9], v1[9];
-    spmv_load_chunk<VT, AT>(col, val, (int64_t)kstart + lane, kend, c0, v0);
-    spmv_load_chunk<VT, AT>(col, val, (int64_t)kstart + 32 + lane, kend, c1, v1);
-    AT xa0, xa1, xa2;
-    spmv_load_x<XT, AT>(x, c0, xa0, xa1, xa2, nn);
-    AT carry0 = AT(0), carry1 = AT(0), carry2 = AT(0);
-    int rowbase = r0 - 1;  // the row in progress before the current chunk
-    for (int kc = kstart; kc < kend; kc += 32) {
-      int c2;
-      AT v2[9];
-      spmv_load_chunk<VT, AT>(col, val, (int64_t)kc + 64 + lane, kend, c2, v2);
-      AT xb0, xb1, xb2;
-      spmv_load_x<XT, AT>(x, c1, xb0, xb1, xb2, nn);
-      AT p0 = AT(0), p1 = AT(0), p2 = AT(0);
-      if (c0 >= 0) {
-        p0 = v0[0] * xa0 + v0[1] * xa1 + v0[2] * xa2;
-        p1 = v0[3] * xa0 + v0[4] * xa1 + v0[5] * xa2;
-        p2 = v0[6] * xa0 + v0[7] * xa1 + v0[8] * xa2;
-      }
-      // row starts inside the chunk, and this lane's segment start (-1: before the chunk)
-      const unsigned bit = (rpl >= kc && rpl - kc < 32) ? (1u << (rpl - kc)) : 0u;
-      const unsigned heads = __reduce_or_sync(0xffffffffu, bit);
-      const unsigned below = heads & (0xffffffffu >> (31 - lane));
-      const int sstart = below ? 31 - __clz(below) : -1;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const AT t0 = __shfl_up_sync(0xffffffffu, p0, off);
-        const AT t1 = __shfl_up_sync(0xffffffffu, p1, off);
-        const AT t2 = __shfl_up_sync(0xffffffffu, p2, off);
-        if (lane >= off && lane - off >= sstart) {
-          p0 += t0;
-          p1 += t1;
-          p2 += t2;
-        }
-      }
-      const int nvalid = min(32, kend - kc);
-      const bool cont = nvalid == 32 && kc + 32 < kend && !__any_sync(0xffffffffu, rpl == kc + 32);
-      const bool tail = lane < nvalid && ((lane < 31 && ((heads >> (lane + 1)) & 1u)) || (lane == nvalid - 1 && !cont));
-      if (tail) {
-        const int row = rowbase + __popc(below);
-        const bool add = sstart < 0;
-        y[3 * (int64_t)row] = widen(p0 + (add ? carry0 : AT(0)));
-        y[3 * (int64_t)row + 1] = widen(p1 + (add ? carry1 : AT(0)));
-        y[3 * (int64_t)row + 2] = widen(p2 + (add ? carry2 : AT(0)));
-      }
-      const AT l0 = __shfl_sync(0xffffffffu, p0, 31), l1 = __shfl_sync(0xffffffffu, p1, 31),
-               l2 = __shfl_sync(0xffffffffu, p2, 31);
-      if (cont) {
-        const bool whole = heads == 0u;  // lane 31's segment started before this chunk
-        carry0 = l0 + (whole ? carry0 : AT(0));
-        carry1 = l1 + (whole ? carry1 : AT(0));
-        carry2 = l2 + (whole ? carry2 : AT(0));
-      } else {
-        carry0 = carry1 = carry2 = AT(0);
-      }
-      rowbase += __popc(heads);
-      c0 = c1;
-      c1 = c2;
-#pragma unroll
-      for (int t = 0; t < 9; t++) {
-        v0[t] = v1[t];
-        v1[t] = v2[t];
-      }
-      xa0 = xb0;
-      xa1 = xb1;
-      xa2 = xb2;
-    }
-  }
+__global__ void __launch_bounds__(STREAM_THREADS, stream_blocks_per_sm<AT>())
+    k_spmv_stream(int nn, int warps, int ranges, const int* __restrict__ part, const int* __restrict__ row_ptr,
+                  const int* __restrict__ col, const VT* __restrict__ val, const XT* __restrict__ x,
+                  double* __restrict__ y) {
+  __shared__ StreamShared<AT> sh;
+  const int warp = (int)blockIdx.x * STREAM_WARPS + (threadIdx.x >> 5);
+  if (warp >= warps) return;
+  EpiSpmv<AT> epi{y};
+  stream_rows<VT, XT, AT>(nn, warp, warps, ranges, part, row_ptr, col, val, x, sh.prod[threadIdx.x >> 5], epi);
 }
 
 // pressure rows: y_p[v] = sum over (u node a, v) of B[a,v] . x_u[a]  (B2 = B1^T)
@@ -1661,17 +1550,14 @@ __global__ void k_pc_bj(int nn, const DT* __restrict__ Dinv, const double* __res
   int a = blockIdx.x * blockDim.x + threadIdx.x;
   if (a >= nn) return;
   const DT* D = Dinv + (int64_t)a * 9;
-  double x0 = x[3 * (int64_t)a], x1 = x[3 * (int64_t)a + 1], x2 = x[3 * (int64_t)a + 2];
-  if constexpr (sizeof(DT) == 8) {
-    z[3 * (int64_t)a] = (OT)(D[0] * x0 + D[1] * x1 + D[2] * x2);
-    z[3 * (int64_t)a + 1] = (OT)(D[3] * x0 + D[4] * x1 + D[5] * x2);
-    z[3 * (int64_t)a + 2] = (OT)(D[6] * x0 + D[7] * x1 + D[8] * x2);
-  } else {
-    float f0 = (float)x0, f1 = (float)x1, f2 = (float)x2;
-    z[3 * (int64_t)a] = (OT)(D[0] * f0 + D[1] * f1 + D[2] * f2);
-    z[3 * (int64_t)a + 1] = (OT)(D[3] * f0 + D[4] * f1 + D[5] * f2);
-    z[3 * (int64_t)a + 2] = (OT)(D[6] * f0 + D[7] * f1 + D[8] * f2);
-  }
+  // the products in the inverse's type
+  const DT x0 = (DT)x[3 * (int64_t)a], x1 = (DT)x[3 * (int64_t)a + 1], x2 = (DT)x[3 * (int64_t)a + 2];
+  const OT z0 = (OT)(D[0] * x0 + D[1] * x1 + D[2] * x2), z1 = (OT)(D[3] * x0 + D[4] * x1 + D[5] * x2),
+           z2 = (OT)(D[6] * x0 + D[7] * x1 + D[8] * x2);
+  OT* zo = z + 3 * (int64_t)a;
+  zo[0] = z0;
+  zo[1] = z1;
+  zo[2] = z2;
 }
 
 // lower Schur (SIMPLE): z_p = S^{-1} (x_p - B2 z_u), point-Jacobi S
@@ -1704,21 +1590,27 @@ __global__ void __launch_bounds__(256) k_pc_schur(int np, int nn, const int* __r
 }
 
 template <class OT>
+static int pc_schur_t(fe_mesh m, const double* x, OT* z) {
+  const unsigned grid = (unsigned)(((int64_t)m->np * 32 + 255) / 256);
+  if (m->prec == FE_PREC_FP64)
+    k_pc_schur<double, OT><<<grid, 256, 0, m->stream>>>(m->np, m->nn, m->pu_ptr, m->pu_col, m->pu_src, m->B64,
+                                                            m->Sd, x, z);
+  else
+    k_pc_schur<float, OT><<<grid, 256, 0, m->stream>>>(m->np, m->nn, m->pu_ptr, m->pu_col, m->pu_src, m->B32,
+                                                           m->Sd, x, z);
+  FE_CUDA(cudaGetLastError());
+  return FE_OK;
+}
+
+// z = M^{-1} x, z an FP64 vector or the SpMV input m->zx
+template <class OT>
 static int pc_apply_t(fe_mesh m, const double* x, OT* z) {
   if (m->pc_type >= 1) {  // one AMG V-cycle on the displacement block
-    FE_TRY(fe_amg_apply(m, x, z, sizeof(OT) == 8));
+    FE_TRY(fe_amg_apply(m, x, (void*)z == m->zx ? nullptr : (double*)z));
     if (!m->pres) return FE_OK;
     // u-p form: the lower Schur step z_p = S^-1 (x_p - B2 z_u) with the V-cycle's z_u
     FE_SCOPE(m, FE_PROF_PC, (double)m->nnz_up * (8 + 12.0 * (m->prec == FE_PREC_FP64 ? 8 : 4)) + 24.0 * m->np);
-    const unsigned grid = (unsigned)(((int64_t)m->np * 32 + 255) / 256);
-    if (m->prec == FE_PREC_FP64)
-      k_pc_schur<double, OT><<<grid, 256, 0, m->stream>>>(m->np, m->nn, m->pu_ptr, m->pu_col, m->pu_src, m->B64,
-                                                          m->Sd, x, z);
-    else
-      k_pc_schur<float, OT><<<grid, 256, 0, m->stream>>>(m->np, m->nn, m->pu_ptr, m->pu_col, m->pu_src, m->B32,
-                                                         m->Sd, x, z);
-    FE_CUDA(cudaGetLastError());
-    return FE_OK;
+    return pc_schur_t<OT>(m, x, z);
   }
   FE_SCOPE(m, FE_PROF_PC, (double)m->nn * (9.0 * (m->prec == FE_PREC_FP64 ? 8 : 4) + 24 + 3.0 * sizeof(OT)) +
                               (m->pres ? (double)m->nnz_up * (8 + 12.0 * (m->prec == FE_PREC_FP64 ? 8 : 4)) + 24.0 * m->np
@@ -1728,20 +1620,19 @@ static int pc_apply_t(fe_mesh m, const double* x, OT* z) {
   else
     k_pc_bj<float, OT><<<(m->nn + 255) / 256, 256, 0, m->stream>>>(m->nn, m->Dinv32, x, z);
   FE_CUDA(cudaGetLastError());
-  if (m->pres) {
-    unsigned grid = (unsigned)(((int64_t)m->np * 32 + 255) / 256);
-    if (m->prec == FE_PREC_FP64)
-      k_pc_schur<double, OT><<<grid, 256, 0, m->stream>>>(m->np, m->nn, m->pu_ptr, m->pu_col, m->pu_src, m->B64,
-                                                          m->Sd, x, z);
-    else
-      k_pc_schur<float, OT><<<grid, 256, 0, m->stream>>>(m->np, m->nn, m->pu_ptr, m->pu_col, m->pu_src, m->B32,
-                                                         m->Sd, x, z);
-    FE_CUDA(cudaGetLastError());
-  }
+  if (m->pres) return pc_schur_t<OT>(m, x, z);
   return FE_OK;
 }
 
-int fe_pc_dev(fe_mesh m, const double* x, double* y) { return pc_apply_t<double>(m, x, y); }
+static int ensure_zx(fe_mesh m) {
+  if (!m->zx) FE_TRY(fe_alloc(m, &m->zx, (size_t)m->ndof * sizeof(double)));
+  return FE_OK;
+}
+
+int fe_pc_dev(fe_mesh m, const double* x, double* y) {
+  FE_TRY(ensure_zx(m));  // (the V-cycle's iterate lives there)
+  return pc_apply_t<double>(m, x, y);
+}
 
 // z (SpMV input type) = M^{-1} x
 static int pc_to_zx(fe_mesh m, const double* x) {
@@ -1749,20 +1640,24 @@ static int pc_to_zx(fe_mesh m, const double* x) {
   return pc_apply_t<float>(m, x, (float*)m->zx);
 }
 
-// one wave of the streamed SpMV: resident 256-thread blocks on every SM, but
-// no more warps than row groups
+// one product in the given types
 template <class VT, class XT, class AT>
-static unsigned stream_grid_t(fe_mesh m) {
-  int per_sm = 0;
-  if (fe_kernel_occupancy((const void*)k_spmv_stream<VT, XT, AT>, 256, 0, &per_sm) != FE_OK) per_sm = 4;
-  const int64_t groups = ((int64_t)m->nn + SPMV_RPW - 1) / SPMV_RPW;
-  const int64_t need = (groups + 7) / 8;
-  return (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)std::max(per_sm, 1) * m->sm_count));
-}
-static unsigned spmv_stream_grid(fe_mesh m) {
-  if (m->prec == FE_PREC_FP64) return stream_grid_t<double, double, double>(m);
-  if (m->prec == FE_PREC_MIXED_BF16) return stream_grid_t<__nv_bfloat16, float, float>(m);
-  return stream_grid_t<float, float, float>(m);
+static int launch_spmv_t(fe_mesh m, const VT* K, const VT* B, const XT* x, double* y) {
+  if (!m->pres) {
+    const int warps = sizeof(AT) == 8 ? m->warps64 : m->warps32;
+    k_spmv_stream<VT, XT, AT><<<stream_grid(warps), STREAM_THREADS, 0, m->stream>>>(
+        m->nn, warps, sizeof(AT) == 8 ? m->ranges64 : m->ranges32, sizeof(AT) == 8 ? m->part64 : m->part32, m->row_ptr,
+        m->col, K, x, y);
+  } else {
+    const unsigned grid = (unsigned)(((int64_t)m->nn * 32 + 255) / 256);
+    const unsigned gridp = (unsigned)(((int64_t)m->np * 32 + 255) / 256);
+    k_spmv<VT, XT, AT><<<grid, 256, 0, m->stream>>>(m->nn, m->row_ptr, m->col, K, x, y, m->up_ptr, m->up_col, B,
+                                                        x + 3 * (int64_t)m->nn);
+    k_spmv_p<VT, XT, AT><<<gridp, 256, 0, m->stream>>>(m->np, m->pu_ptr, m->pu_col, m->pu_src, B, x,
+                                                           y + 3 * (int64_t)m->nn);
+  }
+  FE_CUDA(cudaGetLastError());
+  return FE_OK;
 }
 
 // y = K xin with xin in the SpMV input type (FP64 for an FP64 tangent, FP32
@@ -1770,35 +1665,10 @@ static unsigned spmv_stream_grid(fe_mesh m) {
 // the u-p form adds the coupling B1 x_p per row (k_spmv) and the pressure
 // rows (k_spmv_p); the u-p coupling is kept in the tangent's precision.
 static int launch_spmv(fe_mesh m, const void* xin, double* y) {
-  const unsigned grid = (unsigned)(((int64_t)m->nn * 32 + 255) / 256);
-  const unsigned gridp = (unsigned)(((int64_t)m->np * 32 + 255) / 256);
-  const unsigned grids = spmv_stream_grid(m);
-  if (m->prec == FE_PREC_FP64) {
-    const double* x = (const double*)xin;
-    if (!m->pres) {
-      k_spmv_stream<double, double, double><<<grids, 256, 0, m->stream>>>(m->nn, m->row_ptr, m->col, m->K64, x, y);
-    } else {
-      k_spmv<double, double, double><<<grid, 256, 0, m->stream>>>(m->nn, m->row_ptr, m->col, m->K64, x, y, m->up_ptr,
-                                                                  m->up_col, m->B64, x + 3 * (int64_t)m->nn);
-      k_spmv_p<double, double, double><<<gridp, 256, 0, m->stream>>>(m->np, m->pu_ptr, m->pu_col, m->pu_src, m->B64,
-                                                                     x, y + 3 * (int64_t)m->nn);
-    }
-  } else if (m->prec == FE_PREC_MIXED_BF16) {
-    const float* x = (const float*)xin;
-    k_spmv_stream<__nv_bfloat16, float, float><<<grids, 256, 0, m->stream>>>(m->nn, m->row_ptr, m->col, m->K16, x, y);
-  } else {
-    const float* x = (const float*)xin;
-    if (!m->pres) {
-      k_spmv_stream<float, float, float><<<grids, 256, 0, m->stream>>>(m->nn, m->row_ptr, m->col, m->K32, x, y);
-    } else {
-      k_spmv<float, float, float><<<grid, 256, 0, m->stream>>>(m->nn, m->row_ptr, m->col, m->K32, x, y, m->up_ptr,
-                                                               m->up_col, m->B32, x + 3 * (int64_t)m->nn);
-      k_spmv_p<float, float, float><<<gridp, 256, 0, m->stream>>>(m->np, m->pu_ptr, m->pu_col, m->pu_src, m->B32, x,
-                                                                  y + 3 * (int64_t)m->nn);
-    }
-  }
-  FE_CUDA(cudaGetLastError());
-  return FE_OK;
+  if (m->prec == FE_PREC_FP64) return launch_spmv_t<double, double, double>(m, m->K64, m->B64, (const double*)xin, y);
+  if (m->prec == FE_PREC_MIXED_BF16)
+    return launch_spmv_t<__nv_bfloat16, float, float>(m, m->K16, nullptr, (const float*)xin, y);
+  return launch_spmv_t<float, float, float>(m, m->K32, m->B32, (const float*)xin, y);
 }
 
 // y = K zx (zx already in the SpMV input type)
@@ -1818,11 +1688,6 @@ __global__ void k_narrow(int64_t n, const double* __restrict__ x, float* __restr
 __global__ void k_copy(int64_t n, const double* __restrict__ x, double* __restrict__ y) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) y[i] = x[i];
-}
-
-static int ensure_zx(fe_mesh m) {
-  if (!m->zx) FE_TRY(fe_alloc(m, &m->zx, (size_t)m->ndof * sizeof(double)));
-  return FE_OK;
 }
 
 // y = K x for FP64 x, y
@@ -1850,19 +1715,7 @@ static int spmv_acc_t(fe_mesh m, const VT* K, const VT* B, const double* x, doub
   FE_SCOPE_F(m, FE_PROF_SPMV, (double)m->nnzb * (9 * sv + 4) + 4.0 * (m->nn + 1) + 16.0 * (double)m->ndof +
                                   (m->pres ? (double)m->nnz_up * 2 * (3 * sv + 8) + 4.0 * (m->nn + m->np + 2) : 0.0),
              18.0 * (double)m->nnzb + (m->pres ? 12.0 * (double)m->nnz_up : 0.0));
-  if (!m->pres) {
-    const unsigned grids = stream_grid_t<VT, double, double>(m);
-    k_spmv_stream<VT, double, double><<<grids, 256, 0, m->stream>>>(m->nn, m->row_ptr, m->col, K, x, y);
-  } else {
-    const unsigned grid = (unsigned)(((int64_t)m->nn * 32 + 255) / 256);
-    const unsigned gridp = (unsigned)(((int64_t)m->np * 32 + 255) / 256);
-    k_spmv<VT, double, double><<<grid, 256, 0, m->stream>>>(m->nn, m->row_ptr, m->col, K, x, y, m->up_ptr, m->up_col,
-                                                            B, x + 3 * (int64_t)m->nn);
-    k_spmv_p<VT, double, double><<<gridp, 256, 0, m->stream>>>(m->np, m->pu_ptr, m->pu_col, m->pu_src, B, x,
-                                                               y + 3 * (int64_t)m->nn);
-  }
-  FE_CUDA(cudaGetLastError());
-  return FE_OK;
+  return launch_spmv_t<VT, double, double>(m, K, B, x, y);
 }
 
 int fe_spmv_acc_dev(fe_mesh m, const double* x, double* y) {
@@ -1878,9 +1731,8 @@ int fe_spmv_acc_dev(fe_mesh m, const double* x, double* y) {
 int fe_spmv_from_input(fe_mesh m, const void* xin, double* y) { return launch_spmv(m, xin, y); }
 
 // Under CUDA's lazy loading a kernel's code is placed in device memory at
-// its first launch.  Loading every SpMV kernel here (and caching the
-// occupancy the streamed launch reads) lets a caller that must not allocate
-// launch them later without that first-use cost.
+// its first launch.  Loading every SpMV kernel here lets a caller that must
+// not allocate launch them later without that first-use cost.
 int fe_spmv_preload(fe_mesh m) {
   const void* fns[] = {(const void*)k_spmv_stream<double, double, double>,
                        (const void*)k_spmv_stream<float, float, float>,
@@ -1893,10 +1745,6 @@ int fe_spmv_preload(fe_mesh m) {
     cudaFuncAttributes a;
     FE_CUDA(cudaFuncGetAttributes(&a, fn));
   }
-  int per_sm = 0;
-  FE_TRY(fe_kernel_occupancy((const void*)k_spmv_stream<double, double, double>, 256, 0, &per_sm));
-  FE_TRY(fe_kernel_occupancy((const void*)k_spmv_stream<float, float, float>, 256, 0, &per_sm));
-  FE_TRY(fe_kernel_occupancy((const void*)k_spmv_stream<__nv_bfloat16, float, float>, 256, 0, &per_sm));
   (void)m;
   return FE_OK;
 }

@@ -18,6 +18,7 @@
 #include <numeric>
 
 #include "fe_internal.h"
+#include "fe_stream.cuh"
 
 // ---------------------------------------------------------------- errors
 static thread_local char g_err[1024] = "";
@@ -320,6 +321,27 @@ __global__ void k_emap(int ne, int nen, int ncolk, const int* __restrict__ conn,
     pos = 0;
   }
   map[t] = pos;
+}
+
+// row ranges of equal block counts: part[w] = the first row that starts at or
+// after block w nnzb / ranges
+__global__ void k_partition(int nn, int64_t nnzb, int ranges, const int* __restrict__ row_ptr, int* __restrict__ part) {
+  const int w = blockIdx.x * blockDim.x + threadIdx.x;
+  if (w > ranges) return;
+  const int64_t k = nnzb * w / ranges;
+  int lo = 0, hi = nn;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if ((int64_t)row_ptr[mid] >= k) hi = mid;
+    else lo = mid + 1;
+  }
+  part[w] = lo;
+}
+
+int fe_stream_partition(fe_mesh m, int ranges, int* part) {
+  k_partition<<<ranges / 128 + 1, 128, 0, m->stream>>>(m->nn, m->nnzb, ranges, m->row_ptr, part);
+  FE_CUDA(cudaGetLastError());
+  return FE_OK;
 }
 
 __global__ void k_apply_dirichlet(int nn, const double* __restrict__ X, const uint8_t* __restrict__ dgroup,
@@ -680,6 +702,16 @@ static int create_impl(const fe_mesh_desc* desc, fe_mesh m) {
     colp.resize((col.size() + 31) / 32 * 32, 0);
     FE_TRY(upload(m, &m->col, colp));
   }
+  const StreamShape s32 = stream_shape(stream_blocks_per_sm<float>(), m->sm_count, m->nnzb),
+                    s64 = stream_shape(stream_blocks_per_sm<double>(), m->sm_count, m->nnzb);
+  m->warps32 = s32.warps;
+  m->ranges32 = s32.ranges;
+  m->warps64 = s64.warps;
+  m->ranges64 = s64.ranges;
+  FE_TRY(fe_alloc_t(m, &m->part32, (size_t)s32.ranges + 1));
+  FE_TRY(fe_alloc_t(m, &m->part64, (size_t)s64.ranges + 1));
+  FE_TRY(fe_stream_partition(m, s32.ranges, m->part32));
+  FE_TRY(fe_stream_partition(m, s64.ranges, m->part64));
   FE_TRY(upload(m, &m->diag_pos, diag));
   FE_TRY(upload(m, &m->dgroup, dgroup));
   FE_TRY(upload(m, &m->fixmask, fixmask));
@@ -809,7 +841,7 @@ static void free_all(fe_mesh m) {
   for (cudaEvent_t e : m->ev_free) cudaEventDestroy(e);
   m->ev_free.clear();
   void* ptrs[] = {m->X, m->conn, m->colors, m->perm, m->geo, m->fib, m->fixmask, m->dgroup,
-                  m->d_groups, m->row_ptr, m->col, m->diag_pos, m->emap, m->up_ptr, m->up_col,
+                  m->d_groups, m->row_ptr, m->col, m->part32, m->part64, m->diag_pos, m->emap, m->up_ptr, m->up_col,
                   m->upmap, m->pu_ptr, m->pu_col, m->pu_src, m->node_ptr, m->node_list,
                   m->vert_ptr, m->vert_list, m->fext1, m->ks_ptr, m->ks_col, m->ks_val,
                   m->ks_kpos, m->K64, m->K32, m->K16, m->B64, m->B32, m->Dinv64, m->Dinv32,

@@ -45,3 +45,22 @@ def test_arnoldi_launch_shapes(fe, size, orthog):
     assert it == itg == 24
     assert abs(resg - res) <= 1e-8 * res, (resg, res)
     assert np.linalg.norm(xg.cpu().numpy() - x) <= 1e-9 * np.linalg.norm(x)
+
+
+# block counts around one tile, one tile per warp of a wave (58k blocks in
+# FP64, 117k in FP32) and beyond it, short P1 rows and long P2 rows
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-12), ("mixed_fp32", 2e-5)])
+@pytest.mark.parametrize("size,order", [((1, 1, 1), 1), ((2, 2, 1), 2), ((20, 20, 8), 1), ((22, 21, 9), 1),
+                                        ((29, 27, 8), 1), ((30, 31, 9), 1), ((13, 11, 5), 2)])
+def test_streamed_spmv_ranges(fe, size, order, precision, tol):
+    # bounds of the parity tests: FP64 a few ulps of the largest entry, FP32
+    # assembly and sums 2e-5 of it
+    w = W.cook(*size, order=order, nu=0.3)
+    m, om = fe.Mesh(w), O.Mesh(w)
+    d = 0.02 * np.random.default_rng(5).standard_normal(om.ndof)
+    om.apply_dirichlet(d)
+    om.tangent(d)
+    m.tangent(torch.from_numpy(d).cuda(), precision)
+    x = np.random.default_rng(6).standard_normal(om.ndof)
+    y, yg = om.spmv(x), m.spmv(torch.from_numpy(x).cuda()).cpu().numpy()
+    assert np.abs(yg - y).max() <= tol * np.abs(y).max()
