@@ -527,22 +527,25 @@ def serve_mix(nreq, max_dofs, slots, batch_dofs, rate, precision, restart, ortho
     return out
 
 
-VC_BOTTOM_MAXN = 256  # nodes per level that the one-block bottom of the V-cycle takes
+VC_BOTTOM_MAXN = 256  # nodes per level that the one-block bottom of the V-cycle takes at most (block counts unknown)
+VC_BOTTOM_MAXNNZ = 640  # blocks per level that it takes
 
 
-def vcycle_kernels(sizes):
+def vcycle_kernels(sizes, blocks=None):
     """Kernels in one launch of the V-cycle's CUDA graph for AMG levels of
     `sizes` nodes (the composition built by vcycle_launches in fe_amg.cu):
     k_vc_init0; per level above the bottom two Chebyshev steps and a
-    restriction; the one-block bottom (the levels of at most VC_BOTTOM_MAXN
-    nodes below level 0, when one of them is smoothed) or the coarsest
+    restriction; the one-block bottom (the levels of at most
+    VC_BOTTOM_MAXNNZ `blocks` below level 0, when one of them is smoothed;
+    by their nodes where `blocks` is not given; none in FP64, whose caller
+    passes infinite counts) or the coarsest
     solve; per level above the bottom a prolongation and two Chebyshev
     steps.  One level: a conversion and the dense solve."""
     L = len(sizes)
     if L <= 1:
         return 2
     q0 = L - 1
-    while q0 > 1 and sizes[q0 - 1] <= VC_BOTTOM_MAXN:
+    while q0 > 1 and (sizes[q0 - 1] <= VC_BOTTOM_MAXN if blocks is None else blocks[q0 - 1] <= VC_BOTTOM_MAXNNZ):
         q0 -= 1
     qf = q0 if q0 <= L - 2 else L - 1
     return 2 + 6 * qf
@@ -726,7 +729,9 @@ def main():
     pc_kernels = 1
     if args.pc in ("amg", "amg_bf16") and w["pressure_order"] == 0:
         try:
-            pc_kernels = vcycle_kernels(m.amg_sizes())
+            lv = m.amg_levels()
+            blocks = [int(l["ptr"][-1]) if args.precision != "fp64" and "ptr" in l else float("inf") for l in lv]
+            pc_kernels = vcycle_kernels([l["n"] for l in lv], blocks)
         except Exception:  # a count only: never fail the run over it
             pc_kernels = 1
     # only converged solves count (a solve that stops at max_it or diverges is

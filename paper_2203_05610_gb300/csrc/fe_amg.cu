@@ -63,7 +63,9 @@ constexpr int AMG_NS = 6;        // near null space vectors
 constexpr int AMG_DENSE_MAX = 96;
 constexpr int AMG_POWER_STEPS = 15;
 constexpr double AMG_QR_DROP = 1e-8;
-constexpr int AMG_RED_BLOCKS = 256;
+// one level's device scalars (AmgHier::scal): spectral radius, last sum of
+// squares, next scale factor, prolongator weight
+constexpr int SC_RHO = 0, SC_SS = 1, SC_F = 2, SC_OMEGA = 3, SC_N = 4;
 
 uint64_t mix64(uint64_t z) {  // splitmix64 (Steele, Lea and Flood; Vigna's constants)
   z += 0x9E3779B97F4A7C15ULL;
@@ -90,9 +92,16 @@ struct AmgLevel {
   int* own = nullptr;        // one allocation holding this level's int arrays
   unsigned char* absent = nullptr;
   int *agg = nullptr, *pptr = nullptr, *pcol = nullptr, *prow = nullptr;
+  int2* pk_ptr = nullptr;    // the blocks of each P entry (k_amg_plists), its place in R
+  int *pk = nullptr, *rpos = nullptr;
+  int64_t *apoff = nullptr, *raoff = nullptr;  // starts of each fine row's places, each coarse row's products below
+  int* apidx = nullptr;                   // places of the products in their A P row (k_amg_ap)
+  int2* ralist = nullptr;                 // (P entry, A P entry) of the products of each entry of A_{l+1} (k_amg_rap)
+  int64_t* lend = nullptr;                // their ends
+  int* crow = nullptr;                    // row of each entry of A_{l+1}
+  float* tnode32 = nullptr;               // tnode in FP32
   int *rptr = nullptr, *rcol = nullptr, *rsrc = nullptr;
-  int *apptr = nullptr, *apcol = nullptr, *aprow = nullptr;
-  int* crow = nullptr;       // row of each entry of A_l (level >= 1)
+  int *apptr = nullptr, *apcol = nullptr;
   double* tnode = nullptr;   // [n][b*6] tentative block of each node
   // numbers (device)
   double* val64 = nullptr;  // level >= 1: [nnz][b*b]
@@ -118,8 +127,9 @@ struct AmgHier {
   AmgLevel lev[AMG_MAXLEV];
   int vec_elem = 0;          // bytes per V-cycle vector element allocated (0: none yet)
   double* pw = nullptr;      // power iterations: x, y [2][max n*b]
-  double* part = nullptr;    // [2][AMG_RED_BLOCKS] partial sums
-  double* scal = nullptr;    // [4] rho, 1/|y|
+  double* part = nullptr;    // partial sums of a power step, one per block
+  unsigned* ticket = nullptr;
+  double* scal = nullptr;    // [AMG_MAXLEV][SC_N]
   std::vector<void*> allocs; // device buffers owned by the hierarchy
   int64_t bytes = 0;         // their size (counted in the mesh's device bytes)
   bool ready = false;        // numbers formed for the current tangent
@@ -148,6 +158,7 @@ struct HostLevel {
   std::vector<double> ns;  // [n*b][6]
   std::vector<int> agg, pptr, pcol, rptr, rcol, rsrc, apptr, apcol;
   std::vector<double> tnode;  // [n][b*6]
+  std::vector<int64_t> apoff, raoff;
 };
 
 uint8_t full_mask(int b) { return (uint8_t)((1u << b) - 1u); }
@@ -264,12 +275,14 @@ void coarsen(HostLevel& L, HostLevel& C) {
   // A P: row i takes the P rows of its neighbours
   L.apptr.assign(n + 1, 0);
   L.apcol.clear();
+  L.apoff.assign(n + 1, 0);
   for (int i = 0; i < n; i++) {
     tmp.clear();
     for (int k = L.ptr[i]; k < L.ptr[i + 1]; k++) {
       const int j = L.col[k];
       tmp.insert(tmp.end(), L.pcol.begin() + L.pptr[j], L.pcol.begin() + L.pptr[j + 1]);
     }
+    L.apoff[i + 1] = L.apoff[i] + (int64_t)tmp.size();
     sort_unique(tmp);
     L.apcol.insert(L.apcol.end(), tmp.begin(), tmp.end());
     L.apptr[i + 1] = (int)L.apcol.size();
@@ -288,6 +301,11 @@ void coarsen(HostLevel& L, HostLevel& C) {
         L.rcol[s] = i;
         L.rsrc[s] = q;
       }
+  }
+  L.raoff.assign(nc + 1, 0);
+  for (int a = 0; a < nc; a++) {
+    L.raoff[a + 1] = L.raoff[a];
+    for (int q = L.rptr[a]; q < L.rptr[a + 1]; q++) L.raoff[a + 1] += L.apptr[L.rcol[q] + 1] - L.apptr[L.rcol[q]];
   }
   // coarse pattern: row a takes the A P rows of its P^T row, and the diagonal
   C.ptr.assign(nc + 1, 0);
@@ -326,335 +344,405 @@ __device__ __forceinline__ T ldt(const V* p) {
   else return (T)__ldg(p);
 }
 
-// entry c of block k in the setup's arithmetic type C: level 0 reads the
-// tangent in its tiled layout, coarser levels their block-major values
+// a block-major 6x6 block with 16-byte loads (from a device allocation, so
+// 16-byte aligned)
+template <class T>
+__device__ __forceinline__ void load_block6(const T* val, int64_t k, T (&v)[AMG_NS * AMG_NS]) {
+  constexpr int N = AMG_NS * AMG_NS;
+  if constexpr (sizeof(T) == 4) {
+    const float4* p4 = reinterpret_cast<const float4*>(val + k * N);
+#pragma unroll
+    for (int t = 0; t < N / 4; t++) {
+      const float4 u = __ldg(p4 + t);
+      v[4 * t] = u.x;
+      v[4 * t + 1] = u.y;
+      v[4 * t + 2] = u.z;
+      v[4 * t + 3] = u.w;
+    }
+  } else {
+    const double2* p2 = reinterpret_cast<const double2*>(val + k * N);
+#pragma unroll
+    for (int t = 0; t < N / 2; t++) {
+      const double2 u = __ldg(p2 + t);
+      v[2 * t] = u.x;
+      v[2 * t + 1] = u.y;
+    }
+  }
+}
+
+// entry c of block k, or the whole block, in the setup's arithmetic type C:
+// level 0 (B = 3) reads the tangent in its tiled layout, coarser levels (B =
+// 6) their block-major values
 template <class C, class V, int B>
 struct Vals {
   const V* v;
-  bool tiled;
   __device__ __forceinline__ C operator()(int64_t k, int c) const {
-    return tiled ? ldt<C, V>(v + kv_index(k, c)) : ldt<C, V>(v + k * (B * B) + c);
+    return B == 3 ? ldt<C, V>(v + kv_index(k, c)) : ldt<C, V>(v + k * (B * B) + c);
+  }
+  __device__ __forceinline__ void block(int64_t k, C (&a)[B * B]) const {
+    if constexpr (B == 3) {
+#pragma unroll
+      for (int c = 0; c < 9; c++) a[c] = ldt<C, V>(v + kv_index(k, c));
+    } else {
+      load_block6<C>(v, k, a);
+    }
   }
 };
-
-__device__ __forceinline__ int find_col(const int* __restrict__ col, int lo, int hi, int c) {
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    const int v = __ldg(col + mid);
-    if (v == c) return mid;
-    if (v < c) lo = mid + 1;
-    else hi = mid;
-  }
-  return -1;
-}
-
-// inverse of a B x B matrix by Gauss-Jordan elimination with partial pivoting
-template <int B>
-__device__ void gj_inverse(double (&a)[B][B], double (&inv)[B][B]) {
-  for (int i = 0; i < B; i++)
-    for (int j = 0; j < B; j++) inv[i][j] = i == j ? 1.0 : 0.0;
-  for (int c = 0; c < B; c++) {
-    int p = c;
-    for (int r = c + 1; r < B; r++)
-      if (fabs(a[r][c]) > fabs(a[p][c])) p = r;
-    if (p != c)
-      for (int j = 0; j < B; j++) {
-        double t = a[c][j];
-        a[c][j] = a[p][j];
-        a[p][j] = t;
-        t = inv[c][j];
-        inv[c][j] = inv[p][j];
-        inv[p][j] = t;
-      }
-    const double piv = a[c][c];
-    for (int j = 0; j < B; j++) {
-      a[c][j] /= piv;
-      inv[c][j] /= piv;
-    }
-    for (int r = 0; r < B; r++) {
-      if (r == c) continue;
-      const double f = a[r][c];
-      if (f == 0.0) continue;
-      for (int j = 0; j < B; j++) {
-        a[r][j] -= f * a[c][j];
-        inv[r][j] -= f * inv[c][j];
-      }
-    }
-  }
-}
 
 // ---------------------------------------------------------------- numeric setup kernels
 // C is the setup's arithmetic type: FP64 for an FP64 tangent, FP32 for the
 // mixed forms (whose V-cycle runs in FP32; GB300's FP32 rate is tens of
-// times its FP64 rate).  The dense coarsest inverse is always formed in FP64.
-template <class C, class V, int B>
-__global__ void k_amg_dinv(int n, const int* __restrict__ diag, Vals<C, V, B> A, C* __restrict__ dinv) {
+// times its FP64 rate).  The block inverses and the dense coarsest inverse are
+// always formed in FP64, with one reciprocal per pivot (an FP64 division is
+// about 7 multiplications' issue time).
+template <class T>
+__device__ __forceinline__ void swap_if(bool s, T& a, T& b) {
+  const T t = a;
+  a = s ? b : a;
+  b = s ? t : b;
+}
+
+// level 0: one thread per 3x3 block, Gauss-Jordan in registers (fixed loops:
+// with run-time pivot indices the matrices lived in local memory, 82 us for
+// 160k blocks)
+template <class C, class V>
+__global__ void k_amg_dinv3(int n, const int* __restrict__ diag, Vals<C, V, 3> A, C* __restrict__ dinv) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  double a[B][B], inv[B][B];
+  double a[3][3], v[3][3];
   const int64_t k = diag[i];
-  for (int r = 0; r < B; r++)
-    for (int c = 0; c < B; c++) a[r][c] = (double)A(k, B * r + c);
-  gj_inverse<B>(a, inv);
-  for (int r = 0; r < B; r++)
-    for (int c = 0; c < B; c++) dinv[(int64_t)i * B * B + B * r + c] = (C)inv[r][c];
+#pragma unroll
+  for (int r = 0; r < 3; r++)
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+      a[r][c] = (double)A(k, 3 * r + c);
+      v[r][c] = r == c ? 1.0 : 0.0;
+    }
+#pragma unroll
+  for (int c = 0; c < 3; c++) {
+    int p = c;
+    double best = fabs(a[c][c]);
+#pragma unroll
+    for (int r = c + 1; r < 3; r++)
+      if (fabs(a[r][c]) > best) {
+        best = fabs(a[r][c]);
+        p = r;
+      }
+#pragma unroll
+    for (int r = c + 1; r < 3; r++)
+#pragma unroll
+      for (int j = 0; j < 3; j++) {
+        swap_if(p == r, a[c][j], a[r][j]);
+        swap_if(p == r, v[c][j], v[r][j]);
+      }
+    const double inv = 1.0 / a[c][c];
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+      if (j > c) a[c][j] *= inv;
+      v[c][j] *= inv;
+    }
+#pragma unroll
+    for (int r = 0; r < 3; r++) {
+      if (r == c) continue;
+      const double f = a[r][c];
+#pragma unroll
+      for (int j = 0; j < 3; j++) {
+        if (j > c) a[r][j] -= f * a[c][j];
+        v[r][j] -= f * v[c][j];
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 3; r++)
+#pragma unroll
+    for (int c = 0; c < 3; c++) dinv[(int64_t)i * 9 + 3 * r + c] = (C)v[r][c];
 }
 
-// y = D^-1 (A x), one warp per block row
-template <class C, class V, int B>
-__global__ void __launch_bounds__(256) k_amg_dmv(int n, const int* __restrict__ ptr, const int* __restrict__ col,
-                                                 Vals<C, V, B> A, const C* __restrict__ dinv,
-                                                 const C* __restrict__ x, C* __restrict__ y) {
-  const int row = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row >= n) return;
-  C s[B];
-  for (int r = 0; r < B; r++) s[r] = C(0);
-  for (int k = ptr[row] + lane; k < ptr[row + 1]; k += 32) {
-    const int c = col[k];
+// coarse levels: 16 lanes per 6x6 block, lane j < 12 holds column j of
+// [A | I]; the pivot column's entries reach the other lanes by shuffles
+template <class C, class V>
+__global__ void __launch_bounds__(128) k_amg_dinv6(int n, const int* __restrict__ diag, Vals<C, V, AMG_NS> A,
+                                                   C* __restrict__ dinv) {
+  constexpr int B = AMG_NS;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = min(t / 16, n - 1), j = t % 16;  // (the last blocks' spare lanes repeat block n - 1)
+  const int64_t k = diag[i];
+  double a[B];
+#pragma unroll
+  for (int r = 0; r < B; r++) a[r] = j < B ? (double)A(k, B * r + j) : (j - B == r ? 1.0 : 0.0);
+#pragma unroll
+  for (int c = 0; c < B; c++) {
+    // pivot row of column c (the first of the largest), found by lane c
+    int p = c;
+    double best = fabs(a[c]);
+#pragma unroll
+    for (int r = c + 1; r < B; r++)
+      if (fabs(a[r]) > best) {
+        best = fabs(a[r]);
+        p = r;
+      }
+    p = __shfl_sync(0xffffffffu, p, c, 16);
+#pragma unroll
+    for (int r = c + 1; r < B; r++) swap_if(p == r, a[c], a[r]);
+    double f[B];
+#pragma unroll
+    for (int r = 0; r < B; r++) f[r] = __shfl_sync(0xffffffffu, a[r], c, 16);
+    a[c] *= 1.0 / f[c];
+#pragma unroll
     for (int r = 0; r < B; r++)
-      for (int j = 0; j < B; j++) s[r] += A(k, B * r + j) * x[(int64_t)B * c + j];
+      if (r != c) a[r] -= f[r] * a[c];
   }
-  for (int r = 0; r < B; r++)
-    for (int off = 16; off > 0; off >>= 1) s[r] += __shfl_xor_sync(0xffffffffu, s[r], off);
-  if (lane == 0)
-    for (int r = 0; r < B; r++) {
-      C t = C(0);
-      for (int j = 0; j < B; j++) t += dinv[(int64_t)row * B * B + B * r + j] * s[j];
-      y[(int64_t)B * row + r] = t;
-    }
+  if (t / 16 < n && j >= B && j < 2 * B)
+#pragma unroll
+    for (int r = 0; r < B; r++) dinv[(int64_t)i * B * B + B * r + (j - B)] = (C)a[r];
 }
 
 template <class C>
-__global__ void k_amg_start(int64_t N, C* __restrict__ x) {
+__global__ void k_amg_start(int64_t N, C* __restrict__ x, double* __restrict__ scal) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k < N) x[k] = (C)((double)(mix64_d((uint64_t)k) >> 11) * (1.0 / 9007199254740992.0) - 0.5);
+  if (k == 0) {
+    scal[SC_F] = 1.0;
+    scal[SC_SS] = 1.0;
+  }
 }
 
-// partial sums of x.x and y.y over a fixed grid (fixed order: deterministic), in FP64
+// Power iteration on D^-1 A, rho = |y| / |x| of the last step.  A step is one
+// kernel: the product, D^-1, the sums of squares (FP64, one partial per block)
+// and, in the last block to finish, the sum of the partials in block order and
+// the next factor; the last step also leaves rho, the prolongator's omega and
+// the Chebyshev coefficients in device memory, so the host reads all levels'
+// radii once, after the whole setup.  (Before: three kernels per step, the
+// scaling one adding 512 partials in one thread of every block: 31-80 us.)
+//   FP64: x_{k+1} = f_k D^-1 A x_k, f_k the power of two that brings |x_{k+1}|
+// near 1 (scaling by it is exact).
+//   FP32: x is y / |y| rounded to FP32, formed where it is read.  The rounding
+// of the coarse operators is amplified by their condition (1e-4 to 1e-3 in a
+// V-cycle's result), and one unit in the last place of omega changes all of
+// it, so each FP32 sum of the setup keeps a fixed order of its own -- a row's
+// blocks over 32 lanes, a product's terms in list order -- that no launch
+// shape changes.
+struct PowerArgs {
+  double* part;      // [2][blocks]
+  unsigned* ticket;
+  double* scal;      // this level's SC_* values
+  double* coef64;    // Chebyshev coefficients {1/theta, c1, c2}
+  float* coef32;
+};
+
+// what the next step multiplies the iterate by
 template <class C>
-__global__ void __launch_bounds__(256) k_amg_sumsq2(int64_t N, const C* __restrict__ x, const C* __restrict__ y,
-                                                    double* __restrict__ part) {
-  __shared__ double sh[2][8];
-  double sx = 0.0, sy = 0.0;
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
-    const double a = (double)x[k], c = (double)y[k];
-    sx += a * a;
-    sy += c * c;
+struct PowerScale;
+template <>
+struct PowerScale<double> {  // (applied when y was written)
+  __device__ __forceinline__ explicit PowerScale(double) {}
+  __device__ __forceinline__ double operator()(double y) const { return y; }
+};
+template <>
+struct PowerScale<float> {  // y f rounded once: f = h + l, y h + its error + y l
+  float h, l;
+  __device__ __forceinline__ explicit PowerScale(double f) : h((float)f), l((float)(f - (double)h)) {}
+  __device__ __forceinline__ float operator()(float y) const {
+    const float p = y * h;
+    return p + fmaf(y, l, fmaf(y, h, -p));
   }
-  for (int off = 16; off > 0; off >>= 1) {
-    sx += __shfl_xor_sync(0xffffffffu, sx, off);
-    sy += __shfl_xor_sync(0xffffffffu, sy, off);
-  }
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) {
-    sh[0][w] = sx;
-    sh[1][w] = sy;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0.0, c = 0.0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); i++) {
-      a += sh[0][i];
-      c += sh[1][i];
-    }
-    part[blockIdx.x] = a;
-    part[gridDim.x + blockIdx.x] = c;
-  }
-}
+};
 
-// rho = |y| / |x|, x = y / |y|
+// from the sums of squares ss of y and (FP32, last step) xx of x
 template <class C>
-__global__ void k_amg_power_step(int64_t N, int nblk, const double* __restrict__ part, const C* __restrict__ y,
-                                 C* __restrict__ x, double* __restrict__ scal) {
-  __shared__ double s_inv;
+__device__ __forceinline__ void power_result(const PowerArgs& a, double ss, double xx, bool last_step) {
+  double rho = 0.0;
+  if (sizeof(C) == 8) {
+    const double f = a.scal[SC_F];
+    rho = sqrt(ss) / (sqrt(a.scal[SC_SS]) * f);
+    a.scal[SC_SS] = ss;
+    a.scal[SC_F] = ss > 0.0 && isfinite(ss) ? ldexp(1.0, -(ilogb(ss) >> 1)) : 1.0;
+  } else {
+    a.scal[SC_F] = 1.0 / sqrt(ss);
+    if (last_step) rho = sqrt(ss) / sqrt(xx);
+  }
+  if (!last_step) return;
+  a.scal[SC_RHO] = rho;
+  a.scal[SC_OMEGA] = 4.0 / (3.0 * rho);
+  const double lo = rho / 30.0, hi = 1.1 * rho;
+  const double theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo), sigma = theta / delta;
+  const double r0 = 1.0 / sigma, r1 = 1.0 / (2.0 * sigma - r0);
+  const double c[3] = {1.0 / theta, r1 * r0, 2.0 * r1 / delta};
+  for (int q = 0; q < 3; q++) {
+    a.coef64[q] = c[q];
+    a.coef32[q] = (float)c[q];
+  }
+}
+
+// block sum of ss (result in thread 0); every thread of the block calls it
+__device__ __forceinline__ double power_block_sum(double ss, double* sh) {
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x < 32) {
+    t = (int)threadIdx.x < (int)(blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  }
+  return t;
+}
+
+template <class C>
+__device__ __forceinline__ void power_finish(const PowerArgs& a, double ss, double xx, double* sh, bool last_step) {
+  __shared__ bool last;
+  const bool two = sizeof(C) == 4 && last_step;
+  const double bs = power_block_sum(ss, sh), bx = two ? power_block_sum(xx, sh) : 0.0;
   if (threadIdx.x == 0) {
-    double xx = 0.0, yy = 0.0;
-    for (int i = 0; i < nblk; i++) {
-      xx += part[i];
-      yy += part[nblk + i];
-    }
-    scal[0] = sqrt(yy) / sqrt(xx);
-    s_inv = 1.0 / sqrt(yy);
+    a.part[blockIdx.x] = bs;
+    if (two) a.part[gridDim.x + blockIdx.x] = bx;
+    __threadfence();
+    last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x)
-    x[k] = (C)((double)y[k] * s_inv);
+  if (!last) return;
+  __threadfence();
+  double s = 0.0, t = 0.0;
+  for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
+    s += ((volatile double*)a.part)[b];
+    if (two) t += ((volatile double*)a.part)[gridDim.x + b];
+  }
+  s = power_block_sum(s, sh);
+  if (two) t = power_block_sum(t, sh);
+  if (threadIdx.x == 0) {
+    *a.ticket = 0u;
+    power_result<C>(a, s, t, last_step);
+  }
 }
 
-// P entry q = (row i, aggregate a): [agg(i) = a] T_i - omega sum_{k: agg(col k) = a} D_i^-1 A_k T_col(k)
+template <class C>
+struct EpiPower {
+  const C* dinv;
+  C* y;
+  C f;
+  double ss;
+  C di[9];
+  __device__ __forceinline__ void prefetch(int, int, int) {}
+  __device__ __forceinline__ void load(int r0, int, int nd, int lane) {
+    if (lane < nd)
+#pragma unroll
+      for (int q = 0; q < 9; q++) di[q] = dinv[9 * (int64_t)(r0 + lane) + q];
+  }
+  __device__ __forceinline__ void finish(int row, const C (&s)[3]) {
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      const C v = f * (di[3 * q] * s[0] + di[3 * q + 1] * s[1] + di[3 * q + 2] * s[2]);
+      y[3 * (int64_t)row + q] = v;
+      ss += (double)v * (double)v;
+    }
+  }
+};
+
+// level 0 in FP64: the streamed product of fe_stream.cuh
+template <class C, class V>
+__global__ void __launch_bounds__(STREAM_THREADS, stream_blocks_per_sm<C>())
+    k_amg_power0(int n, int warps, int ranges, const int* __restrict__ part, const int* __restrict__ row_ptr,
+                 const int* __restrict__ col, const V* __restrict__ val, const C* __restrict__ dinv,
+                 const C* __restrict__ x, C* __restrict__ y, PowerArgs a, bool last_step) {
+  __shared__ StreamShared<C> sh;
+  __shared__ double red[32];
+  const int warp = (int)blockIdx.x * STREAM_WARPS + (threadIdx.x >> 5);
+  EpiPower<C> epi;
+  epi.dinv = dinv;
+  epi.y = y;
+  epi.f = (C)a.scal[SC_F];
+  epi.ss = 0.0;
+  stream_rows<V, C, C>(n, warp < warps ? warp : ranges, warps, ranges, part, row_ptr, col, val, x,
+                       sh.prod[threadIdx.x >> 5], epi);
+  power_finish<C>(a, epi.ss, 0.0, red, last_step);
+}
+
+// one row of a step by a warp: y_row = D^-1 (A x)_row (FP64: times f); lane
+// q < B adds the square of its component to ss and, if asked, of x to xx
 template <class C, class V, int B>
-__global__ void k_amg_pvals(int64_t nnzp, const int* __restrict__ prow, const int* __restrict__ pcol,
-                            const int* __restrict__ ptr, const int* __restrict__ col, Vals<C, V, B> A,
-                            const int* __restrict__ agg, const C* __restrict__ dinv,
-                            const double* __restrict__ tnode, C omega, C* __restrict__ p) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nnzp) return;
-  const int i = prow[q], a = pcol[q];
-  C acc[B][AMG_NS];
-  for (int r = 0; r < B; r++)
-    for (int c = 0; c < AMG_NS; c++)
-      acc[r][c] = agg[i] == a ? (C)tnode[(int64_t)i * B * AMG_NS + AMG_NS * r + c] : C(0);
-  C D[B][B];
-  for (int r = 0; r < B; r++)
-    for (int c = 0; c < B; c++) D[r][c] = dinv[(int64_t)i * B * B + B * r + c];
-  for (int k = ptr[i]; k < ptr[i + 1]; k++) {
-    const int j = col[k];
-    if (agg[j] != a) continue;
-    C DA[B][B];
-    for (int r = 0; r < B; r++)
-      for (int c = 0; c < B; c++) {
-        C s = C(0);
-        for (int l = 0; l < B; l++) s += D[r][l] * A(k, B * l + c);
-        DA[r][c] = s;
-      }
-    const double* T = tnode + (int64_t)j * B * AMG_NS;
-    for (int r = 0; r < B; r++)
-      for (int c = 0; c < AMG_NS; c++) {
-        C s = C(0);
-        for (int l = 0; l < B; l++) s += DA[r][l] * (C)T[AMG_NS * l + c];
-        acc[r][c] -= omega * s;
-      }
+__device__ __forceinline__ void power_row(int row, int lane, const int* ptr, const int* col, const Vals<C, V, B>& A,
+                                          const C* dinv, const C* x, C* y, C f, const PowerScale<C>& sc, bool want_xx,
+                                          double& ss, double& xx) {
+  C dq[B], s[B];
+#pragma unroll
+  for (int j = 0; j < B; j++) {
+    dq[j] = lane < B ? dinv[(int64_t)row * B * B + B * lane + j] : C(0);
+    s[j] = C(0);
   }
-  for (int r = 0; r < B; r++)
-    for (int c = 0; c < AMG_NS; c++) p[q * B * AMG_NS + AMG_NS * r + c] = acc[r][c];
+  for (int k = ptr[row] + lane; k < ptr[row + 1]; k += 32) {
+    const int c = __ldg(col + k);
+    C v[B * B], g[B];
+    A.block(k, v);
+#pragma unroll
+    for (int j = 0; j < B; j++) g[j] = sc(x[(int64_t)B * c + j]);
+#pragma unroll
+    for (int q = 0; q < B; q++)
+#pragma unroll
+      for (int j = 0; j < B; j++) s[q] += v[B * q + j] * g[j];
+  }
+#pragma unroll
+  for (int q = 0; q < B; q++)
+    for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+  if (lane >= B) return;
+  C t = C(0);
+#pragma unroll
+  for (int j = 0; j < B; j++) t += dq[j] * s[j];
+  if (sizeof(C) == 8) t *= f;
+  y[(int64_t)B * row + lane] = t;
+  ss += (double)t * (double)t;
+  if (want_xx) {
+    const double xv = (double)sc(x[(int64_t)B * row + lane]);
+    xx += xv * xv;
+  }
 }
 
-// A P entry (row i, aggregate a) = sum_k A_k P_(col k, a)
+// coarse levels, and level 0 in FP32: a warp per row, rows strided over at
+// most POWER_BLOCKS_PER_SM blocks per SM (a partial sum and a ticket each).
+// Level 0 of Cook P2 64x64x8: 45 us, of which the values are 23 us at the copy
+// rate (before 100 us in three kernels); a coarse level's 14 us are latency.
+constexpr int POWER_BLOCKS_PER_SM = 8;
 template <class C, class V, int B>
-__global__ void k_amg_ap(int64_t nnzap, const int* __restrict__ aprow, const int* __restrict__ apcol,
-                         const int* __restrict__ ptr, const int* __restrict__ col, Vals<C, V, B> A,
-                         const int* __restrict__ pptr, const int* __restrict__ pcol, const C* __restrict__ p,
-                         C* __restrict__ ap) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nnzap) return;
-  const int i = aprow[e], a = apcol[e];
-  C acc[B][AMG_NS];
-  for (int r = 0; r < B; r++)
-    for (int c = 0; c < AMG_NS; c++) acc[r][c] = C(0);
-  for (int k = ptr[i]; k < ptr[i + 1]; k++) {
-    const int j = col[k];
-    const int q = find_col(pcol, pptr[j], pptr[j + 1], a);
-    if (q < 0) continue;
-    const C* P = p + (int64_t)q * B * AMG_NS;
-    for (int r = 0; r < B; r++) {
-      C Ar[B];
-      for (int l = 0; l < B; l++) Ar[l] = A(k, B * r + l);
-      for (int c = 0; c < AMG_NS; c++) {
-        C s = C(0);
-        for (int l = 0; l < B; l++) s += Ar[l] * P[AMG_NS * l + c];
-        acc[r][c] += s;
-      }
-    }
-  }
-  for (int r = 0; r < B; r++)
-    for (int c = 0; c < AMG_NS; c++) ap[e * B * AMG_NS + AMG_NS * r + c] = acc[r][c];
+__global__ void __launch_bounds__(256) k_amg_power(int n, const int* __restrict__ ptr, const int* __restrict__ col,
+                                                   Vals<C, V, B> A, const C* __restrict__ dinv,
+                                                   const C* __restrict__ x, C* __restrict__ y, PowerArgs a,
+                                                   bool last_step) {
+  __shared__ double red[32];
+  const double f = a.scal[SC_F];
+  const PowerScale<C> sc(f);
+  const int lane = threadIdx.x & 31, nw = (int)((gridDim.x * blockDim.x) >> 5);
+  double ss = 0.0, xx = 0.0;
+  for (int row = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); row < n; row += nw)
+    power_row<C, V, B>(row, lane, ptr, col, A, dinv, x, y, (C)f, sc, sizeof(C) == 4 && last_step, ss, xx);
+  power_finish<C>(a, ss, xx, red, last_step);
 }
 
-// coarse entry (a, c) = sum over P^T row a (fine node i, P entry q) of P_q^T (A P)_(i, c);
-// absent coarse components get a unit diagonal
-template <class C, int B>
-__global__ void k_amg_rap(int64_t nnzc, const int* __restrict__ crow, const int* __restrict__ ccol,
-                          const int* __restrict__ rptr, const int* __restrict__ rcol, const int* __restrict__ rsrc,
-                          const int* __restrict__ apptr, const int* __restrict__ apcol, const C* __restrict__ p,
-                          const C* __restrict__ ap, const unsigned char* __restrict__ cabsent, C* __restrict__ out) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nnzc) return;
-  const int a = crow[e], cc = ccol[e];
-  C acc[AMG_NS][AMG_NS];
-  for (int r = 0; r < AMG_NS; r++)
-    for (int c = 0; c < AMG_NS; c++) acc[r][c] = C(0);
-  for (int s = rptr[a]; s < rptr[a + 1]; s++) {
-    const int i = rcol[s];
-    const int pe = find_col(apcol, apptr[i], apptr[i + 1], cc);
-    if (pe < 0) continue;
-    const C* P = p + (int64_t)rsrc[s] * B * AMG_NS;
-    const C* Q = ap + (int64_t)pe * B * AMG_NS;
-    for (int r = 0; r < AMG_NS; r++)
-      for (int c = 0; c < AMG_NS; c++) {
-        C v = C(0);
-        for (int l = 0; l < B; l++) v += P[AMG_NS * l + r] * Q[AMG_NS * l + c];
-        acc[r][c] += v;
-      }
+// The smallest levels: all 15 steps in one block, while its one SM is done
+// before 15 launches are.  The whole setup, in one block and as launches, for
+// levels of 884, 1,794 and 2,113 blocks: FP32 1.19 and 1.23, 0.98 and 0.95,
+// 1.40 and 1.35 ms; FP64 2.38 and 2.12, 2.58 and 1.93, 3.04 and 2.34 ms.
+template <class C>
+constexpr int AMG_POWER_SMALL = sizeof(C) == 4 ? 1024 : 256;  // blocks of the level
+template <class C>
+__global__ void __launch_bounds__(512) k_amg_power_small(int n, int steps, const int* __restrict__ ptr,
+                                                         const int* __restrict__ col, Vals<C, C, AMG_NS> A,
+                                                         const C* __restrict__ dinv, C* x, C* y, PowerArgs a) {
+  __shared__ double red[32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int it = 0; it < steps; it++) {
+    const double f = ((volatile double*)a.scal)[SC_F];
+    const PowerScale<C> sc(f);
+    const bool last = it == steps - 1;
+    double ss = 0.0, xx = 0.0;
+    for (int row = wid; row < n; row += nw)
+      power_row<C, C, AMG_NS>(row, lane, ptr, col, A, dinv, x, y, (C)f, sc, sizeof(C) == 4 && last, ss, xx);
+    ss = power_block_sum(ss, red);  // (its barriers order this step's rows before the next one's)
+    xx = power_block_sum(xx, red);
+    if (threadIdx.x == 0) power_result<C>(a, ss, xx, last);
+    __syncthreads();
+    C* t = x;
+    x = y;
+    y = t;
   }
-  if (a == cc) {
-    const unsigned m = cabsent[a];
-    for (int c = 0; c < AMG_NS; c++)
-      if ((m >> c) & 1u) acc[c][c] = C(1);
-  }
-  for (int r = 0; r < AMG_NS; r++)
-    for (int c = 0; c < AMG_NS; c++) out[e * AMG_NS * AMG_NS + AMG_NS * r + c] = acc[r][c];
-}
-
-// R = P^T values: R entry s holds the transpose of P entry rsrc[s]
-template <class C, int B>
-__global__ void k_amg_rvals(int64_t nnzr, const int* __restrict__ rsrc, const C* __restrict__ p, C* __restrict__ rv) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= nnzr) return;
-  const C* P = p + (int64_t)rsrc[s] * B * AMG_NS;
-  for (int c = 0; c < AMG_NS; c++)
-    for (int r = 0; r < B; r++) rv[s * B * AMG_NS + B * c + r] = P[AMG_NS * r + c];
-}
-
-// dense inverse of the coarsest operator (N <= 96): one block, Gauss-Jordan
-// with partial pivoting in shared memory (first maximal pivot on ties), FP64
-template <class C, class V, int B>
-__global__ void __launch_bounds__(1024) k_amg_dense_inverse(int n, const int* __restrict__ ptr,
-                                                            const int* __restrict__ col, Vals<C, V, B> A,
-                                                            double* __restrict__ inv) {
-  extern __shared__ double sm[];
-  const int N = n * B;
-  double* M = sm;
-  double* I = sm + N * N;
-  double* fac = sm + 2 * N * N;  // column c before the elimination step
-  __shared__ int s_piv;
-  for (int t = threadIdx.x; t < N * N; t += blockDim.x) {
-    M[t] = 0.0;
-    I[t] = (t / N == t % N) ? 1.0 : 0.0;
-  }
-  __syncthreads();
-  for (int a = threadIdx.x; a < n; a += blockDim.x)
-    for (int k = ptr[a]; k < ptr[a + 1]; k++)
-      for (int r = 0; r < B; r++)
-        for (int c = 0; c < B; c++) M[(B * a + r) * N + B * col[k] + c] = (double)A(k, B * r + c);
-  __syncthreads();
-  for (int c = 0; c < N; c++) {
-    if (threadIdx.x == 0) {
-      int p = c;
-      for (int r = c + 1; r < N; r++)
-        if (fabs(M[r * N + c]) > fabs(M[p * N + c])) p = r;
-      s_piv = p;
-    }
-    __syncthreads();
-    const int p = s_piv;
-    if (p != c)
-      for (int j = threadIdx.x; j < N; j += blockDim.x) {
-        double t = M[c * N + j];
-        M[c * N + j] = M[p * N + j];
-        M[p * N + j] = t;
-        t = I[c * N + j];
-        I[c * N + j] = I[p * N + j];
-        I[p * N + j] = t;
-      }
-    __syncthreads();
-    const double piv = M[c * N + c];
-    __syncthreads();
-    for (int j = threadIdx.x; j < N; j += blockDim.x) {
-      M[c * N + j] /= piv;
-      I[c * N + j] /= piv;
-    }
-    for (int r = threadIdx.x; r < N; r += blockDim.x) fac[r] = M[r * N + c];
-    __syncthreads();
-    for (int t = threadIdx.x; t < N * N; t += blockDim.x) {
-      const int r = t / N, j = t % N;
-      const double f = fac[r];
-      if (r == c || f == 0.0) continue;
-      M[r * N + j] -= f * M[c * N + j];
-      I[r * N + j] -= f * I[c * N + j];
-    }
-    __syncthreads();
-  }
-  for (int t = threadIdx.x; t < N * N; t += blockDim.x) inv[t] = I[t];
 }
 
 __global__ void k_amg_to_f32(int64_t n, const double* __restrict__ a, float* __restrict__ b) {
@@ -662,14 +750,382 @@ __global__ void k_amg_to_f32(int64_t n, const double* __restrict__ a, float* __r
   if (i < n) b[i] = (float)a[i];
 }
 
-// block-major blocks of nv values -> the tiled layout
-template <int NV, class T>
-__global__ void k_amg_tile(int64_t nblocks, const T* __restrict__ src, T* __restrict__ dst) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nblocks * NV) return;
-  const int64_t k = i / NV;
-  const int c = (int)(i % NV);
-  dst[tix<NV>(k, c)] = (T)src[i];
+// Once per mesh: the blocks of every fine row grouped by the aggregate of
+// their column, one list per P entry (pk[pk_ptr[q].x .. pk_ptr[q].y)), and
+// the place of each P entry in R = P^T.
+__global__ void k_amg_plists(int n, const int* __restrict__ ptr, const int* __restrict__ col,
+                             const int* __restrict__ agg, const int* __restrict__ pptr, const int* __restrict__ pcol,
+                             int2* __restrict__ pk_ptr, int* __restrict__ pk) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  int o = ptr[i];
+  for (int q = pptr[i]; q < pptr[i + 1]; q++) {
+    const int a = pcol[q], o0 = o;
+    for (int k = ptr[i]; k < ptr[i + 1]; k++)
+      if (agg[col[k]] == a) pk[o++] = k;
+    pk_ptr[q] = make_int2(o0, o);
+  }
+}
+__global__ void k_amg_rpos(int64_t nnzr, const int* __restrict__ rsrc, int* __restrict__ rpos) {
+  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (s < nnzr) rpos[rsrc[s]] = (int)s;
+}
+
+// P entry q = (row i, aggregate a): [agg(i) = a] T_i - omega sum over the row's
+// blocks k with agg(col k) = a of (D_i^-1 A_k) T_col(k), k ascending.  B
+// threads per entry, one row each: the blocks come from the entry's list (a
+// thread per entry that scanned its whole row took 632 us for 629k entries),
+// the block and T's rows are shared by neighbouring threads.  Also writes the
+// V-cycle's tiled copy pt and the transpose R (their own kernels took 30 and
+// 58 us).  Cook P2 64x64x8: level 0 176 us (before 447), level 1 119.
+template <class C, class V, int B>
+__global__ void __launch_bounds__(B == 3 ? 192 : 64) k_amg_pvals(int64_t nnzp, const int* __restrict__ prow,
+                                                   const int* __restrict__ pcol, const int2* __restrict__ pk_ptr,
+                                                   const int* __restrict__ pk, const int* __restrict__ col,
+                                                   Vals<C, V, B> A, const int* __restrict__ agg,
+                                                   const C* __restrict__ dinv, const C* __restrict__ tnode,
+                                                   const double* __restrict__ scal, const int* __restrict__ rpos,
+                                                   C* __restrict__ p, C* __restrict__ pt, C* __restrict__ rv) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t q = t / B;
+  const int r = (int)(t % B);
+  if (q >= nnzp) return;
+  const int i = prow[q];
+  const C omega = (C)scal[SC_OMEGA];
+  const bool own = agg[i] == pcol[q];
+  C acc[AMG_NS], d[B];
+#pragma unroll
+  for (int c = 0; c < AMG_NS; c++) acc[c] = own ? tnode[((int64_t)i * B + r) * AMG_NS + c] : C(0);
+#pragma unroll
+  for (int l = 0; l < B; l++) d[l] = dinv[((int64_t)i * B + r) * B + l];
+  const int2 lst = pk_ptr[q];
+  int k = lst.x < lst.y ? pk[lst.x] : 0, j = lst.x < lst.y ? col[k] : 0;
+  for (int e = lst.x; e < lst.y; e++) {
+    const C* T = tnode + (int64_t)j * B * AMG_NS;
+    C av[B * B], da[B];
+    A.block(k, av);
+    if (e + 1 < lst.y) {
+      k = pk[e + 1];
+      j = col[k];
+    }
+#pragma unroll
+    for (int c = 0; c < B; c++) {
+      C v = C(0);
+#pragma unroll
+      for (int l = 0; l < B; l++) v += d[l] * av[B * l + c];
+      da[c] = v;
+    }
+#pragma unroll
+    for (int c = 0; c < AMG_NS; c++) {
+      C v = C(0);
+#pragma unroll
+      for (int l = 0; l < B; l++) v += da[l] * T[AMG_NS * l + c];
+      acc[c] -= omega * v;
+    }
+  }
+  const int64_t rp = (int64_t)rpos[q] * B * AMG_NS;
+#pragma unroll
+  for (int c = 0; c < AMG_NS; c++) {
+    p[q * B * AMG_NS + AMG_NS * r + c] = acc[c];
+    pt[tix<B * AMG_NS>(q, AMG_NS * r + c)] = acc[c];
+    rv[rp + B * c + r] = acc[c];
+  }
+}
+
+// place of c among the m ascending values of list, -1 if absent
+__device__ __forceinline__ int find_sorted(const int* list, int m, int c) {
+  int lo = 0;
+  for (int len = m; len > 0;) {  // first place whose value is not below c
+    const int half = len >> 1;
+    const bool below = list[lo + half] < c;
+    lo = below ? lo + half + 1 : lo;
+    len = below ? len - half - 1 : half;
+  }
+  return lo < m && list[lo] == c ? lo : -1;
+}
+
+// Once per mesh: the place in its A P row of every product A_k P_q of a fine
+// row (k in order, then q in P row col k).
+__global__ void k_amg_apidx(int n, const int* __restrict__ ptr, const int* __restrict__ col,
+                            const int* __restrict__ pptr, const int* __restrict__ pcol, const int* __restrict__ apptr,
+                            const int* __restrict__ apcol, const int64_t* __restrict__ off, int* __restrict__ idx) {
+  const int i = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (i >= n) return;
+  int64_t o = off[i];
+  const int a0 = apptr[i], m = apptr[i + 1] - a0;
+  for (int k = ptr[i]; k < ptr[i + 1]; k++) {
+    const int j = col[k], q0 = pptr[j], q1 = pptr[j + 1];
+    for (int q = q0 + lane; q < q1; q += 32) idx[o + (q - q0)] = find_sorted(apcol + a0, m, pcol[q]);
+    o += q1 - q0;
+  }
+}
+// Once per mesh: the products P_q^T (A P)_e of every coarse entry (q of P^T row
+// a in order, e the entry of q's node in the coarse column), one list per
+// entry, and the entry's row.  A warp per coarse row counts, sums the counts
+// and fills; the entries of one A P row have distinct places.
+__global__ void k_amg_raplists(int nc, const int* __restrict__ cptr, const int* __restrict__ ccol,
+                               const int* __restrict__ rptr, const int* __restrict__ rcol,
+                               const int* __restrict__ rsrc, const int* __restrict__ apptr,
+                               const int* __restrict__ apcol, const int64_t* __restrict__ raoff,
+                               int64_t* lend, int* crow, int2* __restrict__ list) {
+  const int a = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (a >= nc) return;
+  const int c0 = cptr[a], m = cptr[a + 1] - c0;
+  for (int t = lane; t < m; t += 32) {
+    lend[c0 + t] = 0;
+    crow[c0 + t] = a;
+  }
+  __syncwarp();
+  for (int pass = 0; pass < 2; pass++) {
+    for (int s = rptr[a]; s < rptr[a + 1]; s++) {
+      const int e1 = apptr[rcol[s] + 1];
+      for (int e = apptr[rcol[s]] + lane; e < e1; e += 32) {
+        const int pos = find_sorted(ccol + c0, m, apcol[e]);
+        if (pos < 0) continue;
+        const int64_t o = lend[c0 + pos]++;
+        if (pass) list[o] = make_int2(rsrc[s], e);
+      }
+      __syncwarp();
+    }
+    if (pass) break;
+    int64_t base = raoff[a];  // counts -> starts; the fill leaves the ends
+    for (int t0 = 0; t0 < m; t0 += 32) {
+      const int64_t v = t0 + lane < m ? lend[c0 + t0 + lane] : 0;
+      int64_t inc = v;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int64_t u = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += u;
+      }
+      if (t0 + lane < m) lend[c0 + t0 + lane] = base + inc - v;
+      base += __shfl_sync(0xffffffffu, inc, 31);
+    }
+    __syncwarp();
+  }
+}
+
+// A P, one warp per fine row: the row's blocks A_k (staged in shared memory,
+// 32 at a time) times the P rows of their columns, five P entries of a row at
+// a time (lane 6 g + c: entry g, column c), added up in shared memory at the
+// product's place in the A P row (a list made once per mesh: searched for
+// here, the places took more instructions than the products).  Rows longer than
+// AMG_CHUNK entries are taken in chunks.  The entries of one P row have
+// distinct places and block k + 1 follows block k after a warp barrier: no
+// atomics, a fixed order.  Bound by the
+// FP32 and shared-memory instructions of the products: about 500 us on level 0
+// of Cook P2 64x64x8 (113k rows, 1.9 M entries).  Before, a thread per output
+// entry that searched the P rows of all the row's columns: 638 us there, and
+// 204 us on the next level, now 51.
+constexpr int AMG_CHUNK = 64;
+template <class C, int B>
+struct ApShared {
+  C acc[AMG_CHUNK * B * AMG_NS];
+  C a[32][B * B];
+};
+template <class C, int B>
+__host__ __device__ constexpr int ap_warps() { return B == 3 && sizeof(C) == 4 ? 8 : 4; }
+
+template <class C, class V, int B>
+__global__ void __launch_bounds__(32 * ap_warps<C, B>())
+    k_amg_ap(int n, const int* __restrict__ ptr, const int* __restrict__ col, Vals<C, V, B> A,
+             const int* __restrict__ pptr, const C* __restrict__ p, const int* __restrict__ apptr,
+             const int64_t* __restrict__ apoff, const int* __restrict__ apidx, C* __restrict__ ap) {
+  constexpr int BN = B * AMG_NS;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  ApShared<C, B>& sh = reinterpret_cast<ApShared<C, B>*>(smraw)[wid];
+  const int i = blockIdx.x * ap_warps<C, B>() + wid;
+  if (i >= n) return;
+  const int g = lane / AMG_NS, c = lane % AMG_NS;
+  const int ks = ptr[i], ke = ptr[i + 1], a0 = apptr[i], ae = apptr[i + 1];
+  for (int cb = a0; cb < ae; cb += AMG_CHUNK) {
+    const int m = min(AMG_CHUNK, ae - cb);
+    const int* ix = apidx + apoff[i];  // places of the next block's products
+    for (int t = lane; t < m * BN; t += 32) sh.acc[t] = C(0);
+    for (int k0 = ks; k0 < ke; k0 += 32) {
+      const int cnt = min(32, ke - k0);
+      int q0 = 0, q1 = 0;
+      if (lane < cnt) {
+        const int j = col[k0 + lane];
+        q0 = pptr[j];
+        q1 = pptr[j + 1];
+        C av[B * B];
+        A.block(k0 + lane, av);
+#pragma unroll
+        for (int t = 0; t < B * B; t++) sh.a[lane][t] = av[t];
+      }
+      __syncwarp();
+      for (int kk = 0; kk < cnt; kk++) {
+        const int qa = __shfl_sync(0xffffffffu, q0, kk), len = __shfl_sync(0xffffffffu, q1, kk) - qa;
+        if (g < 5)
+          for (int u = g; u < len; u += 5) {
+            const int e = (int)ix[u] - (cb - a0);
+            const C* P = p + (int64_t)(qa + u) * BN + c;
+            C pv[B];
+#pragma unroll
+            for (int l = 0; l < B; l++) pv[l] = P[AMG_NS * l];
+            if (e >= 0 && e < m) {
+              C* o = sh.acc + e * BN + c;
+#pragma unroll
+              for (int r = 0; r < B; r++) {
+                C s = C(0);
+#pragma unroll
+                for (int l = 0; l < B; l++) s += sh.a[kk][B * r + l] * pv[l];
+                o[AMG_NS * r] += s;
+              }
+            }
+          }
+        ix += len;
+        __syncwarp();
+      }
+    }
+    for (int t = lane; t < m * BN; t += 32) ap[(int64_t)cb * BN + t] = sh.acc[t];
+    __syncwarp();
+  }
+}
+
+// Coarse operator: entry e = (a, b) is the sum over its list (q ascending) of
+// P_q^T (A P)_(node of q, b); absent components get a unit diagonal.  B = 3
+// (level 0, many entries with some hundred products each): six threads per
+// entry, one row each, the A P values shared by neighbouring threads.  B = 6
+// (few entries, long lists, bound by the latency of the loads): 36 threads, one
+// value each, eight products in flight.  404 us on level 0 of Cook P2 64x64x8
+// and 167 us on level 1 (a thread per entry that searched the
+// A P rows of all the row's nodes: 979 and 849 us).
+template <class C, int B>
+__global__ void __launch_bounds__(B == 3 ? 192 : 64)
+    k_amg_rap(int64_t nnzc, const int* __restrict__ crow, const int* __restrict__ ccol,
+              const int64_t* __restrict__ lend, const int64_t* __restrict__ raoff, const int2* __restrict__ list,
+              const C* __restrict__ p, const C* __restrict__ ap, const unsigned char* __restrict__ cabsent,
+              C* __restrict__ out) {
+  constexpr int BN = B * AMG_NS, NN = AMG_NS * AMG_NS;
+  constexpr int PER = B == 3 ? AMG_NS : 1, TPE = NN / PER;  // values per thread, threads per entry
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t e = t / TPE;
+  if (e >= nnzc) return;
+  const int u = (int)(t % TPE), r = PER == 1 ? u / AMG_NS : u, cc = PER == 1 ? u % AMG_NS : 0;
+  const int a = crow[e];
+  C acc[PER];
+#pragma unroll
+  for (int c = 0; c < PER; c++) acc[c] = C(0);
+  const int64_t l1 = lend[e];
+  constexpr int U = B == 3 ? 2 : (sizeof(C) == 4 ? 8 : 4);  // products in flight
+  int64_t l = e > 0 && crow[e - 1] == a ? lend[e - 1] : raoff[a];
+  auto add = [&](const C (&P)[B], const C (&Q)[B][PER]) {
+#pragma unroll
+    for (int c = 0; c < PER; c++) {
+      C v = C(0);
+#pragma unroll
+      for (int k = 0; k < B; k++) v += P[k] * Q[k][c];
+      acc[c] += v;
+    }
+  };
+  auto load = [&](int2 it, C (&P)[B], C (&Q)[B][PER]) {
+    const C* pp = p + (int64_t)it.x * BN + r;
+    const C* qq = ap + (int64_t)it.y * BN + cc;
+#pragma unroll
+    for (int k = 0; k < B; k++) {
+      P[k] = __ldg(pp + AMG_NS * k);
+#pragma unroll
+      for (int c = 0; c < PER; c++) Q[k][c] = __ldg(qq + AMG_NS * k + c);
+    }
+  };
+  for (; l + U <= l1; l += U) {
+    C P[U][B], Q[U][B][PER];
+#pragma unroll
+    for (int w = 0; w < U; w++) load(list[l + w], P[w], Q[w]);
+#pragma unroll
+    for (int w = 0; w < U; w++) add(P[w], Q[w]);
+  }
+  for (; l < l1; l++) {
+    C P[B], Q[B][PER];
+    load(list[l], P, Q);
+    add(P, Q);
+  }
+  const bool unit = ccol[e] == a && ((cabsent[a] >> r) & 1u);
+#pragma unroll
+  for (int c = 0; c < PER; c++) out[e * NN + AMG_NS * r + cc + c] = unit && cc + c == r ? C(1) : acc[c];
+}
+
+// dense inverse of the coarsest operator (N <= 96): one block, Gauss-Jordan
+// in place in shared memory with partial pivoting (first maximal pivot on
+// ties, found by one warp on the bit patterns), FP64; the row exchanges
+// become column exchanges of the inverse.  The FP64 pipe bounds it: N^2
+// products per column instead of the 2 N^2 of [A | I] (N = 24: 41 us;
+// N = 66 took 525 us as [A | I] with a serial pivot search).
+template <class C, class V, int B>
+__global__ void __launch_bounds__(1024) k_amg_dense_inverse(int n, const int* __restrict__ ptr,
+                                                            const int* __restrict__ col, Vals<C, V, B> A,
+                                                            double* __restrict__ inv, float* __restrict__ inv32) {
+  extern __shared__ double sm[];
+  const int N = n * B;
+  double* M = sm;
+  double* fac = sm + N * N;       // column c before the elimination step
+  double* row = fac + N;          // row c after scaling
+  __shared__ int s_piv[AMG_DENSE_MAX];
+  __shared__ double s_rp;
+  for (int t = threadIdx.x; t < N * N; t += blockDim.x) M[t] = 0.0;
+  __syncthreads();
+  for (int a = threadIdx.x; a < n; a += blockDim.x)
+    for (int k = ptr[a]; k < ptr[a + 1]; k++)
+      for (int r = 0; r < B; r++)
+        for (int c = 0; c < B; c++) M[(B * a + r) * N + B * col[k] + c] = (double)A(k, B * r + c);
+  __syncthreads();
+  for (int c = 0; c < N; c++) {
+    if (threadIdx.x < 32) {
+      unsigned long long best = 0;
+      int p = c;
+      for (int r = c + (int)threadIdx.x; r < N; r += 32) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(M[r * N + c]) & 0x7fffffffffffffffULL;
+        if (b > best) {
+          best = b;
+          p = r;
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long b = __shfl_xor_sync(0xffffffffu, best, o);
+        const int q = __shfl_xor_sync(0xffffffffu, p, o);
+        if (b > best || (b == best && q < p)) {
+          best = b;
+          p = q;
+        }
+      }
+      if (threadIdx.x == 0) {
+        s_piv[c] = p;
+        s_rp = 1.0 / M[p * N + c];
+      }
+    }
+    __syncthreads();
+    const int p = s_piv[c];
+    const double rp = s_rp;
+    // row c <- row p / pivot (with 1 in column c), row p <- row c
+    for (int j = threadIdx.x; j < N; j += blockDim.x) {
+      const double vp = M[p * N + j], vc = M[c * N + j];
+      row[j] = (j == c ? 1.0 : vp) * rp;
+      if (p != c) M[p * N + j] = vc;
+    }
+    __syncthreads();
+    for (int r = threadIdx.x; r < N; r += blockDim.x) fac[r] = r == c ? 0.0 : M[r * N + c];
+    __syncthreads();
+    for (int t = threadIdx.x; t < N * N; t += blockDim.x) {
+      const int r = t / N, j = t - r * N;
+      M[t] = r == c ? row[j] : (j == c ? 0.0 : M[t]) - fac[r] * row[j];
+    }
+    __syncthreads();
+  }
+  for (int c = N - 1; c >= 0; c--) {
+    const int p = s_piv[c];
+    if (p != c)
+      for (int r = threadIdx.x; r < N; r += blockDim.x) {
+        const double t = M[r * N + c];
+        M[r * N + c] = M[r * N + p];
+        M[r * N + p] = t;
+      }
+    __syncthreads();
+  }
+  for (int t = threadIdx.x; t < N * N; t += blockDim.x) {
+    inv[t] = M[t];
+    if (inv32) inv32[t] = (float)M[t];
+  }
 }
 
 // ---------------------------------------------------------------- V-cycle kernels
@@ -981,26 +1437,8 @@ __device__ __forceinline__ void vc_cheb_row(int row, int lane, int n, const int*
   for (int q = 0; q < B; q++) s[q] = T(0);
   for (int k = ptr[row] + lane; k < ptr[row + 1]; k += 32) {
     const int c = fe_idx(__ldg(col + k), n);
-    T v[B * B];  // the block, block-major: B * B * sizeof(T) bytes, a multiple of 16
-    if constexpr (sizeof(T) == 4) {
-      const float4* p4 = reinterpret_cast<const float4*>(val + (int64_t)k * B * B);
-#pragma unroll
-      for (int t = 0; t < B * B / 4; t++) {
-        const float4 u = __ldg(p4 + t);
-        v[4 * t] = u.x;
-        v[4 * t + 1] = u.y;
-        v[4 * t + 2] = u.z;
-        v[4 * t + 3] = u.w;
-      }
-    } else {
-      const double2* p2 = reinterpret_cast<const double2*>(val + (int64_t)k * B * B);
-#pragma unroll
-      for (int t = 0; t < B * B / 2; t++) {
-        const double2 u = __ldg(p2 + t);
-        v[2 * t] = u.x;
-        v[2 * t + 1] = u.y;
-      }
-    }
+    T v[B * B];
+    load_block6<T>(val, k, v);
     T gv[B];
 #pragma unroll
     for (int j = 0; j < B; j++) gv[j] = g[(int64_t)B * c + j];
@@ -1038,8 +1476,13 @@ __device__ __forceinline__ void vc_cheb_row(int row, int lane, int n, const int*
   }
 }
 
+// (FP64, two rows per block: a level of 227 rows spreads over 114 SMs, not 29,
+// V-cycles of 12^3 to 30x26x6 meshes are 4-8 % faster; FP32 7.3 us with eight
+// rows per block there, 8.1 with two)
+template <class T>
+constexpr int VC_CHEB_THREADS = sizeof(T) == 8 ? 64 : 256;
 template <class T, int B>
-__global__ void __launch_bounds__(256) k_vc_cheb(int n, const int* __restrict__ ptr, const int* __restrict__ col,
+__global__ void __launch_bounds__(VC_CHEB_THREADS<T>) k_vc_cheb(int n, const int* __restrict__ ptr, const int* __restrict__ col,
                                                  const T* __restrict__ val, const T* __restrict__ dinv,
                                                  const T* __restrict__ g, T* __restrict__ x, T* __restrict__ r,
                                                  T* __restrict__ dout, T cx, const T* __restrict__ coef,
@@ -1199,17 +1642,20 @@ __global__ void __launch_bounds__(256) k_vc_prolong(int n, const int* __restrict
   vc_prolong_thread<T, BF, LPR>((int64_t)blockIdx.x * blockDim.x + threadIdx.x, n, pptr, pcol, pv, xc, x, e, ncoarse);
 }
 
-// The bottom of the V-cycle in one block.  Below a few hundred nodes per
-// level the coarse kernels are a few blocks each, and their cost is launch
-// latency, not bytes: levels q0..L-1 (each at most VC_BOTTOM_MAXN nodes,
-// q0 >= 1) run as one launch of one block -- smoothing, restriction, the
-// coarsest solve, prolongation and smoothing again, separated by block
-// barriers.  Each stage runs the same device functions as the per-level
-// kernels, with the same assignment of rows and entries to warps, lanes and
-// 128-thread groups, so the result is identical to theirs.
-template <class T>
-__host__ __device__ constexpr int vc_bottom_threads() { return sizeof(T) == 8 ? 512 : 1024; }
-constexpr int VC_BOTTOM_MAXN = 256;
+// The bottom of the V-cycle in one block (FP32).  The smallest coarse levels'
+// kernels cost their launches, not bytes: levels q0..L-1 (each at most
+// VC_BOTTOM_MAXNNZ blocks, q0 >= 1) run as one launch of one block --
+// smoothing, restriction, the coarsest solve, prolongation and smoothing
+// again, separated by block barriers.  Each stage runs the same device
+// functions as the per-level kernels, with the same assignment of rows and
+// entries to warps, lanes and 128-thread groups, so the result is identical.
+// One SM works through the blocks, so the form pays for few of them only, a
+// level of n blocks costing in the whole V-cycle, fused and as launches: 317
+// blocks 296 and 300 us, 884 blocks 72 and 71, 1,794: 80 and 68, 4,267: 122
+// and 69, 9,073: 195 and 86.  In FP64 (884: 208 and 133 us; 317: 1,022 and
+// 983) the launches win throughout.
+constexpr int VC_BOTTOM_THREADS = 1024;
+constexpr int64_t VC_BOTTOM_MAXNNZ = 640;
 
 template <class T>
 struct VcLevelArgs {  // one level of the bottom (device pointers)
@@ -1230,8 +1676,8 @@ struct VcBottomArgs {
 };
 
 template <class T>
-__global__ void __launch_bounds__(vc_bottom_threads<T>()) k_vc_bottom(const VcBottomArgs<T> P) {
-  constexpr int NT = vc_bottom_threads<T>();
+__global__ void __launch_bounds__(VC_BOTTOM_THREADS) k_vc_bottom(const VcBottomArgs<T> P) {
+  constexpr int NT = VC_BOTTOM_THREADS;
   constexpr int NW = NT / 32;
   constexpr int NG = NT / VC_RESTRICT_THREADS;
   __shared__ T sh[NG][4][AMG_NS];
@@ -1367,18 +1813,13 @@ int build_structure(fe_mesh m) {
       A.diag = m->diag_pos;
       A.nnz = m->nnzb;
     } else {
-      int *p = nullptr, *c = nullptr, *d = nullptr, *cr = nullptr;
+      int *p = nullptr, *c = nullptr, *d = nullptr;
       FE_TRY(upload(m, &p, H.ptr));
       FE_TRY(upload(m, &c, H.col));
       FE_TRY(upload(m, &d, H.diag));
-      std::vector<int> crow(H.col.size());
-      for (int a = 0; a < H.n; a++)
-        for (int k = H.ptr[a]; k < H.ptr[a + 1]; k++) crow[k] = a;
-      FE_TRY(upload(m, &cr, crow));
       A.ptr = p;
       A.col = c;
       A.diag = d;
-      A.crow = cr;
       A.nnz = (int64_t)H.col.size();
     }
     FE_TRY(upload(m, &A.absent, H.absent));
@@ -1386,37 +1827,56 @@ int build_structure(fe_mesh m) {
       FE_TRY(upload(m, &A.agg, H.agg));
       FE_TRY(upload(m, &A.pptr, H.pptr));
       FE_TRY(upload(m, &A.pcol, H.pcol));
-      std::vector<int> prow(H.pcol.size()), aprow(H.apcol.size());
-      for (int i = 0; i < H.n; i++) {
+      std::vector<int> prow(H.pcol.size());
+      for (int i = 0; i < H.n; i++)
         for (int k = H.pptr[i]; k < H.pptr[i + 1]; k++) prow[k] = i;
-        for (int k = H.apptr[i]; k < H.apptr[i + 1]; k++) aprow[k] = i;
-      }
       FE_TRY(upload(m, &A.prow, prow));
       FE_TRY(upload(m, &A.rptr, H.rptr));
       FE_TRY(upload(m, &A.rcol, H.rcol));
       FE_TRY(upload(m, &A.rsrc, H.rsrc));
       FE_TRY(upload(m, &A.apptr, H.apptr));
       FE_TRY(upload(m, &A.apcol, H.apcol));
-      FE_TRY(upload(m, &A.aprow, aprow));
       FE_TRY(upload(m, &A.tnode, H.tnode));
       A.nnzp = (int64_t)H.pcol.size();
       A.nnzr = A.nnzp;
       A.nnzap = (int64_t)H.apcol.size();
+      FE_TRY(dev_alloc(m, &A.pk_ptr, (size_t)A.nnzp));
+      FE_TRY(dev_alloc(m, &A.pk, (size_t)A.nnz));
+      FE_TRY(dev_alloc(m, &A.rpos, (size_t)A.nnzr));
+      k_amg_plists<<<blocks_for(A.n, 128), 128, 0, m->stream>>>(A.n, A.ptr, A.col, A.agg, A.pptr, A.pcol, A.pk_ptr,
+                                                                A.pk);
+      k_amg_rpos<<<blocks_for(A.nnzr, 256), 256, 0, m->stream>>>(A.nnzr, A.rsrc, A.rpos);
+      FE_CUDA(cudaGetLastError());
+      FE_TRY(upload(m, &A.apoff, H.apoff));
+      FE_TRY(upload(m, &A.raoff, H.raoff));
+      FE_TRY(dev_alloc(m, &A.apidx, (size_t)H.apoff.back()));
+      FE_TRY(dev_alloc(m, &A.ralist, (size_t)H.raoff.back()));
+      FE_TRY(dev_alloc(m, &A.tnode32, H.tnode.size()));
+      k_amg_to_f32<<<blocks_for((int64_t)H.tnode.size(), 256), 256, 0, m->stream>>>((int64_t)H.tnode.size(), A.tnode,
+                                                                                   A.tnode32);
+      FE_CUDA(cudaGetLastError());
+      k_amg_apidx<<<blocks_for((int64_t)A.n * 32, 256), 256, 0, m->stream>>>(A.n, A.ptr, A.col, A.pptr, A.pcol, A.apptr,
+                                                                           A.apcol, A.apoff, A.apidx);
+      FE_CUDA(cudaGetLastError());
     }
+  }
+  for (int q = 0; q < nlev - 1; q++) {
+    AmgLevel &A = h->lev[q], &Cq = h->lev[q + 1];
+    FE_TRY(dev_alloc(m, &A.lend, (size_t)Cq.nnz));
+    FE_TRY(dev_alloc(m, &A.crow, (size_t)Cq.nnz));
+    k_amg_raplists<<<blocks_for((int64_t)Cq.n * 32, 256), 256, 0, m->stream>>>(
+        Cq.n, Cq.ptr, Cq.col, A.rptr, A.rcol, A.rsrc, A.apptr, A.apcol, A.raoff, A.lend, A.crow, A.ralist);
+    FE_CUDA(cudaGetLastError());
   }
   int64_t maxN = 0;
   for (int q = 0; q < nlev; q++) maxN = std::max<int64_t>(maxN, (int64_t)h->lev[q].n * h->lev[q].b);
   FE_TRY(dev_alloc(m, &h->pw, (size_t)2 * maxN));
-  FE_TRY(dev_alloc(m, &h->part, (size_t)2 * AMG_RED_BLOCKS));
-  FE_TRY(dev_alloc(m, &h->scal, 4));
+  const size_t blocks = std::max<size_t>(stream_grid(m->warps64), (size_t)POWER_BLOCKS_PER_SM * m->sm_count);
+  FE_TRY(dev_alloc(m, &h->part, 2 * blocks));
+  FE_TRY(dev_alloc(m, &h->ticket, 4));
+  FE_CUDA(cudaMemsetAsync(h->ticket, 0, 4 * sizeof(unsigned), m->stream));
+  FE_TRY(dev_alloc(m, &h->scal, (size_t)AMG_MAXLEV * SC_N));
   FE_CUDA(cudaStreamSynchronize(m->stream));  // host vectors above go out of scope
-  return FE_OK;
-}
-
-int to_f32(fe_mesh m, const double* a, float** b, int64_t n) {
-  if (!*b) FE_TRY(dev_alloc(m, b, (size_t)n));
-  k_amg_to_f32<<<blocks_for(n, 256), 256, 0, m->stream>>>(n, a, *b);
-  FE_CUDA(cudaGetLastError());
   return FE_OK;
 }
 
@@ -1428,6 +1888,7 @@ struct Arr {
   static C*& p(AmgLevel& L);
   static C*& ap(AmgLevel& L);
   static C*& r(AmgLevel& L);
+  static C*& pt(AmgLevel& L);
 };
 template <>
 struct Arr<double> {
@@ -1436,6 +1897,7 @@ struct Arr<double> {
   static double*& p(AmgLevel& L) { return L.p64; }
   static double*& ap(AmgLevel& L) { return L.ap64; }
   static double*& r(AmgLevel& L) { return L.r64; }
+  static double*& pt(AmgLevel& L) { return L.pt64; }
 };
 template <>
 struct Arr<float> {
@@ -1444,109 +1906,113 @@ struct Arr<float> {
   static float*& p(AmgLevel& L) { return L.p32; }
   static float*& ap(AmgLevel& L) { return L.ap32; }
   static float*& r(AmgLevel& L) { return L.r32; }
+  static float*& pt(AmgLevel& L) { return L.pt32; }
 };
 
-// numbers of level q (A_q already numeric) in arithmetic type C: D^-1, rho,
-// P, AP, R and A_{q+1}; the coarsest level's dense inverse (FP64, with an
-// FP32 copy for the mixed forms)
+// one power step of level q, x -> y
 template <class C, class V, int B>
-int numeric_level(fe_mesh m, int q, Vals<C, V, B> A) {
+int power_step(fe_mesh m, AmgLevel& L, const V* A, const C* dinv, const C* x, C* y, const PowerArgs& pa, bool last) {
+  FE_SCOPE(m, FE_PROF_OTHER, (double)L.nnz * (B * B * sizeof(V) + 4) + 2.0 * sizeof(C) * L.n * B);
+  if constexpr (B == 3 && sizeof(C) == 8)
+    k_amg_power0<C, V><<<stream_grid(m->warps64), STREAM_THREADS, 0, m->stream>>>(
+        L.n, m->warps64, m->ranges64, m->part64, L.ptr, L.col, A, dinv, x, y, pa, last);
+  else
+    k_amg_power<C, V, B><<<std::min<unsigned>(blocks_for((int64_t)L.n * 32, 256), POWER_BLOCKS_PER_SM * m->sm_count),
+                           256, 0, m->stream>>>(L.n, L.ptr, L.col, Vals<C, V, B>{A}, dinv, x, y, pa, last);
+  FE_CUDA(cudaGetLastError());
+  return FE_OK;
+}
+
+// numbers of level q (A_q already numeric) in arithmetic type C: D^-1, rho,
+// P (with its tiled copy and transpose), AP and A_{q+1}; the coarsest level's
+// dense inverse (FP64, with an FP32 copy for the mixed forms).  Everything is
+// queued; the host reads nothing.
+template <class C, class V, int B>
+int numeric_level(fe_mesh m, int q, const V* val) {
   AmgHier* h = m->amg;
   AmgLevel& L = h->lev[q];
+  const Vals<C, V, B> A{val};
   const int64_t N = (int64_t)L.n * L.b;
   C*& dinv = Arr<C>::dinv(L);
   if (!dinv) FE_TRY(dev_alloc(m, &dinv, (size_t)L.n * B * B));
   {
     FE_SCOPE(m, FE_PROF_OTHER, (double)L.n * B * B * (8 + sizeof(C)));
-    k_amg_dinv<C, V, B><<<blocks_for(L.n, 128), 128, 0, m->stream>>>(L.n, L.diag, A, dinv);
+    if constexpr (B == 3)
+      k_amg_dinv3<C, V><<<blocks_for(L.n, 128), 128, 0, m->stream>>>(L.n, L.diag, A, dinv);
+    else
+      k_amg_dinv6<C, V><<<blocks_for((int64_t)L.n * 16, 128), 128, 0, m->stream>>>(L.n, L.diag, A, dinv);
   }
   FE_CUDA(cudaGetLastError());
   if (q == h->nlev - 1) {  // coarsest: dense inverse
     const int Nd = L.n * B;
     if (!L.inv64) FE_TRY(dev_alloc(m, &L.inv64, (size_t)Nd * Nd));
-    const int smem = (2 * Nd * Nd + Nd) * (int)sizeof(double);
+    if (sizeof(C) == 4 && !L.inv32) FE_TRY(dev_alloc(m, &L.inv32, (size_t)Nd * Nd));
+    const int smem = (Nd * Nd + 2 * Nd) * (int)sizeof(double);
     FE_TRY(fe_kernel_smem((const void*)k_amg_dense_inverse<C, V, B>, smem));
-    {
-      FE_SCOPE(m, FE_PROF_OTHER, 8.0 * Nd * Nd);
-      k_amg_dense_inverse<C, V, B><<<1, 1024, smem, m->stream>>>(L.n, L.ptr, L.col, A, L.inv64);
-    }
+    FE_SCOPE(m, FE_PROF_OTHER, 8.0 * Nd * Nd);
+    k_amg_dense_inverse<C, V, B><<<1, 1024, smem, m->stream>>>(L.n, L.ptr, L.col, A, L.inv64,
+                                                              sizeof(C) == 4 ? L.inv32 : nullptr);
     FE_CUDA(cudaGetLastError());
-    if (!std::is_same<C, double>::value) FE_TRY(to_f32(m, L.inv64, &L.inv32, (int64_t)Nd * Nd));
     return FE_OK;
   }
   // rho: power steps on D^-1 A
+  if (!L.coef64) FE_TRY(dev_alloc(m, &L.coef64, 4));
+  if (!L.coef32) FE_TRY(dev_alloc(m, &L.coef32, 4));
+  double* scal = h->scal + q * SC_N;
+  const PowerArgs pa{h->part, h->ticket, scal, L.coef64, L.coef32};
   C* x = (C*)h->pw;
   C* y = x + N;
-  k_amg_start<C><<<blocks_for(N, 256), 256, 0, m->stream>>>(N, x);
-  for (int it = 0; it < AMG_POWER_STEPS; it++) {
-    {
-      FE_SCOPE(m, FE_PROF_OTHER, (double)L.nnz * (B * B * sizeof(V) + 4) + 2.0 * sizeof(C) * N);
-      k_amg_dmv<C, V, B><<<blocks_for((int64_t)L.n * 32, 256), 256, 0, m->stream>>>(L.n, L.ptr, L.col, A, dinv, x, y);
-    }
-    k_amg_sumsq2<C><<<AMG_RED_BLOCKS, 256, 0, m->stream>>>(N, x, y, h->part);
-    k_amg_power_step<C><<<blocks_for(N, 256), 256, 0, m->stream>>>(N, AMG_RED_BLOCKS, h->part, y, x, h->scal);
-  }
+  k_amg_start<C><<<blocks_for(N, 256), 256, 0, m->stream>>>(N, x, scal);
   FE_CUDA(cudaGetLastError());
-  FE_CUDA(cudaMemcpyAsync(m->h_scal + 20, h->scal, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
-  FE_CUDA(cudaStreamSynchronize(m->stream));
-  L.rho = m->h_scal[20];
-  if (!(L.rho > 0.0) || !std::isfinite(L.rho))
-    return fe_set_error("AMG: spectral radius estimate %g on level %d", L.rho, q), FE_ERR_STATE;
-  const C omega = (C)(4.0 / (3.0 * L.rho));
+  bool small = false;
+  if constexpr (B == AMG_NS) {
+    if (L.nnz <= AMG_POWER_SMALL<C>) {
+      small = true;
+      FE_SCOPE(m, FE_PROF_OTHER, AMG_POWER_STEPS * ((double)L.nnz * (B * B * sizeof(V) + 4) + 2.0 * sizeof(C) * N));
+      k_amg_power_small<C><<<1, 512, 0, m->stream>>>(L.n, AMG_POWER_STEPS, L.ptr, L.col, A, dinv, x, y, pa);
+      FE_CUDA(cudaGetLastError());
+    }
+  }
+  if (!small)
+    for (int it = 0; it < AMG_POWER_STEPS; it++) {
+      FE_TRY((power_step<C, V, B>(m, L, val, dinv, x, y, pa, it == AMG_POWER_STEPS - 1)));
+      std::swap(x, y);
+    }
   C*& p = Arr<C>::p(L);
   C*& ap = Arr<C>::ap(L);
   C*& r = Arr<C>::r(L);
+  C*& pt = Arr<C>::pt(L);
   if (!p) FE_TRY(dev_alloc(m, &p, (size_t)L.nnzp * B * AMG_NS));
+  if (!pt) FE_TRY(dev_alloc(m, &pt, (size_t)tiled_count(L.nnzp, B * AMG_NS)));
   if (!ap) FE_TRY(dev_alloc(m, &ap, (size_t)L.nnzap * B * AMG_NS));
   if (!r) FE_TRY(dev_alloc(m, &r, (size_t)L.nnzr * B * AMG_NS));
   AmgLevel& Cq = h->lev[q + 1];
   C*& cval = Arr<C>::val(Cq);
   if (!cval) FE_TRY(dev_alloc(m, &cval, (size_t)Cq.nnz * AMG_NS * AMG_NS));
   {
-    FE_SCOPE(m, FE_PROF_OTHER, (double)L.nnzp * B * AMG_NS * sizeof(C));
-    k_amg_pvals<C, V, B><<<blocks_for(L.nnzp, 128), 128, 0, m->stream>>>(L.nnzp, L.prow, L.pcol, L.ptr, L.col, A,
-                                                                        L.agg, dinv, L.tnode, omega, p);
+    FE_SCOPE(m, FE_PROF_OTHER, 3.0 * L.nnzp * B * AMG_NS * sizeof(C));
+    const C* tn = nullptr;
+    if constexpr (sizeof(C) == 8) tn = L.tnode;
+    else tn = L.tnode32;
+    k_amg_pvals<C, V, B><<<blocks_for(L.nnzp * B, B == 3 ? 192 : 64), B == 3 ? 192 : 64, 0, m->stream>>>(
+        L.nnzp, L.prow, L.pcol, L.pk_ptr, L.pk, L.col, A, L.agg, dinv, tn, scal, L.rpos, p, pt, r);
   }
   FE_CUDA(cudaGetLastError());
   {
     FE_SCOPE(m, FE_PROF_OTHER, (double)L.nnzap * B * AMG_NS * sizeof(C));
-    k_amg_ap<C, V, B><<<blocks_for(L.nnzap, 128), 128, 0, m->stream>>>(L.nnzap, L.aprow, L.apcol, L.ptr, L.col, A,
-                                                                      L.pptr, L.pcol, p, ap);
+    constexpr int W = ap_warps<C, B>();
+    const int smem = W * (int)sizeof(ApShared<C, B>);
+    FE_TRY(fe_kernel_smem((const void*)k_amg_ap<C, V, B>, smem));
+    k_amg_ap<C, V, B><<<blocks_for(L.n, W), 32 * W, smem, m->stream>>>(L.n, L.ptr, L.col, A, L.pptr, p, L.apptr,
+                                                                      L.apoff, L.apidx, ap);
   }
   FE_CUDA(cudaGetLastError());
   {
     FE_SCOPE(m, FE_PROF_OTHER, (double)Cq.nnz * AMG_NS * AMG_NS * sizeof(C));
-    k_amg_rap<C, B><<<blocks_for(Cq.nnz, 128), 128, 0, m->stream>>>(Cq.nnz, Cq.crow, Cq.col, L.rptr, L.rcol, L.rsrc,
-                                                                    L.apptr, L.apcol, p, ap, Cq.absent, cval);
+    k_amg_rap<C, B><<<blocks_for(Cq.nnz * (B == 3 ? AMG_NS : AMG_NS * AMG_NS), B == 3 ? 192 : 64), B == 3 ? 192 : 64, 0, m->stream>>>(
+        Cq.nnz, L.crow, Cq.col, L.lend, L.raoff, L.ralist, p, ap, Cq.absent, cval);
   }
   FE_CUDA(cudaGetLastError());
-  k_amg_rvals<C, B><<<blocks_for(L.nnzr, 256), 256, 0, m->stream>>>(L.nnzr, L.rsrc, p, r);
-  FE_CUDA(cudaGetLastError());
-  return FE_OK;
-}
-
-int store_coeffs(fe_mesh m);
-
-template <int NV, class T>
-int tile_one(fe_mesh m, const T* src, T** dst, int64_t nblocks) {
-  if (!*dst) FE_TRY(dev_alloc(m, dst, (size_t)tiled_count(nblocks, NV)));
-  k_amg_tile<NV, T><<<blocks_for(nblocks * NV, 256), 256, 0, m->stream>>>(nblocks, src, *dst);
-  FE_CUDA(cudaGetLastError());
-  return FE_OK;
-}
-
-// tiled V-cycle copies of the prolongators
-template <class C>
-int tile_copies(fe_mesh m) {
-  AmgHier* h = m->amg;
-  for (int q = 0; q < h->nlev; q++) {
-    AmgLevel& L = h->lev[q];
-    C** pt = std::is_same<C, double>::value ? (C**)&L.pt64 : (C**)&L.pt32;
-    if (q < h->nlev - 1) {
-      if (L.b == 3) FE_TRY((tile_one<3 * AMG_NS, C>(m, Arr<C>::p(L), pt, L.nnzp)));
-      else FE_TRY((tile_one<AMG_NS * AMG_NS, C>(m, Arr<C>::p(L), pt, L.nnzp)));
-    }
-  }
   return FE_OK;
 }
 
@@ -1554,11 +2020,18 @@ int tile_copies(fe_mesh m) {
 template <class C, class V>
 int numeric_all(fe_mesh m, const V* K0) {
   AmgHier* h = m->amg;
-  FE_TRY((numeric_level<C, V, 3>(m, 0, Vals<C, V, 3>{K0, true})));
-  for (int q = 1; q < h->nlev; q++)
-    FE_TRY((numeric_level<C, C, AMG_NS>(m, q, Vals<C, C, AMG_NS>{Arr<C>::val(h->lev[q]), false})));
-  FE_TRY(store_coeffs(m));
-  return tile_copies<C>(m);
+  FE_TRY((numeric_level<C, V, 3>(m, 0, K0)));
+  for (int q = 1; q < h->nlev; q++) FE_TRY((numeric_level<C, C, AMG_NS>(m, q, Arr<C>::val(h->lev[q]))));
+  double sc[AMG_MAXLEV * SC_N];
+  FE_CUDA(cudaMemcpyAsync(sc, h->scal, sizeof(sc), cudaMemcpyDeviceToHost, m->stream));
+  FE_CUDA(cudaStreamSynchronize(m->stream));
+  for (int q = 0; q < h->nlev - 1; q++) {
+    const double rho = sc[q * SC_N + SC_RHO];
+    if (!(rho > 0.0) || !std::isfinite(rho))
+      return fe_set_error("AMG: spectral radius estimate %g on level %d", rho, q), FE_ERR_STATE;
+    h->lev[q].rho = rho;
+  }
+  return FE_OK;
 }
 
 int ensure_vectors(fe_mesh m, int elem) {
@@ -1577,39 +2050,6 @@ int ensure_vectors(fe_mesh m, int elem) {
     }
   }
   h->vec_elem = elem;
-  return FE_OK;
-}
-
-struct Cheb {
-  double inv_theta, c1, c2;
-};
-Cheb cheb_coeffs(double rho) {
-  const double lo = rho / 30.0, hi = 1.1 * rho;
-  const double theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo), sigma = theta / delta;
-  const double r0 = 1.0 / sigma, r1 = 1.0 / (2.0 * sigma - r0);
-  return Cheb{1.0 / theta, r1 * r0, 2.0 * r1 / delta};
-}
-
-// Chebyshev coefficients of every smoothed level into device memory
-int store_coeffs(fe_mesh m) {
-  AmgHier* h = m->amg;
-  for (int q = 0; q < h->nlev - 1; q++) {
-    AmgLevel& L = h->lev[q];
-    if (!L.coef64) FE_TRY(dev_alloc(m, &L.coef64, 4));
-    if (!L.coef32) FE_TRY(dev_alloc(m, &L.coef32, 4));
-    const Cheb c = cheb_coeffs(L.rho);
-    double* hd = m->h_scal + 24;  // pinned staging, consumed before the next sync
-    float* hf = (float*)(m->h_scal + 28);
-    hd[0] = c.inv_theta;
-    hd[1] = c.c1;
-    hd[2] = c.c2;
-    hf[0] = (float)c.inv_theta;
-    hf[1] = (float)c.c1;
-    hf[2] = (float)c.c2;
-    FE_CUDA(cudaMemcpyAsync(L.coef64, hd, 3 * sizeof(double), cudaMemcpyHostToDevice, m->stream));
-    FE_CUDA(cudaMemcpyAsync(L.coef32, hf, 3 * sizeof(float), cudaMemcpyHostToDevice, m->stream));
-    FE_CUDA(cudaStreamSynchronize(m->stream));
-  }
   return FE_OK;
 }
 
@@ -1651,7 +2091,7 @@ int vcycle_launches(fe_mesh m, cudaStream_t st, const V* K0, const double* b, do
           Lq.n, h->shape0.warps, h->shape0.ranges, h->part0, Lq.ptr, Lq.col, K0, dinv(0), g, X(0), (T*)Lq.r, dout,
           (T)cx, coef(0), flags);
     else
-      k_vc_cheb<T, AMG_NS><<<blocks_for((int64_t)Lq.n * 32, 256), 256, 0, st>>>(
+      k_vc_cheb<T, AMG_NS><<<blocks_for((int64_t)Lq.n * 32, VC_CHEB_THREADS<T>), VC_CHEB_THREADS<T>, 0, st>>>(
           Lq.n, Lq.ptr, Lq.col, vals(q), dinv(q), g, X(q), (T*)Lq.r, dout, (T)cx, coef(q), flags);
     FE_CUDA(cudaGetLastError());
     return FE_OK;
@@ -1669,7 +2109,7 @@ int vcycle_launches(fe_mesh m, cudaStream_t st, const V* K0, const double* b, do
   // the bottom levels q0..L-1 (at most VC_BOTTOM_MAXN nodes each, q0 >= 1)
   // run in one block when at least one of them is smoothed
   int q0 = L - 1;
-  while (q0 > 1 && h->lev[q0 - 1].n <= VC_BOTTOM_MAXN) q0--;
+  while (!D && q0 > 1 && h->lev[q0 - 1].nnz <= VC_BOTTOM_MAXNNZ) q0--;
   const bool fused = q0 <= L - 2;
   const int qf = fused ? q0 : L - 1;  // the per-level kernels run on levels 0..qf-1
   // downward: pre-smoothing, restriction
@@ -1736,7 +2176,7 @@ int vcycle_launches(fe_mesh m, cudaStream_t st, const V* K0, const double* b, do
         *flops += 2.0 * N * N;
       }
     }
-    k_vc_bottom<T><<<1, vc_bottom_threads<T>(), 0, st>>>(a);
+    if constexpr (!D) k_vc_bottom<T><<<1, VC_BOTTOM_THREADS, 0, st>>>(a);
     FE_CUDA(cudaGetLastError());
   } else {  // coarsest
     AmgLevel& Lc = h->lev[L - 1];

@@ -64,3 +64,35 @@ def test_streamed_spmv_ranges(fe, size, order, precision, tol):
     x = np.random.default_rng(6).standard_normal(om.ndof)
     y, yg = om.spmv(x), m.spmv(torch.from_numpy(x).cuda()).cpu().numpy()
     assert np.abs(yg - y).max() <= tol * np.abs(y).max()
+
+
+# coarse rows of more than one chunk of the products (70 to 85 entries), the
+# power steps in one launch (38 rows, 884 blocks) and in 15 (73 rows on)
+@pytest.mark.parametrize("n", [4, 6, 8, 12])
+def test_amg_setup_sizes(fe, n):
+    # bounds of the hierarchy test: radii 1e-12, operators 1e-11, prolongators
+    # 1e-12 of the largest entry; FP32 arithmetic 2e-5 per product of three
+    # factors, 1e-4 for the sums of a row
+    w = W.twist(n)
+    m, om = fe.Mesh(w), O.Mesh(w)
+    d = 0.002 * np.random.default_rng(7).standard_normal(om.ndof)
+    om.apply_dirichlet(d)
+    dg = torch.from_numpy(d).cuda()
+    om.set_pc("amg")
+    om.tangent(d)
+    m.set_pc("amg")
+    x = np.random.default_rng(8).standard_normal(om.ndof)
+    z = om.pc(x)
+    for prec, tr, tv, tz in (("fp64", 1e-12, 1e-11, 1e-10), ("mixed_fp32", 1e-5, 1e-4, 2e-3)):
+        m.tangent(dg, prec)
+        ol, gl = om.amg_levels(), m.amg_levels()
+        assert len(ol) == len(gl)
+        for lv, (o, g) in enumerate(zip(ol, gl)):
+            if lv < len(ol) - 1:
+                assert abs(g["rho"] - o["rho"]) <= tr * o["rho"], lv
+                assert np.abs(g["pval"] - o["pval"]).max() <= tv * np.abs(o["pval"]).max(), lv
+            if lv > 0:
+                assert np.array_equal(g["col"], o["col"])
+                assert np.abs(g["val"] - o["val"]).max() <= tv * np.abs(o["val"]).max(), lv
+        zg = m.pc(torch.from_numpy(x).cuda()).cpu().numpy()
+        assert np.abs(zg - z).max() <= tz * np.abs(z).max(), prec
