@@ -7,10 +7,9 @@
 // contributions (QP lanes reduced with warp shuffles), then one thread per
 // node gathers its incident contributions in a fixed order, adds loads and
 // springs, masks prescribed components and reduces ||R||^2 deterministically.
-// Tangent: elements in colour order (no two elements of a colour share a
-// node), a CTA per group of elements: material tangent per QP in shared
-// memory, then G_a^T A G_b block products written straight into the
-// block-CSR values (read-modify-write, no atomics).
+// Tangent: the element matrices into a workspace, then a warp per block row
+// adds its node's elements in colour order into the block-CSR values.
+#include <algorithm>
 #include <cmath>
 
 #include "fe_element.cuh"
@@ -177,6 +176,512 @@ int fe_energy_dev(fe_mesh m, const double* d, double* out) {
 
 // ---------------------------------------------------------------- tangent
 
+// ---------------------------------------------------------------- tangent
+// Two kernels.  k_elem_blocks64 / k_elem_blocks32 compute every element's
+// matrix once (blocks (a, b), a <= b; the tangent of a potential is symmetric)
+// into a workspace; k_gather_tangent adds, one warp per block row, the
+// contributions of the node's elements in colour order and writes the finished
+// row in the tiled layout.  Each block is written once, in 128-byte runs.
+// (Before: one launch per colour, elements spread over a block's threads,
+// scattered 4-byte read-modify-writes, each its own 32-byte sector of eight.
+// Cook P2 64x64x8 in FP32: 38 launches, 1,580 us; now 171 + 183 us, the blocks
+// 64 us of traffic at the copy rate each way.  Cardiac shell of 149,760 P1 tets
+// in FP64: 3.1 ms; now 486 us, bound by the FP64 pipe, + 148 us.)  A mesh whose workspace does not fit is assembled colour by colour
+// (k_elem_tangent).
+//
+// FP64: at a quadrature point the material tangent A enters the element matrix
+// only through the four barycentric gradients G_k: M_kl[i][j] = sum_JL G_kJ
+// A_iJjL G_lL, k, l = 0..3.  qp_blocks forms M from the law's own terms (F G_k,
+// H G_k, fibre-frame strains of the directions e_i x G_k), 6 pairs of 9 values,
+// without the 81 entries of A (for the fibre law about a sixth of the FP64
+// operations, which bound it); the pairs with G_0 = -(G_1 + G_2 + G_3) follow
+// by sums.  P1: K_ab = w M_ab.  P2: K_ab = sum_q w sum_kl c_ak(q) c_bl(q)
+// M_kl(q) with at most two k per node and coefficients that depend on q only
+// through lambda_k(q) = beta + (alpha - beta) delta_kq.
+__device__ __forceinline__ constexpr int pair4(int k, int l) {  // k <= l < 4
+  return k * 4 - k * (k - 1) / 2 + (l - k);
+}
+
+template <class T>
+__device__ void qp_blocks(const MatParams& mp, const double* __restrict__ fib, const QPState<T>& s, const T (*G)[3],
+                          T* __restrict__ M) {
+  const T* F = s.F;
+  const T* H = s.H;
+  T FG[3][3], HG[3][3];  // [k - 1][i]
+#pragma unroll
+  for (int k = 0; k < 3; k++)
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+      FG[k][i] = F[3 * i] * G[k + 1][0] + F[3 * i + 1] * G[k + 1][1] + F[3 * i + 2] * G[k + 1][2];
+      HG[k][i] = H[3 * i] * G[k + 1][0] + H[3 * i + 1] * G[k + 1][1] + H[3 * i + 2] * G[k + 1][2];
+    }
+  auto put = [&](int k, int l, int i, int j, T v) { M[9 * pair4(k + 1, l + 1) + 3 * i + j] = v; };
+  if (mp.kind == FE_MAT_COOK_NH) {
+    const T j13 = dcbrt(s.J);
+    const T mj = (T)mp.mu / (j13 * j13), cv = (T)mp.cvol, J2 = s.J * s.J;
+    const T c23 = -mj * (T(2) / T(3)), chh = mj * (T(2) / T(9)) * s.I1 + T(4) * cv * J2,
+            cht = mj * s.I1 / T(3) - T(2) * cv * (J2 - T(1));
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+#pragma unroll
+      for (int l = k; l < 3; l++) {
+        const T gg = mj * (G[k + 1][0] * G[l + 1][0] + G[k + 1][1] * G[l + 1][1] + G[k + 1][2] * G[l + 1][2]);
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+          const T ah = c23 * FG[k][i] + chh * HG[k][i], af = c23 * HG[k][i], at = cht * HG[l][i];
+#pragma unroll
+          for (int j = 0; j < 3; j++)
+            put(k, l, i, j, ah * HG[l][j] + af * FG[l][j] + at * HG[k][j] + (i == j ? gg : T(0)));
+        }
+      }
+  } else if (mp.kind == FE_MAT_TH_NH) {
+    const T mu = (T)mp.mu, pJ = s.p * s.J;
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+#pragma unroll
+      for (int l = k; l < 3; l++) {
+        const T gg = mu * (G[k + 1][0] * G[l + 1][0] + G[k + 1][1] * G[l + 1][1] + G[k + 1][2] * G[l + 1][2]);
+#pragma unroll
+        for (int i = 0; i < 3; i++)
+#pragma unroll
+          for (int j = 0; j < 3; j++)
+            put(k, l, i, j, (mu + pJ) * (HG[l][i] * HG[k][j]) - pJ * (HG[k][i] * HG[l][j]) + (i == j ? gg : T(0)));
+      }
+  } else if (mp.kind == FE_MAT_POLYCONVEX) {
+    const T a = (T)mp.ap, b = (T)mp.bp, c = (T)mp.clog, pJ = s.p * s.J;
+    T Bm[9];  // F F^T
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+      for (int j = 0; j < 3; j++)
+        Bm[3 * i + j] = F[3 * i] * F[3 * j] + F[3 * i + 1] * F[3 * j + 1] + F[3 * i + 2] * F[3 * j + 2];
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+#pragma unroll
+      for (int l = k; l < 3; l++) {
+        const T gg = G[k + 1][0] * G[l + 1][0] + G[k + 1][1] * G[l + 1][1] + G[k + 1][2] * G[l + 1][2];
+        const T ff = FG[k][0] * FG[l][0] + FG[k][1] * FG[l][1] + FG[k][2] * FG[l][2];
+        const T dg = T(2) * a * gg + T(2) * b * (s.I1 * gg - ff);
+#pragma unroll
+        for (int i = 0; i < 3; i++)
+#pragma unroll
+          for (int j = 0; j < 3; j++)
+            put(k, l, i, j,
+                T(2) * b * (T(2) * FG[l][j] * FG[k][i] - FG[l][i] * FG[k][j] - Bm[3 * i + j] * gg) +
+                    (c + pJ) * (HG[l][i] * HG[k][j]) - pJ * (HG[k][i] * HG[l][j]) + (i == j ? dg : T(0)));
+      }
+  } else {
+    T fr[9];  // rows f, s, n
+#pragma unroll
+    for (int q = 0; q < 9; q++) fr[q] = (T)fib[q];
+    T Fr[9], Gr[3][3];  // rows of F and the gradients in the fibre frame
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+      for (int al = 0; al < 3; al++) {
+        Fr[3 * i + al] = F[3 * i] * fr[3 * al] + F[3 * i + 1] * fr[3 * al + 1] + F[3 * i + 2] * fr[3 * al + 2];
+        Gr[i][al] = fr[3 * al] * G[i + 1][0] + fr[3 * al + 1] * G[i + 1][1] + fr[3 * al + 2] * G[i + 1][2];
+      }
+    const T ce = (T)mp.C * s.eQ;
+    // strain of the direction e_i x G_k: (ff, ss, nn, fs, fn, sn), and D : dE
+    T E[3][3][6], d[3][3], SG[3][3];
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      T DG[3];
+#pragma unroll
+      for (int q = 0; q < 3; q++) {
+        DG[q] = s.D[3 * q] * G[k + 1][0] + s.D[3 * q + 1] * G[k + 1][1] + s.D[3 * q + 2] * G[k + 1][2];
+        SG[k][q] = ce * DG[q];  // S = C e^Q D
+      }
+#pragma unroll
+      for (int i = 0; i < 3; i++) {
+        const T* f = Fr + 3 * i;
+        const T* g = Gr[k];
+        E[k][i][0] = f[0] * g[0];
+        E[k][i][1] = f[1] * g[1];
+        E[k][i][2] = f[2] * g[2];
+        E[k][i][3] = T(0.5) * (f[0] * g[1] + g[0] * f[1]);
+        E[k][i][4] = T(0.5) * (f[0] * g[2] + g[0] * f[2]);
+        E[k][i][5] = T(0.5) * (f[1] * g[2] + g[1] * f[2]);
+        d[k][i] = F[3 * i] * DG[0] + F[3 * i + 1] * DG[1] + F[3 * i + 2] * DG[2];
+      }
+    }
+    const T bf = (T)mp.bf, bt = (T)mp.bt, bfs = (T)mp.bfs;
+    const T wt[6] = {ce * bf, ce * bt, ce * bt, T(2) * ce * bfs, T(2) * ce * bfs, T(2) * ce * bt};
+    const T lJ = dlog(s.J);
+    const T phi = T(0.5) * (T)mp.kappa * (s.J * lJ + s.J - T(1));
+    const T dphiJ = T(0.5) * (T)mp.kappa * (lJ + T(2)) * s.J;
+    const T ga = (T)mp.gamma / s.an, ian2 = T(1) / (s.an * s.an);
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+#pragma unroll
+      for (int l = k; l < 3; l++) {
+        const T act = ga * Gr[k][0] * Gr[l][0];
+        const T gsg = G[l + 1][0] * SG[k][0] + G[l + 1][1] * SG[k][1] + G[l + 1][2] * SG[k][2];
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+          T we[6];
+#pragma unroll
+          for (int q = 0; q < 6; q++) we[q] = wt[q] * E[k][i][q];
+          const T dd = T(2) * ce * d[k][i], dh = dphiJ * HG[k][i], ph = phi * HG[l][i], aa = act * s.a[i] * ian2;
+#pragma unroll
+          for (int j = 0; j < 3; j++) {
+            T v = dd * d[l][j] + dh * HG[l][j] - ph * HG[k][j] - aa * s.a[j];
+#pragma unroll
+            for (int q = 0; q < 6; q++) v += we[q] * E[l][j][q];
+            put(k, l, i, j, v + (i == j ? gsg + act : T(0)));
+          }
+        }
+      }
+  }
+  // pairs with G_0: M_0l = -(M_1l + M_2l + M_3l), M_00 = -(M_10 + M_20 + M_30)
+  auto get = [&](int k, int l, int i, int j) { return k <= l ? M[9 * pair4(k, l) + 3 * i + j] : M[9 * pair4(l, k) + 3 * j + i]; };
+#pragma unroll
+  for (int i = 0; i < 3; i++)
+#pragma unroll
+    for (int j = 0; j < 3; j++)
+#pragma unroll
+      for (int l = 1; l < 4; l++)
+        M[9 * pair4(0, l) + 3 * i + j] = -(get(1, l, i, j) + get(2, l, i, j) + get(3, l, i, j));
+#pragma unroll
+  for (int i = 0; i < 3; i++)
+#pragma unroll
+    for (int j = 0; j < 3; j++)
+      M[3 * i + j] = -(M[9 * pair4(0, 1) + 3 * j + i] + M[9 * pair4(0, 2) + 3 * j + i] + M[9 * pair4(0, 3) + 3 * j + i]);
+}
+
+template <int ORDER>
+struct Blk64Cfg {
+  static constexpr int NEN = ORDER == 1 ? 4 : 10;
+  static constexpr int NQ = ORDER == 1 ? 1 : 4;
+  static constexpr int NPAIR = NEN * (NEN + 1) / 2;
+  static constexpr int EB = ORDER == 1 ? 64 : 16;      // elements per block
+  static constexpr int THREADS = ORDER == 1 ? 64 : 144;  // P2: one per (element, block entry) in the second phase
+  static constexpr int MS = 91;                         // stride of a point's M (odd: no bank conflicts)
+};
+
+// FP64: the element's blocks (a, b), a <= b, [NPAIR][9], and the u-p coupling
+// [NEN][npl][3]; inertia (mass_c M) included
+template <int ORDER, class T>
+__global__ void __launch_bounds__(Blk64Cfg<ORDER>::THREADS)
+    k_elem_blocks64(int ne, const int* __restrict__ conn, const double* __restrict__ geo, const double* __restrict__ d,
+                  int nn, int pres, MatParams mp, const double* __restrict__ fib, double mass_c, T* __restrict__ Ke,
+                  T* __restrict__ Be) {
+  using C = Blk64Cfg<ORDER>;
+  constexpr int NEN = C::NEN, NQ = C::NQ, EB = C::EB, MS = C::MS;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  T* Ms = reinterpret_cast<T*>(smraw);   // [EB * NQ][MS]
+  T* Hs = Ms + EB * NQ * MS;             // u-p: [EB * NQ][12] -J H G_k
+  __shared__ T vols[EB];
+  const int e0 = blockIdx.x * EB;
+  const int eb = min(EB, ne - e0);
+  for (int t = threadIdx.x; t < eb * NQ; t += blockDim.x) {
+    const int e = e0 + t / NQ, q = t % NQ;
+    T G[4][3], vol, lam[4];
+    QPState<T> s;
+    qp_point<ORDER, T>(e, q, conn + (size_t)e * NEN, geo, d, nn, pres, mp, fib, s, G, lam, vol, [](int, const T (&)[3]) {});
+    qp_blocks<T>(mp, fib ? fib + (size_t)e * 9 : nullptr, s, G, Ms + t * MS);
+    if (pres)
+#pragma unroll
+      for (int k = 0; k < 4; k++)
+#pragma unroll
+        for (int i = 0; i < 3; i++)
+          Hs[t * 12 + 3 * k + i] = -s.J * (s.H[3 * i] * G[k][0] + s.H[3 * i + 1] * G[k][1] + s.H[3 * i + 2] * G[k][2]);
+    if (q == 0) vols[t / NQ] = vol;
+  }
+  __syncthreads();
+  if (ORDER == 1) {  // K_ab = vol M_ab, written in the elements' order
+    for (int t = threadIdx.x; t < eb * 90; t += blockDim.x) {
+      const int le = t / 90, r = t - le * 90, ij = r % 9;
+      T v = vols[le] * Ms[le * MS + r];
+      if (mass_c != 0.0 && ij % 4 == 0) {
+        const int p = r / 9, a = p < 4 ? 0 : (p < 7 ? 1 : (p < 9 ? 2 : 3)), b = p - pair4(a, a) + a;
+        v += (T)(mass_c * (double)vols[le] * mass_hat(1, a, b));
+      }
+      Ke[(size_t)(e0 + le) * 90 + r] = v;
+    }
+    return;
+  }
+  // P2: thread (element, entry ij), the 16 ordered barycentric pairs of its
+  // entry at the four points in registers
+  constexpr int ep[6] = {0, 0, 0, 1, 1, 2}, eq[6] = {1, 2, 3, 2, 3, 3};
+  const int le = threadIdx.x / 9, ij = threadIdx.x % 9, ji = 3 * (ij % 3) + ij / 3;
+  if (le < eb) {
+    const T w = vols[le] / T(NQ);
+    T m[4][4][4], S[4][4];  // [q][k][l], sum over q
+#pragma unroll
+    for (int k = 0; k < 4; k++)
+#pragma unroll
+      for (int l = 0; l < 4; l++) {
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+          m[q][k][l] = w * Ms[(le * 4 + q) * MS + (k <= l ? 9 * pair4(k, l) + ij : 9 * pair4(l, k) + ji)];
+        S[k][l] = (m[0][k][l] + m[1][k][l]) + (m[2][k][l] + m[3][k][l]);
+      }
+    const double al = 0.5854101966249685, be = 0.1381966011250105;
+    const T uv = (T)(4.0 * be - 1.0), ue = (T)(4.0 * be), dl = (T)(4.0 * (al - be));
+    // sum_q (u1 + dl [q = s1]) (u2 + dl [q = s2]) m[q][k][l]
+    auto term = [&](T u1, int s1, T u2, int s2, int k, int l) -> T {
+      if (s1 == s2) return u1 * u2 * S[k][l] + dl * (u1 + u2 + dl) * m[s1][k][l];
+      return u1 * u2 * S[k][l] + dl * u1 * m[s2][k][l] + dl * u2 * m[s1][k][l];
+    };
+    T* out = Ke + (size_t)(e0 + le) * (C::NPAIR * 9) + ij;
+    const bool mass = mass_c != 0.0 && ij % 4 == 0;
+    const double mv = mass ? mass_c * (double)vols[le] : 0.0;
+    int pr = 0;
+#pragma unroll
+    for (int a = 0; a < 10; a++)
+#pragma unroll
+      for (int b = a; b < 10; b++) {
+        T v;
+        if (b < 4) {
+          v = term(uv, a, uv, b, a, b);
+        } else if (a < 4) {
+          const int p = ep[b - 4], r = eq[b - 4];  // node b: 4 (lambda_p G_r + lambda_r G_p)
+          v = term(uv, a, ue, p, a, r) + term(uv, a, ue, r, a, p);
+        } else {
+          const int p = ep[a - 4], r = eq[a - 4], s = ep[b - 4], t = eq[b - 4];
+          v = (term(ue, p, ue, s, r, t) + term(ue, p, ue, t, r, s)) + (term(ue, r, ue, s, p, t) + term(ue, r, ue, t, p, s));
+        }
+        if (mass) v += (T)(mv * mass_hat(2, a, b));
+        out[9 * pr] = v;
+        pr++;
+      }
+  }
+  // u-p coupling: sum_q w lv(q) sum_J (-J H)_iJ g_aJ over the element's local
+  // pressure values (P1: 4 vertices, P0: 1)
+  if (pres) {
+    const int npl = pres == 2 ? 1 : 4;
+    for (int t = threadIdx.x; t < eb * NEN * npl; t += blockDim.x) {
+      const int v = t % npl, a = (t / npl) % NEN, l = t / (npl * NEN);
+      T acc[3] = {T(0), T(0), T(0)};
+      for (int q = 0; q < NQ; q++) {
+        const T* h = Hs + (l * NQ + q) * 12;
+        const T lv = pres == 2 ? T(1) : (T)lam_q<ORDER>(q, v);
+        for (int i = 0; i < 3; i++) {
+          T g;
+          if (a < 4) g = (T)(4.0 * lam_q<ORDER>(q, a) - 1.0) * h[3 * a + i];
+          else
+            g = T(4) * ((T)lam_q<ORDER>(q, ep[a - 4]) * h[3 * eq[a - 4] + i] +
+                        (T)lam_q<ORDER>(q, eq[a - 4]) * h[3 * ep[a - 4] + i]);
+          acc[i] += lv * g;
+        }
+      }
+      const T w = vols[l] / T(NQ);
+      for (int i = 0; i < 3; i++) Be[((size_t)(e0 + l) * NEN * npl + a * npl + v) * 3 + i] = w * acc[i];
+    }
+  }
+}
+
+// FP32: the same blocks in the arithmetic of tangent_tile (A per point, C_b =
+// A g_b, K_ab = sum_q w g_a C_b), bit for bit: the FP32 V-cycle amplifies the
+// rounding of the tangent by the condition of its coarse operators, so the
+// values keep their order of operations whichever kernel forms them.  C_b
+// stays in registers: a thread takes rows i of the blocks (., b) of its b (P2:
+// of b and 9 - b, eleven blocks each), reading A's rows and the gradients from
+// shared memory by 16 bytes.
+template <int ORDER>
+struct Blk32Cfg {
+  static constexpr int NEN = ORDER == 1 ? 4 : 10;
+  static constexpr int NQ = ORDER == 1 ? 1 : 4;
+  static constexpr int NPAIR = NEN * (NEN + 1) / 2;
+  static constexpr int EB = 16;                      // elements per block
+  static constexpr int TPE = ORDER == 1 ? 12 : 15;   // threads per element
+  static constexpr int THREADS = EB * TPE;
+  static constexpr int AROW = 28;                    // one i: 27 values of A, padded
+  static constexpr int SZ_A = NQ * 3 * AROW, SZ_G = NQ * NEN * 4;
+  static constexpr int PER_E = SZ_A + SZ_G + 4;      // floats (the pad spreads the elements over the banks)
+};
+
+template <int ORDER>
+__global__ void __launch_bounds__(Blk32Cfg<ORDER>::THREADS, 2)
+    k_elem_blocks32(int ne, const int* __restrict__ conn, const double* __restrict__ geo, const double* __restrict__ d,
+                    int nn, int pres, MatParams mp, const double* __restrict__ fib, double mass_c,
+                    float* __restrict__ Ke, float* __restrict__ Be) {
+  using C = Blk32Cfg<ORDER>;
+  using T = float;
+  constexpr int NEN = C::NEN, NQ = C::NQ, EB = C::EB;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  T* sm = reinterpret_cast<T*>(smraw);   // [EB][PER_E]: A [NQ][3][AROW], g [NQ][NEN][4]
+  T* dps = sm + EB * C::PER_E;           // u-p: [EB * NQ][9]
+  __shared__ QPState<T> qs[EB * NQ];
+  __shared__ T ws[EB];
+  const int e0 = blockIdx.x * EB, eb = min(EB, ne - e0);
+  for (int k = threadIdx.x; k < eb * NQ; k += blockDim.x) {
+    const int le = k / NQ, q = k % NQ, e = e0 + le;
+    T G[4][3], vol, lam[4];
+    T* gb = sm + le * C::PER_E + C::SZ_A + q * NEN * 4;
+    QPState<T>& s = qs[k];
+    qp_point<ORDER, T>(e, q, conn + (size_t)e * NEN, geo, d, nn, pres, mp, fib, s, G, lam, vol,
+                       [&](int a, const T (&g)[3]) {
+                         *reinterpret_cast<float4*>(gb + 4 * a) = make_float4(g[0], g[1], g[2], 0.f);
+                       });
+    if (q == 0) ws[le] = vol / NQ;
+    if (pres)
+      for (int j = 0; j < 9; j++) dps[k * 9 + j] = -s.J * s.H[j];
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < eb * NQ * 9; k += blockDim.x) {
+    const int lq = k / 9, kl = k % 9, le = lq / NQ, q = lq % NQ;
+    T colv[9];
+    qp_tangent_col(mp, fib ? fib + (size_t)(e0 + le) * 9 : nullptr, qs[lq], kl / 3, kl % 3, colv);
+    T* A = sm + le * C::PER_E + q * 3 * C::AROW;
+#pragma unroll
+    for (int ij = 0; ij < 9; ij++) A[(ij / 3) * C::AROW + (ij % 3) * 9 + kl] = colv[ij];
+  }
+  __syncthreads();
+  const int le = threadIdx.x / C::TPE, r = threadIdx.x % C::TPE, i = r % 3;
+  if (le < eb) {
+    const T* A = sm + le * C::PER_E + i * C::AROW;
+    const T* g = sm + le * C::PER_E + C::SZ_A;
+    const T w = ws[le];
+    T* out = Ke + (size_t)(e0 + le) * (C::NPAIR * 9) + 3 * i;
+#pragma unroll 1
+    for (int h = 0; h < (ORDER == 1 ? 1 : 2); h++) {
+      const int b = h == 0 ? r / 3 : 9 - r / 3;
+      T c[NQ][3][3];
+#pragma unroll
+      for (int q = 0; q < NQ; q++) {
+        T a[C::AROW];
+#pragma unroll
+        for (int t = 0; t < C::AROW / 4; t++)
+          *reinterpret_cast<float4*>(a + 4 * t) = *reinterpret_cast<const float4*>(A + q * 3 * C::AROW + 4 * t);
+        const float4 gb = *reinterpret_cast<const float4*>(g + (q * NEN + b) * 4);
+#pragma unroll
+        for (int J = 0; J < 3; J++)
+#pragma unroll
+          for (int kk = 0; kk < 3; kk++)
+            c[q][J][kk] = a[9 * J + 3 * kk] * gb.x + a[9 * J + 3 * kk + 1] * gb.y + a[9 * J + 3 * kk + 2] * gb.z;
+      }
+#pragma unroll 1
+      for (int a = 0; a <= b; a++) {
+        T acc[3] = {T(0), T(0), T(0)};
+#pragma unroll
+        for (int q = 0; q < NQ; q++) {
+          const float4 g4 = *reinterpret_cast<const float4*>(g + (q * NEN + a) * 4);
+          const T ga[3] = {g4.x, g4.y, g4.z};
+#pragma unroll
+          for (int J = 0; J < 3; J++)
+#pragma unroll
+            for (int kk = 0; kk < 3; kk++) acc[kk] += ga[J] * c[q][J][kk];
+        }
+        if (mass_c != 0.0) {  // inertia of a Newmark step: 4 rho / dt^2 M_ab on the block diagonal
+          const T mv = (T)(mass_c * NQ * mass_hat(ORDER, a, b));
+#pragma unroll
+          for (int kk = 0; kk < 3; kk++)
+            if (kk == i) acc[kk] += mv;
+        }
+        T* o = out + 9 * (a * NEN - a * (a - 1) / 2 + (b - a));
+#pragma unroll
+        for (int kk = 0; kk < 3; kk++) o[kk] = w * acc[kk];
+      }
+    }
+  }
+  if (pres) {  // u-p coupling, as in tangent_tile
+    const int npl = pres == 2 ? 1 : 4;
+    for (int k = threadIdx.x; k < eb * NEN * npl; k += blockDim.x) {
+      const int v = k % npl, a = (k / npl) % NEN, l = k / (npl * NEN);
+      T acc[3] = {T(0), T(0), T(0)};
+      for (int q = 0; q < NQ; q++) {
+        const T* dp = dps + (l * NQ + q) * 9;
+        const T* ga = sm + l * C::PER_E + C::SZ_A + (q * NEN + a) * 4;
+        const T lv = pres == 2 ? T(1) : (T)lam_q<ORDER>(q, v);
+        for (int ii = 0; ii < 3; ii++)
+          acc[ii] += lv * (dp[3 * ii] * ga[0] + dp[3 * ii + 1] * ga[1] + dp[3 * ii + 2] * ga[2]);
+      }
+      for (int ii = 0; ii < 3; ii++) Be[(((size_t)(e0 + l) * NEN + a) * npl + v) * 3 + ii] = ws[l] * acc[ii];
+    }
+  }
+}
+
+// One warp per block row: the row's blocks in shared memory (chunks of
+// TG_CHUNK blocks), the node's elements in colour order (the next element's
+// values are loaded while the current ones are added; a node pair occurs once
+// in an element, so its values have distinct places), prescribed rows and
+// columns zeroed, then the row into the tiles.
+constexpr int TG_CHUNK = 96;
+constexpr int TG_WARPS = 4;
+template <int ORDER, class T>
+__global__ void __launch_bounds__(32 * TG_WARPS)
+    k_gather_tangent(int nn, const int* __restrict__ node_ptr, const int* __restrict__ node_list,
+                     const int* __restrict__ emap, const T* __restrict__ Ke, const int* __restrict__ row_ptr,
+                     const int* __restrict__ col, const uint8_t* __restrict__ fixmask, T* __restrict__ K, int npl,
+                     const int* __restrict__ upmap, const T* __restrict__ Be, const int* __restrict__ up_ptr,
+                     T* __restrict__ B, int64_t nnzb) {
+  using C = Blk64Cfg<ORDER>;  // (the layout of Ke is the same in FP32)
+  constexpr int NEN = C::NEN, NV = (NEN * 9 + 31) / 32;
+  __shared__ T accs[TG_WARPS][TG_CHUNK * 9];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int row = blockIdx.x * TG_WARPS + wid;
+  if (row >= nn) return;
+  T* acc = accs[wid];
+  const int ls = node_ptr[row], lend = node_ptr[row + 1];
+  const int rs = row_ptr[row], re = row_ptr[row + 1];
+  const unsigned fr = fixmask[row];
+  for (int cb = rs; cb < re; cb += TG_CHUNK) {
+    const int m = min(TG_CHUNK, re - cb);
+    for (int t = lane; t < m * 9; t += 32) acc[t] = T(0);
+    __syncwarp();
+    T nv[NV];
+    int np[NV];
+    auto load = [&](int k) {  // this lane's values of the node's k-th element, and their places
+#pragma unroll
+      for (int u = 0; u < NV; u++) {
+        const int t = lane + 32 * u;
+        np[u] = -1;
+        if (k < lend && t < NEN * 9) {
+          const int slot = node_list[k], e = slot / NEN, a = slot - e * NEN, b = t / 9, ij = t - 9 * b;
+          const int lo = min(a, b), hi = max(a, b);
+          const int pr = lo * NEN - lo * (lo - 1) / 2 + (hi - lo);
+          nv[u] = Ke[(size_t)e * (C::NPAIR * 9) + 9 * pr + (a <= b ? ij : 3 * (ij % 3) + ij / 3)];
+          const int pos = fe_idx(emap[(size_t)e * NEN * NEN + a * NEN + b], nnzb) - cb;
+          if (pos >= 0 && pos < m) np[u] = 9 * pos + ij;
+        }
+      }
+    };
+    load(ls);
+    for (int k = ls; k < lend; k++) {
+      T cv[NV];
+      int cp[NV];
+#pragma unroll
+      for (int u = 0; u < NV; u++) {
+        cv[u] = nv[u];
+        cp[u] = np[u];
+      }
+      load(k + 1);
+#pragma unroll
+      for (int u = 0; u < NV; u++)
+        if (cp[u] >= 0) acc[cp[u]] += cv[u];
+      __syncwarp();
+    }
+    for (int pos = lane; pos < m; pos += 32) {
+      const unsigned fc = fixmask[col[cb + pos]];
+#pragma unroll
+      for (int c = 0; c < 9; c++)
+        K[kv_index(cb + pos, c)] = (((fr >> (c / 3)) & 1u) || ((fc >> (c % 3)) & 1u)) ? T(0) : acc[9 * pos + c];
+    }
+    __syncwarp();
+  }
+  if (npl) {
+    const int us = up_ptr[row], ue = up_ptr[row + 1];
+    for (int cb = us; cb < ue; cb += TG_CHUNK) {
+      const int m = min(TG_CHUNK, ue - cb);
+      for (int t = lane; t < m * 3; t += 32) acc[t] = T(0);
+      __syncwarp();
+      for (int k = ls; k < lend; k++) {
+        const int slot = node_list[k];
+        if (lane < npl * 3) {
+          const int pos = upmap[(size_t)slot * npl + lane / 3] - cb;
+          if (pos >= 0 && pos < m) acc[3 * pos + lane % 3] += Be[((size_t)slot * npl + lane / 3) * 3 + lane % 3];
+        }
+        __syncwarp();
+      }
+      for (int t = lane; t < m * 3; t += 32) B[(size_t)cb * 3 + t] = ((fr >> (t % 3)) & 1u) ? T(0) : acc[t];
+      __syncwarp();
+    }
+  }
+}
+
 // One CTA assembles EPB elements of one colour into the block-CSR values.
 template <int ORDER, class T>
 __global__ void __launch_bounds__(256) k_elem_tangent(
@@ -189,13 +694,14 @@ __global__ void __launch_bounds__(256) k_elem_tangent(
 
 // face-pattern blocks: springs (plus 2/dt dashpots while dynamics is on)
 // and the follower-pressure blocks at d, in FP64, prescribed components
-// masked; one thread per node row, the faces of an entry in a fixed order
+// masked; one thread per entry, its faces in a fixed order
 template <int ORDER, class T>
-__global__ void k_add_face_blocks(int nn, const int* __restrict__ ks_ptr, const int* __restrict__ ks_col,
+__global__ void k_add_face_blocks(int64_t nnz_ks, const int* __restrict__ ks_row, const int* __restrict__ ks_col,
                                   const double* __restrict__ ks_val, const int* __restrict__ ks_kpos,
                                   const uint8_t* __restrict__ fixmask, FollowerFaces ff,
                                   const double* __restrict__ d, double load, T* K) {
-  face_blocks_row<ORDER, T>(blockIdx.x * blockDim.x + threadIdx.x, nn, ks_ptr, ks_col, ks_val, ks_kpos, fixmask, ff, d, load, K);
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < nnz_ks) face_block_entry<ORDER, T>((int)k, ks_row[k], ks_col, ks_val, ks_kpos, fixmask, ff, d, load, K);
 }
 
 // unit diagonal at prescribed components, then invert each 3x3 diagonal block
@@ -205,20 +711,23 @@ __global__ void k_diag_inverse(int nn, const int* __restrict__ diag_pos, const u
   diag_inverse_row<T, DT>(blockIdx.x * blockDim.x + threadIdx.x, nn, diag_pos, fixmask, K, Dinv);
 }
 
-// SIMPLE Schur diagonal: S_vv = -sum_{(a,v)} sum_i B[a,v]_i^2 / A_(ai,ai)
+// SIMPLE Schur diagonal: S_vv = -sum_{(a,v)} sum_i B[a,v]_i^2 / A_(ai,ai), a
+// warp per vertex (a thread per vertex walked its 60-odd nodes' three FP64
+// divisions alone: 220 us for 2,197 vertices)
 template <class T>
 __global__ void k_schur_diag(int np, const int* __restrict__ pu_ptr, const int* __restrict__ pu_col,
                              const int* __restrict__ pu_src, const int* __restrict__ diag_pos,
                              const T* __restrict__ K, const T* __restrict__ B, double* Sd) {
-  int v = blockIdx.x * blockDim.x + threadIdx.x;
+  const int v = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (v >= np) return;
   double s = 0.0;
-  for (int k = pu_ptr[v]; k < pu_ptr[v + 1]; k++) {
+  for (int k = pu_ptr[v] + lane; k < pu_ptr[v + 1]; k += 32) {
     const int p = diag_pos[pu_col[k]];
     const T* b = B + (size_t)pu_src[k] * 3;
     for (int i = 0; i < 3; i++) s -= (double)b[i] * (double)b[i] / (double)K[kv_index(p, 4 * i)];
   }
-  Sd[v] = s;
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) Sd[v] = s;
 }
 
 __global__ void k_to_bf16(int64_t n, const float* __restrict__ src, __nv_bfloat16* __restrict__ dst) {
@@ -226,10 +735,62 @@ __global__ void k_to_bf16(int64_t n, const float* __restrict__ src, __nv_bfloat1
   if (i < n) dst[i] = __float2bfloat16_rn(src[i]);
 }
 
+// the element blocks' workspace, kept in the mesh (the larger of the two
+// precisions it was asked for); FE_ERR_OOM where it does not fit
+static int tangent_workspace(fe_mesh m, size_t elem) {
+  const size_t npair = (size_t)m->nen * (m->nen + 1) / 2, npl = m->pres == 0 ? 0 : (m->pres == 2 ? 1 : 4);
+  const size_t bytes = (size_t)m->ne * (9 * npair + 3 * npl * m->nen) * elem;
+  if (m->tan_work_bytes >= bytes) return FE_OK;
+  if (m->tan_work) {
+    FE_CUDA(cudaFreeAsync(m->tan_work, m->stream));
+    m->device_bytes -= (int64_t)m->tan_work_bytes;
+    m->tan_work = nullptr;
+    m->tan_work_bytes = 0;
+  }
+  FE_TRY(fe_alloc(m, &m->tan_work, bytes));
+  m->tan_work_bytes = bytes;
+  return FE_OK;
+}
+
+template <int ORDER, class T>
+static int launch_tangent_blocks(fe_mesh m, const double* d, T* K, T* B) {
+  using C = Blk64Cfg<ORDER>;
+  const double mass = m->dyn ? m->mass_c : 0.0, nen = C::NEN;
+  const int npl = m->pres == 0 ? 0 : (m->pres == 2 ? 1 : 4);
+  T *Ke = (T*)m->tan_work, *Be = Ke + (size_t)m->ne * C::NPAIR * 9;
+  {
+    FE_SCOPE(m, FE_PROF_TANGENT, (double)m->ne * (4 * nen + 84 + 24 * nen + sizeof(T) * (9.0 * C::NPAIR + 3.0 * npl * nen)));
+    if constexpr (sizeof(T) == 8) {
+      const int smem = (int)sizeof(T) * C::EB * C::NQ * (C::MS + (m->pres ? 12 : 0));
+      FE_TRY(fe_kernel_smem((const void*)k_elem_blocks64<ORDER, T>, smem));
+      k_elem_blocks64<ORDER, T><<<(m->ne + C::EB - 1) / C::EB, C::THREADS, smem, m->stream>>>(
+          m->ne, m->conn, m->geo, d, m->nn, m->pres, m->mp, m->fib, mass, Ke, Be);
+    } else {
+      using F = Blk32Cfg<ORDER>;
+      const int smem = (int)sizeof(T) * F::EB * (F::PER_E + (m->pres ? F::NQ * 9 : 0));
+      FE_TRY(fe_kernel_smem((const void*)k_elem_blocks32<ORDER>, smem));
+      k_elem_blocks32<ORDER><<<(m->ne + F::EB - 1) / F::EB, F::THREADS, smem, m->stream>>>(
+          m->ne, m->conn, m->geo, d, m->nn, m->pres, m->mp, m->fib, mass, Ke, Be);
+    }
+    FE_CUDA(cudaGetLastError());
+  }
+  FE_SCOPE(m, FE_PROF_TANGENT, (double)m->ne * (sizeof(T) * (9.0 * C::NPAIR + 3.0 * npl * nen) + 4 * nen * nen) +
+                                   (double)m->nnzb * (9 * sizeof(T) + 4) + 12.0 * m->nn + 3.0 * sizeof(T) * m->nnz_up);
+  k_gather_tangent<ORDER, T><<<(m->nn + TG_WARPS - 1) / TG_WARPS, 32 * TG_WARPS, 0, m->stream>>>(
+      m->nn, m->node_ptr, m->color_list, m->emap, Ke, m->row_ptr, m->col, m->fixmask, K, npl, m->upmap, Be, m->up_ptr,
+      B, m->nnzb);
+  FE_CUDA(cudaGetLastError());
+  return FE_OK;
+}
+
 template <int ORDER, class T>
 static int launch_tangent(fe_mesh m, const double* d, T* K, T* B) {
   using C = TanCfg<ORDER, T>;
   size_t smem = sizeof(T) * C::EPB * C::PER_E;
+  const size_t nval = kv_count(m->nnzb);
+  if (tangent_workspace(m, sizeof(T)) == FE_OK) return launch_tangent_blocks<ORDER, T>(m, d, K, B);
+  FE_CUDA(cudaMemsetAsync(K, 0, nval * sizeof(T), m->stream));
+  if (m->pres) FE_CUDA(cudaMemsetAsync(B, 0, (size_t)std::max<int64_t>(m->nnz_up, 1) * 3 * sizeof(T), m->stream));
   FE_TRY(fe_kernel_smem((const void*)k_elem_tangent<ORDER, T>, (int)smem));
   for (int c = 0; c < m->ncolors; c++) {
     int start = m->h_color_start[c], nel = m->h_color_start[c + 1] - start;
@@ -247,12 +808,23 @@ static int launch_tangent(fe_mesh m, const double* d, T* K, T* B) {
   return FE_OK;
 }
 
+// the tiled values; the last tile's padding is zero (every assembly writes the
+// blocks)
+template <class T>
+static int alloc_values(fe_mesh m, T** K) {
+  const size_t nval = kv_count(m->nnzb);
+  FE_TRY(fe_alloc_t(m, K, nval));
+  FE_CUDA(cudaMemsetAsync(*K, 0, nval * sizeof(T), m->stream));
+  return FE_OK;
+}
+
 template <class T>
 static int add_face_blocks(fe_mesh m, const double* d, T* K) {
   FE_SCOPE(m, FE_PROF_TANGENT, (double)m->nnz_ks * (4 + 4 + 72 + 2 * 9 * sizeof(T)));
   auto kern = m->order == 1 ? k_add_face_blocks<1, T> : k_add_face_blocks<2, T>;
-  kern<<<(m->nn + 255) / 256, 256, 0, m->stream>>>(m->nn, m->ks_ptr, m->ks_col, m->ks_val, m->ks_kpos, m->fixmask,
-                                                   follower_faces(m), d, m->load, K);
+  kern<<<(unsigned)((m->nnz_ks + 127) / 128), 128, 0, m->stream>>>(m->nnz_ks, m->ks_row, m->ks_col, m->ks_val,
+                                                                   m->ks_kpos, m->fixmask, follower_faces(m), d,
+                                                                   m->load, K);
   FE_CUDA(cudaGetLastError());
   return FE_OK;
 }
@@ -264,11 +836,9 @@ int fe_tangent_dev(fe_mesh m, const double* d, int precision) {
   const size_t nval = kv_count(m->nnzb);  // tiles of 32 blocks (the last one zero-padded)
   const size_t nb = (size_t)(m->nnz_up > 0 ? m->nnz_up : 1) * 3;
   if (precision == FE_PREC_FP64) {
-    if (!m->K64) FE_TRY(fe_alloc_t(m, &m->K64, nval));
+    if (!m->K64) FE_TRY(alloc_values(m, &m->K64));
     if (!m->Dinv64) FE_TRY(fe_alloc_t(m, &m->Dinv64, (size_t)m->nn * 9));
     if (m->pres && !m->B64) FE_TRY(fe_alloc_t(m, &m->B64, nb));
-    FE_CUDA(cudaMemsetAsync(m->K64, 0, nval * sizeof(double), m->stream));
-    if (m->pres) FE_CUDA(cudaMemsetAsync(m->B64, 0, nb * sizeof(double), m->stream));
     if (m->order == 1) FE_TRY((launch_tangent<1, double>(m, d, m->K64, m->B64)));
     else FE_TRY((launch_tangent<2, double>(m, d, m->K64, m->B64)));
     if (m->nnz_ks) FE_TRY(add_face_blocks(m, d, m->K64));
@@ -276,11 +846,9 @@ int fe_tangent_dev(fe_mesh m, const double* d, int precision) {
     k_diag_inverse<double, double><<<(m->nn + 255) / 256, 256, 0, m->stream>>>(m->nn, m->diag_pos, m->fixmask,
                                                                                m->K64, m->Dinv64);
   } else {
-    if (!m->K32) FE_TRY(fe_alloc_t(m, &m->K32, nval));
+    if (!m->K32) FE_TRY(alloc_values(m, &m->K32));
     if (!m->Dinv32) FE_TRY(fe_alloc_t(m, &m->Dinv32, (size_t)m->nn * 9));
     if (m->pres && !m->B32) FE_TRY(fe_alloc_t(m, &m->B32, nb));
-    FE_CUDA(cudaMemsetAsync(m->K32, 0, nval * sizeof(float), m->stream));
-    if (m->pres) FE_CUDA(cudaMemsetAsync(m->B32, 0, nb * sizeof(float), m->stream));
     if (m->order == 1) FE_TRY((launch_tangent<1, float>(m, d, m->K32, m->B32)));
     else FE_TRY((launch_tangent<2, float>(m, d, m->K32, m->B32)));
     if (m->nnz_ks) FE_TRY(add_face_blocks(m, d, m->K32));
@@ -300,10 +868,10 @@ int fe_tangent_dev(fe_mesh m, const double* d, int precision) {
     if (!m->Sd) FE_TRY(fe_alloc_t(m, &m->Sd, (size_t)m->np));
     FE_SCOPE(m, FE_PROF_TANGENT, (double)m->nnz_up * (8 + 3.0 * (precision == FE_PREC_FP64 ? 8 : 4) + 4) + 12.0 * m->np);
     if (precision == FE_PREC_FP64)
-      k_schur_diag<double><<<(m->np + 255) / 256, 256, 0, m->stream>>>(m->np, m->pu_ptr, m->pu_col, m->pu_src,
+      k_schur_diag<double><<<(m->np + 7) / 8, 256, 0, m->stream>>>(m->np, m->pu_ptr, m->pu_col, m->pu_src,
                                                                        m->diag_pos, m->K64, m->B64, m->Sd);
     else
-      k_schur_diag<float><<<(m->np + 255) / 256, 256, 0, m->stream>>>(m->np, m->pu_ptr, m->pu_col, m->pu_src,
+      k_schur_diag<float><<<(m->np + 7) / 8, 256, 0, m->stream>>>(m->np, m->pu_ptr, m->pu_col, m->pu_src,
                                                                       m->diag_pos, m->K32, m->B32, m->Sd);
     FE_CUDA(cudaGetLastError());
   }

@@ -634,7 +634,38 @@ struct TanCfg {
   static constexpr int PER_E = SZ_A + SZ_G + SZ_C + SZ_DP + SZ_L + NQ;
 };
 
-// One CTA assembles EPB elements of one colour into the block-CSR values.
+// F, the pressure and the material state at quadrature point q of element e
+// (nodes c); put(a, g) receives the gradient of shape function a
+template <int ORDER, class T, class Put>
+__device__ __forceinline__ void qp_point(int e, int q, const int* c, const double* __restrict__ geo,
+                                         const double* __restrict__ d, int nn, int pres, const MatParams& mp,
+                                         const double* __restrict__ fib, QPState<T>& s, T (&G)[4][3], T (&lam)[4],
+                                         T& vol, Put&& put) {
+  constexpr int NEN = TanCfg<ORDER, T>::NEN;
+  load_G(geo, e, G, vol);
+#pragma unroll
+  for (int k = 0; k < 4; k++) lam[k] = (T)lam_q<ORDER>(q, k);
+#pragma unroll
+  for (int j = 0; j < 9; j++) s.F[j] = (j % 4 == 0) ? T(1) : T(0);
+#pragma unroll
+  for (int a = 0; a < NEN; a++) {
+    T g[3];
+    shape_grad<ORDER>(a, lam, G, g);
+    put(a, g);
+    const double* u = d + 3 * (size_t)c[a];
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+      for (int J = 0; J < 3; J++) s.F[3 * i + J] += (T)u[i] * g[J];
+  }
+  s.p = T(0);
+  if (pres == 1)
+    for (int v = 0; v < 4; v++) s.p += (T)d[3 * (size_t)nn + c[v]] * lam[v];
+  else if (pres == 2)
+    s.p = (T)d[3 * (size_t)nn + e];
+  qp_prepare(mp, fib ? fib + (size_t)e * 9 : nullptr, s);
+}
+
 // One group of EPB elements (tile) of one colour assembled by the whole CTA
 // (phases separated by __syncthreads; a caller looping over tiles puts a
 // __syncthreads between calls)
@@ -672,29 +703,12 @@ __device__ __forceinline__ void tangent_tile(int tile,
     int le = k / NQ, q = k % NQ;
     int e = selem[le];
     if (e < 0) continue;
-    T G[4][3], vol;
-    load_G(geo, e, G, vol);
-    T lam[4];
-    for (int c = 0; c < 4; c++) lam[c] = (T)lam_q<ORDER>(q, c);
+    T G[4][3], vol, lam[4];
     T* gb = Gbuf(le, q);
     QPState<T>& s = qs[k];
-    for (int j = 0; j < 9; j++) s.F[j] = (j % 4 == 0) ? T(1) : T(0);
-    for (int a = 0; a < NEN; a++) {
-      T g[3];
-      shape_grad<ORDER>(a, lam, G, g);
-      gb[3 * a] = g[0];
-      gb[3 * a + 1] = g[1];
-      gb[3 * a + 2] = g[2];
-      const double* u = d + 3 * (size_t)sconn[le][a];
-      for (int i = 0; i < 3; i++)
-        for (int J = 0; J < 3; J++) s.F[3 * i + J] += (T)u[i] * g[J];
-    }
-    s.p = T(0);
-    if (pres == 1)
-      for (int v = 0; v < 4; v++) s.p += (T)d[3 * (size_t)nn + sconn[le][v]] * lam[v];
-    else if (pres == 2)
-      s.p = (T)d[3 * (size_t)nn + selem[le]];
-    qp_prepare(mp, fib ? fib + (size_t)e * 9 : nullptr, s);
+    qp_point<ORDER, T>(e, q, sconn[le], geo, d, nn, pres, mp, fib, s, G, lam, vol, [&](int a, const T (&g)[3]) {
+      for (int j = 0; j < 3; j++) gb[3 * a + j] = g[j];
+    });
     T* lb = Lbuf(le, q);
     // pressure shape functions: P1 the barycentric ones, P0 the constant
     for (int c = 0; c < 4; c++) lb[c] = pres == 2 ? (c == 0 ? T(1) : T(0)) : lam[c];
@@ -802,30 +816,37 @@ __device__ __forceinline__ void tangent_tile(int tile,
 
 // face-pattern blocks: springs (plus 2/dt dashpots while dynamics is on)
 // and the follower-pressure blocks at d, in FP64, prescribed components
-// masked; one thread per node row, the faces of an entry in a fixed order
+// masked, the faces of an entry in a fixed order
+template <int ORDER, class T>
+__device__ __forceinline__ void face_block_entry(int k, int a, const int* __restrict__ ks_col,
+                                  const double* __restrict__ ks_val, const int* __restrict__ ks_kpos,
+                                  const uint8_t* __restrict__ fixmask, const FollowerFaces& ff,
+                                  const double* __restrict__ d, double load, T* K) {
+  uint8_t fa = fixmask[a], fb = fixmask[ks_col[k]];
+  const int p = ks_kpos[k];
+  double blk[9];
+  for (int c = 0; c < 9; c++) blk[c] = ks_val[(size_t)k * 9 + c];
+  if (ff.n)
+    for (int j = ff.blk_ptr[k]; j < ff.blk_ptr[k + 1]; j++) {
+      const int code = ff.blk_list[j], f = fe_idx(code >> 6, ff.n);
+      double fk[9];
+      follower_block<ORDER>(ff.nodes + 6 * (size_t)f, ff.kind[f], ff.data + 3 * (size_t)f, load, (code >> 3) & 7,
+                            code & 7, ff.X, d, fk);
+      for (int c = 0; c < 9; c++) blk[c] += fk[c];
+    }
+  for (int i = 0; i < 3; i++)
+    for (int j = 0; j < 3; j++)
+      if (!((fa >> i) & 1) && !((fb >> j) & 1)) K[kv_index(p, 3 * i + j)] += (T)blk[3 * i + j];
+}
+
 template <int ORDER, class T>
 __device__ __forceinline__ void face_blocks_row(int a, int nn, const int* __restrict__ ks_ptr, const int* __restrict__ ks_col,
                                   const double* __restrict__ ks_val, const int* __restrict__ ks_kpos,
                                   const uint8_t* __restrict__ fixmask, FollowerFaces ff,
                                   const double* __restrict__ d, double load, T* K) {
   if (a >= nn) return;
-  for (int k = ks_ptr[a]; k < ks_ptr[a + 1]; k++) {
-    uint8_t fa = fixmask[a], fb = fixmask[ks_col[k]];
-    const int p = ks_kpos[k];
-    double blk[9];
-    for (int c = 0; c < 9; c++) blk[c] = ks_val[(size_t)k * 9 + c];
-    if (ff.n)
-      for (int j = ff.blk_ptr[k]; j < ff.blk_ptr[k + 1]; j++) {
-        const int code = ff.blk_list[j], f = fe_idx(code >> 6, ff.n);
-        double fk[9];
-        follower_block<ORDER>(ff.nodes + 6 * (size_t)f, ff.kind[f], ff.data + 3 * (size_t)f, load, (code >> 3) & 7,
-                              code & 7, ff.X, d, fk);
-        for (int c = 0; c < 9; c++) blk[c] += fk[c];
-      }
-    for (int i = 0; i < 3; i++)
-      for (int j = 0; j < 3; j++)
-        if (!((fa >> i) & 1) && !((fb >> j) & 1)) K[kv_index(p, 3 * i + j)] += (T)blk[3 * i + j];
-  }
+  for (int k = ks_ptr[a]; k < ks_ptr[a + 1]; k++)
+    face_block_entry<ORDER, T>(k, a, ks_col, ks_val, ks_kpos, fixmask, ff, d, load, K);
 }
 
 // unit diagonal at prescribed components, then invert each 3x3 diagonal block

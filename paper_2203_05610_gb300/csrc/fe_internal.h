@@ -119,6 +119,9 @@ struct fe_mesh_s {
   // residual gather lists: node -> (element*nen + local) ; vertex -> (element*4 + local)
   int* node_ptr = nullptr;
   int* node_list = nullptr;
+  int* color_list = nullptr;  // node_list in the order of the elements' colours
+  void* tan_work = nullptr;   // element blocks of the tangent (launch_tangent in fe_assemble.cu), kept between assemblies
+  size_t tan_work_bytes = 0;
   int* vert_ptr = nullptr;
   int* vert_list = nullptr;
 
@@ -127,6 +130,7 @@ struct fe_mesh_s {
   int64_t nnz_ks = 0;
   int* ks_ptr = nullptr;     // [nn+1] spring matrix (Robin faces)
   int* ks_col = nullptr;
+  int* ks_row = nullptr;      // row of each face-pattern entry
   double* ks_val = nullptr;  // [nnz_ks][9]
   int* ks_kpos = nullptr;    // [nnz_ks] block index in the tangent pattern
   // The face pattern (ks_*) covers the node pairs of every face of kind 2

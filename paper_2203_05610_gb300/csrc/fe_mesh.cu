@@ -721,6 +721,10 @@ static int create_impl(const fe_mesh_desc* desc, fe_mesh m) {
   FE_TRY(upload(m, &m->fext1, fext));
   FE_TRY(upload(m, &m->ks_ptr, ks_ptr));
   FE_TRY(upload(m, &m->ks_col, ks_col));
+  std::vector<int> ks_row(ks_col.size());
+  for (int a = 0; a < nn; a++)
+    for (int k = ks_ptr[a]; k < ks_ptr[a + 1]; k++) ks_row[k] = a;
+  FE_TRY(upload(m, &m->ks_row, ks_row));
   FE_TRY(fe_upload_face_values(m));
   FE_TRY(upload(m, &m->ks_kpos, ks_kpos));
   if (m->nff) {
@@ -813,6 +817,13 @@ static int create_impl(const fe_mesh_desc* desc, fe_mesh m) {
     for (int e = 0; e < ne; e++) perm[fill[colors[e]]++] = e;
   }
   FE_TRY(upload(m, &m->perm, perm));
+  {  // a node's elements in colour order (the order in which the tangent adds them)
+    std::vector<int> clist(nlist.size()), fill(nptr.begin(), nptr.end() - 1);
+    for (int e : perm)
+      for (int a = 0; a < m->nen; a++) clist[fill[conn[(size_t)e * m->nen + a]]++] = e * m->nen + a;
+    FE_TRY(upload(m, &m->color_list, clist));
+    FE_CUDA(cudaStreamSynchronize(m->stream));  // clist goes out of scope
+  }
 
   int64_t tot = (int64_t)ne * m->nen * m->nen;
   FE_TRY(fe_alloc_t(m, &m->emap, (size_t)tot));
@@ -843,7 +854,7 @@ static void free_all(fe_mesh m) {
   void* ptrs[] = {m->X, m->conn, m->colors, m->perm, m->geo, m->fib, m->fixmask, m->dgroup,
                   m->d_groups, m->row_ptr, m->col, m->part32, m->part64, m->diag_pos, m->emap, m->up_ptr, m->up_col,
                   m->upmap, m->pu_ptr, m->pu_col, m->pu_src, m->node_ptr, m->node_list,
-                  m->vert_ptr, m->vert_list, m->fext1, m->ks_ptr, m->ks_col, m->ks_val,
+                  m->vert_ptr, m->vert_list, m->fext1, m->ks_ptr, m->ks_col, m->ks_row, m->ks_val, m->color_list, m->tan_work,
                   m->ks_kpos, m->K64, m->K32, m->K16, m->B64, m->B32, m->Dinv64, m->Dinv32,
                   m->Sd, m->rel, m->relp, m->red, m->red_ticket, m->scal, m->bar, m->xch, m->V,
                   m->H, m->gv, m->w64, m->t64, m->u64, m->zx, m->S, m->Yv, m->nl_R, m->nl_Rn,

@@ -125,6 +125,7 @@ int64_t estimate_footprint(const Request& r, int64_t* ndof_out) {
   b += 24 * nn + ne * (4 * nen + 8 + 80 + 4 * nen * nen + 24 * nen + 8 * nen) + 4 * nnzb + 16 * nn;  // mesh
   if (d.fibers) b += 72 * ne;
   if (d.pressure_order) b += ne * (4 * nen * 4 + 32) + 16 * 12 * nn;  // coupling pattern and values
+  b += ne * sval * (9 * nen * (nen + 1) / 2 + (d.pressure_order ? 12 * nen : 0));  // element blocks of the tangent
   b += 9 * sval * nnzb + 9 * sval * nn + (o.precision == FE_PREC_MIXED_BF16 ? 18 * nnzb : 0);  // tangent
   b += 8 * ndof * (restart + 1) + 8 * (restart + 1) * (restart + 1);                             // Krylov basis
   b += 8 * ndof * (2 * mpairs + 12);                                                              // BFGS pairs, vectors

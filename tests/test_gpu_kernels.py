@@ -96,3 +96,72 @@ def test_amg_setup_sizes(fe, n):
                 assert np.abs(g["val"] - o["val"]).max() <= tv * np.abs(o["val"]).max(), lv
         zg = m.pc(torch.from_numpy(x).cuda()).cpu().numpy()
         assert np.abs(zg - z).max() <= tz * np.abs(z).max(), prec
+
+
+def _hub(order):
+    """A vertex inside a ball of 33 points on a sphere (62 elements): its P2 row has 160 blocks."""
+    from scipy.spatial import ConvexHull
+    k = np.arange(33) + 0.5
+    phi, th = np.arccos(1 - 2 * k / 33), np.pi * (1 + 5 ** 0.5) * k
+    pts = np.stack([np.cos(th) * np.sin(phi), np.sin(th) * np.sin(phi), np.cos(phi)], axis=1)
+    tri = ConvexHull(pts).simplices.astype(np.int64)
+    flip = np.einsum("ij,ij->i", pts[tri[:, 0]], np.cross(pts[tri[:, 1]], pts[tri[:, 2]])) < 0
+    tri[flip] = tri[flip][:, [0, 2, 1]]
+    w = dict(W.cook(1, 1, 1, order=order, nu=0.3))
+    w["coords"] = np.concatenate([np.zeros((1, 3)), pts])
+    w["tets"] = np.concatenate([np.zeros((len(tri), 1), dtype=tri.dtype), tri + 1], axis=1).astype(w["tets"].dtype)
+    w["dir_group"] = np.array([0, 1] + [0] * 32, dtype=w["dir_group"].dtype)
+    w["faces"], w["face_kind"], w["face_data"] = w["faces"][:0], w["face_kind"][:0], w["face_data"][:0]
+    return w
+
+
+# 6 elements (less than a tile of 16 or 64), 96 (six tiles of 16), 144 and 150
+# (a part tile), rows of one chunk of 96 blocks and of two
+TANGENT = {"6": lambda o: W.cook(1, 1, 1, order=o, nu=0.3), "96": lambda o: W.cook(4, 2, 2, order=o, nu=0.3),
+           "144": lambda o: W.cook(4, 3, 2, order=o, nu=0.3), "150": lambda o: W.cook(5, 5, 1, order=o, nu=0.3),
+           "hub": _hub}
+
+
+def _check_tangent(m, om, d, precision, tol):
+    om.tangent(d)
+    m.tangent(torch.from_numpy(d).cuda(), precision)
+    x = np.random.default_rng(6).standard_normal(om.ndof)
+    y = om.spmv(x)
+    for _ in range(2):  # nothing of the first assembly stays in the second
+        yg = m.spmv(torch.from_numpy(x).cuda()).cpu().numpy()
+        assert np.abs(yg - y).max() <= tol * np.abs(y).max()
+        m.tangent(torch.from_numpy(d).cuda(), precision)
+
+
+# bounds of the parity tests: FP64 1e-12, FP32 assembly and sums 2e-5 of the
+# largest entry
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-12), ("mixed_fp32", 2e-5)])
+@pytest.mark.parametrize("order", [1, 2])
+@pytest.mark.parametrize("case", list(TANGENT))
+def test_tangent_tiles_and_rows(fe, case, order, precision, tol):
+    w = TANGENT[case](order)
+    m, om = fe.Mesh(w), O.Mesh(w)
+    d = 0.01 * np.random.default_rng(9).standard_normal(om.ndof)
+    om.apply_dirichlet(d)
+    _check_tangent(m, om, d, precision, tol)
+
+
+def test_tangent_without_workspace(fe):
+    # device memory that holds the matrix but not the element blocks (94 MB
+    # and 128 MB, of 150 MB free): assembled colour by colour, to the same bounds
+    w = W.cook(30, 30, 6, order=2, nu=0.3)
+    m, om = fe.Mesh(w), O.Mesh(w)
+    d = 0.01 * np.random.default_rng(9).standard_normal(om.ndof)
+    om.apply_dirichlet(d)
+    torch.cuda.synchronize()
+    hog = []
+    while True:  # in pieces: the library's pool keeps what it has
+        free = torch.cuda.mem_get_info()[0] - (150 << 20)
+        if free < (2 << 20):
+            break
+        hog.append(torch.empty(min(free, 32 << 30), dtype=torch.uint8, device="cuda"))
+    try:
+        _check_tangent(m, om, d, "fp64", 1e-12)
+    finally:
+        del hog
+        torch.cuda.empty_cache()
