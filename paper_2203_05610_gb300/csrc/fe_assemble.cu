@@ -3,8 +3,8 @@
 // F = I + grad d, P = dPsi/dF; energy of Eq. "minimization"; tangent of
 // Eq. "newton"), materials of Section "Test problems and solvers details".
 //
-// Residual: one thread per (element, quadrature point) writes element-local
-// contributions (QP lanes reduced with warp shuffles), then one thread per
+// Residual: one thread per element (few P2 elements: per quadrature point, the
+// lanes reduced with warp shuffles) writes its contributions, then one thread per
 // node gathers its incident contributions in a fixed order, adds loads and
 // springs, masks prescribed components and reduces ||R||^2 deterministically.
 // Tangent: the element matrices into a workspace, then a warp per block row
@@ -20,9 +20,265 @@ static FollowerFaces follower_faces(fe_mesh m) {
                        m->X};
 }
 
-// MASS adds the inertia of a Newmark step, mass_c M d with mass_c = 4 rho /
-// dt^2 (the step's constant part 4/dt^2 M dhat enters in the gather); the
-// static instantiation carries none of its registers.
+// One thread per element (P1, and P2 meshes of more than RES_ELEMS_PER_SM
+// elements per SM): every quadrature point of the element in turn, FP64.  The FP64
+// pipe bounds it (one warp instruction holds its SM quarter 64 cycles), so the
+// work is counted in FP64 instructions: F comes from differences of the
+// derivatives d u / d lambda_k along the barycentric coordinates and the
+// nodal forces from P G_k, k = 0..3.  P2: with lambda_k(q) = beta + (alpha -
+// beta) delta_kq both split into a part common to the four points and one
+// product per k, about 900 FP64 instructions per element where four lanes
+// that repeat the shape gradients of ten nodes and add 30 forces across
+// lanes take 2,100.  The fibre law works on F in the fibre frame (strains,
+// stress and the active tension are products of its columns): 350
+// instructions per P1 element instead of 650.  Cook P2 64x64x8 (196k elements)
+// 327 us, before 650; 149,760 P1 tets of the fibre law 104 us, before 170.
+//
+// qp_forces: PG[k][i] = w sum_J P_iJ G_kJ, k = 1..3, and J at one point.  At
+// rest (F = I) the terms of the isochoric laws cancel exactly.
+template <int KIND>
+__device__ __forceinline__ void qp_forces(const MatParams& mp, const double* __restrict__ fib, const double (&F)[9],
+                                          double p, const double (&G)[3][3], double w, double (&PG)[3][3], double& J) {
+  double c[9];  // cofactor matrix
+  c[0] = F[4] * F[8] - F[5] * F[7];
+  c[1] = F[5] * F[6] - F[3] * F[8];
+  c[2] = F[3] * F[7] - F[4] * F[6];
+  c[3] = F[2] * F[7] - F[1] * F[8];
+  c[4] = F[0] * F[8] - F[2] * F[6];
+  c[5] = F[1] * F[6] - F[0] * F[7];
+  c[6] = F[1] * F[5] - F[2] * F[4];
+  c[7] = F[2] * F[3] - F[0] * F[5];
+  c[8] = F[0] * F[4] - F[1] * F[3];
+  J = F[0] * c[0] + F[1] * c[1] + F[2] * c[2];
+  if (KIND == FE_MAT_GUCCIONE) {
+    double Fr[3][3], fr[9];  // F f_alpha (columns of F in the fibre frame)
+#pragma unroll
+    for (int q = 0; q < 9; q++) fr[q] = fib[q];
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+      for (int al = 0; al < 3; al++)
+        Fr[i][al] = F[3 * i] * fr[3 * al] + F[3 * i + 1] * fr[3 * al + 1] + F[3 * i + 2] * fr[3 * al + 2];
+    // E_ab = (F f_a . F f_b - f_a . f_b) / 2, S'_ab = C e^Q B_ab E_ab
+    double S[3][3], Q = 0.0;
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+#pragma unroll
+      for (int b = a; b < 3; b++) {
+        const double B = a == 0 ? (b == 0 ? mp.bf : mp.bfs) : mp.bt;
+        const double E = 0.5 * ((Fr[0][a] * Fr[0][b] + Fr[1][a] * Fr[1][b] + Fr[2][a] * Fr[2][b]) -
+                                (fr[3 * a] * fr[3 * b] + fr[3 * a + 1] * fr[3 * b + 1] + fr[3 * a + 2] * fr[3 * b + 2]));
+        const double BE = B * E;
+        Q += (a == b ? 1.0 : 2.0) * BE * E;
+        S[a][b] = S[b][a] = BE;
+      }
+    const double ce = w * mp.C * exp(Q);
+    const double phiJ = w * 0.5 * mp.kappa * (J * log(J) + (J - 1.0)) / J;  // phi / J, phi = kappa/2 (J ln J + J - 1)
+    const double an = sqrt(Fr[0][0] * Fr[0][0] + Fr[1][0] * Fr[1][0] + Fr[2][0] * Fr[2][0]);
+    const double act = w * mp.gamma / an;
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      double gr[3], sg[3];
+#pragma unroll
+      for (int al = 0; al < 3; al++) gr[al] = fr[3 * al] * G[k][0] + fr[3 * al + 1] * G[k][1] + fr[3 * al + 2] * G[k][2];
+#pragma unroll
+      for (int a = 0; a < 3; a++) sg[a] = ce * (S[a][0] * gr[0] + S[a][1] * gr[1] + S[a][2] * gr[2]);
+      sg[0] += act * gr[0];
+#pragma unroll
+      for (int i = 0; i < 3; i++)
+        PG[k][i] = Fr[i][0] * sg[0] + Fr[i][1] * sg[1] + Fr[i][2] * sg[2] +
+                   phiJ * (c[3 * i] * G[k][0] + c[3 * i + 1] * G[k][1] + c[3 * i + 2] * G[k][2]);
+    }
+    return;
+  }
+  const double iJ = 1.0 / J;
+  double P[9];
+  if (KIND == FE_MAT_COOK_NH) {
+    double I1 = 0.0;
+#pragma unroll
+    for (int q = 0; q < 9; q++) I1 += F[q] * F[q];
+    const double r = rcbrt(J);
+    const double c1 = w * mp.mu * (r * r);
+    const double c2 = (w * 2.0 * mp.cvol * (J * J - 1.0) - c1 * (I1 * (1.0 / 3.0))) * iJ;
+#pragma unroll
+    for (int q = 0; q < 9; q++) P[q] = c1 * F[q] + c2 * c[q];
+  } else if (KIND == FE_MAT_TH_NH) {
+    const double c1 = w * mp.mu, c2 = -w * (mp.mu + p * J) * iJ;
+#pragma unroll
+    for (int q = 0; q < 9; q++) P[q] = c1 * F[q] + c2 * c[q];
+  } else {  // P = 2a F + 2b F (tr C I - C) - (c + p J) H
+    double Cm[9];
+    poly_C(F, Cm);
+    const double I1 = Cm[0] + Cm[4] + Cm[8], ch = (mp.clog + p * J) * iJ;
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+      for (int j = 0; j < 3; j++) {
+        const double fc = F[3 * i] * Cm[j] + F[3 * i + 1] * Cm[3 + j] + F[3 * i + 2] * Cm[6 + j];
+        P[3 * i + j] = w * (2.0 * mp.ap * F[3 * i + j] + 2.0 * mp.bp * (I1 * F[3 * i + j] - fc) - ch * c[3 * i + j]);
+      }
+  }
+#pragma unroll
+  for (int k = 0; k < 3; k++)
+#pragma unroll
+    for (int i = 0; i < 3; i++) PG[k][i] = P[3 * i] * G[k][0] + P[3 * i + 1] * G[k][1] + P[3 * i + 2] * G[k][2];
+}
+
+template <int ORDER, bool MASS, int KIND>
+__global__ void __launch_bounds__(128) k_elem_forces(int ne, const int* __restrict__ conn,
+                                                     const double* __restrict__ geo, const double* __restrict__ d,
+                                                     int nn, int pres, MatParams mp, const double* __restrict__ fib,
+                                                     double mass_c, double* __restrict__ rel,
+                                                     double* __restrict__ relp) {
+  constexpr int NEN = ORDER == 1 ? 4 : 10;
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= ne) return;
+  const int* c = conn + (size_t)e * NEN;
+  double u[NEN][3], G[3][3];
+#pragma unroll
+  for (int a = 0; a < NEN; a++) {
+    const double* ua = d + 3 * (size_t)c[a];
+#pragma unroll
+    for (int i = 0; i < 3; i++) u[a][i] = ua[i];
+  }
+  const double* g = geo + (size_t)e * 10;
+#pragma unroll
+  for (int k = 0; k < 3; k++)
+#pragma unroll
+    for (int i = 0; i < 3; i++) G[k][i] = g[3 * k + i];
+  const double vol = g[9];
+  const double* fe = KIND == FE_MAT_GUCCIONE ? fib + (size_t)e * 9 : nullptr;
+  double* out = rel + (size_t)e * NEN * 3;
+  if constexpr (ORDER == 1) {
+    double F[9], PG[3][3], J;
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+      double du[3];
+#pragma unroll
+      for (int k = 0; k < 3; k++) du[k] = u[k + 1][i] - u[0][i];
+#pragma unroll
+      for (int j = 0; j < 3; j++)
+        F[3 * i + j] = (i == j ? 1.0 : 0.0) + du[0] * G[0][j] + du[1] * G[1][j] + du[2] * G[2][j];
+    }
+    qp_forces<KIND>(mp, fe, F, 0.0, G, vol, PG, J);
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+      double r[4] = {-(PG[0][i] + PG[1][i] + PG[2][i]), PG[0][i], PG[1][i], PG[2][i]};
+      if (MASS) {
+        const double mc = mass_c * vol * 0.05, su = (u[0][i] + u[1][i]) + (u[2][i] + u[3][i]);
+#pragma unroll
+        for (int a = 0; a < 4; a++) r[a] += mc * (su + u[a][i]);
+      }
+#pragma unroll
+      for (int a = 0; a < 4; a++) out[3 * a + i] = r[a];
+    }
+    return;
+  } else {
+    constexpr double al = 0.5854101966249685, be = 0.1381966011250105;
+    constexpr double uv = 4.0 * be - 1.0, ue = 4.0 * be, dl = 4.0 * (al - be);
+    // node of the edge between vertices k and l
+    constexpr int ed[4][4] = {{0, 4, 5, 6}, {4, 0, 7, 8}, {5, 7, 0, 9}, {6, 8, 9, 0}};
+    double b[4][3];  // d u / d lambda_k without its delta_kq part
+#pragma unroll
+    for (int k = 0; k < 4; k++)
+#pragma unroll
+      for (int i = 0; i < 3; i++) {
+        double s = 0.0;
+#pragma unroll
+        for (int l = 0; l < 4; l++)
+          if (l != k) s += u[ed[k][l]][i];
+        b[k][i] = uv * u[k][i] + ue * s;
+      }
+    double pv[4] = {0.0, 0.0, 0.0, 0.0}, ps = 0.0;
+    if (pres == 1) {
+#pragma unroll
+      for (int v = 0; v < 4; v++) {
+        pv[v] = d[3 * (size_t)nn + c[v]];
+        ps += pv[v];
+      }
+    } else if (pres == 2) {
+      ps = d[3 * (size_t)nn + e];
+    }
+    const double w = 0.25 * vol;
+    double r[NEN][3], T[4][3], Jm[4];
+#pragma unroll
+    for (int a = 0; a < NEN; a++) r[a][0] = r[a][1] = r[a][2] = 0.0;
+#pragma unroll
+    for (int k = 0; k < 4; k++) T[k][0] = T[k][1] = T[k][2] = 0.0;
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      double F[9], PG[3][3];
+#pragma unroll
+      for (int i = 0; i < 3; i++) {
+        double D[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) D[k] = b[k][i] + dl * u[k == q ? q : ed[k][q]][i];
+#pragma unroll
+        for (int k = 1; k < 4; k++) D[k] -= D[0];
+#pragma unroll
+        for (int j = 0; j < 3; j++)
+          F[3 * i + j] = (i == j ? 1.0 : 0.0) + D[1] * G[0][j] + D[2] * G[1][j] + D[3] * G[2][j];
+      }
+      const double p = pres == 1 ? be * ps + (al - be) * pv[q] : ps;
+      double J;
+      qp_forces<KIND>(mp, fe, F, p, G, w, PG, J);
+      Jm[q] = J - 1.0;
+#pragma unroll
+      for (int i = 0; i < 3; i++) {
+        const double f[4] = {-(PG[0][i] + PG[1][i] + PG[2][i]), PG[0][i], PG[1][i], PG[2][i]};
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+          T[k][i] += f[k];
+          r[k == q ? q : ed[k][q]][i] += dl * f[k];
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        r[k][i] += uv * T[k][i];
+#pragma unroll
+        for (int l = k + 1; l < 4; l++) r[ed[k][l]][i] += ue * (T[k][i] + T[l][i]);
+      }
+      if (MASS) {  // consistent mass through vertex, edge and per-vertex edge sums (mass_hat times 420)
+        const double mc = mass_c * vol * (1.0 / 420.0);
+        const double sv = (u[0][i] + u[1][i]) + (u[2][i] + u[3][i]);
+        double E[4], se = 0.0;
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+          E[k] = 0.0;
+#pragma unroll
+          for (int l = 0; l < 4; l++)
+            if (l != k) E[k] += u[ed[k][l]][i];
+          se += 0.5 * E[k];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+          r[k][i] += mc * (sv + 5.0 * u[k][i] - 6.0 * se + 2.0 * E[k]);
+#pragma unroll
+          for (int l = k + 1; l < 4; l++)
+            r[ed[k][l]][i] += mc * (2.0 * (u[k][i] + u[l][i]) - 6.0 * sv + 8.0 * (se + E[k] + E[l] + u[ed[k][l]][i]));
+        }
+      }
+#pragma unroll
+      for (int a = 0; a < NEN; a++) out[3 * a + i] = r[a][i];
+    }
+    if (pres) {  // R_p = -int (J - 1) q_h: P1 slots per vertex, P0 all in slot 0
+      const double js = (Jm[0] + Jm[1]) + (Jm[2] + Jm[3]);
+#pragma unroll
+      for (int v = 0; v < 4; v++)
+        relp[(size_t)e * 4 + v] = pres == 1 ? -w * (be * js + (al - be) * Jm[v]) : (v == 0 ? -w * js : 0.0);
+    }
+  }
+}
+
+// P2 meshes of fewer elements: a thread per (element, quadrature point).  The
+// element thread's chain of four points is the longer one there (whole residual,
+// Cook and twist P2: 3,072 elements 40 against 51 us, 6,000 to 6,144: 55-56
+// against 51-54, 12,000: 72 against 55, 49,152: 203 against 118; P1 768: 35
+// against 29, 96,000: 62 against 53).
+constexpr int RES_ELEMS_PER_SM = 40;
 template <int ORDER, bool MASS>
 __global__ void __launch_bounds__(128) k_elem_residual(int ne, const int* __restrict__ conn,
                                                        const double* __restrict__ geo,
@@ -52,6 +308,18 @@ __global__ void __launch_bounds__(256) k_gather_residual(
   if (norm2) grid_sum_finish(acc, red, ticket, norm2);
 }
 
+template <int ORDER, bool MASS>
+static int launch_forces(fe_mesh m, const double* d) {
+  auto kern = m->mp.kind == FE_MAT_COOK_NH      ? k_elem_forces<ORDER, MASS, FE_MAT_COOK_NH>
+              : m->mp.kind == FE_MAT_TH_NH      ? k_elem_forces<ORDER, MASS, FE_MAT_TH_NH>
+              : m->mp.kind == FE_MAT_POLYCONVEX ? k_elem_forces<ORDER, MASS, FE_MAT_POLYCONVEX>
+                                                : k_elem_forces<ORDER, MASS, FE_MAT_GUCCIONE>;
+  kern<<<(m->ne + 127) / 128, 128, 0, m->stream>>>(m->ne, m->conn, m->geo, d, m->nn, m->pres, m->mp, m->fib,
+                                                   m->mass_c, m->rel, m->relp);
+  FE_CUDA(cudaGetLastError());
+  return FE_OK;
+}
+
 int fe_residual_dev(fe_mesh m, const double* d, double* r, bool want_norm) {
   int nthr = m->ne * m->nq;
   double eb = (double)m->ne * (4.0 * m->nen + 80.0 + 24.0 * m->nen + (m->fib ? 72.0 : 0.0) + (m->pres ? 32.0 : 0.0)) +
@@ -59,10 +327,15 @@ int fe_residual_dev(fe_mesh m, const double* d, double* r, bool want_norm) {
   {
     FE_SCOPE(m, FE_PROF_RESIDUAL, eb);
     const bool dyn = m->dyn != nullptr;
-    auto kern = m->order == 1 ? (dyn ? k_elem_residual<1, true> : k_elem_residual<1, false>)
-                              : (dyn ? k_elem_residual<2, true> : k_elem_residual<2, false>);
-    kern<<<(nthr + 127) / 128, 128, 0, m->stream>>>(m->ne, m->conn, m->geo, d, m->nn, m->pres, m->mp, m->fib,
-                                                    m->mass_c, m->rel, m->relp);
+    if (m->order == 1) {
+      FE_TRY((dyn ? launch_forces<1, true>(m, d) : launch_forces<1, false>(m, d)));
+    } else if (m->ne >= (int64_t)RES_ELEMS_PER_SM * m->sm_count) {
+      FE_TRY((dyn ? launch_forces<2, true>(m, d) : launch_forces<2, false>(m, d)));
+    } else {
+      auto kern = dyn ? k_elem_residual<2, true> : k_elem_residual<2, false>;
+      kern<<<(nthr + 127) / 128, 128, 0, m->stream>>>(m->ne, m->conn, m->geo, d, m->nn, m->pres, m->mp, m->fib,
+                                                      m->mass_c, m->rel, m->relp);
+    }
   }
   FE_CUDA(cudaGetLastError());
   int rows = m->nn + m->np;

@@ -165,3 +165,36 @@ def test_tangent_without_workspace(fe):
     finally:
         del hog
         torch.cuda.empty_cache()
+
+
+# element kernels of the residual: 6 and more P1 elements, P2 meshes on both sides
+# of 6,080 elements, every law, statically and in a Newmark step
+@pytest.mark.parametrize("case", ["cook1_6", "cook1_390", "cook2_6000", "cook2_6144", "twist_6000", "twist_7986",
+                                  "heart1_12288"])
+def test_residual_element_kernels(fe, case):
+    # FP64 sums of a node's elements in the oracle's terms: a few ulps of the
+    # largest contribution, 1e-12 of the largest entry as in the parity tests
+    w = {"cook1_6": lambda: W.cook(1, 1, 1, order=1, nu=0.3), "cook1_390": lambda: W.cook(13, 5, 1, order=1, nu=0.3),
+         "cook2_6000": lambda: W.cook(20, 10, 5, order=2, nu=0.3),
+         "cook2_6144": lambda: W.cook(16, 16, 4, order=2, nu=0.49),
+         "twist_6000": lambda: W.twist(10), "twist_7986": lambda: W.twist(11),
+         "heart1_12288": lambda: W.heart(nr=2, nc=32, nl=32, order=1)}[case]()
+    m, om = fe.Mesh(w), O.Mesh(w)
+    m.set_load(0.4, 0.1)
+    om.set_load(0.4, 0.1)
+    d = 0.002 * np.random.default_rng(10).standard_normal(om.ndof)
+    om.apply_dirichlet(d)
+    dg = torch.from_numpy(d).cuda()
+    r = om.residual(d)
+    r = r[0] if isinstance(r, tuple) else r
+    rg, norm = m.residual(dg)
+    assert np.abs(rg.cpu().numpy() - r).max() <= 1e-12 * np.abs(r).max()
+    assert abs(norm - np.linalg.norm(r)) <= 1e-12 * np.linalg.norm(r)
+    if case.startswith("twist"):
+        return
+    for mesh in (m, om):
+        mesh.set_dynamics(1e-3, 0.1)
+    r = om.residual(d)
+    r = r[0] if isinstance(r, tuple) else r
+    rg, _ = m.residual(dg)
+    assert np.abs(rg.cpu().numpy() - r).max() <= 1e-12 * np.abs(r).max()
