@@ -198,3 +198,33 @@ def test_residual_element_kernels(fe, case):
     r = r[0] if isinstance(r, tuple) else r
     rg, _ = m.residual(dg)
     assert np.abs(rg.cpu().numpy() - r).max() <= 1e-12 * np.abs(r).max()
+
+
+# unknowns 225 to 1,989: one to eight values per lane of the batch kernel's
+# orthogonalisation; 2,160: beyond it.  Cycles of 20 end in a part block.
+@pytest.mark.parametrize("size", [(4, 4, 2), (5, 5, 2), (7, 7, 2), (8, 8, 3), (9, 9, 3), (10, 9, 3), (13, 12, 2),
+                                  (16, 12, 2), (15, 14, 2)])
+@pytest.mark.parametrize("restart", [20, 100])
+def test_batch_orthogonalisation_sizes(fe, size, restart):
+    # FP64 Newton with tight inner solves ends far below its tolerance, so the
+    # solutions of both paths agree to the residual's 1e-10 times a condition
+    # of 1e2: 1e-8; the CTA shapes agree bit for bit.  Iteration counts are
+    # compared where the cycles hold the whole of the convergence (100 vectors
+    # and up to 1,000 unknowns); short cycles stagnate, and rounding alone
+    # moves their counts by a tenth.
+    w = W.cook(*size, order=1, nu=0.3)
+    opts = dict(ksp_restart=restart, ksp_rtol=1e-6, ksp_atol=0.0, precision="fp64")
+    m = fe.Mesh(w)
+    m.set_load(0.1)
+    out = []
+    for nt in (128, 256):
+        d = m.zeros()
+        st = fe.batch_solve([m], ["NK"], [d], [1e-10], opts=opts, threads=nt)[0]
+        assert st["status"] == 0 and st["rfinal"] <= 1e-10 * st["r0"]
+        out.append((d, st["lit_total"]))
+    assert torch.equal(out[0][0], out[1][0]) and out[0][1] == out[1][1]
+    d, st = m.solve("NK", m.zeros(), tol=1e-10, opts=opts)
+    assert st["status"] == 0
+    assert torch.linalg.norm(out[0][0] - d) <= 1e-8 * torch.linalg.norm(d)
+    if restart == 100 and m.ndof <= 1000:
+        assert st["lit_total"] == out[0][1]
