@@ -295,7 +295,10 @@ typedef struct {
   double dtol;         /* divergence: ||R|| > dtol*||R0||, default 1e4 */
   int32_t apply_dirichlet; /* 1 (default): write prescribed values into d first */
   int32_t orthog;      /* Arnoldi orthogonalisation: 0 (default) the sequential modified
-                          Gram-Schmidt sweep the paper uses (j+2 grid reductions per step);
+                          Gram-Schmidt sweep the paper uses (its coefficients are formed 8
+                          basis vectors at a time as in 2 where the vectors fit one
+                          co-resident grid, and one at a time, j+2 grid reductions per
+                          step, beyond it);
                           1 the same MGS projections in compact-WY form (2 grid
                           reductions per step, ~1.5x the FP64 work, restart <= 128);
                           2 MGS over blocks of 8 basis vectors, the block's

@@ -297,7 +297,6 @@ __device__ __forceinline__ double warp_reduce_scatter(double (&v)[P], int lane) 
 struct ArnShared {
   double wpart[BMGS_P][16];  // block partials by warp (at most 16 warps)
   double wsum[16][BMGS_P];   // gathered partials by warp
-  double part[512];          // one value per thread (sums of one value)
   double h[BMGS_P];          // the last sum's results
   double inv;                // 1 / |w|
   double gj;                 // block 0: g_j
@@ -323,47 +322,28 @@ __device__ __forceinline__ bool xch_reduce(const XchSync& xs, unsigned& seq, dou
   const int G = gridDim.x;
   uint4* set = xs.slots + (size_t)(seq & 1u) * XCH_BLOCKS * BMGS_P;
   double t = 0.0;
-  if (P == 1) {
-    // one value: through shared memory, then one warp (a warp sum in every
-    // warp first would cost five more dependent FP64 steps)
-    sh.part[threadIdx.x] = loc[0];
-    __syncthreads();
-    if (wid == 0) {
-      for (int q = 0; q < nw; q++) t += sh.part[32 * q + lane];
-      t = warp_sum(t);
-      if (G > 1 && lane == 0) xch_post(set + blockIdx.x, t, seq);
-    }
-  } else {
-    const double r = warp_reduce_scatter<P>(loc, lane);
-    if ((lane & (32 / P - 1)) == 0) sh.wpart[lane / (32 / P)][wid] = r;
-    __syncthreads();
-    if (wid == 0) {
-      for (int q = lane / P; q < nw; q += 32 / P) t += sh.wpart[lane % P][q];
+  const double r = warp_reduce_scatter<P>(loc, lane);
+  if ((lane & (32 / P - 1)) == 0) sh.wpart[lane / (32 / P)][wid] = r;
+  __syncthreads();
+  if (wid == 0) {
+    for (int q = lane / P; q < nw; q += 32 / P) t += sh.wpart[lane % P][q];
 #pragma unroll
-      for (int o = P; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      if (G > 1 && lane < P) xch_post(set + blockIdx.x * P + lane, t, seq);
-    }
+    for (int o = P; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (G > 1 && lane < P) xch_post(set + blockIdx.x * P + lane, t, seq);
   }
   if (wid == nw - 1) idle();
   if (G > 1) {
-    if (P == 1) {  // few words: one warp gathers them
-      if (wid == 0) {
-        if (!xch_gather<FL>(xs, set, lane, 32, G, seq, t)) sh.fail = 1;
-        t = warp_sum(t);
-      }
-    } else {
-      double a;
-      if (!xch_gather<FL>(xs, set, threadIdx.x, blockDim.x, G * P, seq, a)) sh.fail = 1;
+    double a;
+    if (!xch_gather<FL>(xs, set, threadIdx.x, blockDim.x, G * P, seq, a)) sh.fail = 1;
 #pragma unroll
-      for (int o = P; o < 32; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-      if (lane < P) sh.wsum[wid][lane] = a;
-      __syncthreads();
-      if (wid == 0) {
-        t = 0.0;
-        for (int q = lane / P; q < nw; q += 32 / P) t += sh.wsum[q][lane % P];
+    for (int o = P; o < 32; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (lane < P) sh.wsum[wid][lane] = a;
+    __syncthreads();
+    if (wid == 0) {
+      t = 0.0;
+      for (int q = lane / P; q < nw; q += 32 / P) t += sh.wsum[q][lane % P];
 #pragma unroll
-        for (int o = P; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      }
+      for (int o = P; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     }
     seq++;
   }
@@ -539,8 +519,10 @@ __device__ __forceinline__ void arnoldi_finish(ArnShared& sh, int j, int ng, dou
 // is loaded once per step and the next block's loads are in flight during
 // the current block's grid sum.
 //
-// Blocked form (SEQ false): modified Gram-Schmidt over the basis in blocks of
-// P vectors.  Inside a block the sequential MGS coefficients follow from the
+// Modified Gram-Schmidt over the basis in blocks of P vectors, for the
+// sequential option (orthog 0) as for the blocked one: the coefficients are
+// the sweep's, in its order.  Inside a block the sequential MGS coefficients
+// follow from the
 // block's inner products with the current w and from its own Gram entries:
 //   <w - sum_{l<m} h_l v_l, v_m> = <w, v_m> - sum_{l<m} h_l <v_l, v_m>,
 // i.e. h_B = (I + L_B)^{-1} V_B^T w with L_B the strictly lower triangle of
@@ -550,9 +532,6 @@ __device__ __forceinline__ void arnoldi_finish(ArnShared& sh, int j, int ng, dou
 // entries <v_{j+1}, v_l>, v_l in the block of v_{j+1}, are summed together
 // with ||w||^2 at the end of step j, and the new row of T_B = (I + L_B)^{-1}
 // is stored, so step j takes ceil((j+1)/P) + 1 grid sums instead of j + 2.
-//
-// Sequential form (SEQ): for i = 0..j: h_ij = <w, V_i>, w -= h_ij V_i, one
-// grid sum each.
 //
 // Then h_{j+1,j} = ||w||, V_{j+1} = w / h_{j+1,j}, z, and block 0 applies the
 // rotations.
@@ -566,10 +545,11 @@ __device__ __forceinline__ void arnoldi_finish(ArnShared& sh, int j, int ng, dou
 // cycles, dependent or not).
 //
 // Measured per launch (before: slices of 6,144 values in shared memory or
-// registers on as few blocks as hold the vector): blocked, 94,800 unknowns,
-// j < 16: 88 -> 28 us; sequential, 178,689 unknowns, j = 24: 173 -> 101 us;
-// sequential, 729 unknowns, j = 95: 402 -> 125 us.
-template <int NPT, bool SEQ, class DT, class ZT>
+// registers on as few blocks as hold the vector): 94,800 unknowns, j < 16: 88
+// -> 28 us; the sequential option with a grid sum per vector: 178,689
+// unknowns, j = 24: 173 -> 101 us spread over every SM and 62 in blocks; 729
+// unknowns, j = 95: 402 -> 125 and 70.
+template <int NPT, class DT, class ZT>
 __global__ void __launch_bounds__(256)
     k_arnoldi_reg(int64_t n, int64_t S, int j, double* __restrict__ V, int64_t ldv, const double* __restrict__ w,
                   double* __restrict__ Hcol, XchSync xs, double* __restrict__ T, double* __restrict__ cs,
@@ -587,7 +567,7 @@ __global__ void __launch_bounds__(256)
   const int64_t len = n - base < S ? n - base : S;
   const int nb = j / P + 1;                     // blocks of the basis v_0..v_j
   const int nlast = j + 1 - (nb - 1) * P;       // vectors in the last block
-  const int ng = SEQ || (j + 1) % P == 0 ? 0 : nlast;  // Gram entries of v_{j+1} (its block is the last one)
+  const int ng = (j + 1) % P == 0 ? 0 : nlast;  // Gram entries of v_{j+1} (its block is the last one)
   if (threadIdx.x == 0) sh.fail = 0;
   if (blockIdx.x == 0) {
     if (threadIdx.x == 0) sh.gj = g[j];
@@ -612,49 +592,30 @@ __global__ void __launch_bounds__(256)
   };
   for (int kb = 0; kb < nb; kb++) {
     const int nc = kb == nb - 1 ? nlast : P;
-    if (SEQ) {
-      if (kb + 1 < nb)
+    double loc[P];
 #pragma unroll
-        for (int m = 0; m < P; m++)
-          load_slice<NPT>(nxt[m], V + (int64_t)((kb + 1) * P + m) * ldv + base, (kb + 1) * P + m <= j ? len : 0);
+    for (int m = 0; m < P; m++) {
+      loc[m] = 0.0;
+#pragma unroll
+      for (int s = 0; s < NPT; s++) loc[m] += wr[s] * cur[m][s];
+    }
+    if (kb + 1 < nb)
 #pragma unroll
       for (int m = 0; m < P; m++)
-        if (m < nc) {
-          double a[1] = {0.0};
+        load_slice<NPT>(nxt[m], V + (int64_t)((kb + 1) * P + m) * ldv + base, (kb + 1) * P + m <= j ? len : 0);
+    if (wid == 0 && lane < nc) {  // T rows of the block (lane m: row kb P + m, entries l < m)
+      const double* tr = T + (int64_t)(kb * P + lane) * P;
 #pragma unroll
-          for (int s = 0; s < NPT; s++) a[0] += wr[s] * cur[m][s];
-          if (!xch_reduce<1, 5>(xs, seq, a, sh, false, 0, false, none)) return;
-          const double h = sh.h[0];
-          if (blockIdx.x == 0 && threadIdx.x == 0) sh.col[kb * P + m] = h;
+      for (int l = 0; l < P - 1; l++)
+        if (l < lane) sh.trow[lane][l] = tr[l];
+    }
+    if (!xch_reduce<P, 5>(xs, seq, loc, sh, true, nc, false, none)) return;
+    if (blockIdx.x == 0 && (int)threadIdx.x < nc) sh.col[kb * P + threadIdx.x] = sh.h[threadIdx.x];
 #pragma unroll
-          for (int s = 0; s < NPT; s++) wr[s] -= h * cur[m][s];
-        }
-    } else {
-      double loc[P];
+    for (int m = 0; m < P; m++) {
+      const double h = m < nc ? sh.h[m] : 0.0;
 #pragma unroll
-      for (int m = 0; m < P; m++) {
-        loc[m] = 0.0;
-#pragma unroll
-        for (int s = 0; s < NPT; s++) loc[m] += wr[s] * cur[m][s];
-      }
-      if (kb + 1 < nb)
-#pragma unroll
-        for (int m = 0; m < P; m++)
-          load_slice<NPT>(nxt[m], V + (int64_t)((kb + 1) * P + m) * ldv + base, (kb + 1) * P + m <= j ? len : 0);
-      if (wid == 0 && lane < nc) {  // T rows of the block (lane m: row kb P + m, entries l < m)
-        const double* tr = T + (int64_t)(kb * P + lane) * P;
-#pragma unroll
-        for (int l = 0; l < P - 1; l++)
-          if (l < lane) sh.trow[lane][l] = tr[l];
-      }
-      if (!xch_reduce<P, 5>(xs, seq, loc, sh, true, nc, false, none)) return;
-      if (blockIdx.x == 0 && (int)threadIdx.x < nc) sh.col[kb * P + threadIdx.x] = sh.h[threadIdx.x];
-#pragma unroll
-      for (int m = 0; m < P; m++) {
-        const double h = m < nc ? sh.h[m] : 0.0;
-#pragma unroll
-        for (int s = 0; s < NPT; s++) wr[s] -= h * cur[m][s];
-      }
+      for (int s = 0; s < NPT; s++) wr[s] -= h * cur[m][s];
     }
     if (kb + 1 < nb)
 #pragma unroll
@@ -662,23 +623,16 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
         for (int s = 0; s < NPT; s++) cur[m][s] = nxt[m][s];
   }
-  // final sum: ||w||^2 and, in the blocked form, the Gram row against the last block
-  if (SEQ) {
-    double a[1] = {0.0};
+  // final sum: ||w||^2 and the Gram row against the last block
+  double loc[P];
 #pragma unroll
-    for (int s = 0; s < NPT; s++) a[0] += wr[s] * wr[s];
-    if (!xch_reduce<1, 5>(xs, seq, a, sh, false, 0, true, rotate)) return;
-  } else {
-    double loc[P];
+  for (int m = 0; m < P; m++) {
+    loc[m] = 0.0;
+    if (m == 0 || m - 1 < ng)
 #pragma unroll
-    for (int m = 0; m < P; m++) {
-      loc[m] = 0.0;
-      if (m == 0 || m - 1 < ng)
-#pragma unroll
-        for (int s = 0; s < NPT; s++) loc[m] += wr[s] * (m == 0 ? wr[s] : cur[m > 0 ? m - 1 : 0][s]);
-    }
-    if (!xch_reduce<P, 5>(xs, seq, loc, sh, false, 0, true, rotate)) return;
+      for (int s = 0; s < NPT; s++) loc[m] += wr[s] * (m == 0 ? wr[s] : cur[m > 0 ? m - 1 : 0][s]);
   }
+  if (!xch_reduce<P, 5>(xs, seq, loc, sh, false, 0, true, rotate)) return;
   const double hn = sh.h[0];
   if (blockIdx.x == 0 && threadIdx.x == 0) *(volatile unsigned*)xs.seq = seq;
   if (hn > 0.0) arnoldi_tail<NPT, DT, ZT>(wr, sh.inv, ws, V + (int64_t)(j + 1) * ldv + base, base, len, Dinv, z);
@@ -691,9 +645,8 @@ __global__ void __launch_bounds__(256)
 // registers; each sweep applies the previous block's update and accumulates
 // the current block's inner products, one vector per pass, with the next
 // pass's vector loaded while the current one is used (a block's second pass
-// over its vectors reads L2).  SEQ: one vector per pass, inner product, grid
-// sum, update.
-template <int NPT, bool SEQ, class DT, class ZT>
+// over its vectors reads L2).
+template <int NPT, class DT, class ZT>
 __global__ void __launch_bounds__(512)
     k_arnoldi_bm(int64_t n, int64_t S, int j, double* __restrict__ V, int64_t ldv, const double* __restrict__ w,
                  double* __restrict__ Hcol, XchSync xs, double* __restrict__ T, double* __restrict__ cs,
@@ -709,7 +662,7 @@ __global__ void __launch_bounds__(512)
   const int64_t len = n - base < S ? n - base : S;
   const int nb = j / P + 1;                // blocks of the basis v_0..v_j
   const int nlast = j + 1 - (nb - 1) * P;  // vectors in the last block
-  const int ng = SEQ || (j + 1) % P == 0 ? 0 : nlast;  // Gram entries of v_{j+1} (its block is the last one)
+  const int ng = (j + 1) % P == 0 ? 0 : nlast;  // Gram entries of v_{j+1} (its block is the last one)
   if (threadIdx.x == 0) sh.fail = 0;
   if (threadIdx.x < P) sh.h[threadIdx.x] = 0.0;
   if (threadIdx.x < P && (int)threadIdx.x <= j) prefetch_l2(V + (int64_t)threadIdx.x * ldv + base, len);
@@ -732,96 +685,69 @@ __global__ void __launch_bounds__(512)
   auto rotate = [&] {
     if (blockIdx.x == 0) arnoldi_rotate(sh, j, Hcol);
   };
-  if (SEQ) {
-    for (int i = 0; i <= j; i++) {
-      double a[1] = {0.0};
-      double b = 0.0;
+  for (int kb = 0; kb <= nb; kb++) {
+    const int np = kb == 0 ? 0 : (kb == nb ? nlast : P);        // previous block: update
+    const int nc = kb == nb ? ng : (kb == nb - 1 ? nlast : P);  // current block (final sweep: Gram row)
+    const double* Vp = V + (int64_t)(kb > 0 ? kb - 1 : 0) * P * ldv + base;
+    const double* Vc = kb < nb ? V + (int64_t)kb * P * ldv + base : Vp;
+    // Passes over one vector each: np update passes (w -= h_m v_m, block B-1),
+    // then nc inner-product passes (block B; final sweep: the Gram row against
+    // block B-1).  The slice of the next pass's vector is loaded into registers
+    // while the current one is used.
+    const int nq = np + nc;
 #pragma unroll
-      for (int s = 0; s < NPT; s += 2) {
-        a[0] += wr[s] * cur[s];
-        b += wr[s + 1] * cur[s + 1];
-      }
-      a[0] += b;
-      if (i < j) load_slice<NPT>(nxt, V + (int64_t)(i + 1) * ldv + base, len);
-      if (i + P <= j && threadIdx.x == 0) prefetch_l2(V + (int64_t)(i + P) * ldv + base, len);
-      if (!xch_reduce<1, 3>(xs, seq, a, sh, false, 0, false, none)) return;
-      const double h = sh.h[0];
-      if (blockIdx.x == 0 && threadIdx.x == 0) sh.col[i] = h;
+    for (int m = 0; m < P; m++) {
+      if (m < np) {
+        if (m + 1 < nq) load_slice<NPT>(nxt, m + 1 < np ? Vp + (int64_t)(m + 1) * ldv : Vc, len);
+        const double h = sh.h[m];
 #pragma unroll
-      for (int s = 0; s < NPT; s++) {
-        wr[s] -= h * cur[s];
-        cur[s] = nxt[s];
+        for (int s = 0; s < NPT; s++) wr[s] -= h * cur[s];
+#pragma unroll
+        for (int s = 0; s < NPT; s++) cur[s] = nxt[s];
       }
     }
-    double a[1] = {0.0};
+    double loc[P];
 #pragma unroll
-    for (int s = 0; s < NPT; s++) a[0] += wr[s] * wr[s];
-    if (!xch_reduce<1, 3>(xs, seq, a, sh, false, 0, true, rotate)) return;
-  } else {
-    for (int kb = 0; kb <= nb; kb++) {
-      const int np = kb == 0 ? 0 : (kb == nb ? nlast : P);        // previous block: update
-      const int nc = kb == nb ? ng : (kb == nb - 1 ? nlast : P);  // current block (final sweep: Gram row)
-      const double* Vp = V + (int64_t)(kb > 0 ? kb - 1 : 0) * P * ldv + base;
-      const double* Vc = kb < nb ? V + (int64_t)kb * P * ldv + base : Vp;
-      // Passes over one vector each: np update passes (w -= h_m v_m, block B-1),
-      // then nc inner-product passes (block B; final sweep: the Gram row against
-      // block B-1).  The slice of the next pass's vector is loaded into registers
-      // while the current one is used.
-      const int nq = np + nc;
+    for (int m = 0; m < P; m++) loc[m] = 0.0;
 #pragma unroll
-      for (int m = 0; m < P; m++) {
-        if (m < np) {
-          if (m + 1 < nq) load_slice<NPT>(nxt, m + 1 < np ? Vp + (int64_t)(m + 1) * ldv : Vc, len);
-          const double h = sh.h[m];
+    for (int m = 0; m < P; m++) {
+      if (m < nc) {
+        if (m + 1 < nc) load_slice<NPT>(nxt, Vc + (int64_t)(m + 1) * ldv, len);
+        double a[2] = {0.0, 0.0};  // two chains: each extra one costs an FP64 add per vector
 #pragma unroll
-          for (int s = 0; s < NPT; s++) wr[s] -= h * cur[s];
+        for (int s = 0; s < NPT; s++) a[s & 1] += wr[s] * cur[s];
+        loc[m] = a[0] + a[1];
 #pragma unroll
-          for (int s = 0; s < NPT; s++) cur[s] = nxt[s];
-        }
+        for (int s = 0; s < NPT; s++) cur[s] = nxt[s];
       }
-      double loc[P];
-#pragma unroll
-      for (int m = 0; m < P; m++) loc[m] = 0.0;
-#pragma unroll
-      for (int m = 0; m < P; m++) {
-        if (m < nc) {
-          if (m + 1 < nc) load_slice<NPT>(nxt, Vc + (int64_t)(m + 1) * ldv, len);
-          double a[2] = {0.0, 0.0};  // two chains: each extra one costs an FP64 add per vector
-#pragma unroll
-          for (int s = 0; s < NPT; s++) a[s & 1] += wr[s] * cur[s];
-          loc[m] = a[0] + a[1];
-#pragma unroll
-          for (int s = 0; s < NPT; s++) cur[s] = nxt[s];
-        }
-      }
-      if (kb == nb) {  // final sweep: [||w||^2, Gram row]
-        double a[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-        for (int s = 0; s < NPT; s++) a[s & 3] += wr[s] * wr[s];
-#pragma unroll
-        for (int m = P - 1; m > 0; m--) loc[m] = loc[m - 1];
-        loc[0] = (a[0] + a[1]) + (a[2] + a[3]);
-      } else {
-        // first pass of the next sweep: the update with this block's v_{kb P}
-        load_slice<NPT>(cur, V + (int64_t)kb * P * ldv + base, len);
-      }
-      // the next block's vectors are read from HBM by the next sweep: start them now
-      if (kb + 1 < nb && threadIdx.x < P && (kb + 1) * P + (int)threadIdx.x <= j)
-        prefetch_l2(V + (int64_t)((kb + 1) * P + threadIdx.x) * ldv + base, len);
-      // T rows of the current block (lane m: row kb P + m, entries l < m)
-      const bool solve = kb < nb;
-      if (wid == 0 && solve && lane < nc) {
-        const double* tr = T + (int64_t)(kb * P + lane) * P;
-#pragma unroll
-        for (int l = 0; l < P - 1; l++)
-          if (l < lane) sh.trow[lane][l] = tr[l];
-      }
-      auto rotate_last = [&] {
-        if (kb == nb) rotate();
-      };
-      if (!xch_reduce<P, 3>(xs, seq, loc, sh, solve, nc, !solve, rotate_last)) return;
-      if (solve && blockIdx.x == 0 && (int)threadIdx.x < nc) sh.col[kb * P + threadIdx.x] = sh.h[threadIdx.x];
     }
+    if (kb == nb) {  // final sweep: [||w||^2, Gram row]
+      double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+      for (int s = 0; s < NPT; s++) a[s & 3] += wr[s] * wr[s];
+#pragma unroll
+      for (int m = P - 1; m > 0; m--) loc[m] = loc[m - 1];
+      loc[0] = (a[0] + a[1]) + (a[2] + a[3]);
+    } else {
+      // first pass of the next sweep: the update with this block's v_{kb P}
+      load_slice<NPT>(cur, V + (int64_t)kb * P * ldv + base, len);
+    }
+    // the next block's vectors are read from HBM by the next sweep: start them now
+    if (kb + 1 < nb && threadIdx.x < P && (kb + 1) * P + (int)threadIdx.x <= j)
+      prefetch_l2(V + (int64_t)((kb + 1) * P + threadIdx.x) * ldv + base, len);
+    // T rows of the current block (lane m: row kb P + m, entries l < m)
+    const bool solve = kb < nb;
+    if (wid == 0 && solve && lane < nc) {
+      const double* tr = T + (int64_t)(kb * P + lane) * P;
+#pragma unroll
+      for (int l = 0; l < P - 1; l++)
+        if (l < lane) sh.trow[lane][l] = tr[l];
+    }
+    auto rotate_last = [&] {
+      if (kb == nb) rotate();
+    };
+    if (!xch_reduce<P, 3>(xs, seq, loc, sh, solve, nc, !solve, rotate_last)) return;
+    if (solve && blockIdx.x == 0 && (int)threadIdx.x < nc) sh.col[kb * P + threadIdx.x] = sh.h[threadIdx.x];
   }
   // sh.h[0] = ||w||, sh.h[1..ng] = <w, v_l> for the last block's vectors
   const double hn = sh.h[0];
@@ -1938,33 +1864,32 @@ static int xch_reserve(fe_mesh m, int sums) {
 // up to 6,144 values per SM; returns 1 without launching for longer ones.
 // fuse_pc: also write z = D^{-1} V_{j+1} into zx.
 //
-// Grid.  A step costs about 16 (blocked: 8 vectors' products and updates) or
-// 2 (sequential) FP64 passes of S / 2 cycles over a block's slice of S values
-// per grid sum, and a grid sum about 3,000 cycles more on several blocks than
-// on one: one block up to 384 (blocked) or 1,536 (sequential) values, above
-// that slices of at least 256 or 512 values on as many SMs as there are.
+// Grid.  A step costs about 16 FP64 passes (8 vectors' products and updates)
+// of S / 2 cycles over a block's slice of S values per grid sum, and a grid sum
+// about 3,000 cycles more on several blocks than on one: one block up to 384
+// values, above that slices of at least 256 values on as many SMs as there are.
 // Threads: of the (threads, values per thread) pairs that hold the slice, the
-// one with the least FP64 issue per SM quarter (the passes, and 9 or 6 steps
-// per warp for the sums).
-template <bool SEQ, class DT, class ZT>
+// one with the least FP64 issue per SM quarter (the passes, and 9 steps per
+// warp for the sums).
+template <class DT, class ZT>
 static int launch_arnoldi_new(fe_mesh m, int j, int kmax, bool fuse_pc, const DT* Dinv, double target, int it0,
                               int max_it) {
   const int64_t n = m->ndof;
   const int sms = std::min(m->sm_count, XCH_BLOCKS);
   int64_t G = 1;
-  if (n > (SEQ ? 1536 : 384)) G = std::min<int64_t>(sms, (n + (SEQ ? 511 : 255)) / (SEQ ? 512 : 256));
+  if (n > 384) G = std::min<int64_t>(sms, (n + 255) / 256);
   const int64_t S = ((n + G - 1) / G + 5) / 6 * 6;
   if (S > 6144) return 1;
   const int grid = (int)((n + S - 1) / S);
   const void* fn = nullptr;
   int nt = 0, npt = 0;
   if (S <= 1536) {
-    const void* fns[3] = {(const void*)k_arnoldi_reg<2, SEQ, DT, ZT>, (const void*)k_arnoldi_reg<4, SEQ, DT, ZT>,
-                          (const void*)k_arnoldi_reg<6, SEQ, DT, ZT>};
+    const void* fns[3] = {(const void*)k_arnoldi_reg<2, DT, ZT>, (const void*)k_arnoldi_reg<4, DT, ZT>,
+                          (const void*)k_arnoldi_reg<6, DT, ZT>};
     int best = INT_MAX;
     for (int t = 128; t <= 256; t += 128)
       for (int q = 0; q < 3; q++) {
-        const int v = 2 * (q + 1), cost = t / 128 * (16 * v + (SEQ ? 48 : 9));
+        const int v = 2 * (q + 1), cost = t / 128 * (16 * v + 9);
         if ((int64_t)t * v >= S && cost < best) {
           best = cost;
           fn = fns[q];
@@ -1973,7 +1898,7 @@ static int launch_arnoldi_new(fe_mesh m, int j, int kmax, bool fuse_pc, const DT
         }
       }
   } else {
-    fn = (const void*)k_arnoldi_bm<12, SEQ, DT, ZT>;
+    fn = (const void*)k_arnoldi_bm<12, DT, ZT>;
     npt = 12;
     nt = (int)((S + 12 * 128 - 1) / (12 * 128) * 128);
   }
@@ -1999,7 +1924,7 @@ static int launch_arnoldi_new(fe_mesh m, int j, int kmax, bool fuse_pc, const DT
                   (void*)&D, (void*)&z, (void*)&target, (void*)&kmax, (void*)&it0, (void*)&max_it};
   // flops: (j+1) inner products and axpys (4 per entry), the norm (2) and the scaling (1) per
   // entry, the blocked form's Gram row, plus 18 per node for the fused block-Jacobi product
-  const int ng = SEQ ? 0 : (j + 1) % BMGS_P;
+  const int ng = (j + 1) % BMGS_P;
   FE_SCOPE_F(m, FE_PROF_ARNOLDI, 8.0 * (double)n * (j + 3) + (fuse_pc ? (double)n * (3.0 * sizeof(DT) + sizeof(ZT)) : 0.0),
              (double)n * (4.0 * (j + 1) + 3.0 + 2.0 * ng) + (fuse_pc ? 6.0 * n : 0.0));
   FE_CUDA(cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(nt), args, smem, m->stream));
@@ -2169,15 +2094,9 @@ static int launch_arnoldi_bm_t(fe_mesh m, int j, int kmax, bool fuse_pc, const D
 
 static int launch_arnoldi(fe_mesh m, int j, int kmax, bool fuse_pc, double target, int it0, int max_it) {
   if (m->orthog != 1) {
-    int r;
-    if (m->orthog == 2)
-      r = m->prec == FE_PREC_FP64
-              ? launch_arnoldi_new<false, double, double>(m, j, kmax, fuse_pc, m->Dinv64, target, it0, max_it)
-              : launch_arnoldi_new<false, float, float>(m, j, kmax, fuse_pc, m->Dinv32, target, it0, max_it);
-    else
-      r = m->prec == FE_PREC_FP64
-              ? launch_arnoldi_new<true, double, double>(m, j, kmax, fuse_pc, m->Dinv64, target, it0, max_it)
-              : launch_arnoldi_new<true, float, float>(m, j, kmax, fuse_pc, m->Dinv32, target, it0, max_it);
+    const int r = m->prec == FE_PREC_FP64
+                      ? launch_arnoldi_new<double, double>(m, j, kmax, fuse_pc, m->Dinv64, target, it0, max_it)
+                      : launch_arnoldi_new<float, float>(m, j, kmax, fuse_pc, m->Dinv32, target, it0, max_it);
     if (r <= 0) return r;
   }
   if (m->orthog == 2) {
