@@ -698,7 +698,7 @@ __device__ __forceinline__ void power_row(int row, int lane, const int* ptr, con
 
 // coarse levels, and level 0 in FP32: a warp per row, rows strided over at
 // most POWER_BLOCKS_PER_SM blocks per SM (a partial sum and a ticket each).
-// Level 0 of Cook P2 64x64x8: 45 us, of which the values are 23 us at the copy
+// Level 0 of Cook P2 45x41x7: 45 us, of which the blocks are 18 us at the copy
 // rate (before 100 us in three kernels); a coarse level's 14 us are latency.
 constexpr int POWER_BLOCKS_PER_SM = 8;
 template <class C, class V, int B>
@@ -777,7 +777,7 @@ __global__ void k_amg_rpos(int64_t nnzr, const int* __restrict__ rsrc, int* __re
 // thread per entry that scanned its whole row took 632 us for 629k entries),
 // the block and T's rows are shared by neighbouring threads.  Also writes the
 // V-cycle's tiled copy pt and the transpose R (their own kernels took 30 and
-// 58 us).  Cook P2 64x64x8: level 0 176 us (before 447), level 1 119.
+// 58 us).  Cook P2 45x41x7: level 0 176 us (before 447), level 1 119.
 template <class C, class V, int B>
 __global__ void __launch_bounds__(B == 3 ? 192 : 64) k_amg_pvals(int64_t nnzp, const int* __restrict__ prow,
                                                    const int* __restrict__ pcol, const int2* __restrict__ pk_ptr,
@@ -912,7 +912,7 @@ __global__ void k_amg_raplists(int nc, const int* __restrict__ cptr, const int* 
 // distinct places and block k + 1 follows block k after a warp barrier: no
 // atomics, a fixed order.  Bound by the
 // FP32 and shared-memory instructions of the products: about 500 us on level 0
-// of Cook P2 64x64x8 (113k rows, 1.9 M entries).  Before, a thread per output
+// of Cook P2 45x41x7 (113k rows, 1.9 M entries).  Before, a thread per output
 // entry that searched the P rows of all the row's columns: 638 us there, and
 // 204 us on the next level, now 51.
 constexpr int AMG_CHUNK = 64;
@@ -988,7 +988,7 @@ __global__ void __launch_bounds__(32 * ap_warps<C, B>())
 // (level 0, many entries with some hundred products each): six threads per
 // entry, one row each, the A P values shared by neighbouring threads.  B = 6
 // (few entries, long lists, bound by the latency of the loads): 36 threads, one
-// value each, eight products in flight.  404 us on level 0 of Cook P2 64x64x8
+// value each, eight products in flight.  404 us on level 0 of Cook P2 45x41x7
 // and 167 us on level 1 (a thread per entry that searched the
 // A P rows of all the row's nodes: 979 and 849 us).
 template <class C, int B>

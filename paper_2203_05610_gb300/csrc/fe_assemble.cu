@@ -457,10 +457,10 @@ int fe_energy_dev(fe_mesh m, const double* d, double* out) {
 // row in the tiled layout.  Each block is written once, in 128-byte runs.
 // (Before: one launch per colour, elements spread over a block's threads,
 // scattered 4-byte read-modify-writes, each its own 32-byte sector of eight.
-// Cook P2 64x64x8 in FP32: 38 launches, 1,580 us; now 171 + 183 us, the blocks
-// 64 us of traffic at the copy rate each way.  Cardiac shell of 149,760 P1 tets
-// in FP64: 3.1 ms; now 486 us, bound by the FP64 pipe, + 148 us.)  A mesh whose workspace does not fit is assembled colour by colour
-// (k_elem_tangent).
+// Cook P2 45x41x7 in FP32: 38 launches, 1,580 us; now 171 + 183 us, the blocks
+// 23 us of traffic at the copy rate each way.  Cardiac shell of 149,760 P1 tets
+// in FP64: 3.1 ms; now 486 us, bound by the FP64 pipe, + 148 us.)  A mesh whose
+// workspace does not fit is assembled colour by colour (k_elem_tangent).
 //
 // FP64: at a quadrature point the material tangent A enters the element matrix
 // only through the four barycentric gradients G_k: M_kl[i][j] = sum_JL G_kJ
