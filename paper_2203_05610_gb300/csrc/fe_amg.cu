@@ -2106,7 +2106,7 @@ int vcycle_launches(fe_mesh m, cudaStream_t st, const V* K0, const double* b, do
     *flops += 2.0 * N * N;
     return FE_OK;
   }
-  // the bottom levels q0..L-1 (at most VC_BOTTOM_MAXN nodes each, q0 >= 1)
+  // the bottom levels q0..L-1 (at most VC_BOTTOM_MAXNNZ blocks each, q0 >= 1)
   // run in one block when at least one of them is smoothed
   int q0 = L - 1;
   while (!D && q0 > 1 && h->lev[q0 - 1].nnz <= VC_BOTTOM_MAXNNZ) q0--;
