@@ -1139,10 +1139,9 @@ enum { VC_SETX = 1, VC_FINAL = 2, VC_KEEPX = 4, VC_START = 8 };
 
 // Level-0 Chebyshev step: the streamed product of fe_stream.cuh with the row
 // updates as its epilogue; a window's g, r, x and block-Jacobi inverses are
-// copied to shared memory while its tiles are multiplied.  Every row of A
-// holds its diagonal block, so no row is empty.  Five blocks per SM (96
-// registers) in FP32: with six the operands spill (48x48x8: 312 against 278 us
-// per V-cycle).
+// copied to shared memory while its tiles are multiplied.  Five blocks per SM
+// (96 registers) in FP32: with six the operands spill (48x48x8: 312 against
+// 278 us per V-cycle).
 template <class T>
 __host__ __device__ constexpr int cheb0_blocks_per_sm() { return sizeof(T) == 8 ? 3 : 5; }
 

@@ -324,12 +324,13 @@ __global__ void k_emap(int ne, int nen, int ncolk, const int* __restrict__ conn,
 }
 
 // row ranges of equal block counts: part[w] = the first row that starts at or
-// after block w nnzb / ranges
+// after block w nnzb / ranges; the last range ends with the last row, also
+// where that one has no blocks (a vertex that no element uses)
 __global__ void k_partition(int nn, int64_t nnzb, int ranges, const int* __restrict__ row_ptr, int* __restrict__ part) {
   const int w = blockIdx.x * blockDim.x + threadIdx.x;
   if (w > ranges) return;
   const int64_t k = nnzb * w / ranges;
-  int lo = 0, hi = nn;
+  int lo = w < ranges ? 0 : nn, hi = nn;
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
     if ((int64_t)row_ptr[mid] >= k) hi = mid;

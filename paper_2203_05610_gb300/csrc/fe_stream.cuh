@@ -15,7 +15,9 @@
 // window carrying its sum; the rows that end there go through the epilogue
 // Epi, lane i on the i-th of them, with operands whose loads are in flight
 // during the sums.  Summation order is fixed by the row pointers and the
-// partition, so results are deterministic.
+// partition, so results are deterministic.  A range may hold no rows (a row
+// longer than a range) or rows without blocks (vertices that no element uses:
+// their sums are zero); the walk goes through it like through any other.
 //
 // What bounds it, and why this form.  HBM, with the latency of the chain
 // column index -> x behind it.  Walking the value tiles where they are aligned
@@ -133,7 +135,7 @@ __device__ __forceinline__ void stream_rows(int n, int range, int step, int rang
       c[t] = stream_load_col(col, kc + 32 * (t + 3) + lane, kstart, kend);
     }
     AT carry[3] = {AT(0), AT(0), AT(0)};  // row r's sum over the earlier windows
-    while (kc < kend) {
+    do {  // (once for a range without blocks: its empty rows' sums, and the next range's loads)
       const int kw = kc;  // the window's first block
       const int kwe = min(kw + STREAM_WIN, kend);
       const int rw = r;
@@ -191,7 +193,7 @@ __device__ __forceinline__ void stream_rows(int n, int range, int step, int rang
         off = (off + RP) & 31;
       }
       __syncwarp();
-    }
+    } while (kc < kend);
     if (range >= ranges) return;
     r = nr;
     rb = nrb;

@@ -228,3 +228,78 @@ def test_batch_orthogonalisation_sizes(fe, size, restart):
     assert torch.linalg.norm(out[0][0] - d) <= 1e-8 * torch.linalg.norm(d)
     if restart == 100 and m.ndof <= 1000:
         assert st["lit_total"] == out[0][1]
+
+
+def _with_unused(w, n):
+    """The mesh with n vertices that no element uses behind its own."""
+    w = dict(w)
+    w["coords"] = np.concatenate([w["coords"], 100.0 + np.arange(3.0 * n).reshape(n, 3)])
+    w["dir_group"] = np.concatenate([w["dir_group"], np.zeros(n, dtype=w["dir_group"].dtype)])
+    return w
+
+
+# rows without blocks behind the last row that has some: one, and more than the
+# warps' share of one row each
+@pytest.mark.parametrize("precision", ["fp64", "mixed_fp32"])
+@pytest.mark.parametrize("unused", [1, 40])
+def test_streamed_spmv_rows_without_blocks(fe, unused, precision):
+    # the mesh without the unused vertices has the same blocks: same sums, bit for bit, and zeros
+    w = W.cook(7, 5, 2, order=1, nu=0.3)
+    m, mu = fe.Mesh(w), fe.Mesh(_with_unused(w, unused))
+    assert mu.nnzb == m.nnzb and mu.ndof == m.ndof + 3 * unused
+    rng = np.random.default_rng(11)
+    d, x = (torch.from_numpy(rng.standard_normal(mu.ndof)).cuda() for _ in range(2))
+    d *= 0.01
+    m.tangent(d[: m.ndof].clone(), precision)
+    mu.tangent(d, precision)
+    y, yu = m.spmv(x[: m.ndof].clone()), mu.spmv(x, torch.full_like(x, float("nan")))
+    assert torch.equal(yu[: m.ndof], y)
+    assert torch.equal(yu[m.ndof:], torch.zeros_like(yu[m.ndof:]))
+
+
+def _stars(n, cook):
+    """n x 100 to 128 tets that share one vertex each (rows of 900 to 1,153 blocks), then Cook's membrane."""
+    rng, X, T, o = np.random.default_rng(0), [], [], 0
+    for i in range(n):
+        k = 100 + i % 29
+        x = rng.standard_normal((k, 3, 3))
+        x /= np.linalg.norm(x, axis=2, keepdims=True)
+        flip = np.linalg.det(x) < 0
+        x[flip] = x[flip][:, [0, 2, 1]]
+        X.append(np.concatenate([np.zeros((1, 3)), x.reshape(-1, 3)]))
+        T.append(o + np.concatenate([np.zeros((k, 1), dtype=int), 1 + np.arange(3 * k).reshape(k, 3)], axis=1))
+        o += len(X[-1])
+    w = dict(W.cook(*cook, order=2, nu=0.3))
+    w["tets"] = np.concatenate(T + [w["tets"] + o]).astype(w["tets"].dtype)
+    w["faces"] = w["faces"] + o
+    w["coords"] = np.concatenate(X + [w["coords"]])
+    w["dir_group"] = np.concatenate([np.zeros(o, dtype=w["dir_group"].dtype), w["dir_group"]])
+    return w
+
+
+def test_streamed_spmv_empty_range(fe):
+    # a row longer than a range leaves a range without rows.  Where that one
+    # starts at a tile's edge and the warp has another range, the warp must
+    # not walk the blocks between the two (about half of all, alone: tens of
+    # milliseconds): the product takes the time of one without such rows, to
+    # a factor that leaves room for anything else.
+    import time
+    m, p = fe.Mesh(_stars(64, (34, 34, 8))), fe.Mesh(W.cook(42, 42, 9, order=2, nu=0.3))
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rp, wave = m.topology()["row_ptr"].astype(np.int64), 3 * sms * 4
+    ranges = 2 * wave
+    part = np.searchsorted(rp[:-1], m.nnzb * np.arange(ranges + 1) // ranges)
+    empty = np.nonzero(part[:-1] == part[1:])[0]
+    if not any(rp[part[e]] % 32 == 0 and e + wave < ranges for e in empty):
+        pytest.skip("no such range on this device")  # (152 SMs have one)
+    t = []
+    for mesh in (m, p):
+        x = torch.from_numpy(np.random.default_rng(12).standard_normal(mesh.ndof)).cuda()
+        mesh.tangent(torch.zeros_like(x))
+        y, best = mesh.spmv(x), 1e9
+        for _ in range(5):
+            t0 = time.perf_counter()
+            mesh.spmv(x, y)
+            best = min(best, time.perf_counter() - t0)
+        t.append(best)
+    assert t[0] < 10 * t[1], t
