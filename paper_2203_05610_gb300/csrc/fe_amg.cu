@@ -410,12 +410,12 @@ __global__ void k_amg_dinv3(int n, const int* __restrict__ diag, Vals<C, V, 3> A
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   double a[3][3], v[3][3];
-  const int64_t k = diag[i];
+  const int64_t k = diag[i];  // (-1: a row without blocks, identity)
 #pragma unroll
   for (int r = 0; r < 3; r++)
 #pragma unroll
     for (int c = 0; c < 3; c++) {
-      a[r][c] = (double)A(k, 3 * r + c);
+      a[r][c] = k >= 0 ? (double)A(k, 3 * r + c) : (r == c ? 1.0 : 0.0);
       v[r][c] = r == c ? 1.0 : 0.0;
     }
 #pragma unroll

@@ -855,6 +855,11 @@ __device__ __forceinline__ void diag_inverse_row(int a, int nn, const int* __res
                                T* K, DT* Dinv) {
   if (a >= nn) return;
   const int p = diag_pos[a];
+  DT* o = Dinv + (size_t)a * 9;
+  if (p < 0) {  // no element uses the node: no blocks, identity
+    for (int k = 0; k < 9; k++) o[k] = DT(k % 4 == 0 ? 1 : 0);
+    return;
+  }
   uint8_t fm = fixmask[a];
   for (int i = 0; i < 3; i++)
     if ((fm >> i) & 1) K[kv_index(p, 4 * i)] = T(1);
@@ -865,7 +870,6 @@ __device__ __forceinline__ void diag_inverse_row(int a, int nn, const int* __res
   T c2 = M[3] * M[7] - M[4] * M[6];
   T det = M[0] * c0 + M[1] * c1 + M[2] * c2;
   T id = T(1) / det;
-  DT* o = Dinv + (size_t)a * 9;
   o[0] = (DT)(c0 * id);
   o[1] = (DT)((M[2] * M[7] - M[1] * M[8]) * id);
   o[2] = (DT)((M[1] * M[5] - M[2] * M[4]) * id);

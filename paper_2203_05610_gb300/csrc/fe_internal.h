@@ -102,7 +102,7 @@ struct fe_mesh_s {
   int64_t nnzb = 0;
   int* row_ptr = nullptr;  // [nn+1]
   int* col = nullptr;      // [nnzb]
-  int* diag_pos = nullptr; // [nn]
+  int* diag_pos = nullptr; // [nn] (-1: a row without blocks)
   int* emap = nullptr;     // [ne][nen*nen]
   int* part32 = nullptr;   // [ranges+1] row ranges of the streamed products (fe_stream.cuh) by accumulation type
   int* part64 = nullptr;

@@ -560,9 +560,10 @@ static int create_impl(const fe_mesh_desc* desc, fe_mesh m) {
   std::vector<int> row_ptr, col;
   build_rows(nn, nptr, nlist, conn, m->nen, m->nen, m->nen, row_ptr, col);
   m->nnzb = (int64_t)col.size();
-  std::vector<int> diag(nn);
+  std::vector<int> diag(nn, -1);  // (-1: a vertex that no element uses has no blocks)
   for (int a = 0; a < nn; a++)
-    diag[a] = (int)(std::lower_bound(col.begin() + row_ptr[a], col.begin() + row_ptr[a + 1], a) - col.begin());
+    if (row_ptr[a] < row_ptr[a + 1])
+      diag[a] = (int)(std::lower_bound(col.begin() + row_ptr[a], col.begin() + row_ptr[a + 1], a) - col.begin());
   std::vector<int> up_ptr, up_col, pu_ptr, pu_col, pu_src;
   if (m->pres) {
     if (m->pres == 1) {

@@ -303,3 +303,24 @@ def test_streamed_spmv_empty_range(fe):
             best = min(best, time.perf_counter() - t0)
         t.append(best)
     assert t[0] < 10 * t[1], t
+
+
+# an unused vertex before, between and behind the others, clamped or not
+@pytest.mark.parametrize("precision", ["fp64", "mixed_fp32"])
+@pytest.mark.parametrize("group", [0, 1])
+def test_tangent_with_unused_vertices(fe, group, precision):
+    # the others' blocks and inverses are those of the mesh without them, bit for bit; theirs the identity
+    w = W.cook(5, 4, 1, order=1, nu=0.3)
+    n = len(w["coords"])
+    ids = np.delete(np.arange(n + 3), [0, 17, n + 2])  # new numbers of the mesh's own vertices
+    u = dict(w, tets=ids[w["tets"]].astype(w["tets"].dtype), faces=ids[w["faces"]].astype(w["faces"].dtype),
+             coords=100.0 + np.arange(3.0 * (n + 3)).reshape(n + 3, 3),
+             dir_group=np.full(n + 3, group, dtype=w["dir_group"].dtype))
+    u["coords"][ids], u["dir_group"][ids] = w["coords"], w["dir_group"]
+    m, mu = fe.Mesh(w), fe.Mesh(u)
+    d = 0.01 * np.random.default_rng(13).standard_normal((n + 3, 3))
+    mu.tangent(torch.from_numpy(d.reshape(-1).copy()).cuda(), precision)
+    m.tangent(torch.from_numpy(d[ids].reshape(-1).copy()).cuda(), precision)
+    (val, _, dinv), (valu, _, dinvu) = m.tangent_copy(), mu.tangent_copy()
+    assert np.array_equal(valu, val) and np.array_equal(dinvu[ids], dinv)
+    assert np.array_equal(dinvu[[0, 17, n + 2]], np.tile(np.eye(3), (3, 1, 1)))
