@@ -1009,18 +1009,28 @@ __global__ void k_to_bf16(int64_t n, const float* __restrict__ src, __nv_bfloat1
 }
 
 // the element blocks' workspace, kept in the mesh (the larger of the two
-// precisions it was asked for); FE_ERR_OOM where it does not fit
+// precisions it was asked for) until another allocation of the mesh needs the
+// memory (fe_alloc); FE_ERR_OOM where it does not fit.  Above
+// TAN_WORK_SMALL it takes at most a quarter of the free memory, so that what
+// the caller and other meshes allocate next finds the rest (P2 in FP64: 4 kB an
+// element, more than the matrix).
+constexpr size_t TAN_WORK_SMALL = (size_t)64 << 20;
 static int tangent_workspace(fe_mesh m, size_t elem) {
   const size_t npair = (size_t)m->nen * (m->nen + 1) / 2, npl = m->pres == 0 ? 0 : (m->pres == 2 ? 1 : 4);
   const size_t bytes = (size_t)m->ne * (9 * npair + 3 * npl * m->nen) * elem;
   if (m->tan_work_bytes >= bytes) return FE_OK;
+  if (bytes > TAN_WORK_SMALL) {
+    size_t free_b = 0, total_b = 0;
+    FE_CUDA(cudaMemGetInfo(&free_b, &total_b));
+    if (bytes > (free_b + m->tan_work_bytes) / 4) return FE_ERR_OOM;
+  }
   if (m->tan_work) {
     FE_CUDA(cudaFreeAsync(m->tan_work, m->stream));
     m->device_bytes -= (int64_t)m->tan_work_bytes;
     m->tan_work = nullptr;
     m->tan_work_bytes = 0;
   }
-  FE_TRY(fe_alloc(m, &m->tan_work, bytes));
+  FE_TRY(fe_alloc_once(m, &m->tan_work, bytes));
   m->tan_work_bytes = bytes;
   return FE_OK;
 }
@@ -1061,7 +1071,9 @@ static int launch_tangent(fe_mesh m, const double* d, T* K, T* B) {
   using C = TanCfg<ORDER, T>;
   size_t smem = sizeof(T) * C::EPB * C::PER_E;
   const size_t nval = kv_count(m->nnzb);
-  if (tangent_workspace(m, sizeof(T)) == FE_OK) return launch_tangent_blocks<ORDER, T>(m, d, K, B);
+  const int rc = tangent_workspace(m, sizeof(T));
+  if (rc == FE_OK) return launch_tangent_blocks<ORDER, T>(m, d, K, B);
+  if (rc != FE_ERR_OOM) return rc;
   FE_CUDA(cudaMemsetAsync(K, 0, nval * sizeof(T), m->stream));
   if (m->pres) FE_CUDA(cudaMemsetAsync(B, 0, (size_t)std::max<int64_t>(m->nnz_up, 1) * 3 * sizeof(T), m->stream));
   FE_TRY(fe_kernel_smem((const void*)k_elem_tangent<ORDER, T>, (int)smem));
@@ -1204,7 +1216,8 @@ static int copy_out(fe_mesh m, double* host, const double* d64, const float* d32
     return FE_OK;
   }
   double* tmp = nullptr;
-  FE_CUDA(cudaMallocAsync((void**)&tmp, n * sizeof(double), m->stream));
+  FE_TRY(fe_alloc_t(m, &tmp, (size_t)n));
+  m->device_bytes -= n * (int64_t)sizeof(double);  // (freed below)
   if (d16) k_widen_bf<<<(unsigned)((n + 255) / 256), 256, 0, m->stream>>>(n, d16, tmp);
   else k_widen<<<(unsigned)((n + 255) / 256), 256, 0, m->stream>>>(n, d32, tmp);
   cudaError_t e = cudaStreamSynchronize(m->stream);

@@ -288,7 +288,9 @@ struct LaunchScope {
 #define FE_SCOPE_F(m, cls, bytes, flops) \
   LaunchScope FE_CAT(fe_scope_, __LINE__)(m, cls, (double)(bytes), (double)(flops))
 
-// allocation helper that tracks the mesh's device footprint
+// Stream-ordered allocation, counted in the mesh's device bytes; out of
+// memory, fe_alloc gives the mesh's optional scratch back and tries once more
+int fe_alloc_once(fe_mesh m, void** p, size_t bytes);
 int fe_alloc(fe_mesh m, void** p, size_t bytes);
 template <class T>
 int fe_alloc_t(fe_mesh m, T** p, size_t count) {

@@ -33,17 +33,38 @@ extern "C" const char* fe_last_error(void) { return g_err; }
 // Stream-ordered allocations on the mesh's stream: freeing them does not
 // synchronise the device, so meshes created and destroyed by the serving
 // loop's workers do not stall the kernels of other requests.
-int fe_alloc(fe_mesh m, void** p, size_t bytes) {
+int fe_alloc_once(fe_mesh m, void** p, size_t bytes) {
   *p = nullptr;
   if (bytes == 0) bytes = 16;
   cudaError_t e = cudaMallocAsync(p, bytes, m->stream);
   if (e != cudaSuccess) {
     fe_set_error("cudaMallocAsync(%zu bytes) failed: %s", bytes, cudaGetErrorString(e));
     cudaGetLastError();
-    return FE_ERR_OOM;
+    return e == cudaErrorMemoryAllocation ? FE_ERR_OOM : FE_ERR_CUDA;
   }
   m->device_bytes += (int64_t)bytes;
   return FE_OK;
+}
+
+// Gives the mesh's optional scratch back to the device (nothing in it outlives
+// the call that filled it, and its users have a form without it); false:
+// there was none.
+static bool release_scratch(fe_mesh m) {
+  if (!m->tan_work) return false;
+  cudaFreeAsync(m->tan_work, m->stream);
+  m->device_bytes -= (int64_t)m->tan_work_bytes;
+  m->tan_work = nullptr;
+  m->tan_work_bytes = 0;
+  cudaStreamSynchronize(m->stream);
+  cudaMemPool_t pool;  // (memory the pool still holds may be in pieces too small for the caller)
+  if (cudaDeviceGetDefaultMemPool(&pool, m->device) == cudaSuccess) cudaMemPoolTrimTo(pool, 0);
+  return true;
+}
+
+int fe_alloc(fe_mesh m, void** p, size_t bytes) {
+  int rc = fe_alloc_once(m, p, bytes);
+  if (rc == FE_ERR_OOM && release_scratch(m)) rc = fe_alloc_once(m, p, bytes);
+  return rc;
 }
 
 // grid-reduction state of the persistent kernels: arrival counter, step
