@@ -84,7 +84,7 @@ __device__ __forceinline__ uint64_t mix64_d(uint64_t z) {
 
 struct AmgLevel {
   int n = 0, b = 3, nc = 0;
-  int64_t nnz = 0, nnzp = 0, nnzap = 0, nnzr = 0;
+  int64_t nnz = 0, nnzp = 0, nnzap = 0, nnzr = 0, napidx = 0, nralist = 0;
   // structure (device)
   const int* ptr = nullptr;  // A_l pattern (level 0: the mesh's)
   const int* col = nullptr;
@@ -95,8 +95,11 @@ struct AmgLevel {
   int2* pk_ptr = nullptr;    // the blocks of each P entry (k_amg_plists), its place in R
   int *pk = nullptr, *rpos = nullptr;
   int64_t *apoff = nullptr, *raoff = nullptr;  // starts of each fine row's places, each coarse row's products below
-  int* apidx = nullptr;                   // places of the products in their A P row (k_amg_ap)
-  int2* ralist = nullptr;                 // (P entry, A P entry) of the products of each entry of A_{l+1} (k_amg_rap)
+  // places of the products in their A P row (k_amg_ap), and (P entry, A P
+  // entry) of the products of each entry of A_{l+1} (k_amg_rap); optional, null
+  // where they do not fit (fe_amg_release_lists)
+  int* apidx = nullptr;
+  int2* ralist = nullptr;
   int64_t* lend = nullptr;                // their ends
   int* crow = nullptr;                    // row of each entry of A_{l+1}
   float* tnode32 = nullptr;               // tnode in FP32
@@ -867,7 +870,7 @@ __global__ void k_amg_raplists(int nc, const int* __restrict__ cptr, const int* 
                                const int* __restrict__ rptr, const int* __restrict__ rcol,
                                const int* __restrict__ rsrc, const int* __restrict__ apptr,
                                const int* __restrict__ apcol, const int64_t* __restrict__ raoff,
-                               int64_t* lend, int* crow, int2* __restrict__ list) {
+                               int64_t* lend, int* crow, int2* __restrict__ list) {  // (no list: the rows alone)
   const int a = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (a >= nc) return;
   const int c0 = cptr[a], m = cptr[a + 1] - c0;
@@ -875,6 +878,7 @@ __global__ void k_amg_raplists(int nc, const int* __restrict__ cptr, const int* 
     lend[c0 + t] = 0;
     crow[c0 + t] = a;
   }
+  if (!list) return;
   __syncwarp();
   for (int pass = 0; pass < 2; pass++) {
     for (int s = rptr[a]; s < rptr[a + 1]; s++) {
@@ -908,7 +912,8 @@ __global__ void k_amg_raplists(int nc, const int* __restrict__ cptr, const int* 
 // a time (lane 6 g + c: entry g, column c), added up in shared memory at the
 // product's place in the A P row (a list made once per mesh: searched for
 // here, the places took more instructions than the products).  Rows longer than
-// AMG_CHUNK entries are taken in chunks.  The entries of one P row have
+// AMG_CHUNK entries are taken in chunks.  Without the list (LIST false) the
+// place is searched, to the same sums.  The entries of one P row have
 // distinct places and block k + 1 follows block k after a warp barrier: no
 // atomics, a fixed order.  Bound by the
 // FP32 and shared-memory instructions of the products: about 500 us on level 0
@@ -924,11 +929,12 @@ struct ApShared {
 template <class C, int B>
 __host__ __device__ constexpr int ap_warps() { return B == 3 && sizeof(C) == 4 ? 8 : 4; }
 
-template <class C, class V, int B>
+template <class C, class V, int B, bool LIST>
 __global__ void __launch_bounds__(32 * ap_warps<C, B>())
     k_amg_ap(int n, const int* __restrict__ ptr, const int* __restrict__ col, Vals<C, V, B> A,
-             const int* __restrict__ pptr, const C* __restrict__ p, const int* __restrict__ apptr,
-             const int64_t* __restrict__ apoff, const int* __restrict__ apidx, C* __restrict__ ap) {
+             const int* __restrict__ pptr, const int* __restrict__ pcol, const C* __restrict__ p,
+             const int* __restrict__ apptr, const int* __restrict__ apcol, const int64_t* __restrict__ apoff,
+             const int* __restrict__ apidx, C* __restrict__ ap) {
   constexpr int BN = B * AMG_NS;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -939,7 +945,7 @@ __global__ void __launch_bounds__(32 * ap_warps<C, B>())
   const int ks = ptr[i], ke = ptr[i + 1], a0 = apptr[i], ae = apptr[i + 1];
   for (int cb = a0; cb < ae; cb += AMG_CHUNK) {
     const int m = min(AMG_CHUNK, ae - cb);
-    const int* ix = apidx + apoff[i];  // places of the next block's products
+    const int* ix = LIST ? apidx + apoff[i] : nullptr;  // places of the next block's products
     for (int t = lane; t < m * BN; t += 32) sh.acc[t] = C(0);
     for (int k0 = ks; k0 < ke; k0 += 32) {
       const int cnt = min(32, ke - k0);
@@ -958,7 +964,7 @@ __global__ void __launch_bounds__(32 * ap_warps<C, B>())
         const int qa = __shfl_sync(0xffffffffu, q0, kk), len = __shfl_sync(0xffffffffu, q1, kk) - qa;
         if (g < 5)
           for (int u = g; u < len; u += 5) {
-            const int e = (int)ix[u] - (cb - a0);
+            const int e = (LIST ? ix[u] : find_sorted(apcol + a0, ae - a0, pcol[qa + u])) - (cb - a0);
             const C* P = p + (int64_t)(qa + u) * BN + c;
             C pv[B];
 #pragma unroll
@@ -974,7 +980,7 @@ __global__ void __launch_bounds__(32 * ap_warps<C, B>())
               }
             }
           }
-        ix += len;
+        if (LIST) ix += len;
         __syncwarp();
       }
     }
@@ -990,12 +996,14 @@ __global__ void __launch_bounds__(32 * ap_warps<C, B>())
 // (few entries, long lists, bound by the latency of the loads): 36 threads, one
 // value each, eight products in flight.  404 us on level 0 of Cook P2 45x41x7
 // and 167 us on level 1 (a thread per entry that searched the
-// A P rows of all the row's nodes: 979 and 849 us).
-template <class C, int B>
+// A P rows of all the row's nodes: 979 and 849 us).  Without the list (LIST
+// false) the A P rows are searched, to the same sums.
+template <class C, int B, bool LIST>
 __global__ void __launch_bounds__(B == 3 ? 192 : 64)
     k_amg_rap(int64_t nnzc, const int* __restrict__ crow, const int* __restrict__ ccol,
               const int64_t* __restrict__ lend, const int64_t* __restrict__ raoff, const int2* __restrict__ list,
-              const C* __restrict__ p, const C* __restrict__ ap, const unsigned char* __restrict__ cabsent,
+              const int* __restrict__ rptr, const int* __restrict__ rcol, const int* __restrict__ rsrc,
+              const int* __restrict__ apptr, const int* __restrict__ apcol, const C* __restrict__ p, const C* __restrict__ ap, const unsigned char* __restrict__ cabsent,
               C* __restrict__ out) {
   constexpr int BN = B * AMG_NS, NN = AMG_NS * AMG_NS;
   constexpr int PER = B == 3 ? AMG_NS : 1, TPE = NN / PER;  // values per thread, threads per entry
@@ -1007,9 +1015,7 @@ __global__ void __launch_bounds__(B == 3 ? 192 : 64)
   C acc[PER];
 #pragma unroll
   for (int c = 0; c < PER; c++) acc[c] = C(0);
-  const int64_t l1 = lend[e];
   constexpr int U = B == 3 ? 2 : (sizeof(C) == 4 ? 8 : 4);  // products in flight
-  int64_t l = e > 0 && crow[e - 1] == a ? lend[e - 1] : raoff[a];
   auto add = [&](const C (&P)[B], const C (&Q)[B][PER]) {
 #pragma unroll
     for (int c = 0; c < PER; c++) {
@@ -1029,17 +1035,29 @@ __global__ void __launch_bounds__(B == 3 ? 192 : 64)
       for (int c = 0; c < PER; c++) Q[k][c] = __ldg(qq + AMG_NS * k + c);
     }
   };
-  for (; l + U <= l1; l += U) {
-    C P[U][B], Q[U][B][PER];
+  if constexpr (LIST) {
+    const int64_t l1 = lend[e];
+    int64_t l = e > 0 && crow[e - 1] == a ? lend[e - 1] : raoff[a];
+    for (; l + U <= l1; l += U) {
+      C P[U][B], Q[U][B][PER];
 #pragma unroll
-    for (int w = 0; w < U; w++) load(list[l + w], P[w], Q[w]);
+      for (int w = 0; w < U; w++) load(list[l + w], P[w], Q[w]);
 #pragma unroll
-    for (int w = 0; w < U; w++) add(P[w], Q[w]);
-  }
-  for (; l < l1; l++) {
-    C P[B], Q[B][PER];
-    load(list[l], P, Q);
-    add(P, Q);
+      for (int w = 0; w < U; w++) add(P[w], Q[w]);
+    }
+    for (; l < l1; l++) {
+      C P[B], Q[B][PER];
+      load(list[l], P, Q);
+      add(P, Q);
+    }
+  } else {
+    for (int s = rptr[a]; s < rptr[a + 1]; s++) {
+      const int f0 = apptr[rcol[s]], pos = find_sorted(apcol + f0, apptr[rcol[s] + 1] - f0, ccol[e]);
+      if (pos < 0) continue;
+      C P[B], Q[B][PER];
+      load(make_int2(rsrc[s], f0 + pos), P, Q);
+      add(P, Q);
+    }
   }
   const bool unit = ccol[e] == a && ((cabsent[a] >> r) & 1u);
 #pragma unroll
@@ -1746,6 +1764,17 @@ int dev_alloc(fe_mesh m, X** p, size_t count) {
   return FE_OK;
 }
 
+// an array the hierarchy can do without: *p stays null where it does not fit
+template <class X>
+int dev_alloc_optional(fe_mesh m, X** p, size_t count) {
+  const int rc = fe_alloc_once(m, reinterpret_cast<void**>(p), std::max<size_t>(count, 1) * sizeof(X));
+  if (rc == FE_ERR_OOM) return FE_OK;
+  FE_TRY(rc);
+  m->amg->allocs.push_back((void*)*p);
+  m->amg->bytes += (int64_t)(std::max<size_t>(count, 1) * sizeof(X));
+  return FE_OK;
+}
+
 template <class X>
 int upload(fe_mesh m, X** p, const std::vector<X>& v) {
   FE_TRY(dev_alloc(m, p, v.size()));
@@ -1848,14 +1877,11 @@ int build_structure(fe_mesh m) {
       FE_CUDA(cudaGetLastError());
       FE_TRY(upload(m, &A.apoff, H.apoff));
       FE_TRY(upload(m, &A.raoff, H.raoff));
-      FE_TRY(dev_alloc(m, &A.apidx, (size_t)H.apoff.back()));
-      FE_TRY(dev_alloc(m, &A.ralist, (size_t)H.raoff.back()));
+      A.napidx = H.apoff.back();
+      A.nralist = H.raoff.back();
       FE_TRY(dev_alloc(m, &A.tnode32, H.tnode.size()));
       k_amg_to_f32<<<blocks_for((int64_t)H.tnode.size(), 256), 256, 0, m->stream>>>((int64_t)H.tnode.size(), A.tnode,
                                                                                    A.tnode32);
-      FE_CUDA(cudaGetLastError());
-      k_amg_apidx<<<blocks_for((int64_t)A.n * 32, 256), 256, 0, m->stream>>>(A.n, A.ptr, A.col, A.pptr, A.pcol, A.apptr,
-                                                                           A.apcol, A.apoff, A.apidx);
       FE_CUDA(cudaGetLastError());
     }
   }
@@ -1863,6 +1889,11 @@ int build_structure(fe_mesh m) {
     AmgLevel &A = h->lev[q], &Cq = h->lev[q + 1];
     FE_TRY(dev_alloc(m, &A.lend, (size_t)Cq.nnz));
     FE_TRY(dev_alloc(m, &A.crow, (size_t)Cq.nnz));
+    FE_TRY(dev_alloc_optional(m, &A.apidx, (size_t)A.napidx));
+    FE_TRY(dev_alloc_optional(m, &A.ralist, (size_t)A.nralist));
+    if (A.apidx)
+      k_amg_apidx<<<blocks_for((int64_t)A.n * 32, 256), 256, 0, m->stream>>>(A.n, A.ptr, A.col, A.pptr, A.pcol, A.apptr,
+                                                                           A.apcol, A.apoff, A.apidx);
     k_amg_raplists<<<blocks_for((int64_t)Cq.n * 32, 256), 256, 0, m->stream>>>(
         Cq.n, Cq.ptr, Cq.col, A.rptr, A.rcol, A.rsrc, A.apptr, A.apcol, A.raoff, A.lend, A.crow, A.ralist);
     FE_CUDA(cudaGetLastError());
@@ -2001,15 +2032,18 @@ int numeric_level(fe_mesh m, int q, const V* val) {
     FE_SCOPE(m, FE_PROF_OTHER, (double)L.nnzap * B * AMG_NS * sizeof(C));
     constexpr int W = ap_warps<C, B>();
     const int smem = W * (int)sizeof(ApShared<C, B>);
-    FE_TRY(fe_kernel_smem((const void*)k_amg_ap<C, V, B>, smem));
-    k_amg_ap<C, V, B><<<blocks_for(L.n, W), 32 * W, smem, m->stream>>>(L.n, L.ptr, L.col, A, L.pptr, p, L.apptr,
-                                                                      L.apoff, L.apidx, ap);
+    auto kern = L.apidx ? k_amg_ap<C, V, B, true> : k_amg_ap<C, V, B, false>;
+    FE_TRY(fe_kernel_smem((const void*)kern, smem));
+    kern<<<blocks_for(L.n, W), 32 * W, smem, m->stream>>>(L.n, L.ptr, L.col, A, L.pptr, L.pcol, p, L.apptr, L.apcol,
+                                                          L.apoff, L.apidx, ap);
   }
   FE_CUDA(cudaGetLastError());
   {
     FE_SCOPE(m, FE_PROF_OTHER, (double)Cq.nnz * AMG_NS * AMG_NS * sizeof(C));
-    k_amg_rap<C, B><<<blocks_for(Cq.nnz * (B == 3 ? AMG_NS : AMG_NS * AMG_NS), B == 3 ? 192 : 64), B == 3 ? 192 : 64, 0, m->stream>>>(
-        Cq.nnz, L.crow, Cq.col, L.lend, L.raoff, L.ralist, p, ap, Cq.absent, cval);
+    auto kern = L.ralist ? k_amg_rap<C, B, true> : k_amg_rap<C, B, false>;
+    kern<<<blocks_for(Cq.nnz * (B == 3 ? AMG_NS : AMG_NS * AMG_NS), B == 3 ? 192 : 64), B == 3 ? 192 : 64, 0, m->stream>>>(
+        Cq.nnz, L.crow, Cq.col, L.lend, L.raoff, L.ralist, L.rptr, L.rcol, L.rsrc, L.apptr, L.apcol, p, ap, Cq.absent,
+        cval);
   }
   FE_CUDA(cudaGetLastError());
   return FE_OK;
@@ -2322,6 +2356,29 @@ int fe_amg_apply(fe_mesh m, const double* x, double* z) {
     FE_CUDA(cudaGetLastError());
   }
   return FE_OK;
+}
+
+// Gives the product lists back (Cook P2 48x48x8: 175 MB, a fifth of what a mesh
+// with the hierarchy holds); the products are searched from then on.  false:
+// there were none.
+bool fe_amg_release_lists(fe_mesh m) {
+  AmgHier* h = m->amg;
+  if (!h) return false;
+  int64_t freed = 0;
+  auto drop = [&](auto*& p, int64_t count) {
+    if (!p) return;
+    h->allocs.erase(std::find(h->allocs.begin(), h->allocs.end(), (void*)p));
+    cudaFreeAsync(p, m->stream);
+    freed += std::max<int64_t>(count, 1) * (int64_t)sizeof(*p);
+    p = nullptr;
+  };
+  for (int q = 0; q < h->nlev; q++) {
+    drop(h->lev[q].apidx, h->lev[q].napidx);
+    drop(h->lev[q].ralist, h->lev[q].nralist);
+  }
+  h->bytes -= freed;
+  m->device_bytes -= freed;
+  return freed > 0;
 }
 
 void fe_amg_free(fe_mesh m) {

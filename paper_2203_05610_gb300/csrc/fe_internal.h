@@ -289,7 +289,7 @@ struct LaunchScope {
   LaunchScope FE_CAT(fe_scope_, __LINE__)(m, cls, (double)(bytes), (double)(flops))
 
 // Stream-ordered allocation, counted in the mesh's device bytes; out of
-// memory, fe_alloc gives the mesh's optional scratch back and tries once more
+// memory, fe_alloc gives the mesh's optional arrays back and tries again
 int fe_alloc_once(fe_mesh m, void** p, size_t bytes);
 int fe_alloc(fe_mesh m, void** p, size_t bytes);
 template <class T>
@@ -333,6 +333,7 @@ int fe_spmv_preload(fe_mesh m);  // loads every SpMV kernel and caches its launc
 int fe_amg_setup(fe_mesh m);
 int fe_amg_apply(fe_mesh m, const double* x, double* z);
 void fe_amg_free(fe_mesh m);
+bool fe_amg_release_lists(fe_mesh m);  // frees the optional arrays of the setup
 // fe_assemble.cu: uploads the face-pattern values (springs plus 2/dt times
 // the dashpots while dynamics is on)
 int fe_upload_face_values(fe_mesh m);

@@ -46,15 +46,18 @@ int fe_alloc_once(fe_mesh m, void** p, size_t bytes) {
   return FE_OK;
 }
 
-// Gives the mesh's optional scratch back to the device (nothing in it outlives
-// the call that filled it, and its users have a form without it); false:
-// there was none.
+// Gives optional arrays of the mesh back to the device, those that have a form
+// without them: the tangent's element blocks (nothing in them outlives an
+// assembly), then the AMG setup's product lists.  false: there were none.
 static bool release_scratch(fe_mesh m) {
-  if (!m->tan_work) return false;
-  cudaFreeAsync(m->tan_work, m->stream);
-  m->device_bytes -= (int64_t)m->tan_work_bytes;
-  m->tan_work = nullptr;
-  m->tan_work_bytes = 0;
+  if (m->tan_work) {
+    cudaFreeAsync(m->tan_work, m->stream);
+    m->device_bytes -= (int64_t)m->tan_work_bytes;
+    m->tan_work = nullptr;
+    m->tan_work_bytes = 0;
+  } else if (!fe_amg_release_lists(m)) {
+    return false;
+  }
   cudaStreamSynchronize(m->stream);
   cudaMemPool_t pool;  // (memory the pool still holds may be in pieces too small for the caller)
   if (cudaDeviceGetDefaultMemPool(&pool, m->device) == cudaSuccess) cudaMemPoolTrimTo(pool, 0);
@@ -63,7 +66,7 @@ static bool release_scratch(fe_mesh m) {
 
 int fe_alloc(fe_mesh m, void** p, size_t bytes) {
   int rc = fe_alloc_once(m, p, bytes);
-  if (rc == FE_ERR_OOM && release_scratch(m)) rc = fe_alloc_once(m, p, bytes);
+  while (rc == FE_ERR_OOM && release_scratch(m)) rc = fe_alloc_once(m, p, bytes);
   return rc;
 }
 

@@ -376,3 +376,36 @@ def test_tangent_workspace_given_back(fe):
         torch.cuda.empty_cache()
     assert torch.linalg.norm(x - want[0]) <= 1e-9 * torch.linalg.norm(want[0])
     assert (y - want[1]).abs().max() <= 1e-12 * want[1].abs().max()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed_fp32"])
+@pytest.mark.parametrize("case", ["cook2", "twist", "heart1"])
+def test_amg_setup_without_product_lists(fe, case, precision):
+    # a basis that does not fit takes the lists with it; the products are then
+    # searched: the same hierarchy and V-cycle, bit for bit
+    w = {"cook2": lambda: W.cook(13, 11, 5, order=2, nu=0.3), "twist": lambda: W.twist(6),
+         "heart1": lambda: W.heart(nr=2, nc=24, nl=20, order=1)}[case]()
+    m, ref = fe.Mesh(w), fe.Mesh(w)
+    rng = np.random.default_rng(16)
+    d, x = (torch.from_numpy(rng.standard_normal(m.ndof)).cuda() for _ in range(2))
+    d *= 0.002
+    for mesh in (m, ref):
+        mesh.set_pc("amg")
+        mesh.tangent(0.5 * d, precision)
+    npair, npl = m.nen * (m.nen + 1) // 2, 4 if case == "twist" else 0
+    work = m.ne * (9 * npair + 3 * npl * m.nen) * (8 if precision == "fp64" else 4)
+    held = _device_bytes(fe, m)
+    hog = _hog(20 << 20)
+    try:
+        with pytest.raises(fe.FEError, match="out of memory"):
+            m.gmres(x, restart=1000)
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    assert _device_bytes(fe, m) <= held - work + 4 * 8 * m.ndof - 100000  # (four vectors of the workspace fitted)
+    for mesh in (m, ref):
+        mesh.tangent(d, precision)
+    for a, b in zip(m.amg_levels(), ref.amg_levels()):
+        assert a["rho"] == b["rho"]
+        assert all(np.array_equal(a[k], b[k]) for k in ("val", "pval") if k in b)
+    assert torch.equal(m.pc(x), ref.pc(x))
