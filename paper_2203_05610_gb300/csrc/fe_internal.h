@@ -72,6 +72,14 @@ struct MatParams {
 };
 
 // ---------------------------------------------------------------- mesh object
+// a device array that knows its own size: asked for more (fe_grow) it is
+// replaced, and a request that ends in FE_ERR_OOM leaves it empty
+struct GrowVec {
+  double* p = nullptr;
+  size_t size = 0;
+  operator double*() const { return p; }
+};
+
 struct fe_mesh_s {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -182,24 +190,22 @@ struct fe_mesh_s {
   double* h_scal = nullptr;  // pinned host mirror [64]
 
   // solver workspace (lazy)
-  int ws_restart = 0;
-  double* V = nullptr;       // [(restart+1)][ldv], rows zero-padded
+  GrowVec V;                 // [(restart+1)][ldv], rows zero-padded
   int64_t ldv = 0;           // leading dimension of V: ndof rounded up to 32
   int orthog = 0;            // 0: sequential MGS sweep, 1: low-synchronisation MGS, 2: blocked MGS
-  double* Lmat = nullptr;    // [(restart+1)^2] strictly lower triangle of V^T V (low-sync MGS)
-  double* hpub = nullptr;    // [restart+1] published MGS coefficients
-  double* partv = nullptr;   // [partv_blocks][2 restart + 1] per-block inner products
+  GrowVec Lmat;              // [(restart+1)^2] strictly lower triangle of V^T V (low-sync MGS)
+  GrowVec hpub;              // [restart+1] published MGS coefficients
+  GrowVec partv;             // [partv_blocks][2 restart + 1] per-block inner products
   int partv_blocks = 0;
-  double* Tbm = nullptr;     // [(restart+2)][BMGS_P] strictly lower rows of (I + L_B)^{-1} (blocked MGS)
-  double* H = nullptr;       // [(restart+1)][restart] column-major by step
-  double* gv = nullptr;      // Givens: cs, sn, g, y [4][restart+1]
+  GrowVec Tbm;               // [(restart+2)][BMGS_P] strictly lower rows of (I + L_B)^{-1} (blocked MGS)
+  GrowVec H;                 // [(restart+1)][restart] column-major by step
+  GrowVec gv;                // Givens: cs, sn, g, y [4][restart+1]
   double* w64 = nullptr;     // [ndof]
   double* t64 = nullptr;     // [ndof]
   double* u64 = nullptr;     // [ndof]
   void* zx = nullptr;        // [ndof] SpMV input (FP32 or FP64); also the V-cycle's level-0 iterate
-  int lb_m = 0;
-  double* S = nullptr;       // [m][ndof]
-  double* Yv = nullptr;      // [m][ndof]
+  GrowVec S;                 // [m][ndof]
+  GrowVec Yv;                // [m][ndof]
   double* nl_R = nullptr, *nl_Rn = nullptr, *nl_dl = nullptr, *nl_t = nullptr;
   double* rho_d = nullptr;   // [LBFGS_MAX] curvature scalars 1/(y.s) of the stored pairs
   double* alpha_d = nullptr; // [LBFGS_MAX] two-loop coefficients alpha_i
@@ -296,6 +302,8 @@ template <class T>
 int fe_alloc_t(fe_mesh m, T** p, size_t count) {
   return fe_alloc(m, reinterpret_cast<void**>(p), count * sizeof(T));
 }
+// at least `count` values (contents are lost where it grows)
+int fe_grow(fe_mesh m, GrowVec* v, size_t count);
 int fe_check_device_error(fe_mesh m);  // syncs the stream and reads the error word
 // Kernel launch facts cached per (kernel, device, shape), safe from several
 // host threads (the serving loop) and from several devices in one process:

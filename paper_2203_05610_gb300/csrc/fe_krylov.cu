@@ -1788,39 +1788,22 @@ int fe_workspace(fe_mesh m, int restart) {
   if (!m->w64) FE_TRY(fe_alloc_t(m, &m->w64, (size_t)m->ndof));
   if (!m->t64) FE_TRY(fe_alloc_t(m, &m->t64, (size_t)m->ndof));
   if (!m->u64) FE_TRY(fe_alloc_t(m, &m->u64, (size_t)m->ndof));
-  if (restart > m->ws_restart) {
-    // basis rows padded to a multiple of 32 values (256 bytes) and zeroed, so
-    // the Arnoldi kernel's 16-byte pair loads stay inside a row
-    const int64_t ldv = (m->ndof + 31) / 32 * 32;
-    if (m->V) {
-      cudaFreeAsync(m->V, m->stream);
-      cudaFreeAsync(m->H, m->stream);
-      cudaFreeAsync(m->gv, m->stream);
-      m->device_bytes -= (int64_t)(m->ws_restart + 1) * m->ldv * 8 + (int64_t)(m->ws_restart + 1) * (m->ws_restart + 1) * 8 +
-                         (int64_t)4 * (m->ws_restart + 2) * 8;
-      m->V = m->H = m->gv = nullptr;
-      cudaFreeAsync(m->Tbm, m->stream);
-      m->device_bytes -= (int64_t)(m->ws_restart + 2) * BMGS_P * 8;
-      m->Tbm = nullptr;
-    }
-    FE_TRY(fe_alloc_t(m, &m->V, (size_t)(restart + 1) * ldv));
-    FE_CUDA(cudaMemsetAsync(m->V, 0, (size_t)(restart + 1) * ldv * sizeof(double), m->stream));
-    FE_TRY(fe_alloc_t(m, &m->H, (size_t)(restart + 1) * (restart + 1)));
-    FE_TRY(fe_alloc_t(m, &m->gv, (size_t)4 * (restart + 2)));
-    m->ws_restart = restart;
-    m->ldv = ldv;
-    FE_TRY(fe_alloc_t(m, &m->Tbm, (size_t)(restart + 2) * BMGS_P));
-    if (restart <= LOWSYNC_MAX_RESTART) {  // low-synchronisation MGS: L, h, per-block inner products
-      if (m->Lmat) {
-        cudaFreeAsync(m->Lmat, m->stream);
-        cudaFreeAsync(m->hpub, m->stream);
-        cudaFreeAsync(m->partv, m->stream);
-      }
-      m->partv_blocks = 2 * m->sm_count;
-      FE_TRY(fe_alloc_t(m, &m->Lmat, (size_t)(restart + 1) * (restart + 1)));
-      FE_TRY(fe_alloc_t(m, &m->hpub, (size_t)(restart + 1)));
-      FE_TRY(fe_alloc_t(m, &m->partv, (size_t)m->partv_blocks * (2 * restart + 1)));
-    }
+  // basis rows padded to a multiple of 32 values (256 bytes) and zeroed, so
+  // the Arnoldi kernel's 16-byte pair loads stay inside a row
+  m->ldv = (m->ndof + 31) / 32 * 32;
+  const size_t r1 = (size_t)restart + 1, nv = r1 * (size_t)m->ldv;
+  if (m->V.size < nv) {
+    FE_TRY(fe_grow(m, &m->V, nv));
+    FE_CUDA(cudaMemsetAsync(m->V, 0, nv * sizeof(double), m->stream));
+  }
+  FE_TRY(fe_grow(m, &m->H, r1 * r1));
+  FE_TRY(fe_grow(m, &m->gv, 4 * (r1 + 1)));
+  FE_TRY(fe_grow(m, &m->Tbm, (r1 + 1) * BMGS_P));
+  if (restart <= LOWSYNC_MAX_RESTART) {  // low-synchronisation MGS: L, h, per-block inner products
+    m->partv_blocks = 2 * m->sm_count;
+    FE_TRY(fe_grow(m, &m->Lmat, r1 * r1));
+    FE_TRY(fe_grow(m, &m->hpub, r1));
+    FE_TRY(fe_grow(m, &m->partv, (size_t)m->partv_blocks * (2 * r1 - 1)));
   }
   return FE_OK;
 }

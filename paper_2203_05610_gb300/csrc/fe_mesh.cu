@@ -70,6 +70,20 @@ int fe_alloc(fe_mesh m, void** p, size_t bytes) {
   return rc;
 }
 
+int fe_grow(fe_mesh m, GrowVec* v, size_t count) {
+  if (v->size >= count) return FE_OK;
+  if (v->p) {
+    cudaFreeAsync(v->p, m->stream);
+    m->device_bytes -= (int64_t)(v->size * sizeof(double));
+    *v = GrowVec();
+  }
+  double* p = nullptr;
+  FE_TRY(fe_alloc_t(m, &p, count));
+  v->p = p;
+  v->size = count;
+  return FE_OK;
+}
+
 // grid-reduction state of the persistent kernels: arrival counter, step
 // sequence, and two published-value slots holding the "not yet" sentinel;
 // then the blocked-MGS step's own sequence and its two sets of 8 slots, and

@@ -143,17 +143,8 @@ static int solve_impl(fe_mesh m, int method, double tol, int max_it, double* d, 
   } else {
     const int mcap = o.lbfgs_m;
     if (mcap < 1 || mcap > LBFGS_MAX) return fe_set_error("lbfgs_m must lie in [1, %d]", LBFGS_MAX), FE_ERR_ARG;
-    if (m->lb_m < mcap) {
-      if (m->S) {
-        cudaFreeAsync(m->S, m->stream);
-        cudaFreeAsync(m->Yv, m->stream);
-        m->device_bytes -= 2LL * m->lb_m * n * 8;
-        m->S = m->Yv = nullptr;
-      }
-      FE_TRY(fe_alloc_t(m, &m->S, (size_t)mcap * n));
-      FE_TRY(fe_alloc_t(m, &m->Yv, (size_t)mcap * n));
-      m->lb_m = mcap;
-    }
+    FE_TRY(fe_grow(m, &m->S, (size_t)mcap * n));
+    FE_TRY(fe_grow(m, &m->Yv, (size_t)mcap * n));
     FE_TRY(fe_tangent_dev(m, d, o.precision));  // the one Hessian assembly at d_0
     st.assemblies = 1;
     int head = 0, np = 0;

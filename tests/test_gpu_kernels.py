@@ -409,3 +409,45 @@ def test_amg_setup_without_product_lists(fe, case, precision):
         assert a["rho"] == b["rho"]
         assert all(np.array_equal(a[k], b[k]) for k in ("val", "pval") if k in b)
     assert torch.equal(m.pc(x), ref.pc(x))
+
+
+def test_workspace_after_a_request_that_did_not_fit(fe):
+    # a basis and a set of secant pairs that end in FE_ERR_OOM leave a mesh that solves as before
+    w = W.cook(13, 11, 5, order=2, nu=0.3)
+    m, ref = fe.Mesh(w), fe.Mesh(w)
+    b = torch.from_numpy(np.random.default_rng(17).standard_normal(m.ndof)).cuda()
+    opts = dict(lbfgs_m=4, ksp_restart=6, ksp_max_it=6)
+    out = []
+    for mesh in (m, ref):
+        mesh.set_load(0.1)
+        mesh.tangent(mesh.zeros())
+        out.append([mesh.gmres(b, restart=6, max_it=9)[0], mesh.solve("B", mesh.zeros(), max_it=3, opts=opts)[0]])
+    hog = _hog(20 << 20)
+    try:
+        with pytest.raises(fe.FEError, match="out of memory"):
+            m.gmres(b, restart=1000)
+        with pytest.raises(fe.FEError, match="out of memory"):
+            m.solve("B", m.zeros(), max_it=3, opts=dict(opts, lbfgs_m=1000))
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    for mesh, o in zip((m, ref), out):
+        o.append(mesh.solve("B", mesh.zeros(), max_it=3, opts=opts)[0])
+        mesh.tangent(mesh.zeros())
+        o.append(mesh.gmres(b, restart=6, max_it=9)[0])
+    for x, y in zip(*out):
+        assert torch.equal(x, y)
+
+
+def test_lowsync_workspace_follows_its_own_restart(fe):
+    # the low-synchronisation form's arrays belong to restarts of up to 128: a
+    # longer restart of another form in between does not stand for them
+    w = W.cook(9, 9, 4, order=1, nu=0.3)
+    m, ref = fe.Mesh(w), fe.Mesh(w)
+    b = torch.from_numpy(np.random.default_rng(18).standard_normal(m.ndof)).cuda()
+    for mesh in (m, ref):
+        mesh.tangent(mesh.zeros())
+    for restart in (20, 300):
+        m.gmres(b, restart=restart, max_it=2)
+    x, y = (mesh.gmres(b, rtol=0.0, atol=0.0, restart=128, max_it=128, orthog=1)[0] for mesh in (m, ref))
+    assert torch.equal(x, y)
