@@ -4,7 +4,9 @@
  * A server owns one GPU.  Clients submit nonlinear solves (a mesh
  * description, a method, tolerances, a load step) at any time; a scheduler
  * thread admits queued requests in arrival order as soon as a slot is free
- * and their estimated device footprint fits the HBM budget, and runs every
+ * and their estimated device footprint fits the HBM budget (one beyond the
+ * whole budget runs without the arrays its mesh can do without, if that
+ * fits), and runs every
  * admitted request on its own CUDA stream, so the work of all admitted
  * requests overlaps on the device.  Small requests (fe_batch.h) are instead
  * handed to batcher threads that solve all such requests waiting at that

@@ -1767,6 +1767,7 @@ int dev_alloc(fe_mesh m, X** p, size_t count) {
 // an array the hierarchy can do without: *p stays null where it does not fit
 template <class X>
 int dev_alloc_optional(fe_mesh m, X** p, size_t count) {
+  if (m->lean) return FE_OK;
   const int rc = fe_alloc_once(m, reinterpret_cast<void**>(p), std::max<size_t>(count, 1) * sizeof(X));
   if (rc == FE_ERR_OOM) return FE_OK;
   FE_TRY(rc);

@@ -1019,6 +1019,7 @@ static int tangent_workspace(fe_mesh m, size_t elem) {
   const size_t npair = (size_t)m->nen * (m->nen + 1) / 2, npl = m->pres == 0 ? 0 : (m->pres == 2 ? 1 : 4);
   const size_t bytes = (size_t)m->ne * (9 * npair + 3 * npl * m->nen) * elem;
   if (m->tan_work_bytes >= bytes) return FE_OK;
+  if (m->lean) return FE_ERR_OOM;
   if (bytes > TAN_WORK_SMALL) {
     size_t free_b = 0, total_b = 0;
     FE_CUDA(cudaMemGetInfo(&free_b, &total_b));

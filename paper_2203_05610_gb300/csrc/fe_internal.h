@@ -130,6 +130,7 @@ struct fe_mesh_s {
   int* color_list = nullptr;  // node_list in the order of the elements' colours
   void* tan_work = nullptr;   // element blocks of the tangent (launch_tangent in fe_assemble.cu), kept between assemblies
   size_t tan_work_bytes = 0;
+  bool lean = false;          // take no optional arrays (tan_work, the AMG setup's product lists)
   int* vert_ptr = nullptr;
   int* vert_list = nullptr;
 

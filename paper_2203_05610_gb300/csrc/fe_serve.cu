@@ -55,6 +55,8 @@ struct Request {
   struct CachedMesh* cm = nullptr;  // the resident mesh it runs on, if any
   std::vector<struct CachedMesh*> victims;  // idle meshes evicted to admit it
   int64_t charge = 0;              // budget bytes it holds itself while running
+  int64_t lean_footprint = 0;      // without the mesh's optional arrays
+  bool lean = false;               // runs without them: the budget has no room for the whole footprint
 };
 
 // A mesh kept on the device between requests with the same description:
@@ -98,8 +100,8 @@ std::string mesh_key(const Request& r) {
 // device bytes a request will hold, estimated from its description before
 // anything is allocated (exact node count; block count from the measured
 // blocks per node of tetrahedral meshes, 28 for P2 and 16 for P1, with
-// margin)
-int64_t estimate_footprint(const Request& r, int64_t* ndof_out) {
+// margin); *lean: without the arrays a mesh can do without
+int64_t estimate_footprint(const Request& r, int64_t* ndof_out, int64_t* lean) {
   const fe_mesh_desc& d = r.desc;
   int64_t nv = d.nv, ne = d.ne, nn = nv;
   if (d.order == 2) {
@@ -125,12 +127,14 @@ int64_t estimate_footprint(const Request& r, int64_t* ndof_out) {
   b += 24 * nn + ne * (4 * nen + 8 + 80 + 4 * nen * nen + 24 * nen + 8 * nen) + 4 * nnzb + 16 * nn;  // mesh
   if (d.fibers) b += 72 * ne;
   if (d.pressure_order) b += ne * (4 * nen * 4 + 32) + 16 * 12 * nn;  // coupling pattern and values
-  b += ne * sval * (9 * nen * (nen + 1) / 2 + (d.pressure_order ? 12 * nen : 0));  // element blocks of the tangent
   b += 9 * sval * nnzb + 9 * sval * nn + (o.precision == FE_PREC_MIXED_BF16 ? 18 * nnzb : 0);  // tangent
   b += 8 * ndof * (restart + 1) + 8 * (restart + 1) * (restart + 1);                             // Krylov basis
   b += 8 * ndof * (2 * mpairs + 12);                                                              // BFGS pairs, vectors
-  if (o.pc_type >= 1) b += (d.order == 1 ? 3300 : 7500) * nn;  // AMG: P, A P, P^T in FP64, coarse levels, product lists
+  if (o.pc_type >= 1) b += (d.order == 1 ? 2500 : 6000) * nn;  // AMG: P, A P, P^T in FP64 and coarse levels
   *ndof_out = ndof;
+  *lean = b + b / 8 + (64 << 20);
+  b += ne * sval * (9 * nen * (nen + 1) / 2 + (d.pressure_order ? 12 * nen : 0));  // element blocks of the tangent
+  if (o.pc_type >= 1) b += (d.order == 1 ? 800 : 1500) * nn;                       // AMG: product lists
   return b + b / 8 + (64 << 20);
 }
 
@@ -220,6 +224,7 @@ static void run_request(fe_server s, Request* r) {
   }
   cudaStream_t stream = c->stream;
   fe_mesh m = c->m;
+  if (rc == FE_OK) m->lean = r->lean;
   if (rc == FE_OK) rc = fe_set_load(m, r->load, r->time);
   int64_t ndof = 0;
   if (rc == FE_OK) {
@@ -432,6 +437,10 @@ static void scheduler_loop(fe_server s) {
     bool admitted = false;
     for (auto it = s->queue.begin(); it != s->queue.end();) {
       Request* r = s->reqs[*it].get();
+      if (r->st.footprint > s->budget && r->lean_footprint <= s->budget) {
+        r->lean = true;
+        r->st.footprint = r->lean_footprint;
+      }
       if (r->st.footprint > s->budget) {  // can never fit: reject
         r->st.state = FE_REQ_FAILED;
         r->st.result = FE_ERR_OOM;
@@ -564,7 +573,7 @@ extern "C" int serve_submit(fe_server s, const fe_request* q, int64_t* id_out) {
   r->load = q->load;
   r->time = q->time;
   int64_t ndof = 0;
-  r->st.footprint = estimate_footprint(*r, &ndof);
+  r->st.footprint = estimate_footprint(*r, &ndof, &r->lean_footprint);
   r->mesh_key = mesh_key(*r);
   r->key_hash = std::hash<std::string>{}(r->mesh_key);
   if (q->d0) r->d0.assign(q->d0, q->d0 + ndof);

@@ -164,3 +164,21 @@ def test_resident_meshes_are_evicted_least_recently_used(fe):
     srv.close()
     assert all(x["state"] == "done" for x in res)
     assert [x["mesh_reused"] for x in res] == [False, False, False, True]
+
+
+def test_requests_run_without_optional_arrays_in_a_tight_budget(fe):
+    """A budget below a request's whole footprint but with room for it without
+    the arrays that the mesh can do without (element blocks of the tangent,
+    AMG product lists): it is solved without them, to the same solution."""
+    w = W.cook(12, 12, 4, order=2, nu=0.3)
+    opts = dict(precision="mixed_fp32", pc_type="amg", ksp_restart=30)
+    out = []
+    budget = 0
+    for _ in range(2):
+        srv = fe.Server(hbm_budget=budget, max_active=1, batch_max_dofs=-1)
+        out.append(srv.poll(srv.submit(w, "iNK", tol=1e-8, opts=opts, load=0.2), wait=True))
+        srv.close()
+        budget = out[0]["footprint"] - 1
+    assert [r["state"] for r in out] == ["done", "done"], out[1]
+    assert out[1]["footprint"] <= budget
+    assert np.array_equal(out[0]["d"], out[1]["d"])
