@@ -2415,9 +2415,11 @@ extern "C" int fe_amg_get_level(fe_mesh m, int level, int64_t* info, double* rho
     info[4] = last ? 0 : L.nnzp;
   }
   if (rho) *rho = L.rho;
-  // values in FP64 (widened from the FP32 numbers of the mixed forms)
+  // values in FP64 (widened from the FP32 numbers of the mixed forms), those of
+  // the last tangent: the arrays of another precision may be there, too
+  const bool f64 = m->prec == FE_PREC_FP64;
   auto copy_vals = [&](double* dst, const double* s64, const float* s32, int64_t count) -> int {
-    if (s64) {
+    if (f64) {
       FE_CUDA(cudaMemcpy(dst, s64, sizeof(double) * count, cudaMemcpyDeviceToHost));
     } else {
       std::vector<float> tmp(count);

@@ -451,3 +451,22 @@ def test_lowsync_workspace_follows_its_own_restart(fe):
         m.gmres(b, restart=restart, max_it=2)
     x, y = (mesh.gmres(b, rtol=0.0, atol=0.0, restart=128, max_it=128, orthog=1)[0] for mesh in (m, ref))
     assert torch.equal(x, y)
+
+
+def test_amg_levels_follow_the_last_tangent(fe):
+    # an FP64 tangent, then a mixed one elsewhere on the same mesh: the levels
+    # are those of the second, as on a mesh that has seen nothing else
+    w = W.twist(6)
+    m, ref = fe.Mesh(w), fe.Mesh(w)
+    rng = np.random.default_rng(19)
+    a, b = (torch.from_numpy(0.002 * rng.standard_normal(m.ndof)).cuda() for _ in range(2))
+    for mesh in (m, ref):
+        mesh.set_pc("amg")
+    m.tangent(a, "fp64")
+    first = m.amg_levels()
+    m.tangent(b, "mixed_fp32")
+    ref.tangent(b, "mixed_fp32")
+    for f, g, r in zip(first, m.amg_levels(), ref.amg_levels()):
+        for k in ("val", "pval"):
+            if k in r:
+                assert np.array_equal(g[k], r[k]) and not np.array_equal(g[k], f[k]), k
