@@ -136,6 +136,7 @@ struct AmgHier {
   std::vector<void*> allocs; // device buffers owned by the hierarchy
   int64_t bytes = 0;         // their size (counted in the mesh's device bytes)
   bool ready = false;        // numbers formed for the current tangent
+  int prec = -1;             // its precision
   // the V-cycle captured as a CUDA graph, output lev[0].x; its first kernel
   // reads the caller's vector (argument `root_arg` of node `root`, set before
   // each launch)
@@ -2326,6 +2327,7 @@ int fe_amg_setup(fe_mesh m) {
   else if (m->prec == FE_PREC_MIXED_BF16) FE_TRY((numeric_all<float, __nv_bfloat16>(m, m->K16)));
   else FE_TRY((numeric_all<float, float>(m, m->K32)));
   m->amg->ready = true;
+  m->amg->prec = m->prec;
   return FE_OK;
 }
 
@@ -2416,8 +2418,8 @@ extern "C" int fe_amg_get_level(fe_mesh m, int level, int64_t* info, double* rho
   }
   if (rho) *rho = L.rho;
   // values in FP64 (widened from the FP32 numbers of the mixed forms), those of
-  // the last tangent: the arrays of another precision may be there, too
-  const bool f64 = m->prec == FE_PREC_FP64;
+  // the last setup: the arrays of another precision may be there, too
+  const bool f64 = h->prec == FE_PREC_FP64;
   auto copy_vals = [&](double* dst, const double* s64, const float* s32, int64_t count) -> int {
     if (f64) {
       FE_CUDA(cudaMemcpy(dst, s64, sizeof(double) * count, cudaMemcpyDeviceToHost));

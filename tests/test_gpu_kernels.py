@@ -470,3 +470,7 @@ def test_amg_levels_follow_the_last_tangent(fe):
         for k in ("val", "pval"):
             if k in r:
                 assert np.array_equal(g[k], r[k]) and not np.array_equal(g[k], f[k]), k
+    m.set_pc("bj")
+    m.tangent(a, "fp64")  # no hierarchy is made for this one: they stay
+    for g, r in zip(m.amg_levels(), ref.amg_levels()):
+        assert all(np.array_equal(g[k], r[k]) for k in ("val", "pval") if k in r)
