@@ -57,6 +57,7 @@ int fe_dbg_bounds_assemble(void);
 int fe_dbg_bounds_krylov(void);
 int fe_dbg_bounds_amg(void);
 int fe_dbg_bounds_batch(void);
+int fe_dbg_bounds_batch_p2(void);
 #else
 __device__ __forceinline__ int fe_idx(int i, int64_t) { return i; }
 #define FE_DBG_BOUNDS_READER(name)

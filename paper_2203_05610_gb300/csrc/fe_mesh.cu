@@ -157,7 +157,7 @@ int fe_check_device_error(fe_mesh m) {
   FE_CUDA(cudaStreamSynchronize(m->stream));
 #ifdef FE_DEBUG_BOUNDS
   if (h == DEV_OK && (fe_dbg_bounds_mesh() | fe_dbg_bounds_assemble() | fe_dbg_bounds_krylov() | fe_dbg_bounds_amg() |
-                        fe_dbg_bounds_batch()))
+                        fe_dbg_bounds_batch() | fe_dbg_bounds_batch_p2()))
     h = DEV_ERR_BOUNDS;
 #endif
   if (h == DEV_OK) return FE_OK;

@@ -37,3 +37,25 @@ def test_library_exports_every_declared_symbol():
 def test_binding_signatures_cover_the_header():
     import paper_2203_05610_gb300 as fe
     assert set(_declared()) == set(fe.SIGNATURES)
+
+
+def test_every_unit_with_index_checks_has_its_flag_read():
+    """The FE_DEBUG_BOUNDS flag is one per translation unit: each source whose
+    kernels use fe_idx defines a reader, and fe_check_device_error calls it."""
+    from paper_2203_05610_gb300 import build as B
+
+    def text(name, seen):
+        src = open(os.path.join(B.CSRC, name)).read()
+        for inc in re.findall(r'#include "(\w+\.cuh)"', src):
+            if inc not in seen:
+                seen.add(inc)
+                src += text(inc, seen)
+        return src
+    mesh = open(os.path.join(B.CSRC, "fe_mesh.cu")).read()
+    check = mesh[mesh.index("int fe_check_device_error"):]
+    check = check[: check.index("#endif")]
+    for name in B.SOURCES:
+        if "fe_idx(" in text(name, set()):
+            reader = re.search(r"^FE_DBG_BOUNDS_READER\((\w+)\)", open(os.path.join(B.CSRC, name)).read(), flags=re.M)
+            assert reader, name
+            assert reader.group(1) + "()" in check, name

@@ -40,3 +40,16 @@ def test_debug_bounds_build_runs_the_parity_subset_clean():
                        cwd=ROOT, env=env, capture_output=True, text=True, timeout=1200)
     assert r.returncode == 0, r.stdout[-4000:] + r.stderr[-2000:]
     assert " passed" in r.stdout and "failed" not in r.stdout
+
+
+def test_debug_bounds_build_runs_batches_clean():
+    """Batched solves of both orders (a translation unit each) against that build."""
+    pytest.importorskip("torch")
+    from paper_2203_05610_gb300 import build as B
+    B.build(debug_bounds=True)
+    env = dict(os.environ, FE_LIB_VARIANT="debug_bounds")
+    r = subprocess.run([sys.executable, "-m", "pytest", "-q", "-x", "-m", "gpu", "-p", "no:cacheprovider",
+                        "tests/test_gpu_batch.py::test_batch_matches_the_oracle_fp64",
+                        "tests/test_gpu_batch.py::test_batch_mixed_precision_error"],
+                       cwd=ROOT, env=env, capture_output=True, text=True, timeout=1200)
+    assert r.returncode == 0, r.stdout[-4000:] + r.stderr[-2000:]
