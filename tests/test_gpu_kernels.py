@@ -474,3 +474,92 @@ def test_amg_levels_follow_the_last_tangent(fe):
     m.tangent(a, "fp64")  # no hierarchy is made for this one: they stay
     for g, r in zip(m.amg_levels(), ref.amg_levels()):
         assert all(np.array_equal(g[k], r[k]) for k in ("val", "pval") if k in r)
+
+
+# the waits of the forms that the limit's other test does not reach:
+# compact-WY, long slices (1,644 values per block of 512 threads) and the two
+# forms beyond 6,144 values per SM (956,961 unknowns on 152 SMs)
+@pytest.mark.parametrize("size,orthog", [((24, 24, 20), 1), ((50, 50, 31), 2), ((68, 68, 66), 0), ((68, 68, 66), 2)])
+def test_bounded_waits_of_every_form(fe, size, orthog):
+    # with no polls allowed a multi-block step's waits give up, the call
+    # returns FE_ERR_TIMEOUT, and the mesh then solves as before, bit for bit
+    m = fe.Mesh(W.cook(*size, order=1, nu=0.3))
+    m.tangent(m.zeros())
+    b = torch.from_numpy(np.random.default_rng(20).standard_normal(m.ndof)).cuda()
+    args = dict(rtol=0.0, atol=0.0, restart=12, max_it=12, orthog=orthog)
+    x = m.gmres(b, **args)[0]
+    m.set_wait_limit(0)
+    with pytest.raises(fe.FEError) as e:
+        m.gmres(b, **args)
+    assert e.value.code == -4 and "wait" in str(e.value)
+    m.set_wait_limit()
+    assert torch.equal(m.gmres(b, **args)[0], x)
+
+
+def _product(ptr, col, val):
+    """x -> A x for block-CSR arrays."""
+    n, k = len(ptr) - 1, val.shape[1]
+    row = torch.from_numpy(np.repeat(np.arange(n), np.diff(ptr))).cuda()
+    col, val = torch.from_numpy(col.astype(np.int64)).cuda(), torch.from_numpy(val).cuda()
+
+    def apply(x):
+        y = torch.zeros(n, k, dtype=torch.float64, device="cuda")
+        return y.index_add_(0, row, torch.einsum("qij,qj->qi", val, x.view(n, k)[col])).view(-1)
+    return apply
+
+
+def _vcycle(levels, A0, D0, b, lv=0):
+    """The V-cycle in FP64 on the hierarchy's own numbers: degree-2 Chebyshev
+    steps in D^-1 A on [rho / 30, 1.1 rho] before and after the coarse
+    correction, the inverse on the coarsest level."""
+    L = levels[lv]
+    n, k = L["n"], L["b"]
+    if lv == 0:
+        A, D = A0, D0
+    else:
+        A = _product(L["ptr"], L["col"], L["val"])
+        row = np.repeat(np.arange(n), np.diff(L["ptr"]))
+        D = torch.linalg.inv(torch.from_numpy(L["val"][row == L["col"]]).cuda())
+    if lv == len(levels) - 1:
+        return torch.linalg.solve(torch.stack([A(c) for c in torch.eye(n * k, dtype=b.dtype, device="cuda")], 1), b)
+    lo, hi = L["rho"] / 30.0, 1.1 * L["rho"]
+    theta, delta = 0.5 * (hi + lo), 0.5 * (hi - lo)
+    r0 = delta / theta
+    r1 = 1.0 / (2.0 / r0 - r0)
+
+    def jac(r):
+        return torch.einsum("aij,aj->ai", D, r.view(n, k)).reshape(-1)
+
+    def smooth(x, r):
+        d = jac(r) / theta
+        x, r = x + d, r - A(d)
+        d = r1 * r0 * d + 2.0 * r1 / delta * jac(r)
+        return x + d, r - A(d)
+    x, r = smooth(torch.zeros_like(b), b)
+    row = torch.from_numpy(np.repeat(np.arange(n), np.diff(L["pptr"]))).cuda()
+    col, pv = torch.from_numpy(L["pcol"].astype(np.int64)).cuda(), torch.from_numpy(L["pval"]).cuda()
+    rc = torch.zeros(L["nc"], 6, dtype=torch.float64, device="cuda")
+    rc.index_add_(0, col, torch.einsum("qij,qi->qj", pv, r.view(n, k)[row]))
+    xc = _vcycle(levels, A0, D0, rc.view(-1), lv + 1).view(-1, 6)
+    e = torch.zeros_like(r).view(n, k).index_add_(0, row, torch.einsum("qij,qj->qi", pv, xc[col])).view(-1)
+    return smooth(x + e, r - A(e))[0]
+
+
+# level 0 with several windows (more than nine tiles) and several row ranges per
+# warp in both precisions, and the FP32 form of the largest meshes (16-row
+# groups that fill the wave four times: from about 233,000 nodes on 152 SMs)
+@pytest.mark.parametrize("size,precision,tol", [((48, 48, 8), "fp64", 1e-10), ((48, 48, 8), "mixed_fp32", 2e-3),
+                                                ((64, 64, 8), "mixed_fp32", 2e-3)])
+def test_vcycle_of_large_levels(fe, size, precision, tol):
+    # the reference runs in FP64 on the numbers of the device's hierarchy;
+    # bounds of the V-cycle's other tests
+    m = fe.Mesh(W.cook(*size, order=2, nu=0.3))
+    d = torch.from_numpy(0.01 * np.random.default_rng(21).standard_normal(m.ndof)).cuda()
+    m.set_pc("amg")
+    m.tangent(d, precision)
+    b = torch.from_numpy(np.random.default_rng(22).standard_normal(m.ndof)).cuda()
+    z = m.pc(b)
+    top = m.topology()
+    val, _, dinv = m.tangent_copy()
+    want = _vcycle(m.amg_levels(), _product(top["row_ptr"], top["col"], val), torch.from_numpy(dinv).cuda(), b)
+    assert (z - want).abs().max() <= tol * want.abs().max()
