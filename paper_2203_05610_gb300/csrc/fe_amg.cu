@@ -40,8 +40,8 @@
 // the block-Jacobi product and the direction and iterate updates of its
 // rows (r stays b - A x throughout, so the residual for the restriction
 // comes for free); level 0 reads the tangent in its tiled layout, coarser
-// levels their 6x6 blocks block-major with 16-byte loads.  The levels of at
-// most a few hundred nodes below level 0 run in one block (one launch
+// levels their 6x6 blocks block-major with 16-byte loads.  FP32 levels of at
+// most VC_BOTTOM_MAXNNZ blocks below level 0 run in one thread block (one launch
 // instead of seven or more latency-bound ones), and the whole V-cycle is
 // captured as one CUDA graph.
 #include <algorithm>
@@ -2107,21 +2107,27 @@ int vcycle_launches(fe_mesh m, cudaStream_t st, const V* K0, const double* b, do
   const double sv = sizeof(T), s0 = sizeof(V);
   // level 0: the scan form where its 16-row groups fill the wave four times
   // (FP32 and BF16 values; see k_vc_cheb0_scan)
-  int per_sm = 0;
-  FE_TRY(fe_kernel_occupancy((const void*)k_vc_cheb0_scan<V, T>, 256, 0, &per_sm));
-  const int64_t groups = ((int64_t)m->nn + VC_RPW - 1) / VC_RPW, wave = (int64_t)std::max(per_sm, 1) * m->sm_count;
-  const bool scan = !D && groups >= 4 * 8 * wave;
-  const unsigned grid_scan = (unsigned)wave;
+  unsigned grid_scan = 0;
+  if constexpr (!D) {
+    int per_sm = 0;
+    FE_TRY(fe_kernel_occupancy((const void*)k_vc_cheb0_scan<V, T>, 256, 0, &per_sm));
+    const int64_t groups = ((int64_t)m->nn + VC_RPW - 1) / VC_RPW, wave = (int64_t)std::max(per_sm, 1) * m->sm_count;
+    if (groups >= 4 * 8 * wave) grid_scan = (unsigned)wave;
+  }
   // Chebyshev step on level q (fused SpMV)
   auto step = [&](int q, const T* g, T* dout, double cx, int flags) -> int {
     AmgLevel& Lq = h->lev[q];
     const int B = Lq.b;
     *bytes += (double)Lq.nnz * (B * B * (q == 0 ? s0 : sv) + 4) + 4.0 * (Lq.n + 1) + (double)Lq.n * B * (sv * 5 + B * sv);
     *flops += 2.0 * Lq.nnz * B * B;
-    if (q == 0 && scan)
-      k_vc_cheb0_scan<V, T><<<grid_scan, 256, 0, st>>>(Lq.n, Lq.ptr, Lq.col, K0, dinv(0), g, X(0), (T*)Lq.r, dout,
-                                                       (T)cx, coef(0), flags);
-    else if (q == 0)
+    if constexpr (!D)
+      if (q == 0 && grid_scan) {
+        k_vc_cheb0_scan<V, T><<<grid_scan, 256, 0, st>>>(Lq.n, Lq.ptr, Lq.col, K0, dinv(0), g, X(0), (T*)Lq.r, dout,
+                                                         (T)cx, coef(0), flags);
+        FE_CUDA(cudaGetLastError());
+        return FE_OK;
+      }
+    if (q == 0)
       k_vc_cheb0<V, T><<<stream_grid(h->shape0.warps), STREAM_THREADS, 0, st>>>(
           Lq.n, h->shape0.warps, h->shape0.ranges, h->part0, Lq.ptr, Lq.col, K0, dinv(0), g, X(0), (T*)Lq.r, dout,
           (T)cx, coef(0), flags);

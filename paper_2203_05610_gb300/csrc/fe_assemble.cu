@@ -448,8 +448,6 @@ int fe_energy_dev(fe_mesh m, const double* d, double* out) {
 }
 
 // ---------------------------------------------------------------- tangent
-
-// ---------------------------------------------------------------- tangent
 // Two kernels.  k_elem_blocks64 / k_elem_blocks32 compute every element's
 // matrix once (blocks (a, b), a <= b; the tangent of a potential is symmetric)
 // into a workspace; k_gather_tangent adds, one warp per block row, the

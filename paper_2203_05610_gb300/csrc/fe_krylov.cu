@@ -478,13 +478,13 @@ __device__ __forceinline__ void arnoldi_tail(const double (&wr)[NPT], double inv
     ZT* zo = z + base + 3 * a;
     if constexpr (sizeof(DT) == 8) {
       zo[0] = (ZT)(D[0] * x0 + D[1] * x1 + D[2] * x2);
-          zo[1] = (ZT)(D[3] * x0 + D[4] * x1 + D[5] * x2);
-          zo[2] = (ZT)(D[6] * x0 + D[7] * x1 + D[8] * x2);
+      zo[1] = (ZT)(D[3] * x0 + D[4] * x1 + D[5] * x2);
+      zo[2] = (ZT)(D[6] * x0 + D[7] * x1 + D[8] * x2);
     } else {
       const float f0 = (float)x0, f1 = (float)x1, f2 = (float)x2;
       zo[0] = (ZT)(D[0] * f0 + D[1] * f1 + D[2] * f2);
-          zo[1] = (ZT)(D[3] * f0 + D[4] * f1 + D[5] * f2);
-          zo[2] = (ZT)(D[6] * f0 + D[7] * f1 + D[8] * f2);
+      zo[1] = (ZT)(D[3] * f0 + D[4] * f1 + D[5] * f2);
+      zo[2] = (ZT)(D[6] * f0 + D[7] * f1 + D[8] * f2);
     }
   }
 }
@@ -536,7 +536,7 @@ __device__ __forceinline__ void arnoldi_finish(ArnShared& sh, int j, int ng, dou
 // GB300 issues about two FP64 lane-operations per clock per SM, so a step
 // costs 2 (j+1) n / grid FP64 cycles plus its grid sums: the slice is spread
 // over every SM as soon as the vector is longer than a few hundred values
-// (launch_arnoldi_new), with only as many threads as the slice has values
+// (launch_arnoldi_reg), with only as many threads as the slice has values
 // for (idle lanes of a warp cost FP64 issue like busy ones, and so does every
 // step of a warp sum: one FP64 warp instruction holds its SM quarter 64
 // cycles, dependent or not).
@@ -1852,7 +1852,7 @@ static int xch_reserve(fe_mesh m, int sums) {
 // one with the least FP64 issue per SM quarter (the passes, and 9 steps per
 // warp for the sums).
 template <class DT, class ZT>
-static int launch_arnoldi_new(fe_mesh m, int j, int kmax, bool fuse_pc, const DT* Dinv, double target, int it0,
+static int launch_arnoldi_reg(fe_mesh m, int j, int kmax, bool fuse_pc, const DT* Dinv, double target, int it0,
                               int max_it) {
   const int64_t n = m->ndof;
   const int sms = std::min(m->sm_count, XCH_BLOCKS);
@@ -1916,24 +1916,15 @@ template <class DT, class ZT>
 static int launch_arnoldi_t(fe_mesh m, int j, int kmax, bool fuse_pc, const DT* Dinv, double target, int it0,
                             int max_it) {
   const int64_t n = m->ndof;
-  const void* fns[1] = {(const void*)k_arnoldi<24, DT, ZT>};
-  const int npts[1] = {24};
-  const int bds[1] = {256};
-  int which = -1, grid = 0;
-  {
-    const int q = 0;
-    size_t smem = (size_t)npts[q] * bds[q] * sizeof(double);
-    FE_TRY(fe_kernel_smem(fns[q], (int)smem));
-    int per_sm = 0;
-    FE_TRY(fe_kernel_occupancy(fns[q], bds[q], smem, &per_sm));
-    int64_t need = (n + (int64_t)npts[q] * bds[q] - 1) / ((int64_t)npts[q] * bds[q]);
-    if (per_sm >= 1 && need <= (int64_t)per_sm * m->sm_count && need <= RED_SLOTS) {
-      which = q;
-      grid = (int)need;
-    }
-  }
-  if (which < 0) return fe_set_error("vector too long for the persistent Arnoldi kernel (n = %lld)", (long long)n), FE_ERR_ARG;
-  size_t smem = (size_t)npts[which] * bds[which] * sizeof(double);
+  constexpr int NPT = 24, THREADS = 256;
+  const void* fn = (const void*)k_arnoldi<NPT, DT, ZT>;
+  const size_t smem = (size_t)NPT * THREADS * sizeof(double);
+  FE_TRY(fe_kernel_smem(fn, (int)smem));
+  int per_sm = 0;
+  FE_TRY(fe_kernel_occupancy(fn, THREADS, smem, &per_sm));
+  const int64_t grid = (n + NPT * THREADS - 1) / (NPT * THREADS);
+  if (grid > (int64_t)per_sm * m->sm_count || grid > RED_SLOTS)
+    return fe_set_error("vector too long for the persistent Arnoldi kernel (n = %lld)", (long long)n), FE_ERR_ARG;
   double* V = m->V;
   int64_t ldv = m->ldv;
   double* Hcol = m->H + (int64_t)j * (kmax + 1);
@@ -1952,7 +1943,7 @@ static int launch_arnoldi_t(fe_mesh m, int j, int kmax, bool fuse_pc, const DT* 
   // per entry, plus 18 per node for the fused block-Jacobi product
   FE_SCOPE_F(m, FE_PROF_ARNOLDI, 8.0 * (double)n * (j + 3) + (fuse_pc ? (double)n * (3.0 * sizeof(DT) + sizeof(ZT)) : 0.0),
              (double)n * (4.0 * (j + 1) + 3.0) + (fuse_pc ? 6.0 * n : 0.0));
-  FE_CUDA(cudaLaunchCooperativeKernel(fns[which], dim3(grid), dim3(bds[which]), args, smem, m->stream));
+  FE_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)grid), dim3(THREADS), args, smem, m->stream));
   return FE_OK;
 }
 
@@ -2075,8 +2066,8 @@ static int launch_arnoldi_bm_t(fe_mesh m, int j, int kmax, bool fuse_pc, const D
 static int launch_arnoldi(fe_mesh m, int j, int kmax, bool fuse_pc, double target, int it0, int max_it) {
   if (m->orthog != 1) {
     const int r = m->prec == FE_PREC_FP64
-                      ? launch_arnoldi_new<double, double>(m, j, kmax, fuse_pc, m->Dinv64, target, it0, max_it)
-                      : launch_arnoldi_new<float, float>(m, j, kmax, fuse_pc, m->Dinv32, target, it0, max_it);
+                      ? launch_arnoldi_reg<double, double>(m, j, kmax, fuse_pc, m->Dinv64, target, it0, max_it)
+                      : launch_arnoldi_reg<float, float>(m, j, kmax, fuse_pc, m->Dinv32, target, it0, max_it);
     if (r <= 0) return r;
   }
   if (m->orthog == 2) {
