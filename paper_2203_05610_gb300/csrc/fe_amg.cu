@@ -1667,11 +1667,13 @@ __global__ void __launch_bounds__(256) k_vc_prolong(int n, const int* __restrict
 // again, separated by block barriers.  Each stage runs the same device
 // functions as the per-level kernels, with the same assignment of rows and
 // entries to warps, lanes and 128-thread groups, so the result is identical.
-// One SM works through the blocks, so the form pays for few of them only, a
-// level of n blocks costing in the whole V-cycle, fused and as launches: 317
-// blocks 296 and 300 us, 884 blocks 72 and 71, 1,794: 80 and 68, 4,267: 122
-// and 69, 9,073: 195 and 86.  In FP64 (884: 208 and 133 us; 317: 1,022 and
-// 983) the launches win throughout.
+// One SM works through the blocks, so the form pays for few of them only.  A
+// preconditioner call whose largest fused level has n blocks, fused and as
+// launches: 257 blocks 54.1 and 57.0 us, 317: 292 and 298, 393: 67.9 and 69.0,
+// 455: 55.2 and 57.0, 521: 54.5 and 54.4, 566: 87.4 and 86.5; V-cycles alone
+// with 884: 72 and 71 us, 1,794: 80 and 68, 4,267: 122 and 69, 9,073: 195 and
+// 86.  The gain is 2 to 5% up to about 500 blocks and none to the line.  In FP64
+// (884: 208 and 133 us; 317: 1,022 and 983) the launches win throughout.
 constexpr int VC_BOTTOM_THREADS = 1024;
 constexpr int64_t VC_BOTTOM_MAXNNZ = 640;
 

@@ -10,9 +10,9 @@
 // values and the gather of x of tiles i + 1 and i + 2 and the column indices
 // of the three tiles after them are in flight.  The three products of every block
 // go to the warp's window in shared memory; when the window is full or the
-// range ends, four lanes per row add the rows' products from it (every fourth
-// place, each in order), 8 rows at a time, a row that runs on into the next
-// window carrying its sum; the rows that end there go through the epilogue
+// range ends, four lanes per row (FP32: two) add the rows' products from it
+// (every fourth or second place, each in order), 8 or 16 rows at a time, a row
+// that runs on into the next window carrying its sum; the rows that end there go through the epilogue
 // Epi, lane i on the i-th of them, with operands whose loads are in flight
 // during the sums.  Summation order is fixed by the row pointers and the
 // partition, so results are deterministic.  A range may hold no rows (a row
