@@ -218,41 +218,49 @@ __device__ __forceinline__ void grid_reduce_w0(const GridSync& gs, double* part,
 // distributed shared memory below the exchange 3.0-5.8 us, 4 to 16 copies of
 // the words against polling contention 2.1-2.4 us.
 struct XchSync {
-  ulonglong2* slots;  // [2][XCH_BLOCKS][BMGS_P]
+  uint4* slots;    // [2][XCH_BLOCKS][BMGS_P]
   unsigned* seq;   // sequence number of the next sum
   int* err;
   unsigned limit;  // polls before a wait gives up (fe_set_wait_limit)
 };
 
-__device__ __forceinline__ ulonglong2 ld_relaxed_v2(const ulonglong2* p) {
-  ulonglong2 v;
-  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+// (the words in 32-bit registers: a tag is compared as it lies there)
+__device__ __forceinline__ uint4 ld_relaxed_word(const uint4* p) {
+  uint4 v;
+  asm volatile(
+      "{ .reg .b64 a, b; ld.relaxed.gpu.global.v2.b64 {a, b}, [%4]; mov.b64 {%0, %1}, a; mov.b64 {%2, %3}, b; }"
+      : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+      : "l"(p)
+      : "memory");
   return v;
 }
-__device__ __forceinline__ void st_relaxed_v2(ulonglong2* p, ulonglong2 v) {
-  asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(v.x), "l"(v.y) : "memory");
+__device__ __forceinline__ void st_relaxed_word(uint4* p, uint4 v) {
+  asm volatile(
+      "{ .reg .b64 a, b; mov.b64 a, {%1, %2}; mov.b64 b, {%3, %4}; st.relaxed.gpu.global.v2.b64 [%0], {a, b}; }" ::"l"(p),
+      "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+      : "memory");
 }
-__device__ __forceinline__ void xch_post(ulonglong2* p, double v, unsigned tag) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(v), t = (unsigned long long)tag << 32;
-  st_relaxed_v2(p, make_ulonglong2((u & 0xffffffffull) | t, (u >> 32) | t));
+__device__ __forceinline__ void xch_post(uint4* p, double v, unsigned tag) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+  st_relaxed_word(p, make_uint4((unsigned)u, tag, (unsigned)(u >> 32), tag));
 }
 // Sum of the words idx, idx + step, ... (< cnt) of a set, in that order, once
 // each carries `tag`; up to FL polls in flight.  false: a wait ran out.
 template <int FL>
-__device__ __forceinline__ bool xch_gather(const XchSync& xs, const ulonglong2* set, int idx, int step, int cnt,
+__device__ __forceinline__ bool xch_gather(const XchSync& xs, const uint4* set, int idx, int step, int cnt,
                                            unsigned tag, double& sum) {
   sum = 0.0;
   for (; idx < cnt; idx += FL * step) {
-    ulonglong2 v[FL];
+    uint4 v[FL];
     unsigned spins = 0;
     for (;;) {
       bool all = true;
 #pragma unroll
       for (int q = 0; q < FL; q++)
-        if (idx + q * step < cnt) v[q] = ld_relaxed_v2(set + idx + q * step);
+        if (idx + q * step < cnt) v[q] = ld_relaxed_word(set + idx + q * step);
 #pragma unroll
       for (int q = 0; q < FL; q++)
-        if (idx + q * step < cnt) all = all && (unsigned)(v[q].x >> 32) == tag && (unsigned)(v[q].y >> 32) == tag;
+        if (idx + q * step < cnt) all = all && v[q].y == tag && v[q].w == tag;
       if (all) break;
       if (++spins > xs.limit || *(volatile int*)xs.err != DEV_OK) {
         atomicCAS(xs.err, DEV_OK, DEV_ERR_TIMEOUT);
@@ -262,7 +270,7 @@ __device__ __forceinline__ bool xch_gather(const XchSync& xs, const ulonglong2* 
 #pragma unroll
     for (int q = 0; q < FL; q++)
       if (idx + q * step < cnt)
-        sum += __longlong_as_double((long long)((v[q].y << 32) | (v[q].x & 0xffffffffull)));
+        sum += __longlong_as_double((long long)(((unsigned long long)v[q].z << 32) | v[q].x));
   }
   return true;
 }
@@ -317,7 +325,7 @@ __device__ __forceinline__ bool xch_reduce(const XchSync& xs, unsigned& seq, dou
                                            bool solve, int nc, bool last, Idle idle) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int G = gridDim.x;
-  ulonglong2* set = xs.slots + (size_t)(seq & 1u) * XCH_BLOCKS * BMGS_P;
+  uint4* set = xs.slots + (size_t)(seq & 1u) * XCH_BLOCKS * BMGS_P;
   double t = 0.0;
   const double r = warp_reduce_scatter<P>(loc, lane);
   if ((lane & (32 / P - 1)) == 0) sh.wpart[lane / (32 / P)][wid] = r;
@@ -1825,7 +1833,7 @@ static GridSync grid_sync(fe_mesh m) {
 
 static XchSync xch_sync(fe_mesh m) {
   XchSync xs;
-  xs.slots = (ulonglong2*)m->xch;
+  xs.slots = (uint4*)m->xch;
   xs.seq = m->bar + XCH_SEQ_WORD;
   xs.err = m->err;
   xs.limit = m->wait_limit;
