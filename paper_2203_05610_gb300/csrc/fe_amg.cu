@@ -720,30 +720,30 @@ __global__ void __launch_bounds__(256) k_amg_power(int n, const int* __restrict_
   power_finish<C>(a, ss, xx, red, last_step);
 }
 
-// The smallest levels: all 15 steps in one block, while its one SM is done
-// before 15 launches are.  The whole setup, in one block and as launches, for
-// levels of 884, 1,794 and 2,113 blocks: FP32 1.19 and 1.23, 0.98 and 0.95,
-// 1.40 and 1.35 ms; FP64 2.38 and 2.12, 2.58 and 1.93, 3.04 and 2.34 ms.
-template <class C>
-constexpr int AMG_POWER_SMALL = sizeof(C) == 4 ? 1024 : 256;  // blocks of the level
-template <class C>
+// The smallest FP32 levels: all 15 steps in one block, while its one SM is
+// done before 15 launches are.  The whole setup, in one block and as launches,
+// for levels of 144, 250, 455, 884, 1,794 and 2,113 blocks: 391 and 440 us, 443
+// and 478, 563 and 609, 663 and 696 (884 blocks of another mesh 1.19 and 1.23
+// ms), 0.98 and 0.95 ms, 1.40 and 1.35 ms.  In FP64 the launches win throughout
+// (144: 748 and 649 us, 250: 952 and 666, 884: 2.38 and 2.12 ms).
+constexpr int AMG_POWER_SMALL = 1024;  // blocks of the level
 __global__ void __launch_bounds__(512) k_amg_power_small(int n, int steps, const int* __restrict__ ptr,
-                                                         const int* __restrict__ col, Vals<C, C, AMG_NS> A,
-                                                         const C* __restrict__ dinv, C* x, C* y, PowerArgs a) {
+                                                         const int* __restrict__ col, Vals<float, float, AMG_NS> A,
+                                                         const float* __restrict__ dinv, float* x, float* y, PowerArgs a) {
   __shared__ double red[32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int it = 0; it < steps; it++) {
     const double f = ((volatile double*)a.scal)[SC_F];
-    const PowerScale<C> sc(f);
+    const PowerScale<float> sc(f);
     const bool last = it == steps - 1;
     double ss = 0.0, xx = 0.0;
     for (int row = wid; row < n; row += nw)
-      power_row<C, C, AMG_NS>(row, lane, ptr, col, A, dinv, x, y, (C)f, sc, sizeof(C) == 4 && last, ss, xx);
+      power_row<float, float, AMG_NS>(row, lane, ptr, col, A, dinv, x, y, (float)f, sc, last, ss, xx);
     ss = power_block_sum(ss, red);  // (its barriers order this step's rows before the next one's)
     xx = power_block_sum(xx, red);
-    if (threadIdx.x == 0) power_result<C>(a, ss, xx, last);
+    if (threadIdx.x == 0) power_result<float>(a, ss, xx, last);
     __syncthreads();
-    C* t = x;
+    float* t = x;
     x = y;
     y = t;
   }
@@ -1999,11 +1999,11 @@ int numeric_level(fe_mesh m, int q, const V* val) {
   k_amg_start<C><<<blocks_for(N, 256), 256, 0, m->stream>>>(N, x, scal);
   FE_CUDA(cudaGetLastError());
   bool small = false;
-  if constexpr (B == AMG_NS) {
-    if (L.nnz <= AMG_POWER_SMALL<C>) {
+  if constexpr (B == AMG_NS && sizeof(C) == 4) {
+    if (L.nnz <= AMG_POWER_SMALL) {
       small = true;
       FE_SCOPE(m, FE_PROF_OTHER, AMG_POWER_STEPS * ((double)L.nnz * (B * B * sizeof(V) + 4) + 2.0 * sizeof(C) * N));
-      k_amg_power_small<C><<<1, 512, 0, m->stream>>>(L.n, AMG_POWER_STEPS, L.ptr, L.col, A, dinv, x, y, pa);
+      k_amg_power_small<<<1, 512, 0, m->stream>>>(L.n, AMG_POWER_STEPS, L.ptr, L.col, A, dinv, x, y, pa);
       FE_CUDA(cudaGetLastError());
     }
   }
